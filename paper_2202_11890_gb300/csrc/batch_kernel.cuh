@@ -1,10 +1,5 @@
 // batch_kernel.cuh — the persistent batch kernel (device code). Included by
-// mprk_kernels.cu only: the FP64 tile body is a non-inlined template, and
-// a translation unit compiles its own copy of each instantiation it uses.
-// With the batch kernel in the same unit as the single-instance stage
-// kernel, both call one compiled copy, so an instance gives bitwise the
-// same result alone and in a batch (two copies were seen to contract
-// floating-point operations differently with the general bases).
+// mprk_kernels.cu only.
 //
 // Work items (instance, stage, a run of consecutive tiles) are listed
 // stage-major; see mprk_batch.cu for the list, the dependencies and the
@@ -66,6 +61,17 @@ __device__ __noinline__ void batch_tile_mixed(const StageArgs& a, int tile, Mixe
   stage_tile_mixed<PAR>(a, tile, S);
 }
 
+// The FP64 tile of a work item: dynamic shared memory holds the item's stage
+// arguments, then the tile. A function of its own, so that the persistent
+// loop's state does not add to the tile's registers.
+constexpr int BATCH_ARGS_BYTES = (int)((sizeof(StageArgs) + 127) / 128 * 128);
+template <bool GEN, int ROWS>
+__device__ __noinline__ void batch_tile_fp64(int tile) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  stage_tile<GEN, NTHREADS, ROWS>(*reinterpret_cast<const StageArgs*>(smem_raw), tile,
+                                  *reinterpret_cast<TileSmem<ROWS>*>(smem_raw + BATCH_ARGS_BYTES));
+}
+
 // three CTAs per SM in both precisions (80 and 72 registers; the FP32-flux
 // form spills some, and still runs faster than at two CTAs). ROWS: rows of
 // the FP64 tile, TZ (one thread per cell) or TZ / 2 (two threads per cell);
@@ -81,7 +87,8 @@ __global__ void __launch_bounds__(batch_threads(PREC), 3) batch_kernel(const Bat
   __shared__ int s_ok;
   // the item's stage arguments, one copy for the CTA: the tile reads its
   // launch constants from shared memory instead of a per-thread local copy
-  __shared__ __align__(16) StageArgs s_a;
+  __shared__ __align__(16) unsigned char s_args[PREC == 0 ? 16 : sizeof(StageArgs)];
+  StageArgs& s_a = *reinterpret_cast<StageArgs*>(PREC == 0 ? smem_raw : s_args);
   cuda::atomic_ref<int, cuda::thread_scope_device> nxt(*A.next);
   if (threadIdx.x == 0) s_item[0] = nxt.fetch_add(1, cuda::memory_order_relaxed);
   __syncthreads();
@@ -108,11 +115,9 @@ __global__ void __launch_bounds__(batch_threads(PREC), 3) batch_kernel(const Bat
         for (int t = 0; t < item.count; t++) {
           if (t > 0) __syncthreads();  // the previous tile is done with shared memory
           if (PREC == 0 && s_a.g.gen)  // a general s-stage base (RK3, RK4)
-            stage_tile<double, double, true, NTHREADS, ROWS>(s_a, item.tile + t,
-                                                             *reinterpret_cast<TileSmem<double, ROWS>*>(smem_raw));
+            batch_tile_fp64<true, ROWS>(item.tile + t);
           else if (PREC == 0)
-            stage_tile<double, double, false, NTHREADS, ROWS>(s_a, item.tile + t,
-                                                              *reinterpret_cast<TileSmem<double, ROWS>*>(smem_raw));
+            batch_tile_fp64<false, ROWS>(item.tile + t);
           else if (s_a.stage & 1)  // the FP32-flux tile compiled per stage parity
             batch_tile_mixed<1>(s_a, item.tile + t, *reinterpret_cast<MixedTileSmem*>(smem_raw));
           else

@@ -43,6 +43,30 @@ constexpr unsigned ST_NONFINITE = 1u;
 constexpr unsigned ST_CFL = 2u;
 constexpr unsigned ST_TIMEOUT = 4u;
 
+// A factor of a fixed-point product, hi 2^32 + lo with lo signed (fixed_point.cuh).
+struct FxW {
+  int lo, hi;
+};
+// Coefficients of the viscous face flux over half the divergence factor.
+enum {
+  FXC_A,  // (8/3) mu / d_n: sigma_nn from the normal difference of u_n
+  FXC_B,  // -mu / (3 d_t): sigma_nn from the two cells' tangential differences of u_t
+  FXC_C,  // 2 mu / d_n: sigma_nt from the normal difference of u_t
+  FXC_D,  // mu / (2 d_t): sigma_nt from the two cells' tangential differences of u_n
+  FXC_K,  // 2 kappa gamma (gamma - 1) / d_n: heat flux from the difference of e
+  FXC_N
+};
+
+// Fixed-point constants of the FP64 tile's face fluxes (fixed_point.cuh).
+struct FxConst {
+  int on;              // every factor below fits its scale: the fluxes run in fixed point
+  int square;          // dx = dz1 = dz2: x and z differences add before the scaling
+  double scale;        // their factor: 2^-57 of half of 1/dx
+  FxW gm1;             // (gamma - 1).61
+  FxW gg;              // gamma (gamma - 1).62
+  FxW fc[2][2][FXC_N]; // viscous coefficients per direction (x, z) and fluid, .62
+};
+
 // Physics and grid of one instance, constant over its life.
 struct Geom {
   int nx, pitch, nz;
@@ -112,11 +136,28 @@ struct StageArgs {
   int bulk;           // FP32-flux: interior tiles stage their float planes by
                       // tensor copies (set by launch_stage when maps exist)
   unsigned* status;   // status word for device-side errors, or null
+  FxConst fx;         // FP64, 2-D
 };
+
+// The viscous coefficient j of direction dir (0 x, 1 z) in fluid fl (0, 1),
+// over half the divergence factor 1/d_n of the direction.
+__host__ __device__ inline double visc_coef(const Geom& g, int dir, int fl, int j) {
+  const double iz = fl ? g.inv_dz2 : g.inv_dz1, mu = fl ? g.mu2 : g.mu1;
+  const double in = dir ? iz : g.inv_dx, it = dir ? g.inv_dx : iz;
+  switch (j) {
+    case FXC_A: return 8.0 / 3.0 * mu * in;
+    case FXC_B: return -mu * it / 3.0;
+    case FXC_C: return 2.0 * mu * in;
+    case FXC_D: return 0.5 * mu * it;
+    default: return 2.0 * (fl ? g.kap2 : g.kap1) * g.gamma * g.gm1 * in;
+  }
+}
+// Fills the fixed-point constants of a geometry (mprk_runtime.cu).
+void fixed_point_const(const Geom& g, FxConst* out);
 
 // Arguments of stage st of one slow step: F rows ping-pong between the A and
 // B buffers at every fast substep.
-__host__ __device__ inline StageArgs stage_args(const Geom& g, const Bufs& b, int st) {
+inline StageArgs stage_args(const Geom& g, const Bufs& b, int st) {
   StageArgs a{};
   a.g = g;
   a.b = b;
@@ -129,6 +170,7 @@ __host__ __device__ inline StageArgs stage_args(const Geom& g, const Bufs& b, in
   a.row0 = st < g.s ? 0 : g.nS_r;  // S rows only during the first substep
   a.tiles_x = (g.nx + TX - 1) / TX;
   a.tz = b.dA ? MTZ : TZ;  // float shadows exist only in the FP32-flux mode
+  if (!b.dA && g.ny == 1) fixed_point_const(g, &a.fx);
   return a;
 }
 __host__ __device__ inline int stage_tiles(const StageArgs& a) {

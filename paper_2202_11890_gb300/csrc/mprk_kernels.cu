@@ -27,12 +27,12 @@ namespace mprk {
 // thread per cell: 80 registers, a few spilled in the tile (three 32 x 8
 // CTAs per SM). NT = 2 TX TZR: two threads per cell for launches with no
 // more tiles than SMs.
-template <typename Real, typename Store, bool GEN = false, int NT = NTHREADS, int TZR = TZ>
+template <bool GEN = false, int NT = NTHREADS, int TZR = TZ>
 __global__ void __launch_bounds__(NT, NT == TX * TZR ? 3 * NTHREADS / NT : 1)
-    stage_kernel(const StageArgs a) {
+    stage_kernel(const __grid_constant__ StageArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  TileSmem<Real, TZR>& S = *reinterpret_cast<TileSmem<Real, TZR>*>(smem_raw);
-  stage_tile<Real, Store, GEN, NT, TZR>(a, blockIdx.x, S);
+  TileSmem<TZR>& S = *reinterpret_cast<TileSmem<TZR>*>(smem_raw);
+  stage_tile<GEN, NT, TZR>(a, blockIdx.x, S);
 }
 
 // FP32-flux stage kernel: one CTA per tile, blockIdx = (tile column, tile
@@ -86,22 +86,22 @@ cudaError_t launch_stage3(const StageArgs& a, cudaStream_t stream) {
 }
 
 size_t stage_smem_bytes(int precision) {
-  return precision == 0 ? sizeof(TileSmem<double>) : sizeof(MixedTileSmem);
+  return precision == 0 ? BATCH_ARGS_BYTES + sizeof(TileSmem<>) : sizeof(MixedTileSmem);
 }
 
 cudaError_t prepare_kernels() {
-  cudaError_t e = cudaFuncSetAttribute(stage_kernel<double, double>,
+  cudaError_t e = cudaFuncSetAttribute(stage_kernel<>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sizeof(TileSmem<double>));
+                                       (int)sizeof(TileSmem<>));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(stage_kernel<double, double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sizeof(TileSmem<double>));
+  e = cudaFuncSetAttribute(stage_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)sizeof(TileSmem<>));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(stage_kernel<double, double, false, 2 * NTHREADS>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem<double>));
+  e = cudaFuncSetAttribute(stage_kernel<false, 2 * NTHREADS>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem<>));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(stage_kernel<double, double, true, 2 * NTHREADS>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem<double>));
+  e = cudaFuncSetAttribute(stage_kernel<true, 2 * NTHREADS>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem<>));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(yface3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(YfaceSmem));
   if (e != cudaSuccess) return e;
@@ -176,15 +176,15 @@ namespace {
 template <int TZR>
 void launch_fp64(const StageArgs& a, int n_tiles, bool wide, cudaStream_t stream) {
   constexpr int NT1 = TX * TZR, NT2 = 2 * TX * TZR;
-  const size_t smem = sizeof(TileSmem<double, TZR>);
+  const size_t smem = sizeof(TileSmem<TZR>);
   if (wide && a.g.gen)
-    stage_kernel<double, double, true, NT2, TZR><<<n_tiles, NT2, smem, stream>>>(a);
+    stage_kernel<true, NT2, TZR><<<n_tiles, NT2, smem, stream>>>(a);
   else if (wide)
-    stage_kernel<double, double, false, NT2, TZR><<<n_tiles, NT2, smem, stream>>>(a);
+    stage_kernel<false, NT2, TZR><<<n_tiles, NT2, smem, stream>>>(a);
   else if (a.g.gen)
-    stage_kernel<double, double, true, NT1, TZR><<<n_tiles, NT1, smem, stream>>>(a);
+    stage_kernel<true, NT1, TZR><<<n_tiles, NT1, smem, stream>>>(a);
   else
-    stage_kernel<double, double, false, NT1, TZR><<<n_tiles, NT1, smem, stream>>>(a);
+    stage_kernel<false, NT1, TZR><<<n_tiles, NT1, smem, stream>>>(a);
 }
 }  // namespace
 

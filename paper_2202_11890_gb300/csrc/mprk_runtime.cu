@@ -320,6 +320,36 @@ static void set_base(int base, Geom* g) {
   g->gen = base != MPRK_BASE_RK2;
 }
 
+// The fixed-point form needs gamma (gamma - 1) < 1.9 and every viscous
+// coefficient (the inverse of a cell Reynolds number; 0.1 at 2048 columns)
+// below 1, so that each fits its scale with a bit to spare; otherwise the
+// tile's faces run in double.
+void mprk::fixed_point_const(const Geom& g, FxConst* out) {
+  auto factor = [](double x, int digits) {
+    const long long v = llround(ldexp(x, digits));
+    FxW w;
+    w.lo = (int)(unsigned)(v & 0xffffffffll);
+    w.hi = (int)((v - w.lo) >> 32);
+    return w;
+  };
+  FxConst& f = *out;
+  f = FxConst{};
+  f.square = g.inv_dx == g.inv_dz1 && g.inv_dx == g.inv_dz2;
+  f.scale = ldexp(0.5 * g.inv_dx, -57);
+  const double gg = g.gamma * g.gm1;
+  if (!(gg < 1.9)) return;
+  for (int dir = 0; dir < 2; dir++)
+    for (int fl = 0; fl < 2; fl++)
+      for (int j = 0; j < FXC_N; j++) {
+        const double x = visc_coef(g, dir, fl, j);
+        if (!(std::fabs(x) < 1.0)) return;
+        f.fc[dir][fl][j] = factor(x, 62);
+      }
+  f.gm1 = factor(g.gm1, 61);
+  f.gg = factor(gg, 62);
+  f.on = 1;
+}
+
 void mprk::geom_from_config(const mprk_config& c, int pitch, Geom* gp) {
   Geom& g = *gp;
   memset(&g, 0, sizeof g);

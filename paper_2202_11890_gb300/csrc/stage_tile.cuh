@@ -1,116 +1,94 @@
 // stage_tile.cuh — the fused right-hand-side + stage-combination tile of one
-// MPRK2 stage (device code; included by the kernel translation units).
+// MPRK2 stage in FP64 (device code; included by the kernel translation units).
 //
-// One CTA of TX x TZR threads owns a TX x TZR tile of cells (TZR = TZ rows,
-// or TZ/2 or TZ/4 for launches of few tiles). It
+// One CTA owns a TX x TZR tile of cells (TZR = TZ rows, or TZ/2 or TZ/4 for
+// launches of few tiles). It
 //   1. stages the stage state of the tile plus a two-cell halo in shared
-//      memory (x periodic; stage values q + h R_a rebuilt on the fly),
-//   2. computes u, w, T on the tile plus a one-cell ring, and the interface
-//      state (bulk fluxes and wall states of App. B) when the tile touches it,
-//   3. computes the cell slopes: central differences of the conserved
-//      variables (reconstruction) and of u, w (tangential viscous gradients),
-//      with mirror or wall-state ghosts beyond walls and the interface; the
-//      differences are stored unscaled and their factors (1/4 for the
-//      reconstruction, 1/(2 d) for a derivative) taken up where they are used,
+//      memory (x periodic; stage values q + h R_a rebuilt on the fly in
+//      double), as doubles and as 64-bit fixed point,
+//   2. computes u, w and e = T / (gamma (gamma - 1)) on the tile plus a
+//      one-cell ring, and the interface state (bulk fluxes and wall states of
+//      App. B) when the tile touches it,
+//   3. computes the central differences of u, w along the faces (tangential
+//      viscous gradients), with wall-state ghosts beyond walls and the
+//      interface,
 //   4. computes every x and z face flux of the tile once (Lax–Friedrichs
-//      inviscid flux of Sec. 2.1 minus the common-value viscous flux of
-//      App. B), in one direction-generic routine written in the face frame;
-//      each flux comes out multiplied by the 1/dx or 1/dz of the divergence,
+//      inviscid flux of Sec. 2.1 on the linear reconstruction of the
+//      conserved variables, minus the common-value viscous flux of App. B),
+//      in one direction-generic routine written in the face frame,
 //   5. forms R = -div F* + s per cell and applies the partition's stage
 //      combination (Eq. MRK2 in low-storage form) in double precision.
 //
-// Real is the arithmetic type of steps 1-5 up to R (double, or float in the
-// FP32-flux mode); Store is the type of the saved stage-one right-hand side.
+// Phases 2 to 4 run in 64-bit fixed point (fixed_point.cuh): as double
+// arithmetic they were 300 of the tile's 309 operations per cell on a pipe
+// that completes two per clock and SM, which bound every FP64 launch: the
+// pipe was 86 % busy. Measured: a slow step of 2048 x 1024 cells with m = 8
+// 11.74 -> 2.36 ms (B and F rows of one stage 649 -> 129 to 141 us), 64 x 64
+// with m = 4 165 -> 86 us. Errors of the right-hand side against 80-bit
+// arithmetic fell from 3e-16..1e-15 to 2e-17..5e-16 (rms per component; rest
+// state with 1 % bumps to 25 % cell noise). A face
+// with a state outside the fixed-point range takes the same formulas in
+// double (slow_faces); which form a face takes depends on its own cells
+// alone, so results do not depend on the tile shape or the launch.
 #pragma once
 
+#include "fixed_point.cuh"
 #include "fp64_recip.cuh"
 #include "mprk_internal.h"
 
 namespace mprk {
 
-// Face constants of one face direction in one fluid (scaled by the divergence
-// factor sc = 1/dx at x faces, 1/dz of the fluid at z faces; d_n and d_t are
-// the spacings normal and tangential to the face).
-enum {
-  FC_HS,  // sc / 2: the averages of the Lax–Friedrichs flux
-  FC_A,   // (4/3) mu sc / d_n: sigma_nn from the normal difference of u_n
-  FC_B,   // mu sc / (6 d_t): sigma_nn from the two cells' tangential differences of u_t
-  FC_C,   // mu sc / d_n: sigma_nt from the normal difference of u_t
-  FC_D,   // mu sc / (4 d_t): sigma_nt from the two cells' tangential differences of u_n
-  FC_K,   // kappa gamma (gamma - 1) sc / d_n: heat flux from the normal difference of e = T / (gamma (gamma - 1))
-  FC_SC,  // sc
-  FC_N
-};
+using fx::i64;
 
-template <typename Real, int TZR = TZ>
+template <int TZR = TZ>
 struct TileSmem {
-  Real q[4][TZR + 4][TX + 4];   // stage state, rows k0-2.., cols i0-2..
-  Real v[3][TZR + 2][TX + 2];   // u, w, e = T / (gamma (gamma - 1)), rows k0-1.., cols i0-1..
-  Real hx[4][TZR][TX + 2];      // central x differences of q, cols i0-1..
-  Real hz[4][TZR + 2][TX];      // central z differences of q, rows k0-1..
-  Real tz[2][TZR][TX + 2];      // central z differences of u, w (tangential at x faces)
-  Real tx[2][TZR + 2][TX];      // central x differences of u, w (tangential at z faces)
-  Real fx[4][TZR][TX + 1];      // x face fluxes / dx, face f between cols f-1, f
-  Real fz[4][TZR + 1][TX];      // z face fluxes / dz seen from above
-  Real fg[4][TX];              // interface flux / dz1 seen from fluid 1 (below)
-  double gam[4][TX + 2];       // sigma_xz, Pi_z, u_w, T_w per column i0-1..
-  Real fc[2][2][FC_N];         // face constants per direction (x, z) and fluid (1, 2)
+  static constexpr int NZF = (TZR + 1) * TX, NXF = TZR * (TX + 1);  // z and x faces
+  double q[4][TZR + 4][TX + 4];  // stage state, rows k0-2.., cols i0-2..
+  i64 qi[4][TZR + 4][TX + 4];    // the same: rho, rho E .58, momenta .60
+  i64 v[3][TZR + 2][TX + 2];     // u, w, e (.59), rows k0-1.., cols i0-1..
+  i64 tz[2][TZR][TX + 2];        // central z differences of u, w (tangential at x faces)
+  i64 tx[2][TZR + 2][TX];        // central x differences of u, w (tangential at z faces)
+  // face fluxes over half the divergence factor (.57; a slow face's as the
+  // bits of a double)
+  i64 fx[4][TZR][TX + 1];  // face f between cols f-1, f
+  i64 fz[4][TZR + 1][TX];  // seen from above at the interface
+  i64 fg[4][TX];           // the interface seen from fluid 1 (below)
+  double gam[3][TX + 2];   // sigma_xz, Pi_z, u_w per column i0-1..
+  i64 gam_fx[3][TX + 2];   // 2 u_w .59, 2 sigma_xz .57, 2 (u_w sigma_xz - Pi_z) .57
+  double fc[2][2][FXC_N];  // viscous coefficients of the double pass
+  unsigned char gam_ok[TX + 2];
+  unsigned char slow[NZF + NXF + TX];  // per face: z, x, interface from below
 };
 
-template <typename Real>
-__device__ __forceinline__ Real rsq(Real x);
-template <>
-__device__ __forceinline__ double rsq<double>(double x) { return rsqrt_f64(x); }
-template <>
-__device__ __forceinline__ float rsq<float>(float x) { return rsqrtf(x); }
-
-template <typename Real>
-__device__ __forceinline__ Real sqr(Real x);
-template <>
-__device__ __forceinline__ double sqr<double>(double x) { return sqrt_f64(x); }
-template <>
-__device__ __forceinline__ float sqr<float>(float x) { return x * rsqrtf(x); }
-
-template <typename Real>
-__device__ __forceinline__ Real rcp(Real x);
-template <>
-__device__ __forceinline__ double rcp<double>(double x) { return recip_f64(x); }
-template <>
-__device__ __forceinline__ float rcp<float>(float x) { return 1.0f / x; }
-
-// Lax–Friedrichs flux in the face frame. A state is (rho, m_n, m_t, rho E):
-// m_n is the momentum along the face normal, m_t along the face. Output is
-// sc (F_rho, F_mn, F_mt, F_E) - sub, where hs = sc/2 and each component is
-// hs (f(q_L) + f(q_R) + lambda (q_L - q_R)) - sub: sub carries the viscous
-// or interface part of the face flux, taken off in the last fused
-// multiply-add. lambda is the largest |u_n| + a over the left, right and
-// Roe-averaged states (Sec. 2.1); the Roe weights sqrt(rho)/(sqrt(rho_L) +
-// sqrt(rho_R)) times the enthalpy H = (rho E + p)/rho are formed as
-// (rho E + p)/sqrt(rho).
-template <typename Real>
-__device__ __forceinline__ void lf_face(Real lr, Real lmn, Real lmt, Real lE, Real rr, Real rmn,
-                                        Real rmt, Real rE, Real gamma, Real gm1, Real hs, const Real sub[4],
-                                        Real out[4]) {
-  const Real half = Real(0.5);
-  const Real rsL = rsq(lr), rsR = rsq(rr);
-  const Real invL = rsL * rsL, invR = rsR * rsR;
-  const Real sL = lr * rsL, sR = rr * rsR;  // sqrt(rho)
-  const Real unL = lmn * invL, utL = lmt * invL;
-  const Real unR = rmn * invR, utR = rmt * invR;
-  const Real pL = gm1 * (lE - half * (lmn * unL + lmt * utL));
-  const Real pR = gm1 * (rE - half * (rmn * unR + rmt * utR));
-  const Real cL = sqr(gamma * pL * invL), cR = sqr(gamma * pR * invR);
-  const Real eL = lE + pL, eR = rE + pR;
-  const Real den = rcp(sL + sR);
-  const Real un = (sL * unL + sR * unR) * den;
-  const Real ut = (sL * utL + sR * utR) * den;
-  const Real H = (eL * rsL + eR * rsR) * den;
-  const Real c = sqr(gm1 * (H - half * (un * un + ut * ut)));
-  const Real lam = max_speed(max_speed(fabs(unL) + cL, fabs(unR) + cR), fabs(un) + c);
-  out[0] = hs * fma(lam, lr - rr, lmn + rmn) - sub[0];
-  out[1] = fma(hs, fma(lam, lmn - rmn, (lmn * unL + pL) + (rmn * unR + pR)), -sub[1]);
-  out[2] = fma(hs, fma(lam, lmt - rmt, lmt * unL + rmt * unR), -sub[2]);
-  out[3] = fma(hs, fma(lam, lE - rE, unL * eL + unR * eR), -sub[3]);
+// Lax–Friedrichs flux in the face frame, in double (faces outside the
+// fixed-point range). A state is (rho, m_n, m_t, rho E): m_n is the momentum
+// along the face normal, m_t along the face. Output is f(q_L) + f(q_R) +
+// lambda (q_L - q_R) - sub: sub carries the viscous or interface part.
+// lambda is the largest |u_n| + a over the left, right and Roe-averaged
+// states (Sec. 2.1); the Roe weights sqrt(rho)/(sqrt(rho_L) + sqrt(rho_R))
+// times the enthalpy H = (rho E + p)/rho are formed as (rho E + p)/sqrt(rho).
+__device__ __forceinline__ void lf_face(double lr, double lmn, double lmt, double lE, double rr, double rmn, double rmt,
+                                        double rE, double gamma, double gm1, const double sub[4], double out[4]) {
+  const double rsL = rsqrt_f64(lr), rsR = rsqrt_f64(rr);
+  const double invL = __dmul_rn(rsL, rsL), invR = __dmul_rn(rsR, rsR);
+  const double sL = __dmul_rn(lr, rsL), sR = __dmul_rn(rr, rsR);  // sqrt(rho)
+  const double unL = __dmul_rn(lmn, invL), utL = __dmul_rn(lmt, invL);
+  const double unR = __dmul_rn(rmn, invR), utR = __dmul_rn(rmt, invR);
+  const double kL = __fma_rn(lmt, utL, __dmul_rn(lmn, unL)), kR = __fma_rn(rmt, utR, __dmul_rn(rmn, unR));
+  const double pL = __dmul_rn(gm1, __fma_rn(-0.5, kL, lE)), pR = __dmul_rn(gm1, __fma_rn(-0.5, kR, rE));
+  const double cL = sqrt_f64(__dmul_rn(__dmul_rn(gamma, pL), invL));
+  const double cR = sqrt_f64(__dmul_rn(__dmul_rn(gamma, pR), invR));
+  const double eL = __dadd_rn(lE, pL), eR = __dadd_rn(rE, pR);
+  const double den = recip_f64(__dadd_rn(sL, sR));
+  const double un = __dmul_rn(__fma_rn(sR, unR, __dmul_rn(sL, unL)), den);
+  const double ut = __dmul_rn(__fma_rn(sR, utR, __dmul_rn(sL, utL)), den);
+  const double H = __dmul_rn(__fma_rn(eR, rsR, __dmul_rn(eL, rsL)), den);
+  const double c = sqrt_f64(__dmul_rn(gm1, __fma_rn(-0.5, __fma_rn(ut, ut, __dmul_rn(un, un)), H)));
+  const double lam = max_speed(max_speed(__dadd_rn(fabs(unL), cL), __dadd_rn(fabs(unR), cR)), __dadd_rn(fabs(un), c));
+  out[0] = __dsub_rn(__fma_rn(lam, __dsub_rn(lr, rr), __dadd_rn(lmn, rmn)), sub[0]);
+  out[1] = __dsub_rn(__fma_rn(lam, __dsub_rn(lmn, rmn), __dadd_rn(__fma_rn(lmn, unL, pL), __fma_rn(rmn, unR, pR))), sub[1]);
+  out[2] = __dsub_rn(__fma_rn(lam, __dsub_rn(lmt, rmt), __fma_rn(rmt, unR, __dmul_rn(lmt, unL))), sub[2]);
+  out[3] = __dsub_rn(__fma_rn(lam, __dsub_rn(lE, rE), __fma_rn(unR, eR, __dmul_rn(unL, eL))), sub[3]);
 }
 
 // Viscous flux in the face frame from the common values of App. B: face
@@ -134,25 +112,6 @@ __device__ __forceinline__ void visc_face(Real unL, Real utL, Real TL, Real gnL,
   out[1] = snn;
   out[2] = snt;
   out[3] = un * snn + ut * snt + kap * dn_T;
-}
-
-// visc_face with the spacings, viscosity and divergence factor folded into
-// the face constants fc (FC_*): the tangential inputs gn, gt are the cells'
-// unscaled central differences of u_n, u_t along the face, and TL, TR the
-// cells' temperatures in the units of fc[FC_K] (the tile passes e = T /
-// (gamma (gamma - 1)) and folds that factor into FC_K). Output
-// sc (0, sigma_nn, sigma_nt, u.sigma_n + kappa dT/dn); the same sums as
-// visc_face, regrouped.
-template <typename Real>
-__device__ __forceinline__ void visc_face_fc(Real unL, Real utL, Real TL, Real gnL, Real gtL, Real unR,
-                                             Real utR, Real TR, Real gnR, Real gtR, const Real* fc,
-                                             Real out[4]) {
-  const Real snn = fc[FC_A] * (unR - unL) - fc[FC_B] * (gtL + gtR);
-  const Real snt = fc[FC_C] * (utR - utL) + fc[FC_D] * (gnL + gnR);
-  out[0] = Real(0);
-  out[1] = snn;
-  out[2] = snt;
-  out[3] = Real(0.5) * ((unL + unR) * snn + (utL + utR) * snt) + fc[FC_K] * (TR - TL);
 }
 
 __device__ __forceinline__ int wrap_col(int i, int nx) {
@@ -182,10 +141,6 @@ __device__ __forceinline__ int halo_col(int i, int nx, int xwall, bool* ghost) {
 // Is halo column i an x-wall ghost?
 __device__ __forceinline__ bool x_ghost(int i, int nx, int xwall) { return xwall && (i < 0 || i >= nx); }
 
-// The tile body. tile = linear tile index within the launch's row range.
-// Not inlined: the single-instance kernel and the persistent batch kernel
-// then run the very same compiled body, so an instance's results are bitwise
-// the same alone and in a batch.
 // The stage value of a general s-stage base (GEN): base + h sum_{q<p}
 // A_pq R_q over the R_a slots of the current substep (slot q at
 // Ra + q * slot); p = 0 gives the base value. Every product-sum is an
@@ -208,6 +163,394 @@ __device__ __forceinline__ double gen_weighted_sum(const Geom& g, const double* 
   return __fma_rn(g.bb[g.s - 1], r, sum);
 }
 
+// The stage state lies inside the fixed-point range (fixed_point.cuh)?
+// NaN, zero and negative densities and energies do not.
+__device__ __forceinline__ bool cell_in_range(double r, double mu, double mw, double E) {
+  const unsigned hr = (unsigned)__double2hiint(r), he = (unsigned)__double2hiint(E);
+  const unsigned hm = max((unsigned)__double2hiint(mu) & 0x7fffffffu, (unsigned)__double2hiint(mw) & 0x7fffffffu);
+  return hr - fx::RHO_LO < fx::RHO_HI - fx::RHO_LO && he - fx::E_LO < fx::E_HI - fx::E_LO && hm < fx::MOM_HI;
+}
+
+// Cell values of the two arithmetics: i64 (fixed point) or double.
+template <typename T>
+struct Arith;
+template <>
+struct Arith<i64> {
+  template <int TZR>
+  static __device__ __forceinline__ const i64* q(const TileSmem<TZR>& S) { return &S.qi[0][0][0]; }
+  // q + (upper - lower neighbour) / 4
+  static __device__ __forceinline__ i64 rec(i64 a, i64 up, i64 dn) { return (a << 2) + (up - dn); }
+  // u, w, e of a cell
+  static __device__ __forceinline__ void prims(i64 r, i64 mu, i64 mw, i64 E, i64 out[3]) {
+    const FxW inv = fx::split(fx::recip(r << 2));
+    const FxW m1 = fx::split(mu << 2), m2 = fx::split(mw << 2);
+    out[0] = fx::mul(m1, inv);
+    out[1] = fx::mul(m2, inv);
+    const i64 k = fx::mul(m1, fx::split(out[0])) + fx::mul(m2, fx::split(out[1]));  // .57; k/2 is .58
+    out[2] = fx::mul(fx::split((E - k) << 2), inv) << 2;
+  }
+};
+template <>
+struct Arith<double> {
+  template <int TZR>
+  static __device__ __forceinline__ const double* q(const TileSmem<TZR>& S) { return &S.q[0][0][0]; }
+  static __device__ __forceinline__ double rec(double a, double up, double dn) { return __fma_rn(0.25, __dsub_rn(up, dn), a);
+  }
+  static __device__ __forceinline__ void prims(double r, double mu, double mw, double E, double out[3]) {
+    const double inv = recip_f64(r);
+    out[0] = __dmul_rn(mu, inv);
+    out[1] = __dmul_rn(mw, inv);
+    out[2] = __dmul_rn(__fma_rn(-0.5, __fma_rn(mw, out[1], __dmul_rn(mu, out[0])), E), inv);
+  }
+};
+
+// ---- phase 2: u, w, e on the one-cell ring ---------------------------------
+template <typename T, int NT, int TZR>
+__device__ __forceinline__ void ring_phase(const Geom& g, TileSmem<TZR>& S, int k0, int i0) {
+  T* v = reinterpret_cast<T*>(&S.v[0][0][0]);
+  const T* q = Arith<T>::q(S);
+  constexpr int QP = (TZR + 4) * (TX + 4), VP = (TZR + 2) * (TX + 2);
+  for (int e = threadIdx.x; e < VP; e += NT) {
+    const int rr = e / (TX + 2), cc = e - rr * (TX + 2);
+    const int k = k0 - 1 + rr;
+    if (k < 0 || k >= g.nz) continue;
+    const T* p = q + (rr + 1) * (TX + 4) + cc + 1;
+    T o[3];
+    Arith<T>::prims(p[0], p[QP], p[2 * QP], p[3 * QP], o);
+    v[e] = o[0];
+    // the mirror state's u is already flipped; a no-slip x wall flips w too
+    v[VP + e] = (x_ghost(i0 - 1 + cc, g.nx, g.xwall) && g.wall == 0) ? -o[1] : o[1];
+    v[2 * VP + e] = o[2];
+  }
+}
+
+// ---- phase 3: central differences of u, w along the faces ------------------
+template <typename T>
+__device__ __forceinline__ T lid_u2(double uw, i64 uw_fx);  // 2 u_w
+template <>
+__device__ __forceinline__ i64 lid_u2<i64>(double, i64 uw_fx) { return uw_fx; }
+template <>
+__device__ __forceinline__ double lid_u2<double>(double uw, i64) { return __dmul_rn(2.0, uw); }
+
+template <typename T, int NT, int TZR>
+__device__ __forceinline__ void diff_phase(const Geom& g, TileSmem<TZR>& S, int k0, int row_hi) {
+  const T* v = reinterpret_cast<const T*>(&S.v[0][0][0]);
+  T* tz = reinterpret_cast<T*>(&S.tz[0][0][0]);
+  T* tx = reinterpret_cast<T*>(&S.tx[0][0][0]);
+  constexpr int VP = (TZR + 2) * (TX + 2), ZP = TZR * (TX + 2), XP = (TZR + 2) * TX;
+  for (int e = threadIdx.x; e < ZP + XP; e += NT) {
+    if (e < ZP) {
+      const int rr = e / (TX + 2), cc = e - rr * (TX + 2), k = k0 + rr;
+      if (k >= row_hi) continue;
+      const T* p = v + (rr + 1) * (TX + 2) + cc;
+      const T u = p[0], w = p[VP];
+      T uu, wu, ud, wd;  // values above and below, or their ghosts
+      if (k + 1 == g.nz) { uu = g.wall ? u : -u; wu = -w; }
+      else if (k + 1 == g.n1) { uu = lid_u2<T>(S.gam[2][cc], S.gam_fx[0][cc]) - u; wu = -w; }
+      else { uu = p[TX + 2]; wu = p[VP + TX + 2]; }
+      if (k == 0) { ud = g.wall ? u : -u; wd = -w; }
+      else if (k == g.n1) { ud = lid_u2<T>(S.gam[2][cc], S.gam_fx[0][cc]) - u; wd = -w; }
+      else { ud = p[-(TX + 2)]; wd = p[VP - (TX + 2)]; }
+      tz[e] = uu - ud;
+      tz[ZP + e] = wu - wd;
+    } else {
+      const int x = e - ZP, rr = x / TX, cc = x - rr * TX, k = k0 - 1 + rr;
+      if (k < 0 || k >= g.nz) continue;
+      const T* p = v + rr * (TX + 2) + cc;
+      tx[x] = p[2] - p[0];
+      tx[XP + x] = p[VP + 2] - p[VP];
+    }
+  }
+}
+
+// ---- phase 4: face fluxes ---------------------------------------------------
+// Face e of the tile: z faces by rows, then x faces by rows, then the
+// interface seen from below. False if no cell of the tile needs it.
+struct FaceId {
+  int isx, f, c;  // z: face row f, column c; x: tile row f, face column c
+  int ku;         // row above a z face, or the row of an x face
+  int below;      // the interface from fluid 1
+};
+template <int TZR>
+__device__ __forceinline__ bool face_id(const Geom& g, int e, int k0, int row_hi, FaceId* id) {
+  constexpr int NZF = TileSmem<TZR>::NZF, NXF = TileSmem<TZR>::NXF;
+  id->below = 0;
+  if (e < NZF) {
+    id->isx = 0;
+    id->f = e / TX;
+    id->c = e - id->f * TX;
+    id->ku = k0 + id->f;
+    // needed by the cell below (f >= 1) or above (f < TZR); at the interface
+    // this is the side of fluid 2
+    return id->ku - 1 < row_hi && !(id->f == TZR && id->ku == g.n1);
+  }
+  if (e < NZF + NXF) {
+    const int x = e - NZF;
+    id->isx = 1;
+    id->f = x / (TX + 1);
+    id->c = x - id->f * (TX + 1);
+    id->ku = k0 + id->f;
+    return id->ku < row_hi;
+  }
+  id->isx = 0;
+  id->f = g.n1 - k0;
+  id->c = e - NZF - NXF;
+  id->ku = g.n1;
+  id->below = 1;
+  return id->f >= 1 && id->f <= TZR && g.n1 - 1 < row_hi;
+}
+
+// States of the face in the face frame (rho, m_n, m_t, rho E) on both sides,
+// reconstructed from the four cells across it, and the two cells' velocities,
+// e and tangential differences (un, ut, e, gn, gt). A boundary face (outer
+// wall or interface) has the inner cell's state on one side and its mirror
+// on the other; an outer wall's viscous ghost is 2 wall state - cell. Returns
+// the fluid of the face's coefficients, 2 + fluid at the interface.
+template <typename T, int TZR>
+__device__ __forceinline__ int face_sides(const Geom& g, const TileSmem<TZR>& S, const FaceId& id, T L[4], T R[4],
+                                          T vL[5], T vR[5]) {
+  constexpr int QP = (TZR + 4) * (TX + 4), VP = (TZR + 2) * (TX + 2), ZP = TZR * (TX + 2), XP = (TZR + 2) * TX;
+  const int n1 = g.n1, nz = g.nz, ku = id.ku, kd = ku - 1;
+  // first of the four cells, their stride, and the planes of m_n, m_t
+  const int qs = id.isx ? 1 : TX + 4;
+  const int q0 = id.isx ? (id.f + 2) * (TX + 4) + id.c : id.f * (TX + 4) + id.c + 2;
+  const int pn = id.isx ? QP : 2 * QP, pt = 3 * QP - pn;
+  const bool wall = !id.isx && (ku == 0 || ku == nz), lid = !id.isx && ku == n1;
+  const bool from_above = ku == 0 || (lid && !id.below);  // of a boundary face: the inner cell is the upper one
+  const bool mir0 = !id.isx && (kd == 0 || kd == n1), mir3 = !id.isx && (ku == nz - 1 || ku == n1 - 1);
+  const T* q = Arith<T>::q(S) + q0;
+  auto comp = [&](int plane, bool odd, T& l, T& r) {
+    const T* p = q + plane;
+    T a0 = p[0], a1 = p[qs], a2 = p[2 * qs], a3 = p[3 * qs];
+    if (!id.isx) {  // mirror ghosts beyond a wall or the interface: rho w odd
+      if (wall || lid) {
+        if (from_above) a1 = odd ? -a2 : a2;
+        else a2 = odd ? -a1 : a1;
+      }
+      if (mir0) a0 = odd ? -a1 : a1;
+      if (mir3) a3 = odd ? -a2 : a2;
+    }
+    l = Arith<T>::rec(a1, a2, a0);
+    r = Arith<T>::rec(a2, a1, a3);
+    if (wall || lid) {
+      if (from_above) l = odd ? -r : r;
+      else r = odd ? -l : l;
+    }
+  };
+  comp(0, false, L[0], R[0]);
+  comp(pn, true, L[1], R[1]);
+  comp(pt, false, L[2], R[2]);
+  comp(3 * QP, false, L[3], R[3]);
+  if (lid) return id.below ? 2 : 3;
+  // velocities, e and tangential differences of the cells at the face
+  const T* v = reinterpret_cast<const T*>(&S.v[0][0][0]);
+  const int vo = id.isx ? (id.f + 1) * (TX + 2) + id.c : id.f * (TX + 2) + id.c + 1, vs = id.isx ? 1 : TX + 2;
+  const int vn = id.isx ? 0 : VP, vt = VP - vn;
+  const T* t = id.isx ? reinterpret_cast<const T*>(&S.tz[0][0][0]) + id.f * (TX + 2) + id.c
+                      : reinterpret_cast<const T*>(&S.tx[0][0][0]) + id.f * TX + id.c;
+  const int ts = id.isx ? 1 : TX, tn = id.isx ? 0 : XP, tt = id.isx ? ZP : 0;
+  vL[0] = v[vo + vn], vL[1] = v[vo + vt], vL[2] = v[vo + 2 * VP], vL[3] = t[tn], vL[4] = t[tt];
+  vR[0] = v[vo + vs + vn], vR[1] = v[vo + vs + vt], vR[2] = v[vo + vs + 2 * VP], vR[3] = t[ts + tn],
+  vR[4] = t[ts + tt];
+  if (wall) {
+    const T* c = from_above ? vR : vL;
+    T* o = from_above ? vL : vR;
+    o[0] = -c[0];
+    o[1] = g.wall ? c[1] : -c[1];
+    o[2] = c[2];
+    o[3] = -c[3];
+    o[4] = g.wall ? c[4] : -c[4];
+  }
+  return (id.isx ? ku : (ku == 0 ? 0 : kd)) >= n1;
+}
+
+// The fixed-point face flux over half the divergence factor (.57), or false
+// where a state leaves the range: F = f(q_L) + f(q_R) + lambda (q_L - q_R)
+// - V, lambda the largest |u_n| + a over the left, right and Roe-averaged
+// states.
+struct FxSide {
+  FxW un, mn;
+  i64 un_, ut, mu, p, c2;  // velocities .59, m_n u_n .57, p .57, c^2 .55
+  i64 k;                   // |m|^2 / rho .57
+  i64 eh;                  // rho E + p .59
+};
+__device__ __forceinline__ void fx_side(const FxConst& k, const i64 q[4], FxSide* s, FxW* mt) {
+  const FxW inv = fx::split(fx::recip(q[0]));
+  s->mn = fx::split(q[1]);
+  *mt = fx::split(q[2]);
+  s->un_ = fx::mul(s->mn, inv);
+  s->ut = fx::mul(*mt, inv);
+  s->un = fx::split(s->un_);
+  s->mu = fx::mul(s->mn, s->un);
+  s->k = s->mu + fx::mul(*mt, fx::split(s->ut));
+  const FxW pe = fx::split(q[3] - (s->k << 2));  // p / (gamma - 1) .60
+  s->p = fx::mul(pe, k.gm1);
+  s->c2 = fx::mul(fx::split(fx::mul(pe, inv)), k.gg);
+  s->eh = (q[3] >> 1) + (s->p << 2);
+}
+
+// The Roe-averaged speed |u_n| + a in double from the two states (rarely
+// needed): w the weight sqrt(rho_R) / (sqrt(rho_L) + sqrt(rho_R)), a^2 =
+// (1 - w) a_L^2 + w a_R^2 + (gamma - 1)/2 w (1 - w) |du|^2, which equals the
+// Roe-averaged enthalpy's (gamma - 1)(H - |u|^2 / 2).
+__device__ __noinline__ i64 fx_roe_speed(i64 rL, i64 rR, i64 unL, i64 unR, i64 dut, i64 c2L, i64 c2R, double gm1) {
+  const double w = recip_f64(__dadd_rn(1.0, sqrt_f64(__dmul_rn((double)rL, recip_f64((double)rR)))));
+  const double sv = 1.0 / (double)(1ll << fx::S_VEL), sc = 1.0 / (double)(1ll << 55);
+  const double du = __dmul_rn((double)(unR - unL), sv), dt = __dmul_rn((double)dut, sv);
+  const double un = __fma_rn(w, du, __dmul_rn((double)unL, sv));
+  const double a = __dmul_rn((double)c2L, sc), d = __dmul_rn((double)(c2R - c2L), sc);
+  const double q = __dmul_rn(__dmul_rn(0.5 * gm1, w), __dsub_rn(1.0, w));
+  const double c2 = __fma_rn(q, __fma_rn(du, du, __dmul_rn(dt, dt)), __fma_rn(w, d, a));
+  return __double2ll_rn(__dmul_rn(__dadd_rn(fabs(un), sqrt_f64(c2)), (double)(1ll << fx::S_VEL)));
+}
+
+__device__ __forceinline__ bool fx_flux(const Geom& g, const FxConst& k, const i64 L[4], const i64 R[4], const i64 V[3], i64 F[4]) {
+  FxSide l, r;
+  FxW mtL, mtR;
+  fx_side(k, L, &l, &mtL);
+  fx_side(k, R, &r, &mtR);
+  const int c2l = (int)(l.c2 >> 32), c2r = (int)(r.c2 >> 32);
+  if (min((int)(L[0] >> 32), (int)(R[0] >> 32)) < fx::RHO_MIN ||
+      max((int)(l.k >> 32), (int)(r.k >> 32)) >= fx::KIN_MAX || min(c2l, c2r) < fx::C2_MIN ||
+      max(c2l, c2r) >= fx::C2_MAX)
+    return false;
+  const i64 cl = fx::sqroot(l.c2 << 6), cr = fx::sqroot(r.c2 << 6);
+  const i64 sl = (l.un_ < 0 ? -l.un_ : l.un_) + cl, sr = (r.un_ < 0 ? -r.un_ : r.un_) + cr;
+  i64 lam = sl > sr ? sl : sr;  // .59
+  {
+    // The Roe speed lies below (1 - w) sl + w sr + w (1 - w) / (2 min a) D
+    // with D = (a_L - a_R)^2 + (gamma - 1)/2 |du|^2, so it cannot be the
+    // largest where |sl - sr| max(1, ...) >= D (min a > 0.5, w in [0.2, 0.8]
+    // within the range): all but a few faces of a smooth flow skip it.
+    const float k59 = 5.7646075e17f;
+    const float df = fx::to_float(sl - sr), dc = fx::to_float(cl - cr), dn = fx::to_float(l.un_ - r.un_),
+                dt = fx::to_float(l.ut - r.ut);
+    if (fabsf(df) * k59 < fmaf(dc, dc, 0.5f * g.gm1f * fmaf(dn, dn, dt * dt))) {
+      const i64 roe = fx_roe_speed(L[0], R[0], l.un_, r.un_, r.ut - l.ut, l.c2, r.c2, g.gm1);
+      lam = roe > lam ? roe : lam;
+    }
+  }
+  const FxW lam59 = fx::split(lam), lam61 = fx::split(lam << 2);
+  F[0] = (L[1] >> 5) + (R[1] >> 5) + fx::mul(fx::split(L[0] - R[0]), lam61);
+  F[1] = (l.mu + l.p) + (r.mu + r.p) + fx::mul(fx::split(L[1] - R[1]), lam59) - V[0];
+  F[2] = fx::mul2(mtL, l.un, mtR, r.un) + fx::mul(fx::split(L[2] - R[2]), lam59) - V[1];
+  F[3] = fx::mul(fx::split(l.eh), fx::split(l.un_ << 3)) + fx::mul(fx::split(r.eh), fx::split(r.un_ << 3)) +
+         fx::mul(fx::split(L[3] - R[3]), lam61) - V[2];
+  // room for the sums of phase 5: |F| < 8
+  int top = 0;
+#pragma unroll
+  for (int c = 0; c < 4; c++) {
+    const int h = (int)(F[c] >> 32);
+    top |= h ^ (h >> 31);
+  }
+  return top < (8 << (fx::S_FLUX - 32));
+}
+
+// The viscous flux over half the divergence factor from the common values of
+// App. B: (sigma_nn, sigma_nt, u . sigma_n + kappa dT/dn), .57.
+__device__ __forceinline__ void fx_visc(const FxW* fc, const i64 vL[5], const i64 vR[5], i64 V[3]) {
+  const FxW du = fx::split(vR[0] - vL[0]), dt = fx::split(vR[1] - vL[1]);
+  V[0] = fx::mul2(fc[FXC_A], du, fc[FXC_B], fx::split(vL[4] + vR[4]));
+  V[1] = fx::mul2(fc[FXC_C], dt, fc[FXC_D], fx::split(vL[3] + vR[3]));
+  // (u_L + u_R) / 2 . sigma: .61 x .57 -> .54, half of it at .55
+  const i64 us = fx::mul2(fx::split((vL[0] + vR[0]) << 2), fx::split(V[0]), fx::split((vL[1] + vR[1]) << 2),
+                          fx::split(V[1]));
+  V[2] = (us << 2) + fx::mul(fc[FXC_K], fx::split(vR[2] - vL[2]));
+}
+
+// The same flux in double.
+__device__ __forceinline__ void double_flux(const Geom& g, const double L[4], const double R[4], const double V[3],
+                                            double F[4]) {
+  const double sub[4] = {0.0, V[0], V[1], V[2]};
+  lf_face(L[0], L[1], L[2], L[3], R[0], R[1], R[2], R[3], g.gamma, g.gm1, sub, F);
+}
+__device__ __forceinline__ void double_visc(const double* fc, const double vL[5], const double vR[5], double V[3]) {
+  V[0] = __fma_rn(fc[FXC_A], __dsub_rn(vR[0], vL[0]), __dmul_rn(fc[FXC_B], __dadd_rn(vL[4], vR[4])));
+  V[1] = __fma_rn(fc[FXC_C], __dsub_rn(vR[1], vL[1]), __dmul_rn(fc[FXC_D], __dadd_rn(vL[3], vR[3])));
+  const double us = __fma_rn(__dadd_rn(vL[1], vR[1]), V[1], __dmul_rn(__dadd_rn(vL[0], vR[0]), V[0]));
+  V[2] = __fma_rn(0.5, us, __dmul_rn(fc[FXC_K], __dsub_rn(vR[2], vL[2])));
+}
+
+// Fluxes to shared memory, back in (rho, rho u, rho w, rho E) order.
+template <int TZR>
+__device__ __forceinline__ void store_flux(TileSmem<TZR>& S, const FaceId& id, const i64 F[4]) {
+  i64* p;
+  int plane, n;
+  if (id.isx) {
+    p = &S.fx[0][id.f][id.c], plane = TZR * (TX + 1), n = 1;
+  } else if (id.below) {
+    p = &S.fg[0][id.c], plane = TX, n = 2;
+  } else {
+    p = &S.fz[0][id.f][id.c], plane = (TZR + 1) * TX, n = 2;
+  }
+  p[0] = F[0];
+  p[n * plane] = F[1];
+  p[(3 - n) * plane] = F[2];
+  p[3 * plane] = F[3];
+}
+
+// Do the cells that face id reads (four across it, and the tangential
+// neighbours of the two at it), and the interface states if it reads any,
+// lie in the fixed-point range? Asked only in tiles where some cell does not.
+template <int TZR>
+__device__ __noinline__ bool face_in_range(const Geom& g, const TileSmem<TZR>& S, const FaceId id, int k0) {
+  auto cell = [&](int r, int c) {  // halo row and column
+    const int k = k0 - 2 + r;
+    return k < 0 || k >= g.nz || cell_in_range(S.q[0][r][c], S.q[1][r][c], S.q[2][r][c], S.q[3][r][c]);
+  };
+  bool ok = true;
+  if (id.isx) {
+    for (int j = 0; j < 4; j++) ok = ok && cell(id.f + 2, id.c + j);
+    for (int j = 0; j < 4; j++) ok = ok && cell(id.f + 1 + 2 * (j >> 1), id.c + 1 + (j & 1));
+    if (id.ku == g.n1 || id.ku == g.n1 - 1) ok = ok && S.gam_ok[id.c] && S.gam_ok[id.c + 1];
+  } else {
+    for (int j = 0; j < 4; j++) ok = ok && cell(id.f + j, id.c + 2);
+    for (int j = 0; j < 4; j++) ok = ok && cell(id.f + 1 + (j >> 1), id.c + 1 + 2 * (j & 1));
+    if (id.ku == g.n1) ok = ok && S.gam_ok[id.c + 1];
+  }
+  return ok;
+}
+
+// The faces marked slow, in double: phases 2 and 3 again as doubles (in the
+// same storage), then their fluxes. Ends with the tile's barrier.
+template <int NT, int TZR>
+__device__ __noinline__ void slow_faces(const Geom& g, TileSmem<TZR>& S, int k0, int i0, int row_hi) {
+  ring_phase<double, NT, TZR>(g, S, k0, i0);
+  if (threadIdx.x < 4 * FXC_N) {
+    const int j = threadIdx.x % FXC_N, f = threadIdx.x / FXC_N;
+    S.fc[f >> 1][f & 1][j] = visc_coef(g, f >> 1, f & 1, j);
+  }
+  __syncthreads();
+  diff_phase<double, NT, TZR>(g, S, k0, row_hi);
+  __syncthreads();
+  for (int e = threadIdx.x; e < TileSmem<TZR>::NZF + TileSmem<TZR>::NXF + TX; e += NT) {
+    FaceId id;
+    if (!face_id<TZR>(g, e, k0, row_hi, &id) || !S.slow[e]) continue;
+    double L[4], R[4], vL[5], vR[5], V[3], F[4];
+    const int fl = face_sides<double, TZR>(g, S, id, L, R, vL, vR);
+    if (fl >= 2) {
+      V[0] = 0.0;
+      V[1] = 2.0 * S.gam[0][id.c + 1];
+      V[2] = 2.0 * __fma_rn(S.gam[2][id.c + 1], S.gam[0][id.c + 1], -S.gam[1][id.c + 1]);
+    } else {
+      double_visc(S.fc[id.isx ? 0 : 1][fl], vL, vR, V);
+    }
+    double_flux(g, L, R, V, F);
+    i64 o[4];
+#pragma unroll
+    for (int c = 0; c < 4; c++) o[c] = __double_as_longlong(F[c]);
+    store_flux(S, id, o);
+  }
+  __syncthreads();
+}
+
+// The tile body. tile = linear tile index within the launch's row range.
+// Inlined into each kernel, so that the single-instance kernel takes its
+// arguments from the constant bank and the batch kernel from shared memory;
+// every double operation names its rounding (no contraction is left to the
+// compiler) and the rest is integer, so an instance's results are bitwise
+// the same alone and in a batch.
+//
 // GEN selects the general s-stage base method (Sec. 3 remark) in place of
 // Heun's low-storage path: s R_a slots, the stage values of the region
 // tableaus built from the base, and its weights b in the combinations.
@@ -216,11 +559,8 @@ __device__ __forceinline__ double gen_weighted_sum(const Geom& g, const double* 
 // more warps of the few tiles there are: every phase but the last spreads
 // its work over all threads, and the last (one cell per thread) uses the
 // first TX x TZR. TZR: tile rows.
-template <typename Real, typename Store, bool GEN = false, int NT = NTHREADS, int TZR = TZ>
-__device__ __noinline__ void stage_tile(const StageArgs& __restrict__ a, int tile,
-                                       TileSmem<Real, TZR>& __restrict__ S) {
-  // __restrict__: the argument block and shared memory never alias, so its
-  // fields need not be reloaded after shared-memory stores
+template <bool GEN = false, int NT = NTHREADS, int TZR = TZ>
+__device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSmem<TZR>& S) {
   const Geom& g = a.g;
   const int tid = threadIdx.x;
   const int tzi = tile / a.tiles_x;
@@ -231,268 +571,115 @@ __device__ __noinline__ void stage_tile(const StageArgs& __restrict__ a, int til
   const int row_hi = a.rhs_only ? a.rhs_hi : nz;
   const size_t plane = (size_t)nz * g.pitch;
   const bool odd_stage = !a.rhs_only && (a.stage & 1);  // stages 2, 4, ... (1-based)
-  const Store* Ra = reinterpret_cast<const Store*>(a.b.Ra);
+  const double* Ra = reinterpret_cast<const double*>(a.b.Ra);
   const double hF = g.hF;
 
+  // stage value of component c at row k, column i of the grid
+  auto stage_value = [&](int c, int k, int i) -> double {
+    const size_t off = (size_t)c * plane + (size_t)k * g.pitch + i;
+    if (a.rhs_only) return a.rhs_in[off];
+    const bool slow_rows = k < g.n1_r;
+    const double* base = slow_rows ? a.b.qA : a.qF;
+    const double h = slow_rows ? g.dt : hF;
+    if (GEN) return gen_stage_value(g, base, Ra, 4 * plane, off, a.stage % g.s, h);
+    return odd_stage ? __fma_rn(h, Ra[off], base[off]) : base[off];
+  };
+
   // ---- 1. stage state of the tile and its halo --------------------------
-  if (tid < 4) {
-    // face constants of direction tid >> 1 (x, z) in fluid tid & 1
-    const int dir = tid >> 1, fl = tid & 1;
-    const double inv_dz = fl ? g.inv_dz2 : g.inv_dz1;
-    const double mu = fl ? g.mu2 : g.mu1, kap = fl ? g.kap2 : g.kap1;
-    const double inv_dn = dir ? inv_dz : g.inv_dx, inv_dt = dir ? g.inv_dx : inv_dz;
-    const double sc = inv_dn;  // the divergence factor is the normal one
-    Real* fc = S.fc[dir][fl];
-    fc[FC_HS] = (Real)(0.5 * sc);
-    fc[FC_A] = (Real)(4.0 / 3.0 * mu * inv_dn * sc);
-    fc[FC_B] = (Real)(mu * inv_dt * sc / 6.0);
-    fc[FC_C] = (Real)(mu * inv_dn * sc);
-    fc[FC_D] = (Real)(0.25 * mu * inv_dt * sc);
-    fc[FC_K] = (Real)(kap * inv_dn * sc * (g.gamma * g.gm1));  // times the factor T / e of S.v[2]
-    fc[FC_SC] = (Real)sc;
-  }
-  for (int e = tid; e < 4 * (TZR + 4) * (TX + 4); e += NT) {
-    const int c = e / ((TZR + 4) * (TX + 4));
-    const int rem = e - c * ((TZR + 4) * (TX + 4));
-    const int rr = rem / (TX + 4), cc = rem - rr * (TX + 4);
+  bool bad = !a.fx.on;  // some cell outside the fixed-point range
+  for (int e = tid; e < (TZR + 4) * (TX + 4); e += NT) {
+    const int rr = e / (TX + 4), cc = e - rr * (TX + 4);
     const int k = k0 - 2 + rr;
-    Real val = Real(0);
+    double val[4] = {0.0, 0.0, 0.0, 0.0};
     if (k >= 0 && k < nz) {
       bool gh;
       const int i = halo_col(i0 - 2 + cc, nx, g.xwall, &gh);
-      const size_t off = (size_t)c * plane + (size_t)k * g.pitch + i;
-      if (a.rhs_only) {
-        val = (Real)a.rhs_in[off];
-      } else {
-        const double* base = k < g.n1_r ? a.b.qA : a.qF;
-        if (GEN) {
-          val = (Real)gen_stage_value(g, base, reinterpret_cast<const double*>(Ra), 4 * plane, off,
-                                      a.stage % g.s, k < g.n1_r ? g.dt : hF);
-        } else if (odd_stage) {
-          const Real h = (Real)(k < g.n1_r ? g.dt : hF);
-          val = (Real)base[off] + h * (Real)Ra[off];
-        } else {
-          val = (Real)base[off];
-        }
-      }
-      if (gh && c == 1) val = -val;  // mirror state beyond an x wall
+#pragma unroll
+      for (int c = 0; c < 4; c++) val[c] = stage_value(c, k, i);
+      if (gh) val[1] = -val[1];  // mirror state beyond an x wall
+      bad |= !cell_in_range(val[0], val[1], val[2], val[3]);
     }
-    S.q[c][rr][cc] = val;
-  }
-  const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZR);
-  __syncthreads();
-
-  // ---- 2. u, w, T on the one-cell ring; interface state -----------------
-  const Real gamma = (Real)g.gamma, gm1 = (Real)g.gm1;
-  for (int e = tid; e < (TZR + 2) * (TX + 2); e += NT) {
-    const int rr = e / (TX + 2), cc = e - rr * (TX + 2);
-    const int k = k0 - 1 + rr;
-    if (k < 0 || k >= nz) continue;
-    const Real r = S.q[0][rr + 1][cc + 1], mu_ = S.q[1][rr + 1][cc + 1];
-    const Real mw = S.q[2][rr + 1][cc + 1], E = S.q[3][rr + 1][cc + 1];
-    const Real inv = rcp(r);
-    const Real u = mu_ * inv, w = mw * inv;
-    S.v[0][rr][cc] = u;
-    // the mirror state's u is already flipped; a no-slip wall flips w too
-    S.v[1][rr][cc] = (x_ghost(i0 - 1 + cc, nx, g.xwall) && g.wall == 0) ? -w : w;
-    // internal energy per mass e = T / (gamma (gamma - 1)) with T = gamma p / rho;
-    // the heat-flux constant carries the factor
-    S.v[2][rr][cc] = (E - Real(0.5) * (mu_ * u + mw * w)) * inv;
-  }
-  if (has_gamma && tid < TX + 2) {
-    // Interface state of column i0-1+tid in double precision from the two
-    // cells touching Gamma (App. B, Eq. bulk-flux and the wall states).
-    bool gh;
-    const int i = halo_col(i0 - 1 + tid, nx, g.xwall, &gh);
-    double u[2], T[2];
-#pragma unroll
-    for (int s = 0; s < 2; s++) {
-      const int k = n1 - 1 + s;
-      double qq[4];
-#pragma unroll
-      for (int c = 0; c < 4; c++) {
-        const size_t off = (size_t)c * plane + (size_t)k * g.pitch + i;
-        if (a.rhs_only) {
-          qq[c] = a.rhs_in[off];
-        } else {
-          const double* base = k < g.n1_r ? a.b.qA : a.qF;
-          if (GEN) {
-            qq[c] = gen_stage_value(g, base, reinterpret_cast<const double*>(Ra), 4 * plane, off, a.stage % g.s,
-                                    k < g.n1_r ? g.dt : hF);
-          } else if (odd_stage) {
-            qq[c] = base[off] + (k < g.n1_r ? g.dt : hF) * (double)Ra[off];
-          } else {
-            qq[c] = base[off];
-          }
-        }
-      }
-      if (gh) qq[1] = -qq[1];  // mirror state beyond an x wall
-      const double inv = 1.0 / qq[0];
-      u[s] = qq[1] * inv;
-      const double w = qq[2] * inv;
-      const double p = g.gm1 * (qq[3] - 0.5 * (qq[1] * u[s] + qq[2] * w));
-      T[s] = g.gamma * p * inv;
-    }
-    const double sig = g.bu * (u[1] - u[0]);
-    const double Pi = -g.bT * (T[1] - T[0]);
-    S.gam[0][tid] = sig;
-    S.gam[1][tid] = Pi;
-    S.gam[2][tid] = u[0] + sig * g.cu1;
-    S.gam[3][tid] = T[0] - Pi * g.cT1;
-  }
-  __syncthreads();
-
-  // ---- 3. slopes ---------------------------------------------------------
-  // (a) central x differences of q on tile rows, cols i0-1 .. i0+TX
-  for (int e = tid; e < TZR * (TX + 2); e += NT) {
-    const int rr = e / (TX + 2), cc = e - rr * (TX + 2);
-    if (k0 + rr >= row_hi) continue;
-#pragma unroll
-    for (int c = 0; c < 4; c++) S.hx[c][rr][cc] = S.q[c][rr + 2][cc + 2] - S.q[c][rr + 2][cc];
-    // z differences of u, w at the same cells (tangential at x faces)
-    const int k = k0 + rr;
-    const Real u = S.v[0][rr + 1][cc], w = S.v[1][rr + 1][cc];
-    Real uu, wu, ud, wd;  // values above and below, or their ghosts
-    const bool top_wall = (k + 1 == nz), bot_wall = (k == 0);
-    const bool top_gam = (k + 1 == n1), bot_gam = (k == n1);
-    if (top_wall) { uu = g.wall ? u : -u; wu = -w; }
-    else if (top_gam) { uu = Real(2) * (Real)S.gam[2][cc] - u; wu = -w; }
-    else { uu = S.v[0][rr + 2][cc]; wu = S.v[1][rr + 2][cc]; }
-    if (bot_wall) { ud = g.wall ? u : -u; wd = -w; }
-    else if (bot_gam) { ud = Real(2) * (Real)S.gam[2][cc] - u; wd = -w; }
-    else { ud = S.v[0][rr][cc]; wd = S.v[1][rr][cc]; }
-    S.tz[0][rr][cc] = uu - ud;
-    S.tz[1][rr][cc] = wu - wd;
-  }
-  // (b) central z differences of q on ring rows k0-1 .. k0+TZR, tile cols
-  for (int e = tid; e < (TZR + 2) * TX; e += NT) {
-    const int rr = e / TX, cc = e - rr * TX;
-    const int k = k0 - 1 + rr;
-    if (k < 0 || k >= nz) continue;
-    const bool up_in = (k + 1 < nz) && ((k + 1 < n1) == (k < n1));
-    const bool dn_in = (k - 1 >= 0) && ((k - 1 < n1) == (k < n1));
 #pragma unroll
     for (int c = 0; c < 4; c++) {
-      const Real own = S.q[c][rr + 1][cc + 2];
-      const Real mir = (c == 2) ? -own : own;  // mirror ghost: rho w odd
-      const Real up = up_in ? S.q[c][rr + 2][cc + 2] : mir;
-      const Real dn = dn_in ? S.q[c][rr][cc + 2] : mir;
-      S.hz[c][rr][cc] = up - dn;
+      S.q[c][rr][cc] = val[c];
+      S.qi[c][rr][cc] =
+          fx::from_double(__double_as_longlong(val[c]), c == 1 || c == 2 ? fx::S_MOM - 2 : fx::S_RHO - 2);
     }
-    S.tx[0][rr][cc] = S.v[0][rr][cc + 2] - S.v[0][rr][cc];
-    S.tx[1][rr][cc] = S.v[1][rr][cc + 2] - S.v[1][rr][cc];
   }
+  const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZR);
+  bad = __syncthreads_or(bad);
+
+  // ---- 2. u, w, e on the one-cell ring; interface state ------------------
+  ring_phase<i64, NT, TZR>(g, S, k0, i0);
+  if (has_gamma) {
+    bool lid_bad = false;
+    if (tid < TX + 2) {
+      // Interface state of column i0-1+tid in double precision from the two
+      // cells touching Gamma (App. B, Eq. bulk-flux and the wall states).
+      bool gh;
+      const int i = halo_col(i0 - 1 + tid, nx, g.xwall, &gh);
+      double u[2], T[2];
+#pragma unroll
+      for (int s = 0; s < 2; s++) {
+        double qq[4];
+#pragma unroll
+        for (int c = 0; c < 4; c++) qq[c] = stage_value(c, n1 - 1 + s, i);
+        if (gh) qq[1] = -qq[1];  // mirror state beyond an x wall
+        const double inv = 1.0 / qq[0];
+        u[s] = __dmul_rn(qq[1], inv);
+        const double w = __dmul_rn(qq[2], inv);
+        const double k = __fma_rn(qq[2], w, __dmul_rn(qq[1], u[s]));
+        const double p = __dmul_rn(g.gm1, __fma_rn(-0.5, k, qq[3]));
+        T[s] = __dmul_rn(__dmul_rn(g.gamma, p), inv);
+      }
+      const double sig = __dmul_rn(g.bu, __dsub_rn(u[1], u[0]));
+      const double Pi = __dmul_rn(-g.bT, __dsub_rn(T[1], T[0]));
+      const double uw = __fma_rn(sig, g.cu1, u[0]), En = __fma_rn(uw, sig, -Pi);
+      S.gam[0][tid] = sig;
+      S.gam[1][tid] = Pi;
+      S.gam[2][tid] = uw;
+      const bool ok = fabs(uw) < 1.9 && fabs(sig) < 2.0 && fabs(En) < 2.0;  // false for NaN
+      S.gam_ok[tid] = ok;
+      lid_bad = !ok;
+      S.gam_fx[0][tid] = __double2ll_rn(ok ? uw * (double)(2ll << fx::S_VEL) : 0.0);
+      S.gam_fx[1][tid] = __double2ll_rn(ok ? sig * (double)(2ll << fx::S_FLUX) : 0.0);
+      S.gam_fx[2][tid] = __double2ll_rn(ok ? En * (double)(2ll << fx::S_FLUX) : 0.0);
+    }
+    bad |= __syncthreads_or(lid_bad) != 0;
+  } else {
+    __syncthreads();
+  }
+
+  // ---- 3. tangential differences ------------------------------------------
+  diff_phase<i64, NT, TZR>(g, S, k0, row_hi);
   __syncthreads();
 
   // ---- 4. face fluxes ----------------------------------------------------
-  // z faces first: (TZR+1) rows of TX faces, one warp per face row; then x
-  // faces. Every warp sees one face kind.
-  const Real quarter = Real(0.25);
-  constexpr int NZF = (TZR + 1) * TX, NXF = TZR * (TX + 1);
-  for (int e = tid; e < NZF + NXF; e += NT) {
-    Real F[4];
-    if (e < NZF) {
-      const int f = e / TX, cc = e - f * TX;
-      const int ku = k0 + f;  // row above the face
-      const int kd = ku - 1;  // row below the face
-      // needed by a cell of the tile: the cell below (f >= 1) or above (f == 0)
-      if (kd >= row_hi) continue;
-      // reconstructed state of the cell at tile row rq (halo rows) / ring row
-      // rh in the face frame (normal = z): q + sq * (central z difference),
-      // sq = +-1/4
-      auto load_side = [&](int rq, int rh, Real& r, Real& mn, Real& mt, Real& E, Real sq) {
-        r = S.q[0][rq][cc + 2] + sq * S.hz[0][rh][cc];
-        mt = S.q[1][rq][cc + 2] + sq * S.hz[1][rh][cc];
-        mn = S.q[2][rq][cc + 2] + sq * S.hz[2][rh][cc];
-        E = S.q[3][rq][cc + 2] + sq * S.hz[3][rh][cc];
-      };
-      if (ku == 0 || ku == nz) {
-        // outer wall: the boundary cell against its mirror (inviscid) and its
-        // ghost 2*wall - interior (viscous); no-slip or slip, adiabatic
-        const bool below = (ku == 0);  // wall under row 0
-        const int rq = below ? f + 2 : f + 1;
-        const int rh = below ? f + 1 : f;
-        const int rv = below ? f + 1 : f;
-        const int k = below ? ku : kd;
-        const Real* fc = S.fc[1][k >= n1];
-        Real r, mn, mt, E;
-        load_side(rq, rh, r, mn, mt, E, below ? -quarter : quarter);
-        Real F[4], FV[4];
-        const Real un = S.v[1][rv][cc + 1], ut = S.v[0][rv][cc + 1], T = S.v[2][rv][cc + 1];
-        const Real gn = S.tx[1][rv][cc], gt = S.tx[0][rv][cc];
-        const Real utg = g.wall ? ut : -ut, gtg = g.wall ? gt : -gt;
-        if (below) visc_face_fc(-un, utg, T, -gn, gtg, un, ut, T, gn, gt, fc, FV);
-        else visc_face_fc(un, ut, T, gn, gt, -un, utg, T, -gn, gtg, fc, FV);
-        if (below) lf_face(r, -mn, mt, E, r, mn, mt, E, gamma, gm1, fc[FC_HS], FV, F);
-        else lf_face(r, mn, mt, E, r, -mn, mt, E, gamma, gm1, fc[FC_HS], FV, F);
-        S.fz[0][f][cc] = F[0];
-        S.fz[1][f][cc] = F[2];
-        S.fz[2][f][cc] = F[1];
-        S.fz[3][f][cc] = F[3];
-      } else if (ku == n1) {
-        // the interface: a rigid lid seen from each fluid (inviscid), the bulk
-        // fluxes of App. B (viscous, shared by both fluids)
-        const double sig = S.gam[0][cc + 1], Pi = S.gam[1][cc + 1], uw = S.gam[2][cc + 1];
-        const Real Vt = (Real)sig, VE = (Real)(uw * sig - Pi);
-        const Real *fc2 = S.fc[1][1], *fc1 = S.fc[1][0];
-        Real r, mn, mt, E, F[4];
-        load_side(f + 2, f + 1, r, mn, mt, E, -quarter);  // fluid 2, above
-        const Real sub2[4] = {Real(0), Real(0), Vt * fc2[FC_SC], VE * fc2[FC_SC]};
-        lf_face(r, -mn, mt, E, r, mn, mt, E, gamma, gm1, fc2[FC_HS], sub2, F);
-        S.fz[0][f][cc] = F[0];
-        S.fz[1][f][cc] = F[2];
-        S.fz[2][f][cc] = F[1];
-        S.fz[3][f][cc] = F[3];
-        load_side(f + 1, f, r, mn, mt, E, quarter);  // fluid 1, below
-        const Real sub1[4] = {Real(0), Real(0), Vt * fc1[FC_SC], VE * fc1[FC_SC]};
-        lf_face(r, mn, mt, E, r, -mn, mt, E, gamma, gm1, fc1[FC_HS], sub1, F);
-        S.fg[0][cc] = F[0];
-        S.fg[1][cc] = F[2];
-        S.fg[2][cc] = F[1];
-        S.fg[3][cc] = F[3];
+  constexpr int NZF = TileSmem<TZR>::NZF, NXF = TileSmem<TZR>::NXF;
+  bool slow = false;
+  const int n_faces = NZF + NXF + (has_gamma ? TX : 0);
+  for (int e = tid; e < n_faces; e += NT) {
+    FaceId id;
+    if (!face_id<TZR>(g, e, k0, row_hi, &id)) continue;
+    bool ok = !bad || (a.fx.on && face_in_range<TZR>(g, S, id, k0));
+    if (ok) {
+      i64 L[4], R[4], vL[5], vR[5], V[3], F[4];
+      const int fl = face_sides<i64, TZR>(g, S, id, L, R, vL, vR);
+      if (fl >= 2) {
+        V[0] = 0;
+        V[1] = S.gam_fx[1][id.c + 1];
+        V[2] = S.gam_fx[2][id.c + 1];
       } else {
-        const Real* fc = S.fc[1][kd >= n1];
-        Real lr, lmn, lmt, lE, rr_, rmn, rmt, rE, F[4], FV[4];
-        load_side(f + 1, f, lr, lmn, lmt, lE, quarter);
-        load_side(f + 2, f + 1, rr_, rmn, rmt, rE, -quarter);
-        visc_face_fc(S.v[1][f][cc + 1], S.v[0][f][cc + 1], S.v[2][f][cc + 1], S.tx[1][f][cc], S.tx[0][f][cc],
-                     S.v[1][f + 1][cc + 1], S.v[0][f + 1][cc + 1], S.v[2][f + 1][cc + 1], S.tx[1][f + 1][cc],
-                     S.tx[0][f + 1][cc], fc, FV);
-        lf_face(lr, lmn, lmt, lE, rr_, rmn, rmt, rE, gamma, gm1, fc[FC_HS], FV, F);
-        S.fz[0][f][cc] = F[0];
-        S.fz[1][f][cc] = F[2];
-        S.fz[2][f][cc] = F[1];
-        S.fz[3][f][cc] = F[3];
+        fx_visc(a.fx.fc[id.isx ? 0 : 1][fl], vL, vR, V);
       }
-    } else {
-      const int x = e - NZF;
-      const int rr = x / (TX + 1), f = x - rr * (TX + 1);
-      const int k = k0 + rr;
-      if (k >= row_hi) continue;
-      // face between columns i0+f-1 (L, ring col f) and i0+f (R, ring col f+1)
-      // q +- 1/4 (central difference); the products are exact, so each sum
-      // rounds once
-      const Real lr = S.q[0][rr + 2][f + 1] + quarter * S.hx[0][rr][f];
-      const Real lmn = S.q[1][rr + 2][f + 1] + quarter * S.hx[1][rr][f];
-      const Real lmt = S.q[2][rr + 2][f + 1] + quarter * S.hx[2][rr][f];
-      const Real lE = S.q[3][rr + 2][f + 1] + quarter * S.hx[3][rr][f];
-      const Real rr_ = S.q[0][rr + 2][f + 2] - quarter * S.hx[0][rr][f + 1];
-      const Real rmn = S.q[1][rr + 2][f + 2] - quarter * S.hx[1][rr][f + 1];
-      const Real rmt = S.q[2][rr + 2][f + 2] - quarter * S.hx[2][rr][f + 1];
-      const Real rE = S.q[3][rr + 2][f + 2] - quarter * S.hx[3][rr][f + 1];
-      const Real* fc = S.fc[0][k >= n1];
-      Real F[4], FV[4];
-      visc_face_fc(S.v[0][rr + 1][f], S.v[1][rr + 1][f], S.v[2][rr + 1][f], S.tz[0][rr][f], S.tz[1][rr][f],
-                   S.v[0][rr + 1][f + 1], S.v[1][rr + 1][f + 1], S.v[2][rr + 1][f + 1], S.tz[0][rr][f + 1],
-                   S.tz[1][rr][f + 1], fc, FV);
-      lf_face(lr, lmn, lmt, lE, rr_, rmn, rmt, rE, gamma, gm1, fc[FC_HS], FV, F);
-      S.fx[0][rr][f] = F[0];
-      S.fx[1][rr][f] = F[1];
-      S.fx[2][rr][f] = F[2];
-      S.fx[3][rr][f] = F[3];
+      ok = fx_flux(g, a.fx, L, R, V, F);
+      if (ok) store_flux(S, id, F);
     }
+    S.slow[e] = !ok;
+    slow |= !ok;
   }
-  __syncthreads();
+  slow = __syncthreads_or(slow);
+  if (slow) slow_faces<NT, TZR>(g, S, k0, i0, row_hi);
 
   // ---- 5. R = -div F* + s and the stage combination ----------------------
   {
@@ -500,24 +687,44 @@ __device__ __noinline__ void stage_tile(const StageArgs& __restrict__ a, int til
     const int k = k0 + rr, i = i0 + cc;
     if (rr >= TZR || k >= row_hi || i >= nx) return;
     const bool under_gamma = (k == n1 - 1);
-    Real R[4];
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-      // the face fluxes carry 1/dx and 1/dz already
-      const Real up = under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc];
-      R[c] = (S.fx[c][rr][cc] - S.fx[c][rr][cc + 1]) + (S.fz[c][rr][cc] - up);
+    const double hx = 0.5 * g.inv_dx, hz = 0.5 * (k < n1 ? g.inv_dz1 : g.inv_dz2);
+    const double s57 = 1.0 / (double)(1ll << fx::S_FLUX);
+    double R[4];
+    bool s0 = false, s1 = false, s2 = false, s3 = false;  // slow faces of the cell: left, right, lower, upper
+    if (slow) {
+      s0 = S.slow[NZF + rr * (TX + 1) + cc];
+      s1 = S.slow[NZF + rr * (TX + 1) + cc + 1];
+      s2 = S.slow[rr * TX + cc];
+      s3 = S.slow[under_gamma ? NZF + NXF + cc : (rr + 1) * TX + cc];
     }
-    const Real Gr = (Real)g.G;
-    R[2] -= S.q[0][rr + 2][cc + 2] * Gr;
-    R[3] -= S.q[2][rr + 2][cc + 2] * Gr;
+    if (s0 || s1 || s2 || s3) {
+#pragma unroll
+      for (int c = 0; c < 4; c++) {
+        auto val = [&](i64 f, bool sl) { return sl ? __longlong_as_double(f) : __dmul_rn((double)f, s57); };
+        const double dx = __dsub_rn(val(S.fx[c][rr][cc], s0), val(S.fx[c][rr][cc + 1], s1));
+        const double dz = __dsub_rn(val(S.fz[c][rr][cc], s2),
+                                    val(under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc], s3));
+        R[c] = __fma_rn(hx, dx, __dmul_rn(hz, dz));
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; c++) {
+        const i64 dx = S.fx[c][rr][cc] - S.fx[c][rr][cc + 1];
+        const i64 dz = S.fz[c][rr][cc] - (under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc]);
+        R[c] = a.fx.square ? __dmul_rn(a.fx.scale, (double)(dx + dz))
+                           : __fma_rn(a.fx.scale, (double)dx, __dmul_rn(__dmul_rn(hz, s57), (double)dz));
+      }
+    }
+    R[2] = __fma_rn(-g.G, S.q[0][rr + 2][cc + 2], R[2]);
+    R[3] = __fma_rn(-g.G, S.q[2][rr + 2][cc + 2], R[3]);
 
     const size_t row_off = (size_t)k * g.pitch + i;
     if (a.rhs_only) {
 #pragma unroll
-      for (int c = 0; c < 4; c++) a.rhs_out[(size_t)c * plane + row_off] = (double)R[c];
+      for (int c = 0; c < 4; c++) a.rhs_out[(size_t)c * plane + row_off] = R[c];
       return;
     }
-    Store* Ra_w = reinterpret_cast<Store*>(a.b.Ra);
+    double* Ra_w = reinterpret_cast<double*>(a.b.Ra);
     const int st = a.stage;
     const double h2 = g.h2;
     if (GEN) {
@@ -531,7 +738,7 @@ __device__ __noinline__ void stage_tile(const StageArgs& __restrict__ a, int til
 #pragma unroll
       for (int c = 0; c < 4; c++) {
         const size_t o = (size_t)c * plane + row_off;
-        const double r = (double)R[c];
+        const double r = R[c];
         if (!sub_end) Rs[(size_t)p * slot + o] = r;
         if (k >= g.n1_r) {
           if (sub_end) a.qF_next[o] = __fma_rn(g.hF, gen_weighted_sum(g, Rs, slot, o, r), a.qF[o]);
@@ -551,12 +758,12 @@ __device__ __noinline__ void stage_tile(const StageArgs& __restrict__ a, int til
       // fast region: m Heun substeps of dt/m
       if (!(st & 1)) {
 #pragma unroll
-        for (int c = 0; c < 4; c++) Ra_w[(size_t)c * plane + row_off] = (Store)R[c];
+        for (int c = 0; c < 4; c++) Ra_w[(size_t)c * plane + row_off] = R[c];
       } else {
 #pragma unroll
         for (int c = 0; c < 4; c++) {
           const size_t o = (size_t)c * plane + row_off;
-          a.qF_next[o] = a.qF[o] + h2 * ((double)Ra[o] + (double)R[c]);
+          a.qF_next[o] = __fma_rn(h2, __dadd_rn(Ra[o], R[c]), a.qF[o]);
         }
       }
     } else if (k >= g.nS_r) {
@@ -568,13 +775,13 @@ __device__ __noinline__ void stage_tile(const StageArgs& __restrict__ a, int til
       for (int c = 0; c < 4; c++) {
         const size_t o = (size_t)c * plane + row_off;
         double* acc = a.b.accB + (size_t)c * pb + ob;
-        if (!(st & 1)) Ra_w[o] = (Store)R[c];
+        if (!(st & 1)) Ra_w[o] = R[c];
         if (st == 0) {
-          *acc = (double)R[c];
+          *acc = R[c];
         } else if (last) {
-          *acc = a.b.qA[o] + h2 * (*acc + (double)R[c]);
+          *acc = __fma_rn(h2, __dadd_rn(*acc, R[c]), a.b.qA[o]);
         } else {
-          *acc = *acc + (double)R[c];
+          *acc = __dadd_rn(*acc, R[c]);
         }
       }
     } else {
@@ -584,9 +791,9 @@ __device__ __noinline__ void stage_tile(const StageArgs& __restrict__ a, int til
       for (int c = 0; c < 4; c++) {
         const size_t o = (size_t)c * plane + row_off;
         if (st == 0) {
-          Ra_w[o] = (Store)R[c];
+          Ra_w[o] = R[c];
         } else {
-          a.b.accS[(size_t)c * ps + row_off] = a.b.qA[o] + g.hdt * ((double)Ra[o] + (double)R[c]);
+          a.b.accS[(size_t)c * ps + row_off] = __fma_rn(g.hdt, __dadd_rn(Ra[o], R[c]), a.b.qA[o]);
         }
       }
     }

@@ -1,0 +1,104 @@
+"""The FP64 tile's face fluxes run in 64-bit fixed point where the states of a
+face lie in its range (density in [0.5, 4), |momentum| below 0.656, energy in
+[1/16, 4), sound speed squared in [0.26, 3.9]) and in double elsewhere. States
+across every edge of that range match the oracle's right-hand side, and a face
+takes the same form in every tile shape and in the batch kernel.
+
+Tolerance: the parity norm of the FP64 path, 1e-12 of the largest |R| per
+component. Both sides round each flux a few dozen times at 2^-53 of its size;
+the states below have jumps that make R at least 1e-2 of flux / dx, so the
+difference stays below 64 * 2^-53 / 1e-2 = 7e-13."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2202_11890_gb300 import workloads as W
+from pairs import oracle_threads, pair, rel_err
+from test_gpu_parity import gpu_rhs
+from test_gpu_tile_shapes import SHAPES, launch_buckets, load_table
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+GRID = W.Grid(75, 13, 6, 22)  # ragged tiles, Gamma inside a tile
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2202_11890_gb300 import build
+    build.build()
+    oracle_threads()
+
+
+def state(kind):
+    """Random cell-to-cell variations of 2 % over the rest state, changed so
+    that some or all faces leave the fixed-point range."""
+    rng = np.random.default_rng(41)
+    rho, p = W.rest_primitives(GRID)
+    r = [0.02 * rng.uniform(-1, 1, rho.shape) for _ in range(4)]
+    rho, p, u, w = rho * (1 + r[0]), p * (1 + r[1]), r[2], r[3]
+    # ramps 0 to 1 to 0 over columns 20-50 and rows 8-27, across Gamma and
+    # tiles; gentle enough that every reconstructed pressure stays positive
+    ramp = [np.minimum(1.0, 1.3 * (1.0 - np.abs(np.linspace(-1, 1, n)))) for n in (20, 31)]
+    part = np.zeros(rho.shape)
+    part[8:28, 20:51] = np.outer(*ramp)
+    if kind == "dense":  # every cell outside
+        rho, p = 8.0 * rho, 8.0 * p
+    elif kind == "dense patch":  # densities up to 4.4 over the edge 4
+        rho, p = rho * 4.3 ** part, p * 2.0 ** part
+    elif kind == "thin patch":  # densities down to 0.25, below 0.5
+        rho, p = rho * 0.25 ** part, p * 0.4 ** part
+    elif kind == "fast patch":  # momenta up to 1, over 0.656
+        u, w = u + part * np.sign(r[2]), w - 0.7 * part
+    elif kind == "cold patch":  # sound speed squared down to 0.13, energy to 0.2
+        p = p * 0.13 ** part
+    elif kind == "hot patch":  # sound speed squared up to 4.6, energy to 8
+        p = p * 4.5 ** part
+    return W.conserved(rho, u, w, p)
+
+
+KINDS = ["inside", "dense", "dense patch", "thin patch", "fast patch", "cold patch", "hot patch"]
+
+
+@pytest.mark.parametrize("xwall,wall", [(0, 0), (1, 1)])
+@pytest.mark.parametrize("kind", KINDS)
+def test_rhs_across_the_range_matches_oracle(kind, xwall, wall):
+    q = state(kind)
+    cfg, P, _ = pair(GRID, 2, dt=0.001, xwall=xwall, wall=wall)
+    err = rel_err(gpu_rhs(cfg, q), O.rhs(P, q))
+    assert np.all(err < 1e-12), err
+
+
+@pytest.mark.parametrize("mu1,mu2", [(0.03, W.MU2), (W.MU1, 0.08), (0.04, 0.04)])
+def test_viscosity_across_the_range_matches_oracle(mu1, mu2):
+    """Coefficients (8/3) mu / dx around 1, where the fixed-point form ends."""
+    q = state("inside")
+    cfg, P, _ = pair(GRID, 2, dt=0.001, mu1=mu1, mu2=mu2)
+    err = rel_err(gpu_rhs(cfg, q), O.rhs(P, q))
+    assert np.all(err < 1e-12), err
+
+
+@pytest.mark.parametrize("kind", ["dense", "dense patch", "fast patch", "hot patch"])
+def test_same_bits_in_every_tile_shape_and_in_a_batch(kind, tmp_path):
+    from paper_2202_11890_gb300 import mprk as M
+    q = state(kind)
+    cfg, _, _ = pair(GRID, 2, dt=0.001)
+    try:
+        results = []
+        for sh in SHAPES:
+            load_table(tmp_path, M, launch_buckets(GRID, 2), sh)
+            with M.Instance(cfg, q) as inst:
+                inst.step(2)
+                results.append(inst.state())
+        M.mprk_tune_clear()
+        with M.Instance(cfg, q) as inst:
+            M.mprk_step_batch([inst.h], 2)
+            results.append(inst.state())
+    finally:
+        M.mprk_tune_clear()
+    assert np.isfinite(results[0]).all()
+    for r in results[1:]:
+        assert np.array_equal(results[0], r)
