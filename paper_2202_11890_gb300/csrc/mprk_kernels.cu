@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(NT, NT == TX * TZR ? 3 * NTHREADS / NT : 1)
     stage_kernel(const __grid_constant__ StageArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   TileSmem<TZR>& S = *reinterpret_cast<TileSmem<TZR>*>(smem_raw);
+  chain_wait();
   stage_tile<GEN, NT, TZR>(a, blockIdx.x, S);
 }
 
@@ -65,24 +66,24 @@ __global__ void __launch_bounds__(MIXED_THREADS, 3)
 // tile of an x-z plane, blockIdx = (tile column, tile row, plane).
 __global__ void __launch_bounds__(NTHREADS, 2) yface3_kernel(const StageArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  chain_wait();
   yface_tile(a, a.row0 + blockIdx.y * TZ, blockIdx.x * TX, blockIdx.z, *reinterpret_cast<YfaceSmem*>(smem_raw));
 }
 
 __global__ void __launch_bounds__(NTHREADS, 2) stage3_kernel(const StageArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  chain_wait();
   stage_tile3(a, a.row0 + blockIdx.y * TZ, blockIdx.x * TX, blockIdx.z, *reinterpret_cast<Tile3Smem*>(smem_raw));
 }
 
-cudaError_t launch_stage3(const StageArgs& a, cudaStream_t stream) {
+cudaError_t launch_stage3(const StageArgs& a, cudaStream_t stream, bool chained) {
   const int hi = a.rhs_only ? a.rhs_hi : a.g.nz;
   const int tz = (hi - a.row0 + TZ - 1) / TZ;
   if (tz <= 0) return cudaSuccess;
   const dim3 grid(a.tiles_x, tz, a.g.ny);
-  yface3_kernel<<<grid, NTHREADS, sizeof(YfaceSmem), stream>>>(a);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_kernel(yface3_kernel, grid, NTHREADS, sizeof(YfaceSmem), stream, chained, a);
   if (e != cudaSuccess) return e;
-  stage3_kernel<<<grid, NTHREADS, sizeof(Tile3Smem), stream>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(stage3_kernel, grid, NTHREADS, sizeof(Tile3Smem), stream, chained, a);
 }
 
 size_t stage_smem_bytes(int precision) {
@@ -174,17 +175,13 @@ int sm_count() {
 namespace {
 // One FP64 stage launch with TZR-row tiles; wide: two threads per cell.
 template <int TZR>
-void launch_fp64(const StageArgs& a, int n_tiles, bool wide, cudaStream_t stream) {
+cudaError_t launch_fp64(const StageArgs& a, int n_tiles, bool wide, cudaStream_t stream, bool chained) {
   constexpr int NT1 = TX * TZR, NT2 = 2 * TX * TZR;
   const size_t smem = sizeof(TileSmem<TZR>);
-  if (wide && a.g.gen)
-    stage_kernel<true, NT2, TZR><<<n_tiles, NT2, smem, stream>>>(a);
-  else if (wide)
-    stage_kernel<false, NT2, TZR><<<n_tiles, NT2, smem, stream>>>(a);
-  else if (a.g.gen)
-    stage_kernel<true, NT1, TZR><<<n_tiles, NT1, smem, stream>>>(a);
-  else
-    stage_kernel<false, NT1, TZR><<<n_tiles, NT1, smem, stream>>>(a);
+  if (wide && a.g.gen) return launch_kernel(stage_kernel<true, NT2, TZR>, n_tiles, NT2, smem, stream, chained, a);
+  if (wide) return launch_kernel(stage_kernel<false, NT2, TZR>, n_tiles, NT2, smem, stream, chained, a);
+  if (a.g.gen) return launch_kernel(stage_kernel<true, NT1, TZR>, n_tiles, NT1, smem, stream, chained, a);
+  return launch_kernel(stage_kernel<false, NT1, TZR>, n_tiles, NT1, smem, stream, chained, a);
 }
 }  // namespace
 
@@ -203,7 +200,7 @@ TileShape default_tile_shape(const StageArgs& a) {
 }
 
 cudaError_t launch_stage(const StageArgs& a, int precision, int n_tiles, cudaStream_t stream,
-                         const StageMaps* maps, const TileShape* shape) {
+                         const StageMaps* maps, const TileShape* shape, bool chained) {
   if (n_tiles <= 0) return cudaSuccess;
   if (precision == 0) {
     // FP64: the shape given, else the tuned one for the launch's size
@@ -219,9 +216,9 @@ cudaError_t launch_stage(const StageArgs& a, int precision, int n_tiles, cudaStr
     s.tz = ts.rows;
     const int n = stage_tiles(s);
     const bool wide = ts.tpc == 2;
-    if (s.tz == TZ) launch_fp64<TZ>(s, n, wide, stream);
-    else if (s.tz == TZ / 2) launch_fp64<TZ / 2>(s, n, wide, stream);
-    else launch_fp64<TZ / 4>(s, n, wide, stream);
+    if (s.tz == TZ) return launch_fp64<TZ>(s, n, wide, stream, chained);
+    if (s.tz == TZ / 2) return launch_fp64<TZ / 2>(s, n, wide, stream, chained);
+    return launch_fp64<TZ / 4>(s, n, wide, stream, chained);
   } else {
     StageArgs s = a;
     CUtensorMap none;
@@ -417,6 +414,7 @@ cudaError_t launch_shadow(const Geom& g, const double* q, const float* rowc, flo
 // Rows k_lo <= k < k_hi (x-rows r = k ny + j).
 __global__ void finalize_kernel(const Geom g, const Bufs b, int m_odd, int vec, int k_lo, int k_hi) {
   const bool mixed = b.dA != nullptr;
+  chain_wait();
   const int c = blockIdx.z;
   for (int r = k_lo * g.ny + blockIdx.y; r < k_hi * g.ny; r += gridDim.y) {
     const int k = r / g.ny;
@@ -443,7 +441,7 @@ __global__ void finalize_kernel(const Geom g, const Bufs b, int m_odd, int vec, 
   }
 }
 
-cudaError_t launch_finalize(const Geom& g, const Bufs& b, int m_odd, cudaStream_t stream) {
+cudaError_t launch_finalize(const Geom& g, const Bufs& b, int m_odd, cudaStream_t stream, bool chained) {
   const int k_lo = 0;
   const int k_hi = (m_odd || b.dA) ? g.nz : g.n1_r;  // rows it completes
   const int rows = k_hi - k_lo;
@@ -454,8 +452,7 @@ cudaError_t launch_finalize(const Geom& g, const Bufs& b, int m_odd, cudaStream_
                       ? 1
                       : 0;
   const dim3 grid((g.nx + 511) / 512, (unsigned)std::min(rows * g.ny, 65535), (unsigned)g.nc);
-  finalize_kernel<<<grid, 256, 0, stream>>>(g, b, m_odd, vec, k_lo, k_hi);
-  return cudaGetLastError();
+  return launch_kernel(finalize_kernel, grid, 256, 0, stream, chained && !b.dA, g, b, m_odd, vec, k_lo, k_hi);
 }
 
 // ---------------------------------------------------------------------------

@@ -199,23 +199,26 @@ void free_instance(mprk_instance* I) {
 // Enqueue the stage launches and the completion of one slow step.
 // after_launch(j), when given, runs after launch j on s (0-based, stages
 // first, the completion last): the profiling hook records events there.
+// chained: consecutive launches overlap at their ends (not with work of the
+// hook between them).
 template <typename F>
-int enqueue_step_with(mprk_instance* I, cudaStream_t s, F after_launch) {
+int enqueue_step_with(mprk_instance* I, cudaStream_t s, bool chained, F after_launch) {
   const Geom& g = I->g;
   for (int st = 0; st < g.s * g.m; st++) {
     StageArgs a = stage_args(g, I->b, st);
     a.status = I->status_dev;
     a.gy = I->gy;
-    CU(g.ny > 1 ? launch_stage3(a, s) : launch_stage(a, I->precision, stage_tiles(a), s, &I->maps));
+    const bool ch = chained && st > 0;
+    CU(g.ny > 1 ? launch_stage3(a, s, ch) : launch_stage(a, I->precision, stage_tiles(a), s, &I->maps, nullptr, ch));
     CU(after_launch(st));
   }
-  CU(launch_finalize(g, I->b, g.m & 1, s));
+  CU(launch_finalize(g, I->b, g.m & 1, s, chained));
   CU(after_launch(g.s * g.m));
   return MPRK_OK;
 }
 
 int enqueue_step(mprk_instance* I, cudaStream_t s) {
-  return enqueue_step_with(I, s, [](int) { return cudaSuccess; });
+  return enqueue_step_with(I, s, true, [](int) { return cudaSuccess; });
 }
 
 int capture(mprk_instance* I, bool with_diag, cudaGraphExec_t* out) {
@@ -821,7 +824,7 @@ int mprk_profile_step(mprk_instance* I, double* launch_ms, long long* launch_cel
   if (rc == MPRK_OK) {
     cudaError_t e = cudaEventRecordWithFlags(ev[0], I->stream, cudaEventRecordExternal);
     if (e == cudaSuccess)
-      rc = enqueue_step_with(I, I->stream, [&](int j) {
+      rc = enqueue_step_with(I, I->stream, false, [&](int j) {
         return cudaEventRecordWithFlags(ev[j + 1], I->stream, cudaEventRecordExternal);
       });
     const cudaError_t e2 = cudaStreamEndCapture(I->stream, &graph);

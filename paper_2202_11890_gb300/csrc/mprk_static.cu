@@ -192,10 +192,10 @@ int mprk_step_static(const mprk_config* cfg, double* q_dev, int n_slow_steps, vo
   for (int step = 0; step < n_slow_steps; step++) {
     for (int st = 0; st < 2 * g.m; st++) {
       const StageArgs a = stage_args(g, b, st);
-      e = launch_stage(a, cfg->precision, stage_tiles(a), s, &maps);
+      e = launch_stage(a, cfg->precision, stage_tiles(a), s, &maps, nullptr, step > 0 || st > 0);
       if (e != cudaSuccess) return sfail(MPRK_ECUDA, std::string("stage launch: ") + cudaGetErrorString(e));
     }
-    e = launch_finalize(g, b, g.m & 1, s);
+    e = launch_finalize(g, b, g.m & 1, s, true);
     if (e != cudaSuccess) return sfail(MPRK_ECUDA, std::string("completion launch: ") + cudaGetErrorString(e));
   }
   return MPRK_OK;

@@ -32,13 +32,11 @@
 // alone, so results do not depend on the tile shape or the launch.
 #pragma once
 
-#include "fixed_point.cuh"
+#include "fixed_flux.cuh"
 #include "fp64_recip.cuh"
 #include "mprk_internal.h"
 
 namespace mprk {
-
-using fx::i64;
 
 template <int TZR = TZ>
 struct TileSmem {
@@ -163,12 +161,9 @@ __device__ __forceinline__ double gen_weighted_sum(const Geom& g, const double* 
   return __fma_rn(g.bb[g.s - 1], r, sum);
 }
 
-// The stage state lies inside the fixed-point range (fixed_point.cuh)?
-// NaN, zero and negative densities and energies do not.
+// The stage state lies inside the fixed-point range?
 __device__ __forceinline__ bool cell_in_range(double r, double mu, double mw, double E) {
-  const unsigned hr = (unsigned)__double2hiint(r), he = (unsigned)__double2hiint(E);
-  const unsigned hm = max((unsigned)__double2hiint(mu) & 0x7fffffffu, (unsigned)__double2hiint(mw) & 0x7fffffffu);
-  return hr - fx::RHO_LO < fx::RHO_HI - fx::RHO_LO && he - fx::E_LO < fx::E_HI - fx::E_LO && hm < fx::MOM_HI;
+  return in_range(r, max(abs_word(mu), abs_word(mw)), E);
 }
 
 // Cell values of the two arithmetics: i64 (fixed point) or double.
@@ -362,88 +357,6 @@ __device__ __forceinline__ int face_sides(const Geom& g, const TileSmem<TZR>& S,
     o[4] = g.wall ? c[4] : -c[4];
   }
   return (id.isx ? ku : (ku == 0 ? 0 : kd)) >= n1;
-}
-
-// The fixed-point face flux over half the divergence factor (.57), or false
-// where a state leaves the range: F = f(q_L) + f(q_R) + lambda (q_L - q_R)
-// - V, lambda the largest |u_n| + a over the left, right and Roe-averaged
-// states.
-struct FxSide {
-  FxW un, mn;
-  i64 un_, ut, mu, p, c2;  // velocities .59, m_n u_n .57, p .57, c^2 .55
-  i64 k;                   // |m|^2 / rho .57
-  i64 eh;                  // rho E + p .59
-};
-__device__ __forceinline__ void fx_side(const FxConst& k, const i64 q[4], FxSide* s, FxW* mt) {
-  const FxW inv = fx::split(fx::recip(q[0]));
-  s->mn = fx::split(q[1]);
-  *mt = fx::split(q[2]);
-  s->un_ = fx::mul(s->mn, inv);
-  s->ut = fx::mul(*mt, inv);
-  s->un = fx::split(s->un_);
-  s->mu = fx::mul(s->mn, s->un);
-  s->k = s->mu + fx::mul(*mt, fx::split(s->ut));
-  const FxW pe = fx::split(q[3] - (s->k << 2));  // p / (gamma - 1) .60
-  s->p = fx::mul(pe, k.gm1);
-  s->c2 = fx::mul(fx::split(fx::mul(pe, inv)), k.gg);
-  s->eh = (q[3] >> 1) + (s->p << 2);
-}
-
-// The Roe-averaged speed |u_n| + a in double from the two states (rarely
-// needed): w the weight sqrt(rho_R) / (sqrt(rho_L) + sqrt(rho_R)), a^2 =
-// (1 - w) a_L^2 + w a_R^2 + (gamma - 1)/2 w (1 - w) |du|^2, which equals the
-// Roe-averaged enthalpy's (gamma - 1)(H - |u|^2 / 2).
-__device__ __noinline__ i64 fx_roe_speed(i64 rL, i64 rR, i64 unL, i64 unR, i64 dut, i64 c2L, i64 c2R, double gm1) {
-  const double w = recip_f64(__dadd_rn(1.0, sqrt_f64(__dmul_rn((double)rL, recip_f64((double)rR)))));
-  const double sv = 1.0 / (double)(1ll << fx::S_VEL), sc = 1.0 / (double)(1ll << 55);
-  const double du = __dmul_rn((double)(unR - unL), sv), dt = __dmul_rn((double)dut, sv);
-  const double un = __fma_rn(w, du, __dmul_rn((double)unL, sv));
-  const double a = __dmul_rn((double)c2L, sc), d = __dmul_rn((double)(c2R - c2L), sc);
-  const double q = __dmul_rn(__dmul_rn(0.5 * gm1, w), __dsub_rn(1.0, w));
-  const double c2 = __fma_rn(q, __fma_rn(du, du, __dmul_rn(dt, dt)), __fma_rn(w, d, a));
-  return __double2ll_rn(__dmul_rn(__dadd_rn(fabs(un), sqrt_f64(c2)), (double)(1ll << fx::S_VEL)));
-}
-
-__device__ __forceinline__ bool fx_flux(const Geom& g, const FxConst& k, const i64 L[4], const i64 R[4], const i64 V[3], i64 F[4]) {
-  FxSide l, r;
-  FxW mtL, mtR;
-  fx_side(k, L, &l, &mtL);
-  fx_side(k, R, &r, &mtR);
-  const int c2l = (int)(l.c2 >> 32), c2r = (int)(r.c2 >> 32);
-  if (min((int)(L[0] >> 32), (int)(R[0] >> 32)) < fx::RHO_MIN ||
-      max((int)(l.k >> 32), (int)(r.k >> 32)) >= fx::KIN_MAX || min(c2l, c2r) < fx::C2_MIN ||
-      max(c2l, c2r) >= fx::C2_MAX)
-    return false;
-  const i64 cl = fx::sqroot(l.c2 << 6), cr = fx::sqroot(r.c2 << 6);
-  const i64 sl = (l.un_ < 0 ? -l.un_ : l.un_) + cl, sr = (r.un_ < 0 ? -r.un_ : r.un_) + cr;
-  i64 lam = sl > sr ? sl : sr;  // .59
-  {
-    // The Roe speed lies below (1 - w) sl + w sr + w (1 - w) / (2 min a) D
-    // with D = (a_L - a_R)^2 + (gamma - 1)/2 |du|^2, so it cannot be the
-    // largest where |sl - sr| max(1, ...) >= D (min a > 0.5, w in [0.2, 0.8]
-    // within the range): all but a few faces of a smooth flow skip it.
-    const float k59 = 5.7646075e17f;
-    const float df = fx::to_float(sl - sr), dc = fx::to_float(cl - cr), dn = fx::to_float(l.un_ - r.un_),
-                dt = fx::to_float(l.ut - r.ut);
-    if (fabsf(df) * k59 < fmaf(dc, dc, 0.5f * g.gm1f * fmaf(dn, dn, dt * dt))) {
-      const i64 roe = fx_roe_speed(L[0], R[0], l.un_, r.un_, r.ut - l.ut, l.c2, r.c2, g.gm1);
-      lam = roe > lam ? roe : lam;
-    }
-  }
-  const FxW lam59 = fx::split(lam), lam61 = fx::split(lam << 2);
-  F[0] = (L[1] >> 5) + (R[1] >> 5) + fx::mul(fx::split(L[0] - R[0]), lam61);
-  F[1] = (l.mu + l.p) + (r.mu + r.p) + fx::mul(fx::split(L[1] - R[1]), lam59) - V[0];
-  F[2] = fx::mul2(mtL, l.un, mtR, r.un) + fx::mul(fx::split(L[2] - R[2]), lam59) - V[1];
-  F[3] = fx::mul(fx::split(l.eh), fx::split(l.un_ << 3)) + fx::mul(fx::split(r.eh), fx::split(r.un_ << 3)) +
-         fx::mul(fx::split(L[3] - R[3]), lam61) - V[2];
-  // room for the sums of phase 5: |F| < 8
-  int top = 0;
-#pragma unroll
-  for (int c = 0; c < 4; c++) {
-    const int h = (int)(F[c] >> 32);
-    top |= h ^ (h >> 31);
-  }
-  return top < (8 << (fx::S_FLUX - 32));
 }
 
 // The viscous flux over half the divergence factor from the common values of
@@ -672,7 +585,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
       } else {
         fx_visc(a.fx.fc[id.isx ? 0 : 1][fl], vL, vR, V);
       }
-      ok = fx_flux(g, a.fx, L, R, V, F);
+      ok = fx_flux<2>(g, a.fx, L, R, V, F);
       if (ok) store_flux(S, id, F);
     }
     S.slow[e] = !ok;
