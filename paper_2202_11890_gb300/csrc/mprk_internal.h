@@ -67,6 +67,24 @@ struct FxConst {
   FxW fc[2][2][FXC_N]; // viscous coefficients per direction (x, z) and fluid, .62
 };
 
+// The same of the 3-D tiles: directions x (tangents y, z), y (x, z) and z
+// (x, y), the coefficients in fixed point and in double.
+enum {
+  F3_A,   // (8/3) mu / d_n: sigma_nn from the normal difference of u_n
+  F3_B1,  // -mu / (3 d_t1): sigma_nn from the differences of u_t1 along t1
+  F3_B2,  // -mu / (3 d_t2): of u_t2 along t2
+  F3_C,   // 2 mu / d_n: sigma_nt from the normal difference of u_t
+  F3_D1,  // mu / (2 d_t1): sigma_nt1 from the differences of u_n along t1
+  F3_D2,  // mu / (2 d_t2)
+  F3_K,   // 2 kappa gamma (gamma - 1) / d_n: heat flux from the difference of e
+  F3_N
+};
+struct Fx3Const {
+  FxConst k;  // its fc unused; square: dx = dy = dz1 = dz2
+  FxW fc[3][2][F3_N];
+  double fd[3][2][F3_N];
+};
+
 // Physics and grid of one instance, constant over its life.
 struct Geom {
   int nx, pitch, nz;
@@ -154,6 +172,7 @@ __host__ __device__ inline double visc_coef(const Geom& g, int dir, int fl, int 
 }
 // Fills the fixed-point constants of a geometry (mprk_runtime.cu).
 void fixed_point_const(const Geom& g, FxConst* out);
+void fixed_point_const3(const Geom& g, Fx3Const* out);
 
 // Arguments of stage st of one slow step: F rows ping-pong between the A and
 // B buffers at every fast substep.

@@ -64,16 +64,19 @@ __global__ void __launch_bounds__(MIXED_THREADS, 3)
 // 3-D stage (App. B in full): the y faces of a plane pair, then the x and z
 // faces, the divergence and the combination of a plane; one CTA per TX x TZ
 // tile of an x-z plane, blockIdx = (tile column, tile row, plane).
-__global__ void __launch_bounds__(NTHREADS, 2) yface3_kernel(const StageArgs a) {
+// Three CTAs per SM in both (80 registers; 52 and 72 KB of shared memory).
+__global__ void __launch_bounds__(NTHREADS, 3)
+    yface3_kernel(const __grid_constant__ StageArgs a, const __grid_constant__ Fx3Const C) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   chain_wait();
-  yface_tile(a, a.row0 + blockIdx.y * TZ, blockIdx.x * TX, blockIdx.z, *reinterpret_cast<YfaceSmem*>(smem_raw));
+  yface_tile(a, C, a.row0 + blockIdx.y * TZ, blockIdx.x * TX, blockIdx.z, *reinterpret_cast<YfaceSmem*>(smem_raw));
 }
 
-__global__ void __launch_bounds__(NTHREADS, 2) stage3_kernel(const StageArgs a) {
+__global__ void __launch_bounds__(NTHREADS, 3)
+    stage3_kernel(const __grid_constant__ StageArgs a, const __grid_constant__ Fx3Const C) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   chain_wait();
-  stage_tile3(a, a.row0 + blockIdx.y * TZ, blockIdx.x * TX, blockIdx.z, *reinterpret_cast<Tile3Smem*>(smem_raw));
+  stage_tile3(a, C, a.row0 + blockIdx.y * TZ, blockIdx.x * TX, blockIdx.z, *reinterpret_cast<Tile3Smem*>(smem_raw));
 }
 
 cudaError_t launch_stage3(const StageArgs& a, cudaStream_t stream, bool chained) {
@@ -81,9 +84,11 @@ cudaError_t launch_stage3(const StageArgs& a, cudaStream_t stream, bool chained)
   const int tz = (hi - a.row0 + TZ - 1) / TZ;
   if (tz <= 0) return cudaSuccess;
   const dim3 grid(a.tiles_x, tz, a.g.ny);
-  cudaError_t e = launch_kernel(yface3_kernel, grid, NTHREADS, sizeof(YfaceSmem), stream, chained, a);
+  Fx3Const C;
+  fixed_point_const3(a.g, &C);
+  cudaError_t e = launch_kernel(yface3_kernel, grid, NTHREADS, sizeof(YfaceSmem), stream, chained, a, C);
   if (e != cudaSuccess) return e;
-  return launch_kernel(stage3_kernel, grid, NTHREADS, sizeof(Tile3Smem), stream, chained, a);
+  return launch_kernel(stage3_kernel, grid, NTHREADS, sizeof(Tile3Smem), stream, true, a, C);
 }
 
 size_t stage_smem_bytes(int precision) {

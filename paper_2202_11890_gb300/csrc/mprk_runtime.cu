@@ -323,34 +323,63 @@ static void set_base(int base, Geom* g) {
   g->gen = base != MPRK_BASE_RK2;
 }
 
+// x as a fixed-point factor with `digits` digits after the point.
+static FxW fx_factor(double x, int digits) {
+  const long long v = llround(ldexp(x, digits));
+  FxW w;
+  w.lo = (int)(unsigned)(v & 0xffffffffll);
+  w.hi = (int)((v - w.lo) >> 32);
+  return w;
+}
+// The constants shared by 2-D and 3-D, with `on` and `square` clear; false
+// where gamma does not fit.
+static bool fx_gas(const Geom& g, FxConst* out) {
+  *out = FxConst{};
+  out->scale = ldexp(0.5 * g.inv_dx, -57);
+  const double gg = g.gamma * g.gm1;
+  if (!(gg < 1.9)) return false;
+  out->gm1 = fx_factor(g.gm1, 61);
+  out->gg = fx_factor(gg, 62);
+  return true;
+}
+
 // The fixed-point form needs gamma (gamma - 1) < 1.9 and every viscous
 // coefficient (the inverse of a cell Reynolds number; 0.1 at 2048 columns)
 // below 1, so that each fits its scale with a bit to spare; otherwise the
 // tile's faces run in double.
 void mprk::fixed_point_const(const Geom& g, FxConst* out) {
-  auto factor = [](double x, int digits) {
-    const long long v = llround(ldexp(x, digits));
-    FxW w;
-    w.lo = (int)(unsigned)(v & 0xffffffffll);
-    w.hi = (int)((v - w.lo) >> 32);
-    return w;
-  };
   FxConst& f = *out;
-  f = FxConst{};
+  bool ok = fx_gas(g, out);
   f.square = g.inv_dx == g.inv_dz1 && g.inv_dx == g.inv_dz2;
-  f.scale = ldexp(0.5 * g.inv_dx, -57);
-  const double gg = g.gamma * g.gm1;
-  if (!(gg < 1.9)) return;
   for (int dir = 0; dir < 2; dir++)
     for (int fl = 0; fl < 2; fl++)
       for (int j = 0; j < FXC_N; j++) {
         const double x = visc_coef(g, dir, fl, j);
-        if (!(std::fabs(x) < 1.0)) return;
-        f.fc[dir][fl][j] = factor(x, 62);
+        ok = ok && std::fabs(x) < 1.0;  // false for NaN
+        if (ok) f.fc[dir][fl][j] = fx_factor(x, 62);
       }
-  f.gm1 = factor(g.gm1, 61);
-  f.gg = factor(gg, 62);
-  f.on = 1;
+  f.on = ok;
+}
+
+void mprk::fixed_point_const3(const Geom& g, Fx3Const* out) {
+  Fx3Const& f = *out;
+  bool ok = fx_gas(g, &f.k);
+  f.k.square = g.inv_dx == g.inv_dy && g.inv_dx == g.inv_dz1 && g.inv_dx == g.inv_dz2;
+  for (int dir = 0; dir < 3; dir++)
+    for (int fl = 0; fl < 2; fl++) {
+      const double iz = fl ? g.inv_dz2 : g.inv_dz1, mu = fl ? g.mu2 : g.mu1, kap = fl ? g.kap2 : g.kap1;
+      const double in = dir == 0 ? g.inv_dx : dir == 1 ? g.inv_dy : iz;
+      const double i1 = dir == 0 ? g.inv_dy : g.inv_dx, i2 = dir == 2 ? g.inv_dy : iz;
+      const double v[F3_N] = {8.0 / 3.0 * mu * in, -mu * i1 / 3.0, -mu * i2 / 3.0,          2.0 * mu * in,
+                              0.5 * mu * i1,       0.5 * mu * i2,  2.0 * kap * g.gamma * g.gm1 * in};
+      for (int j = 0; j < F3_N; j++) {
+        f.fd[dir][fl][j] = v[j];
+        f.fc[dir][fl][j] = FxW{};
+        ok = ok && std::fabs(v[j]) < 1.0;
+        if (ok) f.fc[dir][fl][j] = fx_factor(v[j], 62);
+      }
+    }
+  f.k.on = ok;
 }
 
 void mprk::geom_from_config(const mprk_config& c, int pitch, Geom* gp) {

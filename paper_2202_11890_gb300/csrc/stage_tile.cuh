@@ -61,12 +61,12 @@ struct TileSmem {
 // Lax–Friedrichs flux in the face frame, in double (faces outside the
 // fixed-point range). A state is (rho, m_n, m_t, rho E): m_n is the momentum
 // along the face normal, m_t along the face. Output is f(q_L) + f(q_R) +
-// lambda (q_L - q_R) - sub: sub carries the viscous or interface part.
+// lambda (q_L - q_R) - V: V the viscous or interface part of (m_n, m_t, rho E).
 // lambda is the largest |u_n| + a over the left, right and Roe-averaged
 // states (Sec. 2.1); the Roe weights sqrt(rho)/(sqrt(rho_L) + sqrt(rho_R))
 // times the enthalpy H = (rho E + p)/rho are formed as (rho E + p)/sqrt(rho).
 __device__ __forceinline__ void lf_face(double lr, double lmn, double lmt, double lE, double rr, double rmn, double rmt,
-                                        double rE, double gamma, double gm1, const double sub[4], double out[4]) {
+                                        double rE, double gamma, double gm1, const double V[3], double out[4]) {
   const double rsL = rsqrt_f64(lr), rsR = rsqrt_f64(rr);
   const double invL = __dmul_rn(rsL, rsL), invR = __dmul_rn(rsR, rsR);
   const double sL = __dmul_rn(lr, rsL), sR = __dmul_rn(rr, rsR);  // sqrt(rho)
@@ -83,10 +83,11 @@ __device__ __forceinline__ void lf_face(double lr, double lmn, double lmt, doubl
   const double H = __dmul_rn(__fma_rn(eR, rsR, __dmul_rn(eL, rsL)), den);
   const double c = sqrt_f64(__dmul_rn(gm1, __fma_rn(-0.5, __fma_rn(ut, ut, __dmul_rn(un, un)), H)));
   const double lam = max_speed(max_speed(__dadd_rn(fabs(unL), cL), __dadd_rn(fabs(unR), cR)), __dadd_rn(fabs(un), c));
-  out[0] = __dsub_rn(__fma_rn(lam, __dsub_rn(lr, rr), __dadd_rn(lmn, rmn)), sub[0]);
-  out[1] = __dsub_rn(__fma_rn(lam, __dsub_rn(lmn, rmn), __dadd_rn(__fma_rn(lmn, unL, pL), __fma_rn(rmn, unR, pR))), sub[1]);
-  out[2] = __dsub_rn(__fma_rn(lam, __dsub_rn(lmt, rmt), __fma_rn(rmt, unR, __dmul_rn(lmt, unL))), sub[2]);
-  out[3] = __dsub_rn(__fma_rn(lam, __dsub_rn(lE, rE), __fma_rn(unR, eR, __dmul_rn(unL, eL))), sub[3]);
+  out[0] = __fma_rn(lam, __dsub_rn(lr, rr), __dadd_rn(lmn, rmn));
+  const double f1 = __dsub_rn(__dadd_rn(__fma_rn(lmn, unL, pL), __fma_rn(rmn, unR, pR)), V[0]);
+  out[1] = __fma_rn(lam, __dsub_rn(lmn, rmn), f1);
+  out[2] = __fma_rn(lam, __dsub_rn(lmt, rmt), __fma_rn(rmt, unR, __fma_rn(lmt, unL, -V[1])));
+  out[3] = __fma_rn(lam, __dsub_rn(lE, rE), __fma_rn(unR, eR, __fma_rn(unL, eL, -V[2])));
 }
 
 // Viscous flux in the face frame from the common values of App. B: face
@@ -374,8 +375,7 @@ __device__ __forceinline__ void fx_visc(const FxW* fc, const i64 vL[5], const i6
 // The same flux in double.
 __device__ __forceinline__ void double_flux(const Geom& g, const double L[4], const double R[4], const double V[3],
                                             double F[4]) {
-  const double sub[4] = {0.0, V[0], V[1], V[2]};
-  lf_face(L[0], L[1], L[2], L[3], R[0], R[1], R[2], R[3], g.gamma, g.gm1, sub, F);
+  lf_face(L[0], L[1], L[2], L[3], R[0], R[1], R[2], R[3], g.gamma, g.gm1, V, F);
 }
 __device__ __forceinline__ void double_visc(const double* fc, const double vL[5], const double vR[5], double V[3]) {
   V[0] = __fma_rn(fc[FXC_A], __dsub_rn(vR[0], vL[0]), __dmul_rn(fc[FXC_B], __dadd_rn(vL[4], vR[4])));
@@ -424,10 +424,13 @@ __device__ __noinline__ bool face_in_range(const Geom& g, const TileSmem<TZR>& S
   return ok;
 }
 
-// The faces marked slow, in double: phases 2 and 3 again as doubles (in the
-// same storage), then their fluxes. Ends with the tile's barrier.
+// The faces marked slow (all: every face), in double: phases 2 and 3 again as
+// doubles (in the same storage), then their fluxes. Ends with the tile's
+// barrier. A grid wholly outside the range runs about as fast as the tile
+// that did everything in double (2048 x 1024, m = 8: 12.0 ms per step
+// against 11.7).
 template <int NT, int TZR>
-__device__ __noinline__ void slow_faces(const Geom& g, TileSmem<TZR>& S, int k0, int i0, int row_hi) {
+__device__ __noinline__ void slow_faces(const Geom& g, TileSmem<TZR>& S, int k0, int i0, int row_hi, bool all) {
   ring_phase<double, NT, TZR>(g, S, k0, i0);
   if (threadIdx.x < 4 * FXC_N) {
     const int j = threadIdx.x % FXC_N, f = threadIdx.x / FXC_N;
@@ -438,7 +441,8 @@ __device__ __noinline__ void slow_faces(const Geom& g, TileSmem<TZR>& S, int k0,
   __syncthreads();
   for (int e = threadIdx.x; e < TileSmem<TZR>::NZF + TileSmem<TZR>::NXF + TX; e += NT) {
     FaceId id;
-    if (!face_id<TZR>(g, e, k0, row_hi, &id) || !S.slow[e]) continue;
+    if (!face_id<TZR>(g, e, k0, row_hi, &id) || !(all || S.slow[e])) continue;
+    if (all) S.slow[e] = 1;
     double L[4], R[4], vL[5], vR[5], V[3], F[4];
     const int fl = face_sides<double, TZR>(g, S, id, L, R, vL, vR);
     if (fl >= 2) {
@@ -499,7 +503,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
   };
 
   // ---- 1. stage state of the tile and its halo --------------------------
-  bool bad = !a.fx.on;  // some cell outside the fixed-point range
+  bool bad = !a.fx.on, good = false;  // some cell outside, inside the fixed-point range
   for (int e = tid; e < (TZR + 4) * (TX + 4); e += NT) {
     const int rr = e / (TX + 4), cc = e - rr * (TX + 4);
     const int k = k0 - 2 + rr;
@@ -510,7 +514,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
 #pragma unroll
       for (int c = 0; c < 4; c++) val[c] = stage_value(c, k, i);
       if (gh) val[1] = -val[1];  // mirror state beyond an x wall
-      bad |= !cell_in_range(val[0], val[1], val[2], val[3]);
+      const bool in = cell_in_range(val[0], val[1], val[2], val[3]);
+      bad |= !in;
+      good |= in;
     }
 #pragma unroll
     for (int c = 0; c < 4; c++) {
@@ -521,9 +527,11 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
   }
   const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZR);
   bad = __syncthreads_or(bad);
+  bool none = false;  // no cell inside: every face in double
+  if (bad) none = !a.fx.on || !__syncthreads_or(good);
 
   // ---- 2. u, w, e on the one-cell ring; interface state ------------------
-  ring_phase<i64, NT, TZR>(g, S, k0, i0);
+  if (!none) ring_phase<i64, NT, TZR>(g, S, k0, i0);
   if (has_gamma) {
     bool lid_bad = false;
     if (tid < TX + 2) {
@@ -564,17 +572,19 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
   }
 
   // ---- 3. tangential differences ------------------------------------------
-  diff_phase<i64, NT, TZR>(g, S, k0, row_hi);
-  __syncthreads();
+  if (!none) {
+    diff_phase<i64, NT, TZR>(g, S, k0, row_hi);
+    __syncthreads();
+  }
 
   // ---- 4. face fluxes ----------------------------------------------------
   constexpr int NZF = TileSmem<TZR>::NZF, NXF = TileSmem<TZR>::NXF;
   bool slow = false;
   const int n_faces = NZF + NXF + (has_gamma ? TX : 0);
-  for (int e = tid; e < n_faces; e += NT) {
+  for (int e = none ? n_faces : tid; e < n_faces; e += NT) {
     FaceId id;
     if (!face_id<TZR>(g, e, k0, row_hi, &id)) continue;
-    bool ok = !bad || (a.fx.on && face_in_range<TZR>(g, S, id, k0));
+    bool ok = !bad || face_in_range<TZR>(g, S, id, k0);
     if (ok) {
       i64 L[4], R[4], vL[5], vR[5], V[3], F[4];
       const int fl = face_sides<i64, TZR>(g, S, id, L, R, vL, vR);
@@ -591,8 +601,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
     S.slow[e] = !ok;
     slow |= !ok;
   }
-  slow = __syncthreads_or(slow);
-  if (slow) slow_faces<NT, TZR>(g, S, k0, i0, row_hi);
+  slow = none || __syncthreads_or(slow);
+  if (slow) slow_faces<NT, TZR>(g, S, k0, i0, row_hi, none);
 
   // ---- 5. R = -div F* + s and the stage combination ----------------------
   {
@@ -610,7 +620,15 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
       s2 = S.slow[rr * TX + cc];
       s3 = S.slow[under_gamma ? NZF + NXF + cc : (rr + 1) * TX + cc];
     }
-    if (s0 || s1 || s2 || s3) {
+    if (s0 && s1 && s2 && s3) {
+#pragma unroll
+      for (int c = 0; c < 4; c++) {
+        auto val = [&](i64 f) { return __longlong_as_double(f); };
+        const double dx = __dsub_rn(val(S.fx[c][rr][cc]), val(S.fx[c][rr][cc + 1]));
+        const double dz = __dsub_rn(val(S.fz[c][rr][cc]), val(under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc]));
+        R[c] = __fma_rn(hx, dx, __dmul_rn(hz, dz));
+      }
+    } else if (s0 || s1 || s2 || s3) {
 #pragma unroll
       for (int c = 0; c < 4; c++) {
         auto val = [&](i64 f, bool sl) { return sl ? __longlong_as_double(f) : __dmul_rn((double)f, s57); };

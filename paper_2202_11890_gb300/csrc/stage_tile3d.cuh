@@ -5,7 +5,7 @@
 //
 // A stage is two launches over the active rows:
 //  * yface3: one CTA per TX x TZ tile of an x–z plane j computes the y-face
-//    fluxes G* between planes j and j+1 of its cells and stores G*/dy (face
+//    fluxes G* between planes j and j+1 of its cells and stores them (face
 //    j+1/2 at index j) in a state-sized buffer;
 //  * stage3: one CTA per TX x TZ tile of plane j computes its x and z faces
 //    as the 2-D tile does, takes the y divergence from the stored y faces,
@@ -14,12 +14,18 @@
 // of App. B: mean velocity, two-point normal derivatives, tangential
 // derivatives averaged from the two cells' central differences, sigma =
 // mu (grad u + grad u^T - 2/3 div u I), heat flux -kappa grad T.
-// Central differences are stored unscaled; their factors (1/4 for the
-// reconstruction, 1/(2 d) for a derivative), the viscosity and the
-// divergence's 1/dx, 1/dy, 1/dz are folded into per-face constants, so each
-// face flux comes out multiplied by 1/d of its normal direction.
+//
+// As in the 2-D tile, velocities, differences and fluxes run in 64-bit fixed
+// point (fixed_point.cuh), because the double pipe bound both kernels (80 to
+// 86 % busy with 125 + 238 operations per cell). Measured: a slow step of
+// 512 x 64 x 200 cells with m = 4 44.1 -> 9.7 ms. A face whose own cells leave
+// the range is evaluated in double by a second pass over the tile; which form
+// a face takes depends on its cells alone, so neighbouring tiles agree on the
+// faces they share. Fluxes come over half the divergence factor of their
+// direction, as .57 integers or as doubles (flux_tag).
 #pragma once
 
+#include "fixed_flux.cuh"
 #include "fp64_recip.cuh"
 #include "mprk_internal.h"
 
@@ -27,93 +33,46 @@ namespace mprk {
 
 constexpr int NC3 = 5;
 
-// Face constants of one face direction in one fluid: sc = 1/d_n is the
-// divergence factor, d_n, d_t1, d_t2 the spacings normal to the face and
-// along its two tangents.
-enum {
-  F3_HS,  // sc / 2
-  F3_A,   // (4/3) mu sc / d_n
-  F3_B1,  // mu sc / (6 d_t1)
-  F3_B2,  // mu sc / (6 d_t2)
-  F3_C,   // mu sc / d_n
-  F3_D1,  // mu sc / (4 d_t1)
-  F3_D2,  // mu sc / (4 d_t2)
-  F3_K,   // kappa sc / d_n
-  F3_SC,  // sc
-  F3_N
-};
-
-// The constants of a face with normal spacing inv_dn (= sc) and tangential
-// spacings inv_dt1, inv_dt2 (reciprocals) into fc[F3_N].
-__device__ __forceinline__ void face_consts3(double inv_dn, double inv_dt1, double inv_dt2, double mu, double kap,
-                                             double* fc) {
-  const double sc = inv_dn;
-  fc[F3_HS] = 0.5 * sc;
-  fc[F3_A] = 4.0 / 3.0 * mu * inv_dn * sc;
-  fc[F3_B1] = mu * inv_dt1 * sc / 6.0;
-  fc[F3_B2] = mu * inv_dt2 * sc / 6.0;
-  fc[F3_C] = mu * inv_dn * sc;
-  fc[F3_D1] = 0.25 * mu * inv_dt1 * sc;
-  fc[F3_D2] = 0.25 * mu * inv_dt2 * sc;
-  fc[F3_K] = kap * inv_dn * sc;
-  fc[F3_SC] = sc;
-}
-
-// Lax–Friedrichs flux (Sec. 2.1) in a face frame, times sc = 2 hs: a state
-// is (rho, m_n, m_t1, m_t2, rho E); lambda is the largest |u_n| + a over the
-// left, right and Roe-averaged states. The Roe weights times the enthalpy
-// (rho E + p)/rho are formed as (rho E + p)/sqrt(rho).
-__device__ __forceinline__ void lf_face5(const double l[5], const double r[5], double gamma, double gm1, double hs,
-                                         double out[5]) {
+// Lax–Friedrichs flux (Sec. 2.1) in a face frame, in double: a state is (rho,
+// m_n, m_t1, m_t2, rho E); lambda is the largest |u_n| + a over the left,
+// right and Roe-averaged states. The Roe weights times the enthalpy
+// (rho E + p)/rho are formed as (rho E + p)/sqrt(rho). V: the viscous part.
+__device__ __forceinline__ void lf_face5(const double l[5], const double r[5], double gamma, double gm1,
+                                         const double V[4], double out[5]) {
   const double rsL = rsqrt_f64(l[0]), rsR = rsqrt_f64(r[0]);
-  const double invL = rsL * rsL, invR = rsR * rsR;
-  const double sL = l[0] * rsL, sR = r[0] * rsR;  // sqrt(rho)
-  const double unL = l[1] * invL, t1L = l[2] * invL, t2L = l[3] * invL;
-  const double unR = r[1] * invR, t1R = r[2] * invR, t2R = r[3] * invR;
-  const double pL = gm1 * (l[4] - 0.5 * (l[1] * unL + l[2] * t1L + l[3] * t2L));
-  const double pR = gm1 * (r[4] - 0.5 * (r[1] * unR + r[2] * t1R + r[3] * t2R));
-  const double XL = gamma * pL * invL, XR = gamma * pR * invR;
-  const double cL = XL * rsqrt_f64(XL), cR = XR * rsqrt_f64(XR);
-  const double eL = l[4] + pL, eR = r[4] + pR;
-  const double den = recip_f64(sL + sR);
-  const double un = (sL * unL + sR * unR) * den;
-  const double t1 = (sL * t1L + sR * t1R) * den;
-  const double t2 = (sL * t2L + sR * t2R) * den;
-  const double H = (eL * rsL + eR * rsR) * den;
-  const double X = gm1 * (H - 0.5 * (un * un + t1 * t1 + t2 * t2));
-  const double c = X * rsqrt_f64(X);
-  const double lam = max_speed(max_speed(fabs(unL) + cL, fabs(unR) + cR), fabs(un) + c);
-  const double hl = hs * lam;
-  out[0] = hs * (l[1] + r[1]) + hl * (l[0] - r[0]);
-  out[1] = hs * ((l[1] * unL + pL) + (r[1] * unR + pR)) + hl * (l[1] - r[1]);
-  out[2] = hs * (l[2] * unL + r[2] * unR) + hl * (l[2] - r[2]);
-  out[3] = hs * (l[3] * unL + r[3] * unR) + hl * (l[3] - r[3]);
-  out[4] = hs * (unL * eL + unR * eR) + hl * (l[4] - r[4]);
+  const double invL = __dmul_rn(rsL, rsL), invR = __dmul_rn(rsR, rsR);
+  const double sL = __dmul_rn(l[0], rsL), sR = __dmul_rn(r[0], rsR);  // sqrt(rho)
+  const double unL = __dmul_rn(l[1], invL), t1L = __dmul_rn(l[2], invL), t2L = __dmul_rn(l[3], invL);
+  const double unR = __dmul_rn(r[1], invR), t1R = __dmul_rn(r[2], invR), t2R = __dmul_rn(r[3], invR);
+  const double kL = __fma_rn(l[3], t2L, __fma_rn(l[2], t1L, __dmul_rn(l[1], unL)));
+  const double kR = __fma_rn(r[3], t2R, __fma_rn(r[2], t1R, __dmul_rn(r[1], unR)));
+  const double pL = __dmul_rn(gm1, __fma_rn(-0.5, kL, l[4])), pR = __dmul_rn(gm1, __fma_rn(-0.5, kR, r[4]));
+  const double cL = sqrt_f64(__dmul_rn(__dmul_rn(gamma, pL), invL));
+  const double cR = sqrt_f64(__dmul_rn(__dmul_rn(gamma, pR), invR));
+  const double eL = __dadd_rn(l[4], pL), eR = __dadd_rn(r[4], pR);
+  const double den = recip_f64(__dadd_rn(sL, sR));
+  const double un = __dmul_rn(__fma_rn(sR, unR, __dmul_rn(sL, unL)), den);
+  const double t1 = __dmul_rn(__fma_rn(sR, t1R, __dmul_rn(sL, t1L)), den);
+  const double t2 = __dmul_rn(__fma_rn(sR, t2R, __dmul_rn(sL, t2L)), den);
+  const double H = __dmul_rn(__fma_rn(eR, rsR, __dmul_rn(eL, rsL)), den);
+  const double k = __fma_rn(t2, t2, __fma_rn(t1, t1, __dmul_rn(un, un)));
+  const double c = sqrt_f64(__dmul_rn(gm1, __fma_rn(-0.5, k, H)));
+  const double lam = max_speed(max_speed(__dadd_rn(fabs(unL), cL), __dadd_rn(fabs(unR), cR)), __dadd_rn(fabs(un), c));
+  out[0] = __fma_rn(lam, __dsub_rn(l[0], r[0]), __dadd_rn(l[1], r[1]));
+  const double f1 = __dsub_rn(__dadd_rn(__fma_rn(l[1], unL, pL), __fma_rn(r[1], unR, pR)), V[0]);
+  out[1] = __fma_rn(lam, __dsub_rn(l[1], r[1]), f1);
+  out[2] = __fma_rn(lam, __dsub_rn(l[2], r[2]), __fma_rn(r[2], unR, __fma_rn(l[2], unL, -V[1])));
+  out[3] = __fma_rn(lam, __dsub_rn(l[3], r[3]), __fma_rn(r[3], unR, __fma_rn(l[3], unL, -V[2])));
+  out[4] = __fma_rn(lam, __dsub_rn(l[4], r[4]), __fma_rn(unR, eR, __fma_rn(unL, eL, -V[3])));
 }
 
-// One side of a face in its frame: velocity (u_n, u_t1, u_t2), T, and the
-// cell's central differences (unscaled) of the velocity along t1 (d1) and
-// t2 (d2).
+// One side of a face in its frame: velocity (u_n, u_t1, u_t2), e = T / (gamma
+// (gamma - 1)), and the cell's central differences (unscaled) of u_n and u_t1
+// along t1 (g1) and of u_n and u_t2 along t2 (g2).
+template <typename T>
 struct VSide {
-  double u[3], T, d1[3], d2[3];
+  T u[3], e, g1[2], g2[2];
 };
-
-// Viscous flux in the face frame, times sc: (0, sigma_nn, sigma_nt1,
-// sigma_nt2, u^.sigma_n + kappa dT/dn). With G[a][b] = d u_a / d x_b
-// (b = normal, t1, t2): sigma_nn = mu (4/3 G00 - 2/3 (G11 + G22)),
-// sigma_nt = mu (G_t0 + G_0t); the derivative factors sit in fc.
-__device__ __forceinline__ void visc_face5(const VSide& L, const VSide& R, const double* fc, double out[5]) {
-  const double snn = fc[F3_A] * (R.u[0] - L.u[0]) - fc[F3_B1] * (L.d1[1] + R.d1[1]) -
-                     fc[F3_B2] * (L.d2[2] + R.d2[2]);
-  const double snt1 = fc[F3_C] * (R.u[1] - L.u[1]) + fc[F3_D1] * (L.d1[0] + R.d1[0]);
-  const double snt2 = fc[F3_C] * (R.u[2] - L.u[2]) + fc[F3_D2] * (L.d2[0] + R.d2[0]);
-  out[0] = 0.0;
-  out[1] = snn;
-  out[2] = snt1;
-  out[3] = snt2;
-  out[4] = 0.5 * ((L.u[0] + R.u[0]) * snn + (L.u[1] + R.u[1]) * snt1 + (L.u[2] + R.u[2]) * snt2) +
-           fc[F3_K] * (R.T - L.T);
-}
 
 // ---- shared helpers --------------------------------------------------------
 
@@ -142,498 +101,730 @@ __device__ __forceinline__ int wrap3(int i, int n) {
 }
 
 // The stage value (q_n, or q_n + h R_a on the second stage of a substep) of
-// component c at (k, j, i); the full state given by rhs_in for the test hook.
-__device__ __forceinline__ double stage_val3(const StageArgs& a, const Geo3& G, int c, int k, int j, int i) {
-  const size_t o = G.at(c, k, j, i);
-  if (a.rhs_only) return a.rhs_in[o];
+// every component at (k, j, i); the full state given by rhs_in for the test
+// hook.
+__device__ __forceinline__ void stage_val3(const StageArgs& a, const Geo3& G, int k, int j, int i, double q[5]) {
   const Geom& g = a.g;
-  const double* base = k < g.n1_r ? a.b.qA : a.qF;
+  const bool slow = k < g.n1_r;
+  const double* base = a.rhs_only ? a.rhs_in : (slow ? a.b.qA : a.qF);
+  const size_t o = G.at(0, k, j, i);
+#pragma unroll
+  for (int c = 0; c < 5; c++) q[c] = base[o + c * G.plane];
   if (!a.rhs_only && (a.stage & 1)) {
-    const double h = k < g.n1_r ? g.dt : g.hF;
-    return base[o] + h * reinterpret_cast<const double*>(a.b.Ra)[o];
+    const double h = slow ? g.dt : g.hF;
+    const double* Ra = reinterpret_cast<const double*>(a.b.Ra);
+#pragma unroll
+    for (int c = 0; c < 5; c++) q[c] = __fma_rn(h, Ra[o + c * G.plane], q[c]);
   }
-  return base[o];
+}
+__device__ __forceinline__ bool cell_in_range3(const double q[5]) {
+  return in_range(q[0], max(abs_word(q[1]), max(abs_word(q[2]), abs_word(q[3]))), q[4]);
 }
 
-// (u, v, w, T) from a conserved state; gg = gamma (gamma - 1), T = gamma p / rho
-__device__ __forceinline__ void prim5(const double q[5], double gg, double v[4]) {
-  const double inv = recip_f64(q[0]);
-  v[0] = q[1] * inv;
-  v[1] = q[2] * inv;
-  v[2] = q[3] * inv;
-  v[3] = gg * (q[4] - 0.5 * (q[1] * v[0] + q[2] * v[1] + q[3] * v[2])) * inv;
+// The two arithmetics of the tiles: i64 (fixed point) and double.
+template <typename T>
+struct Arith3;
+template <>
+struct Arith3<i64> {
+  static __device__ __forceinline__ i64 cell(double q, int c) {  // rho, rho E .58, momenta .60
+    return fx::from_double(__double_as_longlong(q), c == 0 || c == 4 ? fx::S_RHO - 2 : fx::S_MOM - 2);
+  }
+  static __device__ __forceinline__ i64 rec(i64 a, i64 up, i64 dn) { return (a << 2) + (up - dn); }
+  static __device__ __forceinline__ void vel(const i64 q[4], i64 v[3]) {
+    const FxW inv = fx::split(fx::recip(q[0] << 2));
+#pragma unroll
+    for (int c = 0; c < 3; c++) v[c] = fx::mul(fx::split(q[c + 1] << 2), inv);
+  }
+  static __device__ __forceinline__ void prims(const i64 q[5], i64 v[4]) {
+    const FxW inv = fx::split(fx::recip(q[0] << 2));
+    i64 k = 0;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      const FxW m = fx::split(q[c + 1] << 2);
+      v[c] = fx::mul(m, inv);
+      k += fx::mul(m, fx::split(v[c]));
+    }
+    v[3] = fx::mul(fx::split((q[4] - k) << 2), inv) << 2;  // k .57: k/2 .58
+  }
+};
+template <>
+struct Arith3<double> {
+  static __device__ __forceinline__ double cell(double q, int) { return q; }
+  static __device__ __forceinline__ double rec(double a, double up, double dn) {
+    return __fma_rn(0.25, __dsub_rn(up, dn), a);
+  }
+  static __device__ __forceinline__ void vel(const double q[4], double v[3]) {
+    const double inv = recip_f64(q[0]);
+#pragma unroll
+    for (int c = 0; c < 3; c++) v[c] = __dmul_rn(q[c + 1], inv);
+  }
+  static __device__ __forceinline__ void prims(const double q[5], double v[4]) {
+    const double inv = recip_f64(q[0]);
+    double k = 0.0;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      v[c] = __dmul_rn(q[c + 1], inv);
+      k = __fma_rn(q[c + 1], v[c], k);
+    }
+    v[3] = __dmul_rn(__fma_rn(-0.5, k, q[4]), inv);
+  }
+};
+
+// A stored flux: the .57 integer itself (|F| < 8, so its top four bits agree)
+// or the bits of a double, whose top four bits differ for 2^-511 <= |F| <
+// 2^513. Smaller doubles store as zero, larger ones and NaN as the positive
+// NaN.
+__device__ __forceinline__ bool flux_is_double(i64 f) {
+  return (unsigned)((int)(f >> 32) + 0x10000000) >= 0x20000000u;
+}
+__device__ __forceinline__ i64 flux_tag(double f) {
+  const unsigned h = (unsigned)__double2hiint(f) & 0x7fffffffu;
+  if (h < 0x20000000u) return 0;
+  return h < 0x60000000u ? __double_as_longlong(f) : 0x7ff8000000000000ll;
+}
+__device__ __forceinline__ double flux_value(i64 f) {
+  if (flux_is_double(f)) return __longlong_as_double(f);
+  return __dmul_rn((double)f, 1.0 / (double)(1ll << fx::S_FLUX));
 }
 
 // Interface state of column (i, j) (App. B, Eq. bulk-flux and the wall
-// states after it): {sigma_xz, sigma_yz, Pi_z, u_w1, v_w1, T_w1, u_w2, v_w2,
-// T_w2}, each fluid using its own formula.
-__device__ __forceinline__ void interface3(const StageArgs& a, const Geo3& G, int j, int i, double out[9]) {
+// states after it), doubled: 2 u_w, 2 v_w of fluid 1 and of fluid 2, each
+// with its own formula, 2 sigma_xz, 2 sigma_yz, and 2 (u_w sigma_xz + v_w
+// sigma_yz - Pi_z) of each fluid.
+enum { L3_U1, L3_V1, L3_U2, L3_V2, L3_SX, L3_SY, L3_E1, L3_E2, L3_N };
+__device__ __forceinline__ void interface3(const StageArgs& a, const Geo3& G, int j, int i, double out[L3_N]) {
   const Geom& g = a.g;
   double v1[4], v2[4], q[5];
+  stage_val3(a, G, G.n1 - 1, j, i, q);
+  Arith3<double>::prims(q, v1);
+  stage_val3(a, G, G.n1, j, i, q);
+  Arith3<double>::prims(q, v2);
+  const double sxz = __dmul_rn(g.bu, __dsub_rn(v2[0], v1[0]));
+  const double syz = __dmul_rn(g.bu, __dsub_rn(v2[1], v1[1]));  // b_v = b_u
+  const double gg = __dmul_rn(g.gamma, g.gm1);                  // T / e
+  const double Pi = __dmul_rn(__dmul_rn(-g.bT, gg), __dsub_rn(v2[3], v1[3]));
+  const double u1 = __fma_rn(sxz, g.cu1, v1[0]), w1 = __fma_rn(syz, g.cu1, v1[1]);
+  const double u2 = __fma_rn(-sxz, g.cu2, v2[0]), w2 = __fma_rn(-syz, g.cu2, v2[1]);
+  out[L3_U1] = 2.0 * u1;
+  out[L3_V1] = 2.0 * w1;
+  out[L3_U2] = 2.0 * u2;
+  out[L3_V2] = 2.0 * w2;
+  out[L3_SX] = 2.0 * sxz;
+  out[L3_SY] = 2.0 * syz;
+  out[L3_E1] = 2.0 * __fma_rn(u1, sxz, __fma_rn(w1, syz, -Pi));
+  out[L3_E2] = 2.0 * __fma_rn(u2, sxz, __fma_rn(w2, syz, -Pi));
+}
+// The same as T into column cc of L (row stride ls); false where a value
+// leaves the fixed-point range.
+template <typename T>
+__device__ __forceinline__ bool store_lid(const double s[L3_N], T* L, int ls);
+template <>
+__device__ __forceinline__ bool store_lid<double>(const double s[L3_N], double* L, int ls) {
 #pragma unroll
-  for (int c = 0; c < 5; c++) q[c] = stage_val3(a, G, c, G.n1 - 1, j, i);
-  prim5(q, g.gamma * g.gm1, v1);
+  for (int q = 0; q < L3_N; q++) L[q * ls] = s[q];
+  return true;
+}
+template <>
+__device__ __forceinline__ bool store_lid<i64>(const double s[L3_N], i64* L, int ls) {
+  bool ok = true;
 #pragma unroll
-  for (int c = 0; c < 5; c++) q[c] = stage_val3(a, G, c, G.n1, j, i);
-  prim5(q, g.gamma * g.gm1, v2);
-  const double sxz = g.bu * (v2[0] - v1[0]);
-  const double syz = g.bu * (v2[1] - v1[1]);  // b_v = b_u
-  const double Pi = -g.bT * (v2[3] - v1[3]);
-  out[0] = sxz;
-  out[1] = syz;
-  out[2] = Pi;
-  out[3] = v1[0] + sxz * g.cu1;
-  out[4] = v1[1] + syz * g.cu1;
-  out[5] = v1[3] - Pi * g.cT1;
-  out[6] = v2[0] - sxz * g.cu2;
-  out[7] = v2[1] - syz * g.cu2;
-  out[8] = v2[3] + Pi * g.cT2;
+  for (int q = 0; q < L3_N; q++) ok = ok && fabs(s[q]) < 3.8;  // false for NaN
+#pragma unroll
+  for (int q = 0; q < L3_N; q++)
+    L[q * ls] = __double2ll_rn(ok ? __dmul_rn(s[q], (double)(1ll << (q < L3_SX ? fx::S_VEL : fx::S_FLUX))) : 0.0);
+  return ok;
 }
 
-// Central z difference (unscaled) of (u, v, w) at row k from the cell (c)
-// and its neighbours above (up) and below (dn), with the ghost
-// 2*(wall state) - interior beyond a wall or Gamma; gam holds the column's
+// Central z differences (unscaled) of the velocities A and B at row k from
+// the cell and its neighbours above and below, with the ghost 2 (wall state)
+// - interior beyond a wall or Gamma; component 2 (w) is normal there. v: the
+// cell's u in a plane of stride vp, rows of stride vr; lid: the column's
 // interface state.
-__device__ __forceinline__ void dz_uvw(const Geom& g, int k, const double* c, const double* up, const double* dn,
-                                       const double* gam, double out[3]) {
-  double U[3], D[3];
-  const int nz = g.nz, n1 = g.n1;
-  const double st = g.wall ? 1.0 : -1.0;  // tangential ghost sign at a slip / no-slip wall
-  if (k + 1 == nz) {
-    U[0] = st * c[0]; U[1] = st * c[1]; U[2] = -c[2];
-  } else if (k + 1 == n1) {  // fluid 1's top row: Gamma above
-    U[0] = 2.0 * gam[3] - c[0]; U[1] = 2.0 * gam[4] - c[1]; U[2] = -c[2];
-  } else {
-    U[0] = up[0]; U[1] = up[1]; U[2] = up[2];
-  }
-  if (k == 0) {
-    D[0] = st * c[0]; D[1] = st * c[1]; D[2] = -c[2];
-  } else if (k == n1) {  // fluid 2's bottom row: Gamma below
-    D[0] = 2.0 * gam[6] - c[0]; D[1] = 2.0 * gam[7] - c[1]; D[2] = -c[2];
-  } else {
-    D[0] = dn[0]; D[1] = dn[1]; D[2] = dn[2];
-  }
+template <typename T>
+__device__ __forceinline__ T dz_vel(const Geom& g, int k, int comp, const T* v, int vr, const T* lid, int ls) {
+  const T c = v[0];
+  T up, dn;
+  if (k + 1 == g.nz) up = (comp == 2 || !g.wall) ? -c : c;
+  else if (k + 1 == g.n1) up = comp == 2 ? -c : lid[(L3_U1 + comp) * ls] - c;  // fluid 1's top row
+  else up = v[vr];
+  if (k == 0) dn = (comp == 2 || !g.wall) ? -c : c;
+  else if (k == g.n1) dn = comp == 2 ? -c : lid[(L3_U2 + comp) * ls] - c;  // fluid 2's bottom row
+  else dn = v[-vr];
+  return up - dn;
+}
+
+// Viscous flux in the face frame over half the divergence factor: (sigma_nn,
+// sigma_nt1, sigma_nt2, u^.sigma_n + kappa dT/dn). With G[a][b] = d u_a /
+// d x_b (b = normal, t1, t2): sigma_nn = mu (4/3 G00 - 2/3 (G11 + G22)),
+// sigma_nt = mu (G_t0 + G_0t); the derivative factors sit in the coefficients.
+__device__ __forceinline__ void visc3(const Fx3Const& c, int dir, int fl, const VSide<i64>& L, const VSide<i64>& R,
+                                      i64 V[4]) {
+  const FxW* f = c.fc[dir][fl];
+  V[0] = fx::mul2(f[F3_A], fx::split(R.u[0] - L.u[0]), f[F3_B1], fx::split(L.g1[1] + R.g1[1])) +
+         fx::mul(fx::split(L.g2[1] + R.g2[1]), f[F3_B2]);
+  V[1] = fx::mul2(f[F3_C], fx::split(R.u[1] - L.u[1]), f[F3_D1], fx::split(L.g1[0] + R.g1[0]));
+  V[2] = fx::mul2(f[F3_C], fx::split(R.u[2] - L.u[2]), f[F3_D2], fx::split(L.g2[0] + R.g2[0]));
+  i64 us = 0;  // (u_L + u_R) . sigma .54
 #pragma unroll
-  for (int a = 0; a < 3; a++) out[a] = U[a] - D[a];
+  for (int q = 0; q < 3; q++) us += fx::mul(fx::split((L.u[q] + R.u[q]) << 2), fx::split(V[q]));
+  V[3] = (us << 2) + fx::mul(fx::split(R.e - L.e), f[F3_K]);
+}
+__device__ __forceinline__ void visc3(const Fx3Const& c, int dir, int fl, const VSide<double>& L,
+                                      const VSide<double>& R, double V[4]) {
+  const double* f = c.fd[dir][fl];
+  V[0] = __fma_rn(f[F3_A], __dsub_rn(R.u[0], L.u[0]),
+                  __fma_rn(f[F3_B1], __dadd_rn(L.g1[1], R.g1[1]), __dmul_rn(f[F3_B2], __dadd_rn(L.g2[1], R.g2[1]))));
+  V[1] = __fma_rn(f[F3_C], __dsub_rn(R.u[1], L.u[1]), __dmul_rn(f[F3_D1], __dadd_rn(L.g1[0], R.g1[0])));
+  V[2] = __fma_rn(f[F3_C], __dsub_rn(R.u[2], L.u[2]), __dmul_rn(f[F3_D2], __dadd_rn(L.g2[0], R.g2[0])));
+  double us = 0.0;
+#pragma unroll
+  for (int q = 0; q < 3; q++) us = __fma_rn(__dadd_rn(L.u[q], R.u[q]), V[q], us);
+  V[3] = __fma_rn(0.5, us, __dmul_rn(f[F3_K], __dsub_rn(R.e, L.e)));
+}
+
+// The face flux, as stored; false where it leaves the fixed-point range.
+__device__ __forceinline__ bool flux3(const Geom& g, const Fx3Const& c, const i64 L[5], const i64 R[5], const i64 V[4],
+                                      i64 F[5]) {
+  return fx_flux<3>(g, c.k, L, R, V, F);
+}
+__device__ __forceinline__ bool flux3(const Geom& g, const Fx3Const&, const double L[5], const double R[5],
+                                      const double V[4], i64 F[5]) {
+  double o[5];
+  lf_face5(L, R, g.gamma, g.gm1, V, o);
+#pragma unroll
+  for (int q = 0; q < 5; q++) F[q] = flux_tag(o[q]);
+  return true;
 }
 
 // ---- y faces ------------------------------------------------------------------
 
+constexpr int RING3 = (TZ + 2) * (TX + 2);  // tile plus a one-cell ring
 struct YfaceSmem {
-  double q0[5][TZ + 2][TX + 2];  // plane j, rows k0-1.., cols i0-1..
-  double q1[5][TZ + 2][TX + 2];  // plane j+1
-  double qm[5][TZ][TX];          // plane j-1, tile cells
-  double qp[5][TZ][TX];          // plane j+2, tile cells
-  double v0[4][TZ + 2][TX + 2];  // u, v, w, T of plane j on the ring
-  double v1[4][TZ + 2][TX + 2];
-  double gam0[9][TX];            // interface state of the tile columns, planes j and j+1
-  double gam1[9][TX];
-  double fc[2][F3_N];            // y-face constants per fluid
-  double gg;                     // gamma (gamma - 1)
+  i64 q[2][5][TZ + 2][TX + 2];   // planes j and j+1, rows k0-1.., cols i0-1..
+  i64 v[2][4][TZ + 2][TX + 2];   // u, v, w, e on the ring
+  i64 lid[2][L3_N][TX];          // interface state of the tile columns
+  unsigned char ok[2][TZ + 2][TX + 2];
+  unsigned char lid_ok[2][TX];
 };
 
-// The y faces between planes j and j+1 of the TX x TZ tile from row k0,
-// column i0, times 1/dy, written to a.gy at index j.
-__device__ __forceinline__ void yface_tile(const StageArgs& a, int k0, int i0, int j, YfaceSmem& S) {
+// The y face between planes j and j+1 of the thread's cell (k, i), in T, from
+// the tile's cells restaged as T. First pass (T = i64): returns whether the
+// face was stored in fixed point; its barrier-separated second pass (T =
+// double) stores the others (want).
+template <typename T>
+__device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C, int k0, int i0, int j, YfaceSmem& S,
+                                           bool want) {
+  constexpr bool FX = sizeof(T) == 8 && (T)0.5 == (T)0;
   const Geom& g = a.g;
   const Geo3 G = geo3(g);
   const int tid = threadIdx.x;
-  const int nz = g.nz, nx = g.nx, ny = g.ny, n1 = g.n1;
+  const int nz = g.nz, n1 = g.n1;
   const int row_hi = a.rhs_only ? a.rhs_hi : nz;
-  const int jm = wrap3(j - 1, ny), j1 = wrap3(j + 1, ny), jp = wrap3(j + 2, ny);
-
-  if (tid < 2) {
-    // y faces: t1 = x, t2 = z
-    face_consts3(g.inv_dy, g.inv_dx, tid ? g.inv_dz2 : g.inv_dz1, tid ? g.mu2 : g.mu1, tid ? g.kap2 : g.kap1,
-                 S.fc[tid]);
-    if (tid == 0) S.gg = g.gamma * g.gm1;
-  }
-  for (int e = tid; e < 5 * (TZ + 2) * (TX + 2); e += NTHREADS) {
-    const int c = e / ((TZ + 2) * (TX + 2)), rem = e - c * (TZ + 2) * (TX + 2);
+  const int j1 = wrap3(j + 1, g.ny);
+  T* Sq = reinterpret_cast<T*>(&S.q[0][0][0][0]);
+  T* Sv = reinterpret_cast<T*>(&S.v[0][0][0][0]);
+  T* Sl = reinterpret_cast<T*>(&S.lid[0][0][0]);
+  bool bad = false;
+  for (int e = tid; e < 2 * RING3; e += NTHREADS) {
+    const int side = e >= RING3, rem = e - side * RING3;
     const int rr = rem / (TX + 2), cc = rem - rr * (TX + 2);
-    const int k = k0 - 1 + rr, i = wrap3(i0 - 1 + cc, nx);
-    double x0 = 0.0, x1 = 0.0;
-    if (k >= 0 && k < nz) {
-      x0 = stage_val3(a, G, c, k, j, i);
-      x1 = stage_val3(a, G, c, k, j1, i);
+    const int k = k0 - 1 + rr;
+    if (k < 0 || k >= nz) continue;
+    double q[5];
+    stage_val3(a, G, k, side ? j1 : j, wrap3(i0 - 1 + cc, g.nx), q);
+    bool in = true;
+    if (FX) {
+      in = cell_in_range3(q);
+      S.ok[side][rr][cc] = in;
+      bad |= !in;
     }
-    S.q0[c][rr][cc] = x0;
-    S.q1[c][rr][cc] = x1;
-  }
-  for (int e = tid; e < 5 * TZ * TX; e += NTHREADS) {
-    const int c = e / (TZ * TX), rem = e - c * TZ * TX;
-    const int rr = rem / TX, cc = rem - rr * TX;
-    const int k = k0 + rr, i = wrap3(i0 + cc, nx);
-    double xm = 0.0, xp = 0.0;
-    if (k < nz) {
-      xm = stage_val3(a, G, c, k, jm, i);
-      xp = stage_val3(a, G, c, k, jp, i);
+    if (FX && !in) continue;  // no face in fixed point reads the cell
+    T t[5], v[4];
+#pragma unroll
+    for (int c = 0; c < 5; c++) {
+      t[c] = Arith3<T>::cell(q[c], c);
+      Sq[(side * 5 + c) * RING3 + rem] = t[c];
     }
-    S.qm[c][rr][cc] = xm;
-    S.qp[c][rr][cc] = xp;
+    Arith3<T>::prims(t, v);
+#pragma unroll
+    for (int c = 0; c < 4; c++) Sv[(side * 4 + c) * RING3 + rem] = v[c];
   }
   const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZ);
   if (has_gamma && tid < 2 * TX) {
     const int side = tid / TX, cc = tid - side * TX;
-    double st[9];
-    interface3(a, G, side ? j1 : j, wrap3(i0 + cc, nx), st);
-#pragma unroll
-    for (int s = 0; s < 9; s++) (side ? S.gam1 : S.gam0)[s][cc] = st[s];
+    double st[L3_N];
+    interface3(a, G, side ? j1 : j, wrap3(i0 + cc, g.nx), st);
+    const bool ok = store_lid<T>(st, Sl + side * L3_N * TX + cc, TX);
+    if (FX) S.lid_ok[side][cc] = ok;
+    bad |= !ok;
   }
-  __syncthreads();
-  for (int e = tid; e < 2 * (TZ + 2) * (TX + 2); e += NTHREADS) {
-    const int side = e / ((TZ + 2) * (TX + 2)), rem = e - side * (TZ + 2) * (TX + 2);
-    const int rr = rem / (TX + 2), cc = rem - rr * (TX + 2);
-    const int k = k0 - 1 + rr;
-    if (k < 0 || k >= nz) continue;
-    double q[5], v[4];
-#pragma unroll
-    for (int c = 0; c < 5; c++) q[c] = side ? S.q1[c][rr][cc] : S.q0[c][rr][cc];
-    prim5(q, S.gg, v);
-#pragma unroll
-    for (int c = 0; c < 4; c++) (side ? S.v1 : S.v0)[c][rr][cc] = v[c];
-  }
-  __syncthreads();
-
   const int rr = tid / TX, cc = tid - rr * TX;
   const int k = k0 + rr, i = i0 + cc;
-  if (k >= row_hi || i >= nx) return;
-  // reconstructed states: d/dy central differences of q at j and j+1
-  double L[5], R[5];
+  const bool mine = k < row_hi && i < g.nx;
+  // the outer two of the four cells across the face
+  T am[5], ap[5];
+  bool out_ok = true;
+  if (mine && want) {
+    double q[5];
+    stage_val3(a, G, k, wrap3(j - 1, g.ny), i, q);
+    out_ok = cell_in_range3(q);
+#pragma unroll
+    for (int c = 0; c < 5; c++) am[c] = Arith3<T>::cell(q[c], c);
+    stage_val3(a, G, k, wrap3(j + 2, g.ny), i, q);
+    out_ok = out_ok && cell_in_range3(q);
+#pragma unroll
+    for (int c = 0; c < 5; c++) ap[c] = Arith3<T>::cell(q[c], c);
+  }
+  if (FX) bad = __syncthreads_or(bad);
+  else __syncthreads();
+  if (!mine || !want) return true;
+  if (FX) {
+    if (bad) {
+      // the face's own cells: the four across it and the x and z neighbours
+      // of the two at it (inside the grid), and the interface states it reads
+      for (int s = 0; s < 2; s++) {
+        out_ok = out_ok && S.ok[s][rr + 1][cc + 1] && S.ok[s][rr + 1][cc] && S.ok[s][rr + 1][cc + 2];
+        if (k > 0) out_ok = out_ok && S.ok[s][rr][cc + 1];
+        if (k + 1 < nz) out_ok = out_ok && S.ok[s][rr + 2][cc + 1];
+        if (k == n1 || k == n1 - 1) out_ok = out_ok && S.lid_ok[s][cc];
+      }
+    }
+    if (!out_ok) return false;
+  }
+  // face frame: normal rho v, t1 rho u, t2 rho w
+  const int at = (rr + 1) * (TX + 2) + cc + 1;
+  T L[5], R[5];
 #pragma unroll
   for (int c = 0; c < 5; c++) {
-    const double a0 = S.q0[c][rr + 1][cc + 1], a1 = S.q1[c][rr + 1][cc + 1];
-    L[c] = a0 + 0.25 * (a1 - S.qm[c][rr][cc]);
-    R[c] = a1 - 0.25 * (S.qp[c][rr][cc] - a0);
+    const int f = c == 1 ? 2 : (c == 2 ? 1 : c);
+    const T a0 = Sq[f * RING3 + at], a1 = Sq[(5 + f) * RING3 + at];
+    L[c] = Arith3<T>::rec(a0, a1, am[f]);
+    R[c] = Arith3<T>::rec(a1, a0, ap[f]);
   }
-  // face frame: normal rho v, tangential rho u, rho w
-  const double lf[5] = {L[0], L[2], L[1], L[3], L[4]}, rf[5] = {R[0], R[2], R[1], R[3], R[4]};
-  const double* fc = S.fc[k >= n1];
-  double FI[5], FV[5];
-  lf_face5(lf, rf, g.gamma, g.gm1, fc[F3_HS], FI);
-  VSide s[2];
+  VSide<T> s[2];
 #pragma unroll
   for (int side = 0; side < 2; side++) {
-    double (*V)[TZ + 2][TX + 2] = side ? S.v1 : S.v0;
-    const double(*gam)[TX] = side ? S.gam1 : S.gam0;
-    // frame order (v, u, w)
-    s[side].u[0] = V[1][rr + 1][cc + 1];
-    s[side].u[1] = V[0][rr + 1][cc + 1];
-    s[side].u[2] = V[2][rr + 1][cc + 1];
-    s[side].T = V[3][rr + 1][cc + 1];
-    // x (t1) differences of (v, u, w)
-    s[side].d1[0] = V[1][rr + 1][cc + 2] - V[1][rr + 1][cc];
-    s[side].d1[1] = V[0][rr + 1][cc + 2] - V[0][rr + 1][cc];
-    s[side].d1[2] = V[2][rr + 1][cc + 2] - V[2][rr + 1][cc];
-    // z (t2) differences of (v, u, w), ghosts beyond a wall or Gamma
-    const double cv[3] = {V[0][rr + 1][cc + 1], V[1][rr + 1][cc + 1], V[2][rr + 1][cc + 1]};
-    const double uv[3] = {V[0][rr + 2][cc + 1], V[1][rr + 2][cc + 1], V[2][rr + 2][cc + 1]};
-    const double dv[3] = {V[0][rr][cc + 1], V[1][rr][cc + 1], V[2][rr][cc + 1]};
-    double gz[9];
-#pragma unroll
-    for (int q = 0; q < 9; q++) gz[q] = has_gamma ? gam[q][cc] : 0.0;
-    double dz[3];
-    dz_uvw(g, k, cv, uv, dv, gz, dz);
-    s[side].d2[0] = dz[1];
-    s[side].d2[1] = dz[0];
-    s[side].d2[2] = dz[2];
+    const T* V = Sv + side * 4 * RING3 + at;
+    const T* lid = Sl + side * L3_N * TX + cc;
+    s[side].u[0] = V[RING3];
+    s[side].u[1] = V[0];
+    s[side].u[2] = V[2 * RING3];
+    s[side].e = V[3 * RING3];
+    s[side].g1[0] = V[RING3 + 1] - V[RING3 - 1];  // x differences of v, u
+    s[side].g1[1] = V[1] - V[-1];
+    s[side].g2[0] = dz_vel(g, k, 1, V + RING3, TX + 2, lid, TX);  // z differences of v, w
+    s[side].g2[1] = dz_vel(g, k, 2, V + 2 * RING3, TX + 2, lid, TX);
   }
-  visc_face5(s[0], s[1], fc, FV);
-  const double F[5] = {FI[0] - FV[0], FI[2] - FV[2], FI[1] - FV[1], FI[3] - FV[3], FI[4] - FV[4]};
+  T V[4];
+  visc3(C, 1, k >= n1, s[0], s[1], V);
+  i64 F[5];
+  if (!flux3(g, C, L, R, V, F)) return false;
 #pragma unroll
-  for (int c = 0; c < 5; c++) a.gy[G.at(c, k, j, i)] = F[c];
+  for (int c = 0; c < 5; c++) {
+    const int f = c == 1 ? 2 : (c == 2 ? 1 : c);
+    reinterpret_cast<i64*>(a.gy)[G.at(f, k, j, i)] = F[c];
+  }
+  return true;
+}
+__device__ __noinline__ void yface_slow(const StageArgs& a, const Fx3Const& C, int k0, int i0, int j, YfaceSmem& S,
+                                        bool want) {
+  yface_pass<double>(a, C, k0, i0, j, S, want);
+}
+__device__ __forceinline__ void yface_tile(const StageArgs& a, const Fx3Const& C, int k0, int i0, int j,
+                                           YfaceSmem& S) {
+  const bool done = C.k.on && yface_pass<i64>(a, C, k0, i0, j, S, true);
+  if (__syncthreads_or(!done)) yface_slow(a, C, k0, i0, j, S, !done);
 }
 
 // ---- x and z faces, divergence and stage combination ----------------------
 
 struct Tile3Smem {
-  double q[5][TZ + 4][TX + 4];   // plane j, rows k0-2.., cols i0-2..
-  double v[4][TZ + 2][TX + 2];   // u, v, w, T on the ring
-  double vy[3][TZ + 2][TX + 2];  // central y differences of u, v, w on the ring
-  double hx[5][TZ][TX + 2];      // central x differences of q, tile rows, cols i0-1..
-  double hz[5][TZ + 2][TX];      // central z differences of q, rows k0-1.., tile cols
-  double tz[3][TZ][TX + 2];      // central z differences of u, v, w at x-face cells
-  double tx[3][TZ + 2][TX];      // central x differences of u, v, w at z-face cells
-  double fx[5][TZ][TX + 1];      // x face fluxes / dx, face f between cols f-1, f
-  double fz[5][TZ + 1][TX];      // z face fluxes / dz seen from above
-  double fg[5][TX];              // interface flux seen from fluid 1
-  double gam[9][TX + 2];         // interface state per ring column
-  double fc[2][2][F3_N];         // face constants per direction (x, z) and fluid
-  double gg;                     // gamma (gamma - 1)
+  static constexpr int NZF = (TZ + 1) * TX, NXF = TZ * (TX + 1);
+  i64 q[5][TZ + 4][TX + 4];   // plane j, rows k0-2.., cols i0-2..
+  i64 v[4][TZ + 2][TX + 2];   // u, v, w, e on the ring
+  i64 vy[3][TZ + 2][TX + 2];  // central y differences of u, v, w on the ring
+  i64 tz[2][TZ][TX + 2];      // central z differences of u, w at x-face cells
+  i64 tx[2][TZ + 2][TX];      // central x differences of u, w at z-face cells
+  i64 fx[5][TZ][TX + 1];      // x face fluxes, face f between cols f-1, f
+  i64 fz[5][TZ + 1][TX];      // z face fluxes seen from above
+  i64 fg[5][TX];              // interface flux seen from fluid 1
+  i64 lid[L3_N][TX + 2];      // interface state per ring column
+  unsigned char ok[TZ + 4][TX + 4];
+  unsigned char oky[TZ + 2][TX + 2];  // the cells in planes j-1 and j+1
+  unsigned char lid_ok[TX + 2];
+  unsigned char slow[NZF + NXF + TX];  // per face: z, x, interface from below
 };
 
-__device__ __forceinline__ void stage_tile3(const StageArgs& a, int k0, int i0, int j, Tile3Smem& S) {
+// Phases 1 to 3 in T: stage state, velocities, y differences, interface
+// state, then the tangential differences. Returns (T = i64) 0, or 1 where
+// some cell or interface state leaves the fixed-point range, or 2 where every
+// cell does. Ends with a barrier.
+template <typename T>
+__device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, int k0, int i0, int j, int row_hi,
+                                            Tile3Smem& S) {
+  constexpr bool FX = (T)0.5 == (T)0;
+  const Geom& g = a.g;
+  const int tid = threadIdx.x, nz = g.nz, n1 = g.n1;
+  const int jm = wrap3(j - 1, g.ny), jp = wrap3(j + 1, g.ny);
+  constexpr int QP = (TZ + 4) * (TX + 4), ZP = TZ * (TX + 2), XP = (TZ + 2) * TX;
+  T* q = reinterpret_cast<T*>(&S.q[0][0][0]);
+  T* v = reinterpret_cast<T*>(&S.v[0][0][0]);
+  T* vy = reinterpret_cast<T*>(&S.vy[0][0][0]);
+  T* tz = reinterpret_cast<T*>(&S.tz[0][0][0]);
+  T* tx = reinterpret_cast<T*>(&S.tx[0][0][0]);
+  T* lid = reinterpret_cast<T*>(&S.lid[0][0]);
+  bool bad = false, good = false;
+  for (int e = tid; e < QP; e += NTHREADS) {
+    const int rr = e / (TX + 4), cc = e - rr * (TX + 4);
+    const int k = k0 - 2 + rr;
+    if (k < 0 || k >= nz) {
+      // read by the faces next to a wall, which replace it by the mirror cell
+#pragma unroll
+      for (int c = 0; c < 5; c++) q[c * QP + e] = (T)0;
+      continue;
+    }
+    double x[5];
+    stage_val3(a, G, k, j, wrap3(i0 - 2 + cc, g.nx), x);
+    if (FX) {
+      const bool in = cell_in_range3(x);
+      S.ok[rr][cc] = in;
+      bad |= !in;
+      good |= in;
+      if (!in) continue;  // no face in fixed point reads the cell
+    }
+    T t[5];
+#pragma unroll
+    for (int c = 0; c < 5; c++) {
+      t[c] = Arith3<T>::cell(x[c], c);
+      q[c * QP + e] = t[c];
+    }
+    // velocities on the one-cell ring
+    if (rr >= 1 && rr <= TZ + 2 && cc >= 1 && cc <= TX + 2) {
+      T o[4];
+      Arith3<T>::prims(t, o);
+#pragma unroll
+      for (int c = 0; c < 4; c++) v[c * RING3 + (rr - 1) * (TX + 2) + cc - 1] = o[c];
+    }
+  }
+  for (int e = tid; e < RING3; e += NTHREADS) {
+    const int rr = e / (TX + 2), cc = e - rr * (TX + 2);
+    const int k = k0 - 1 + rr;
+    if (k < 0 || k >= nz) continue;
+    const int i = wrap3(i0 - 1 + cc, g.nx);
+    double x[5];
+    T t[4], up[3], dn[3];
+    bool in = true;
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+      stage_val3(a, G, k, s ? jm : jp, i, x);
+      if (FX) in = in && cell_in_range3(x);
+      if (!in) break;
+#pragma unroll
+      for (int c = 0; c < 4; c++) t[c] = Arith3<T>::cell(x[c], c);
+      Arith3<T>::vel(t, s ? dn : up);
+    }
+    if (FX) {
+      S.oky[rr][cc] = in;
+      bad |= !in;
+    }
+    if (!in) continue;
+#pragma unroll
+    for (int c = 0; c < 3; c++) vy[c * RING3 + e] = up[c] - dn[c];
+  }
+  const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZ);
+  if (has_gamma && tid < TX + 2) {
+    double st[L3_N];
+    interface3(a, G, j, wrap3(i0 - 1 + tid, g.nx), st);
+    const bool ok = store_lid<T>(st, lid + tid, TX + 2);
+    if (FX) S.lid_ok[tid] = ok;
+    bad |= !ok;
+  }
+  if (FX) {
+    bad = __syncthreads_or(bad);
+    if (bad && !__syncthreads_or(good)) return 2;
+  } else {
+    __syncthreads();
+  }
+  for (int e = tid; e < ZP + XP; e += NTHREADS) {
+    if (e < ZP) {
+      const int rr = e / (TX + 2), cc = e - rr * (TX + 2), k = k0 + rr;
+      if (k >= row_hi) continue;
+      const T* p = v + (rr + 1) * (TX + 2) + cc;
+      tz[e] = dz_vel(g, k, 0, p, TX + 2, lid + cc, TX + 2);
+      tz[ZP + e] = dz_vel(g, k, 2, p + 2 * RING3, TX + 2, lid + cc, TX + 2);
+    } else {
+      const int x = e - ZP, rr = x / TX, cc = x - rr * TX, k = k0 - 1 + rr;
+      if (k < 0 || k >= nz) continue;
+      const T* p = v + rr * (TX + 2) + cc;
+      tx[x] = p[2] - p[0];
+      tx[XP + x] = p[2 * RING3 + 2] - p[2 * RING3];
+    }
+  }
+  __syncthreads();
+  return bad;
+}
+
+// Face e of the tile, numbered and placed as in the 2-D tile.
+struct Face3 {
+  int isx, f, c;  // z: face row f, column c; x: tile row f, face column c
+  int ku;         // row above a z face, or the row of an x face
+  int below;      // the interface from fluid 1
+};
+__device__ __forceinline__ bool face3_id(const Geom& g, int e, int k0, int row_hi, Face3* id) {
+  constexpr int NZF = Tile3Smem::NZF, NXF = Tile3Smem::NXF;
+  id->below = 0;
+  if (e < NZF) {
+    id->isx = 0;
+    id->f = e / TX;
+    id->c = e - id->f * TX;
+    id->ku = k0 + id->f;
+    return id->ku - 1 < row_hi && !(id->f == TZ && id->ku == g.n1);
+  }
+  if (e < NZF + NXF) {
+    const int x = e - NZF;
+    id->isx = 1;
+    id->f = x / (TX + 1);
+    id->c = x - id->f * (TX + 1);
+    id->ku = k0 + id->f;
+    return id->ku < row_hi;
+  }
+  id->isx = 0;
+  id->f = g.n1 - k0;
+  id->c = e - NZF - NXF;
+  id->ku = g.n1;
+  id->below = 1;
+  return id->f >= 1 && id->f <= TZ && g.n1 - 1 < row_hi;
+}
+
+// The flux of face id in T, stored; false where it leaves the range. A
+// boundary face (outer wall or interface) has the inner cell's reconstructed
+// state on one side and its mirror on the other; an outer wall's viscous
+// ghost is 2 wall state - cell.
+template <typename T>
+__device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Smem& S, const Face3& id) {
+  constexpr int QP = (TZ + 4) * (TX + 4), ZP = TZ * (TX + 2), XP = (TZ + 2) * TX;
+  const int n1 = g.n1, nz = g.nz, ku = id.ku, kd = ku - 1;
+  const int qs = id.isx ? 1 : TX + 4;
+  const int q0 = id.isx ? (id.f + 2) * (TX + 4) + id.c : id.f * (TX + 4) + id.c + 2;
+  // component planes of the normal and the tangents: x (u; v, w), z (w; u, v)
+  const int pn = id.isx ? 1 : 3, p1 = id.isx ? 2 : 1, p2 = id.isx ? 3 : 2;
+  const bool wall = !id.isx && (ku == 0 || ku == nz), lidf = !id.isx && ku == n1;
+  const bool from_above = ku == 0 || (lidf && !id.below);
+  const bool mir0 = !id.isx && (kd == 0 || kd == n1), mir3 = !id.isx && (ku == nz - 1 || ku == n1 - 1);
+  const T* q = reinterpret_cast<const T*>(&S.q[0][0][0]) + q0;
+  T L[5], R[5], V[4];
+  auto comp = [&](int plane, bool odd, T& l, T& r) {
+    const T* p = q + plane * QP;
+    T a0 = p[0], a1 = p[qs], a2 = p[2 * qs], a3 = p[3 * qs];
+    if (!id.isx) {
+      if (wall || lidf) {
+        if (from_above) a1 = odd ? -a2 : a2;
+        else a2 = odd ? -a1 : a1;
+      }
+      if (mir0) a0 = odd ? -a1 : a1;
+      if (mir3) a3 = odd ? -a2 : a2;
+    }
+    l = Arith3<T>::rec(a1, a2, a0);
+    r = Arith3<T>::rec(a2, a1, a3);
+    if (wall || lidf) {
+      if (from_above) l = odd ? -r : r;
+      else r = odd ? -l : l;
+    }
+  };
+  if (lidf) {
+    const T* lid = reinterpret_cast<const T*>(&S.lid[0][0]) + id.c + 1;
+    V[0] = 0;
+    V[1] = lid[L3_SX * (TX + 2)];
+    V[2] = lid[L3_SY * (TX + 2)];
+    V[3] = lid[(id.below ? L3_E1 : L3_E2) * (TX + 2)];
+  } else {
+    const T* v = reinterpret_cast<const T*>(&S.v[0][0][0]);
+    const T* vy = reinterpret_cast<const T*>(&S.vy[0][0][0]);
+    const int vo = id.isx ? (id.f + 1) * (TX + 2) + id.c : id.f * (TX + 2) + id.c + 1, vs = id.isx ? 1 : TX + 2;
+    const T* t = id.isx ? reinterpret_cast<const T*>(&S.tz[0][0][0]) + id.f * (TX + 2) + id.c
+                        : reinterpret_cast<const T*>(&S.tx[0][0][0]) + id.f * TX + id.c;
+    const int ts = id.isx ? 1 : TX;
+    VSide<T> s[2];
+#pragma unroll
+    for (int side = 0; side < 2; side++) {
+      const T* p = v + vo + side * vs;
+      const T* y = vy + vo + side * vs;
+      const T* d = t + side * ts;
+      s[side].u[0] = p[(pn - 1) * RING3];
+      s[side].u[1] = p[(p1 - 1) * RING3];
+      s[side].u[2] = p[(p2 - 1) * RING3];
+      s[side].e = p[3 * RING3];
+      if (id.isx) {  // t1 = y: du, dv; t2 = z: du, dw
+        s[side].g1[0] = y[0];
+        s[side].g1[1] = y[RING3];
+        s[side].g2[0] = d[0];
+        s[side].g2[1] = d[ZP];
+      } else {  // t1 = x: dw, du; t2 = y: dw, dv
+        s[side].g1[0] = d[XP];
+        s[side].g1[1] = d[0];
+        s[side].g2[0] = y[2 * RING3];
+        s[side].g2[1] = y[RING3];
+      }
+    }
+    if (wall) {
+      VSide<T> o = from_above ? s[1] : s[0];
+      o.u[0] = -o.u[0];
+      o.g1[0] = -o.g1[0];
+      o.g2[0] = -o.g2[0];
+      if (!g.wall) {
+        o.u[1] = -o.u[1];
+        o.u[2] = -o.u[2];
+        o.g1[1] = -o.g1[1];
+        o.g2[1] = -o.g2[1];
+      }
+      if (from_above) s[0] = o;
+      else s[1] = o;
+    }
+    visc3(C, id.isx ? 0 : 2, (id.isx ? ku : (ku == 0 ? 0 : kd)) >= n1, s[0], s[1], V);
+  }
+  comp(0, false, L[0], R[0]);
+  comp(pn, true, L[1], R[1]);
+  comp(p1, false, L[2], R[2]);
+  comp(p2, false, L[3], R[3]);
+  comp(4, false, L[4], R[4]);
+  i64 F[5];
+  if (!flux3(g, C, L, R, V, F)) return false;
+  i64* o;
+  int plane;
+  if (id.isx) {
+    o = &S.fx[0][id.f][id.c], plane = TZ * (TX + 1);
+  } else if (id.below) {
+    o = &S.fg[0][id.c], plane = TX;
+  } else {
+    o = &S.fz[0][id.f][id.c], plane = (TZ + 1) * TX;
+  }
+  o[0] = F[0];
+  o[pn * plane] = F[1];
+  o[p1 * plane] = F[2];
+  o[p2 * plane] = F[3];
+  o[4 * plane] = F[4];
+  return true;
+}
+
+// Do the cells that face id reads lie in the range? The four across it, the
+// y neighbours and the third-direction neighbours of the two at it, and the
+// interface states. Asked only in tiles where some cell does not.
+__device__ __noinline__ bool face3_in_range(const Geom& g, const Tile3Smem& S, const Face3 id, int k0) {
+  auto cell = [&](int r, int c) {  // halo row and column
+    const int k = k0 - 2 + r;
+    return k < 0 || k >= g.nz || S.ok[r][c];
+  };
+  auto celly = [&](int r, int c) {  // ring row and column
+    const int k = k0 - 1 + r;
+    return k < 0 || k >= g.nz || S.oky[r][c];
+  };
+  bool ok = true;
+  if (id.isx) {
+    for (int s = 0; s < 4; s++) ok = ok && cell(id.f + 2, id.c + s);
+    for (int s = 0; s < 2; s++)
+      ok = ok && cell(id.f + 1, id.c + 1 + s) && cell(id.f + 3, id.c + 1 + s) && celly(id.f + 1, id.c + s);
+    if (id.ku == g.n1 || id.ku == g.n1 - 1) ok = ok && S.lid_ok[id.c] && S.lid_ok[id.c + 1];
+  } else {
+    for (int s = 0; s < 4; s++) ok = ok && cell(id.f + s, id.c + 2);
+    for (int s = 0; s < 2; s++)
+      ok = ok && cell(id.f + 1 + s, id.c + 1) && cell(id.f + 1 + s, id.c + 3) && celly(id.f + s, id.c + 1);
+    if (id.ku == g.n1) ok = ok && S.lid_ok[id.c + 1];
+  }
+  return ok;
+}
+
+// The faces marked slow (all: every face), in double, from the tile's cells
+// restaged as doubles.
+__device__ __noinline__ void slow_faces3(const StageArgs& a, const Fx3Const& C, int k0, int i0, int j, int row_hi,
+                                         Tile3Smem& S, bool all) {
+  tile3_cells<double>(a, geo3(a.g), k0, i0, j, row_hi, S);
+  for (int e = threadIdx.x; e < Tile3Smem::NZF + Tile3Smem::NXF + TX; e += NTHREADS) {
+    Face3 id;
+    if (face3_id(a.g, e, k0, row_hi, &id) && (all || S.slow[e])) face3<double>(a.g, C, S, id);
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ void stage_tile3(const StageArgs& a, const Fx3Const& C, int k0, int i0, int j,
+                                            Tile3Smem& S) {
   const Geom& g = a.g;
   const Geo3 G = geo3(g);
   const int tid = threadIdx.x;
   const int nz = g.nz, nx = g.nx, ny = g.ny, n1 = g.n1;
   const int row_hi = a.rhs_only ? a.rhs_hi : nz;
-  const double gamma = g.gamma, gm1 = g.gm1;
-  const int jm = wrap3(j - 1, ny), jp = wrap3(j + 1, ny);
 
-  // ---- 1. stage state with a two-cell halo; y differences of the velocity
-  // on the ring from planes j-1 and j+1; the interface state
-  if (tid < 4) {
-    // x faces: t1 = y, t2 = z; z faces: t1 = x, t2 = y
-    const int dir = tid >> 1, fl = tid & 1;
-    const double inv_dz = fl ? g.inv_dz2 : g.inv_dz1;
-    const double mu = fl ? g.mu2 : g.mu1, kap = fl ? g.kap2 : g.kap1;
-    if (dir == 0) face_consts3(g.inv_dx, g.inv_dy, inv_dz, mu, kap, S.fc[0][fl]);
-    else face_consts3(inv_dz, g.inv_dx, g.inv_dy, mu, kap, S.fc[1][fl]);
-    if (tid == 0) S.gg = g.gamma * g.gm1;
-  }
-  for (int e = tid; e < 5 * (TZ + 4) * (TX + 4); e += NTHREADS) {
-    const int c = e / ((TZ + 4) * (TX + 4)), rem = e - c * (TZ + 4) * (TX + 4);
-    const int rr = rem / (TX + 4), cc = rem - rr * (TX + 4);
-    const int k = k0 - 2 + rr;
-    S.q[c][rr][cc] = (k >= 0 && k < nz) ? stage_val3(a, G, c, k, j, wrap3(i0 - 2 + cc, nx)) : 0.0;
-  }
-  for (int e = tid; e < (TZ + 2) * (TX + 2); e += NTHREADS) {
-    const int rr = e / (TX + 2), cc = e - rr * (TX + 2);
-    const int k = k0 - 1 + rr;
-    if (k < 0 || k >= nz) continue;
-    const int i = wrap3(i0 - 1 + cc, nx);
-    double up[3], dn[3];
-    {
-      const double inv = recip_f64(stage_val3(a, G, 0, k, jp, i));
-      up[0] = stage_val3(a, G, 1, k, jp, i) * inv;
-      up[1] = stage_val3(a, G, 2, k, jp, i) * inv;
-      up[2] = stage_val3(a, G, 3, k, jp, i) * inv;
-    }
-    {
-      const double inv = recip_f64(stage_val3(a, G, 0, k, jm, i));
-      dn[0] = stage_val3(a, G, 1, k, jm, i) * inv;
-      dn[1] = stage_val3(a, G, 2, k, jm, i) * inv;
-      dn[2] = stage_val3(a, G, 3, k, jm, i) * inv;
-    }
-#pragma unroll
-    for (int q = 0; q < 3; q++) S.vy[q][rr][cc] = up[q] - dn[q];
-  }
-  const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZ);
-  if (has_gamma && tid < TX + 2) {
-    double st[9];
-    interface3(a, G, j, wrap3(i0 - 1 + tid, nx), st);
-#pragma unroll
-    for (int s = 0; s < 9; s++) S.gam[s][tid] = st[s];
-  }
-  __syncthreads();
-
-  // ---- 2. u, v, w, T on the ring --------------------------------------------
-  for (int e = tid; e < (TZ + 2) * (TX + 2); e += NTHREADS) {
-    const int rr = e / (TX + 2), cc = e - rr * (TX + 2);
-    const int k = k0 - 1 + rr;
-    if (k < 0 || k >= nz) continue;
-    double q[5], v[4];
-#pragma unroll
-    for (int c = 0; c < 5; c++) q[c] = S.q[c][rr + 1][cc + 1];
-    prim5(q, S.gg, v);
-#pragma unroll
-    for (int c = 0; c < 4; c++) S.v[c][rr][cc] = v[c];
-  }
-  __syncthreads();
-
-  // ---- 3. slopes and tangential differences --------------------------------
-  for (int e = tid; e < TZ * (TX + 2); e += NTHREADS) {
-    const int rr = e / (TX + 2), cc = e - rr * (TX + 2);
-    const int k = k0 + rr;
-    if (k >= row_hi) continue;
-#pragma unroll
-    for (int c = 0; c < 5; c++) S.hx[c][rr][cc] = S.q[c][rr + 2][cc + 2] - S.q[c][rr + 2][cc];
-    const double cv[3] = {S.v[0][rr + 1][cc], S.v[1][rr + 1][cc], S.v[2][rr + 1][cc]};
-    const double uv[3] = {S.v[0][rr + 2][cc], S.v[1][rr + 2][cc], S.v[2][rr + 2][cc]};
-    const double dv[3] = {S.v[0][rr][cc], S.v[1][rr][cc], S.v[2][rr][cc]};
-    double gz[9];
-#pragma unroll
-    for (int q = 0; q < 9; q++) gz[q] = has_gamma ? S.gam[q][cc] : 0.0;
-    double dz[3];
-    dz_uvw(g, k, cv, uv, dv, gz, dz);
-#pragma unroll
-    for (int q = 0; q < 3; q++) S.tz[q][rr][cc] = dz[q];
-  }
-  for (int e = tid; e < (TZ + 2) * TX; e += NTHREADS) {
-    const int rr = e / TX, cc = e - rr * TX;
-    const int k = k0 - 1 + rr;
-    if (k < 0 || k >= nz) continue;
-    const bool up_in = (k + 1 < nz) && ((k + 1 < n1) == (k < n1));
-    const bool dn_in = (k - 1 >= 0) && ((k - 1 < n1) == (k < n1));
-#pragma unroll
-    for (int c = 0; c < 5; c++) {
-      const double own = S.q[c][rr + 1][cc + 2];
-      const double mir = (c == 3) ? -own : own;  // mirror ghost: rho w odd
-      const double up = up_in ? S.q[c][rr + 2][cc + 2] : mir;
-      const double dn = dn_in ? S.q[c][rr][cc + 2] : mir;
-      S.hz[c][rr][cc] = up - dn;
-    }
-#pragma unroll
-    for (int q = 0; q < 3; q++) S.tx[q][rr][cc] = S.v[q][rr][cc + 2] - S.v[q][rr][cc];
-  }
-  __syncthreads();
+  // ---- 1-3. stage state, velocities, tangential differences -----------------
+  const int out = C.k.on ? tile3_cells<i64>(a, G, k0, i0, j, row_hi, S) : 2;
 
   // ---- 4. face fluxes -----------------------------------------------------
-  constexpr int NZF = (TZ + 1) * TX, NXF = TZ * (TX + 1);
-  const double st = g.wall ? 1.0 : -1.0;
-  for (int e = tid; e < NZF + NXF; e += NTHREADS) {
-    if (e < NZF) {
-      const int f = e / TX, cc = e - f * TX;
-      const int ku = k0 + f, kd = ku - 1;
-      if (kd >= row_hi) continue;
-      // z-frame side of ring row rh (q row rh + 1): (u_n, u_t1, u_t2) = (w, u, v)
-      auto zside = [&](int rh, VSide& s) {
-        s.u[0] = S.v[2][rh][cc + 1];
-        s.u[1] = S.v[0][rh][cc + 1];
-        s.u[2] = S.v[1][rh][cc + 1];
-        s.T = S.v[3][rh][cc + 1];
-        s.d1[0] = S.tx[2][rh][cc];
-        s.d1[1] = S.tx[0][rh][cc];
-        s.d1[2] = S.tx[1][rh][cc];
-        s.d2[0] = S.vy[2][rh][cc + 1];
-        s.d2[1] = S.vy[0][rh][cc + 1];
-        s.d2[2] = S.vy[1][rh][cc + 1];
-      };
-      // reconstructed state of ring row rh in the z frame,
-      // q + sq * (central difference), sq = +-1/4
-      auto zstate = [&](int rh, double sq, double o[5]) {
-        const double x[5] = {S.q[0][rh + 1][cc + 2] + sq * S.hz[0][rh][cc],
-                             S.q[1][rh + 1][cc + 2] + sq * S.hz[1][rh][cc],
-                             S.q[2][rh + 1][cc + 2] + sq * S.hz[2][rh][cc],
-                             S.q[3][rh + 1][cc + 2] + sq * S.hz[3][rh][cc],
-                             S.q[4][rh + 1][cc + 2] + sq * S.hz[4][rh][cc]};
-        o[0] = x[0];
-        o[1] = x[3];
-        o[2] = x[1];
-        o[3] = x[2];
-        o[4] = x[4];
-      };
-      double FI[5], FV[5], Ff[5];
-      if (ku == 0 || ku == nz) {
-        // outer wall: the boundary state against its mirror; the cell
-        // against its ghost 2*wall - interior (adiabatic)
-        const bool below = (ku == 0);
-        const int rh = below ? f + 1 : f;
-        const int k = below ? ku : kd;
-        const double* fc = S.fc[1][k >= n1];
-        double b[5], m[5];
-        zstate(rh, below ? -0.25 : 0.25, b);
-#pragma unroll
-        for (int c = 0; c < 5; c++) m[c] = b[c];
-        m[1] = -b[1];
-        if (below) lf_face5(m, b, gamma, gm1, fc[F3_HS], FI);
-        else lf_face5(b, m, gamma, gm1, fc[F3_HS], FI);
-        VSide C, Gh;
-        zside(rh, C);
-        Gh = C;
-        Gh.u[0] = -C.u[0];
-        Gh.d1[0] = -C.d1[0];
-        Gh.d2[0] = -C.d2[0];
-#pragma unroll
-        for (int q = 1; q < 3; q++) {
-          Gh.u[q] = st * C.u[q];
-          Gh.d1[q] = st * C.d1[q];
-          Gh.d2[q] = st * C.d2[q];
-        }
-        if (below) visc_face5(Gh, C, fc, FV);
-        else visc_face5(C, Gh, fc, FV);
-#pragma unroll
-        for (int c = 0; c < 5; c++) Ff[c] = FI[c] - FV[c];
-        // frame (rho, w, u, v, E) -> (rho, u, v, w, E)
-        S.fz[0][f][cc] = Ff[0];
-        S.fz[1][f][cc] = Ff[2];
-        S.fz[2][f][cc] = Ff[3];
-        S.fz[3][f][cc] = Ff[1];
-        S.fz[4][f][cc] = Ff[4];
-      } else if (ku == n1) {
-        // Gamma: a rigid lid from each side (inviscid) and the bulk fluxes
-        // (viscous) with each side's wall state
-        const double sxz = S.gam[0][cc + 1], syz = S.gam[1][cc + 1], Pi = S.gam[2][cc + 1];
-        const double *fc2 = S.fc[1][1], *fc1 = S.fc[1][0];
-        double b[5], m[5];
-        zstate(f + 1, -0.25, b);  // fluid 2, above
-#pragma unroll
-        for (int c = 0; c < 5; c++) m[c] = b[c];
-        m[1] = -b[1];
-        lf_face5(m, b, gamma, gm1, fc2[F3_HS], FI);
-        S.fz[0][f][cc] = FI[0];
-        S.fz[1][f][cc] = FI[2] - sxz * fc2[F3_SC];
-        S.fz[2][f][cc] = FI[3] - syz * fc2[F3_SC];
-        S.fz[3][f][cc] = FI[1];
-        S.fz[4][f][cc] = FI[4] - (S.gam[6][cc + 1] * sxz + S.gam[7][cc + 1] * syz - Pi) * fc2[F3_SC];
-        zstate(f, 0.25, b);  // fluid 1, below
-#pragma unroll
-        for (int c = 0; c < 5; c++) m[c] = b[c];
-        m[1] = -b[1];
-        lf_face5(b, m, gamma, gm1, fc1[F3_HS], FI);
-        S.fg[0][cc] = FI[0];
-        S.fg[1][cc] = FI[2] - sxz * fc1[F3_SC];
-        S.fg[2][cc] = FI[3] - syz * fc1[F3_SC];
-        S.fg[3][cc] = FI[1];
-        S.fg[4][cc] = FI[4] - (S.gam[3][cc + 1] * sxz + S.gam[4][cc + 1] * syz - Pi) * fc1[F3_SC];
-      } else {
-        const double* fc = S.fc[1][kd >= n1];
-        double l[5], r[5];
-        zstate(f, 0.25, l);
-        zstate(f + 1, -0.25, r);
-        lf_face5(l, r, gamma, gm1, fc[F3_HS], FI);
-        VSide sL, sR;
-        zside(f, sL);
-        zside(f + 1, sR);
-        visc_face5(sL, sR, fc, FV);
-        S.fz[0][f][cc] = FI[0] - FV[0];
-        S.fz[1][f][cc] = FI[2] - FV[2];
-        S.fz[2][f][cc] = FI[3] - FV[3];
-        S.fz[3][f][cc] = FI[1] - FV[1];
-        S.fz[4][f][cc] = FI[4] - FV[4];
-      }
-    } else {
-      const int x = e - NZF;
-      const int rr = x / (TX + 1), f = x - rr * (TX + 1);
-      const int k = k0 + rr;
-      if (k >= row_hi) continue;
-      // face between ring cols f (L) and f+1 (R); frame = Cartesian (n = x)
-      double l[5], r[5], FI[5], FV[5];
-#pragma unroll
-      for (int c = 0; c < 5; c++) {
-        l[c] = S.q[c][rr + 2][f + 1] + 0.25 * S.hx[c][rr][f];
-        r[c] = S.q[c][rr + 2][f + 2] - 0.25 * S.hx[c][rr][f + 1];
-      }
-      const double* fc = S.fc[0][k >= n1];
-      lf_face5(l, r, gamma, gm1, fc[F3_HS], FI);
-      VSide s[2];
-#pragma unroll
-      for (int side = 0; side < 2; side++) {
-        const int col = f + side;
-#pragma unroll
-        for (int q = 0; q < 3; q++) {
-          s[side].u[q] = S.v[q][rr + 1][col];
-          s[side].d1[q] = S.vy[q][rr + 1][col];
-          s[side].d2[q] = S.tz[q][rr][col];
-        }
-        s[side].T = S.v[3][rr + 1][col];
-      }
-      visc_face5(s[0], s[1], fc, FV);
-#pragma unroll
-      for (int c = 0; c < 5; c++) S.fx[c][rr][f] = FI[c] - FV[c];
-    }
+  const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZ);
+  const int n_faces = Tile3Smem::NZF + Tile3Smem::NXF + (has_gamma ? TX : 0);
+  bool slow = false;
+  for (int e = out == 2 ? n_faces : tid; e < n_faces; e += NTHREADS) {
+    Face3 id;
+    if (!face3_id(g, e, k0, row_hi, &id)) continue;
+    const bool ok = (out == 0 || face3_in_range(g, S, id, k0)) && face3<i64>(g, C, S, id);
+    S.slow[e] = !ok;
+    slow |= !ok;
   }
-  __syncthreads();
+  slow = out == 2 || __syncthreads_or(slow);
+  if (slow) slow_faces3(a, C, k0, i0, j, row_hi, S, out == 2);
 
   // ---- 5. R = -div F* + s and the stage combination -------------------------
   const int rr = tid / TX, cc = tid - rr * TX;
   const int k = k0 + rr, i = i0 + cc;
   if (k >= row_hi || i >= nx) return;
   const bool under_gamma = (k == n1 - 1);
-  double R[5];
-#pragma unroll
-  for (int c = 0; c < 5; c++) {
-    // every face flux carries the 1/d of its direction already
-    const double up = under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc];
-    R[c] = (S.fx[c][rr][cc] - S.fx[c][rr][cc + 1]) + (S.fz[c][rr][cc] - up) +
-           (a.gy[G.at(c, k, jm, i)] - a.gy[G.at(c, k, j, i)]);
-  }
-  R[3] -= S.q[0][rr + 2][cc + 2] * g.G;
-  R[4] -= S.q[3][rr + 2][cc + 2] * g.G;
-
   const size_t row = (size_t)(k * ny + j) * g.pitch + i;  // offset within a component
   const size_t plane = G.plane;
+  const int jm = wrap3(j - 1, ny);
+  const i64* gy = reinterpret_cast<const i64*>(a.gy);
+  const double hx = 0.5 * g.inv_dx, hy = 0.5 * g.inv_dy, hz = 0.5 * (k < n1 ? g.inv_dz1 : g.inv_dz2);
+  const double s57 = 1.0 / (double)(1ll << fx::S_FLUX);
+  double R[5];
+  i64 y0[5], y1[5];
+  int any = 0;
+#pragma unroll
+  for (int c = 0; c < 5; c++) {
+    y0[c] = gy[G.at(c, k, jm, i)];
+    y1[c] = gy[G.at(c, k, j, i)];
+    const int h0 = (int)(y0[c] >> 32), h1 = (int)(y1[c] >> 32);
+    any |= (h0 ^ (h0 >> 31)) | (h1 ^ (h1 >> 31));
+  }
+  bool dbl = any >= 0x10000000;  // some y flux is a double
+  if (out == 2) dbl = true;
+  else if (slow)
+    dbl = dbl || S.slow[Tile3Smem::NZF + rr * (TX + 1) + cc] || S.slow[Tile3Smem::NZF + rr * (TX + 1) + cc + 1] ||
+          S.slow[rr * TX + cc] ||
+          S.slow[under_gamma ? Tile3Smem::NZF + Tile3Smem::NXF + cc : (rr + 1) * TX + cc];
+  if (dbl) {
+#pragma unroll
+    for (int c = 0; c < 5; c++) {
+      const double dx = __dsub_rn(flux_value(S.fx[c][rr][cc]), flux_value(S.fx[c][rr][cc + 1]));
+      const double dz = __dsub_rn(flux_value(S.fz[c][rr][cc]),
+                                  flux_value(under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc]));
+      const double dy = __dsub_rn(flux_value(y0[c]), flux_value(y1[c]));
+      R[c] = __fma_rn(hx, dx, __fma_rn(hy, dy, __dmul_rn(hz, dz)));
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 5; c++) {
+      const i64 dx = S.fx[c][rr][cc] - S.fx[c][rr][cc + 1];
+      const i64 dz = S.fz[c][rr][cc] - (under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc]);
+      const i64 dy = y0[c] - y1[c];
+      R[c] = C.k.square ? __dmul_rn(C.k.scale, (double)(dx + dy + dz))
+                        : __fma_rn(C.k.scale, (double)dx,
+                                   __fma_rn(__dmul_rn(hy, s57), (double)dy, __dmul_rn(__dmul_rn(hz, s57), (double)dz)));
+    }
+  }
+  {
+    // the source, from the stage state itself
+    double q[5];
+    stage_val3(a, G, k, j, i, q);
+    R[3] = __fma_rn(-g.G, q[0], R[3]);
+    R[4] = __fma_rn(-g.G, q[3], R[4]);
+  }
+
   if (a.rhs_only) {
 #pragma unroll
     for (int c = 0; c < 5; c++) a.rhs_out[(size_t)c * plane + row] = R[c];
@@ -647,7 +838,7 @@ __device__ __forceinline__ void stage_tile3(const StageArgs& a, int k0, int i0, 
     for (int c = 0; c < 5; c++) {
       const size_t o = (size_t)c * plane + row;
       if (!(sg & 1)) Ra[o] = R[c];
-      else a.qF_next[o] = a.qF[o] + g.h2 * (Ra[o] + R[c]);
+      else a.qF_next[o] = __fma_rn(g.h2, __dadd_rn(Ra[o], R[c]), a.qF[o]);
     }
   } else if (k >= g.nS_r) {
     // buffer: RK2 restarted from q_n each substep, weights 1/(2m)
@@ -660,8 +851,8 @@ __device__ __forceinline__ void stage_tile3(const StageArgs& a, int k0, int i0, 
       double* acc = a.b.accB + (size_t)c * pb + ob;
       if (!(sg & 1)) Ra[o] = R[c];
       if (sg == 0) *acc = R[c];
-      else if (last) *acc = a.b.qA[o] + g.h2 * (*acc + R[c]);
-      else *acc = *acc + R[c];
+      else if (last) *acc = __fma_rn(g.h2, __dadd_rn(*acc, R[c]), a.b.qA[o]);
+      else *acc = __dadd_rn(*acc, R[c]);
     }
   } else {
     // slow region: stages 1 and 2 only (Algorithm 1)
@@ -670,7 +861,7 @@ __device__ __forceinline__ void stage_tile3(const StageArgs& a, int k0, int i0, 
     for (int c = 0; c < 5; c++) {
       const size_t o = (size_t)c * plane + row;
       if (sg == 0) Ra[o] = R[c];
-      else a.b.accS[(size_t)c * ps + row] = a.b.qA[o] + g.hdt * (Ra[o] + R[c]);
+      else a.b.accS[(size_t)c * ps + row] = __fma_rn(g.hdt, __dadd_rn(Ra[o], R[c]), a.b.qA[o]);
     }
   }
 }

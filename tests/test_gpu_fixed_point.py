@@ -14,6 +14,7 @@ import pytest
 from oracle import oracle as O
 from paper_2202_11890_gb300 import workloads as W
 from pairs import oracle_threads, pair, rel_err
+from test_gpu_3d import gpu_rhs3, pair3, rel3
 from test_gpu_parity import gpu_rhs
 from test_gpu_tile_shapes import SHAPES, launch_buckets, load_table
 
@@ -69,6 +70,43 @@ def test_rhs_across_the_range_matches_oracle(kind, xwall, wall):
     q = state(kind)
     cfg, P, _ = pair(GRID, 2, dt=0.001, xwall=xwall, wall=wall)
     err = rel_err(gpu_rhs(cfg, q), O.rhs(P, q))
+    assert np.all(err < 1e-12), err
+
+
+GRID3 = W.Grid3(45, 6, 7, 4, 10)  # ragged tiles, Gamma inside a tile
+
+
+def state3(kind):
+    """As state(), in 3-D: planes 1 to 4 of columns 15-38 and rows 4-17."""
+    rng = np.random.default_rng(43)
+    rho, p = W.rest_primitives(GRID3.column_grid())
+    shape = (GRID3.nz, GRID3.ny, GRID3.nx)
+    r = [0.02 * rng.uniform(-1, 1, shape) for _ in range(5)]
+    rho, p = rho[:, None, :] * (1 + r[0]), p[:, None, :] * (1 + r[1])
+    u, v, w = r[2:]
+    rz, ry, rx = [np.minimum(1.0, 1.3 * (1.0 - np.abs(np.linspace(-1, 1, n)))) for n in (14, 6, 24)]
+    part = np.zeros(shape)
+    part[4:18, :, 15:39] = rz[:, None, None] * ry[None, :, None] * rx
+    if kind == "dense":
+        rho, p = 8.0 * rho, 8.0 * p
+    elif kind == "dense patch":
+        rho, p = rho * 4.3 ** part, p * 2.0 ** part
+    elif kind == "fast patch":
+        u, v, w = u + part, v - 0.8 * part, w + 0.3 * part
+    elif kind == "cold patch":
+        p = p * 0.2 ** part
+    elif kind == "hot patch":
+        p = p * 4.5 ** part
+    return W.conserved3(rho, u, v, w, p)
+
+
+@pytest.mark.parametrize("wall,mu1", [(0, W.MU1), (1, 0.1)])
+@pytest.mark.parametrize("kind", [k for k in KINDS if k != "thin patch"])
+def test_rhs3_across_the_range_matches_oracle(kind, wall, mu1):
+    """mu1 = 0.1 puts fluid 1's coefficients beyond the fixed-point form."""
+    q = state3(kind)
+    cfg, P, _ = pair3(GRID3, 2, dt=0.001, wall=wall, mu1=mu1)
+    err = rel3(gpu_rhs3(cfg, q), O.rhs3(P, q))
     assert np.all(err < 1e-12), err
 
 
