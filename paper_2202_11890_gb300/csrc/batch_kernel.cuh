@@ -149,11 +149,12 @@ template <int PAR>
 __global__ void __launch_bounds__(MIXED_THREADS, 3)
     wave_stage_mixed(const StageArgs* __restrict__ tab, const StageWork* __restrict__ work, int single) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  const StageWork w = single >= 0 ? StageWork{single, (int)blockIdx.x} : work[blockIdx.x];
+  const StageWork w = single >= 0 ? StageWork{single, 3 * (int)blockIdx.x} : work[blockIdx.x];
   const StageArgs& a = tab[w.args];
-  const int tzi = w.tile / a.tiles_x, txi = w.tile - tzi * a.tiles_x;
+  const int t = w.tile / 3, half = w.tile - 3 * t - 1;
+  const int tzi = t / a.tiles_x, txi = t - tzi * a.tiles_x;
   (void)stage_tile_mixed<PAR>(a, a.row0 + tzi * MTZ, txi * TX, *reinterpret_cast<MixedTileSmem*>(smem_raw),
-                              nullptr, nullptr);
+                              nullptr, nullptr, half);
 }
 
 // Step completion of rows r0 .. r0 + fin_rows(nx) - 1 of component c of one

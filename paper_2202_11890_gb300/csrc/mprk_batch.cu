@@ -298,8 +298,17 @@ void build_wave(const std::vector<BatchInst>& hinst, int groups, std::vector<Sta
       for (int j : members[g]) {
         const BatchInst& bi = hinst[j];
         if (st >= bi.g.s * bi.g.m) continue;
-        const int nt = stage_tiles(batch_stage_args(bi, st, MTZ));
-        for (int t = 0; t < nt; t++) work.push_back({bi.args_base + st, t});
+        const StageArgs sa = batch_stage_args(bi, st, MTZ);
+        const int nt = stage_tiles(sa);
+        for (int t = 0; t < nt; t++) {
+          const int k0 = sa.row0 + t / sa.tiles_x * MTZ, i0 = t % sa.tiles_x * TX;
+          if (pair_interior(sa, k0, i0) || k0 + TZ >= bi.g.nz) {
+            work.push_back({bi.args_base + st, 3 * t});
+          } else {
+            work.push_back({bi.args_base + st, 3 * t + 1});
+            work.push_back({bi.args_base + st, 3 * t + 2});
+          }
+        }
         n_in++;
         only = bi.args_base + st;
       }
@@ -354,7 +363,7 @@ void wave_step(const WaveLaunches& L, const BatchInst* d_insts, const StageArgs*
     for (int k = 0; k + 1 < launches; k++) {
       const int one = L.single[g][k];
       if (one >= 0)
-        launch_stage(L.h_args[one], 1, o[k + 1] - o[k], st, &L.h_maps[L.args_inst[one]]);
+        launch_stage(L.h_args[one], 1, stage_tiles(L.h_args[one]), st, &L.h_maps[L.args_inst[one]]);
       else
         wave_launch_stage(k & 1, o[k + 1] - o[k], d_args, d_work + o[k], -1, st);
     }

@@ -197,6 +197,24 @@ __host__ __device__ inline int stage_tiles(const StageArgs& a) {
   return a.tiles_x * ((hi - a.row0 + a.tz - 1) / a.tz);
 }
 
+// FP32-flux tiles: the TX x MTZ tile from row k0, column i0 takes the pair path
+// (stage_tile_mixed.cuh). An interior tile needs none of the ghost rules: rows k0-2 .. k0+MTZ+1 lie
+// inside the grid and inside one fluid, and with x walls its halo columns
+// i0-2 .. i0+TX+1 lie between them. For a stage (not the right-hand-side
+// hook) they also lie on one side of the F-row bound.
+__host__ __device__ inline bool pair_interior(const StageArgs& a, int k0, int i0) {
+  const Geom& g = a.g;
+  const int hi = a.rhs_only ? a.rhs_hi : g.nz;
+  const int lo_h = k0 - 2, hi_h = k0 + MTZ + 2;  // halo rows [lo_h, hi_h)
+  if (lo_h < 0 || hi_h > g.nz || k0 + MTZ > hi || !(g.n1 <= lo_h || g.n1 >= hi_h)) return false;
+  if (g.xwall && (i0 < 2 || i0 + TX + 2 > g.nx)) return false;  // halo columns inside the walls
+  if (a.rhs_only) return true;
+  // S and B rows may share a tile (the combination picks per cell, and both
+  // take their stage values from q_n with dt); the F rows' state and step
+  // differ, so no F row lies within the halo of a tile with S or B rows
+  return g.n1_r <= lo_h || g.n1_r >= hi_h;
+}
+
 // Tensor maps of the FP32-flux float planes ([4][nz][pitch] float each) for
 // the bulk tensor copies of the stage kernel (mprk_kernels.cu).
 struct StageMaps {

@@ -47,13 +47,14 @@ __global__ void __launch_bounds__(MIXED_THREADS, 3)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   MixedKernelSmem& S = *reinterpret_cast<MixedKernelSmem*>(smem_raw);
   const int k0 = a.row0 + blockIdx.y * MTZ, i0 = blockIdx.x * TX;
-  const bool staged = tile_bulk_ok(a, k0, i0);
+  const int half = gridDim.z > 1 ? (int)blockIdx.z : -1;
+  const bool staged = half <= 0 && tile_bulk_ok(a, k0, i0);
   if (staged && threadIdx.x == MIXED_THREADS - 32) {
     mbar_init(&S.bar);
     stage_issue(a, k0, i0, S.stg, &S.bar, &tm_sb, &tm_f, &tm_ra);
   }
   if (staged) __syncthreads();  // the mbarrier is initialised before anyone waits on it
-  if (!stage_tile_mixed<PAR>(a, k0, i0, S.work, staged ? &S.stg : nullptr, &S.bar)) {
+  if (!stage_tile_mixed<PAR>(a, k0, i0, S.work, staged ? &S.stg : nullptr, &S.bar, half)) {
     // a tensor copy never completed within the bound: flag it, give the
     // copies one more bounded wait, and leave
     if (threadIdx.x == 0 && a.status) atomicOr(a.status, ST_TIMEOUT);
@@ -233,7 +234,12 @@ cudaError_t launch_stage(const StageArgs& a, int precision, int n_tiles, cudaStr
     const CUtensorMap& sb = staged ? maps->dA : none;
     const CUtensorMap& f = staged ? (a.dF == a.b.dA ? maps->dA : maps->dB) : none;
     const CUtensorMap& ra = staged ? maps->Ra : none;
-    const dim3 grid(a.tiles_x, n_tiles / a.tiles_x);
+    // a launch whose tiles' halves fit in one wave of three CTAs per SM: the
+    // general path's two halves run side by side, since one such tile takes
+    // about twice a pair tile's time and would end the launch alone (321 x
+    // 273 cells, m = 4: 110.7 -> 71.9 us per step; larger launches start
+    // other tiles meanwhile, and their idle half CTAs would cost more)
+    const dim3 grid(a.tiles_x, n_tiles / a.tiles_x, 2 * n_tiles <= 3 * sm_count() ? 2 : 1);
     const size_t smem = mixed_kernel_smem(a.stage & 1);
     if (a.rhs_only) {
       stage_kernel_mixed<PAR_RT><<<grid, MIXED_THREADS, smem, stream>>>(s, sb, f, ra);

@@ -775,23 +775,6 @@ __device__ __forceinline__ void pair_z_face(PairSmem& S, const PairConst& C, int
   S.fzb[hu - 2][cc] = cat2(sub2(FI[1], FV[0]), sub2(FI[3], FV[2]));
 }
 
-// An interior tile needs none of the ghost rules: rows k0-2 .. k0+MTZ+1 lie
-// inside the grid and inside one fluid, and with x walls its halo columns
-// i0-2 .. i0+TX+1 lie between them. For a stage (not the right-hand-side
-// hook) they also lie on one side of the F-row bound.
-__device__ __forceinline__ bool pair_interior(const StageArgs& a, int k0, int i0) {
-  const Geom& g = a.g;
-  const int hi = a.rhs_only ? a.rhs_hi : g.nz;
-  const int lo_h = k0 - 2, hi_h = k0 + MTZ + 2;  // halo rows [lo_h, hi_h)
-  if (lo_h < 0 || hi_h > g.nz || k0 + MTZ > hi || !(g.n1 <= lo_h || g.n1 >= hi_h)) return false;
-  if (g.xwall && (i0 < 2 || i0 + TX + 2 > g.nx)) return false;  // halo columns inside the walls
-  if (a.rhs_only) return true;
-  // S and B rows may share a tile (the combination picks per cell, and both
-  // take their stage values from q_n with dt); the F rows' state and step
-  // differ, so no F row lies within the halo of a tile with S or B rows
-  return g.n1_r <= lo_h || g.n1_r >= hi_h;
-}
-
 // Stage combination of one cell outside the F rows (B and S rows), the
 // general path's arithmetic with R in float.
 template <int PAR>
@@ -1104,15 +1087,17 @@ union MixedTileSmem {
   PairSmem pair;
 };
 
+// half: a tile on the general path runs as two TX x TZ halves one after the
+// other (-1), or as two CTAs, each with one half (0 and 1; half 1 of a pair
+// tile has nothing to do).
 template <int PAR>
 __device__ __forceinline__ bool stage_tile_mixed(const StageArgs& a, int k0, int i0, MixedTileSmem& S,
-                                                 const Stage* stg, unsigned long long* bar) {
-  if (pair_interior(a, k0, i0)) return pair_tile<PAR>(a, k0, i0, S.pair, stg, bar);
-  mixed_subtile<PAR>(a, k0, i0, S.gen);
+                                                 const Stage* stg, unsigned long long* bar, int half = -1) {
+  if (pair_interior(a, k0, i0)) return half > 0 || pair_tile<PAR>(a, k0, i0, S.pair, stg, bar);
   const int hi = rhs_mode<PAR>(a) ? a.rhs_hi : a.g.nz;
-  if (k0 + TZ < hi) {
-    __syncthreads();  // the first half's phase 3 reads shared memory
-    mixed_subtile<PAR>(a, k0 + TZ, i0, S.gen);
+  for (int h = max(half, 0); h < (half < 0 ? 2 : half + 1) && k0 + h * TZ < hi; h++) {
+    if (half < 0 && h > 0) __syncthreads();  // the first half's phase 3 reads shared memory
+    mixed_subtile<PAR>(a, k0 + h * TZ, i0, S.gen);
   }
   return true;
 }
