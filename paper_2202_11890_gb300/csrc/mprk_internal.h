@@ -263,6 +263,11 @@ cudaError_t launch_stage3(const StageArgs& a, cudaStream_t stream, bool chained 
 // and the float shadow dA = q - q_ref of qA.
 cudaError_t launch_reference(const Geom& g, const double* q, double* refd, float* rowc,
                              cudaStream_t stream);
+// `rows` rows of `width` doubles from src (row stride spitch) to dst (row
+// stride dpitch; null: not copied), and where rowc is given the float shadow
+// of row r = c nz + k into `shadow` (row stride dpitch).
+cudaError_t launch_copy_state(double* dst, size_t dpitch, const double* src, size_t spitch, int width, long long rows,
+                              int nz, const float* rowc, float* shadow, cudaStream_t stream);
 cudaError_t launch_shadow(const Geom& g, const double* q, const float* rowc, float* d,
                           cudaStream_t stream);
 cudaError_t launch_diag(const Geom& g, const double* q, double* partials, int nblocks,
@@ -288,11 +293,11 @@ __device__ __forceinline__ void chain_wait() {
 
 // One launch, chained to the one before it on the stream or not.
 template <typename... P, typename... A>
-cudaError_t launch_kernel(void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, bool chained,
+cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool chained,
                           const A&... args) {
   cudaLaunchConfig_t c = {};
   c.gridDim = grid;
-  c.blockDim = dim3(threads);
+  c.blockDim = block;
   c.dynamicSmemBytes = smem;
   c.stream = s;
   cudaLaunchAttribute at[1];

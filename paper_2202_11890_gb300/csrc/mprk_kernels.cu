@@ -385,26 +385,96 @@ cudaError_t launch_reference(const Geom& g, const double* q, double* refd, float
   return cudaGetLastError();
 }
 
-__global__ void shadow_kernel(const Geom g, const double* __restrict__ q, const float* __restrict__ rowc,
-                              float* d) {
-  const long long total = 4LL * g.nz * g.nx;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(e / ((long long)g.nz * g.nx));
-    const int rem = (int)(e - (long long)c * g.nz * g.nx);
-    const int k = rem / g.nx, i = rem - k * g.nx;
-    const size_t o = ((size_t)c * g.nz + k) * g.pitch + i;
-    d[o] = narrow(q[o] - (double)rowc[4 * k + c]);
+// Blocks of the row kernels below: 256 threads as BX pairs of columns by BY
+// rows, U rows per thread (all its loads in flight before its first store).
+struct RowGrid {
+  dim3 grid, block;
+  bool four;  // U = 4: the rows of a launch that fills the GPU even so; else 1
+};
+namespace {
+RowGrid row_grid(int width, long long rows, int comps) {
+  const int pairs = (width + 1) / 2;
+  unsigned bx = 32;
+  while (bx < 256 && (int)bx < pairs) bx *= 2;
+  const unsigned by = 256 / bx;
+  RowGrid r;
+  r.block = dim3(bx, by);
+  r.four = rows * comps * pairs >= 4LL * 2048 * sm_count();
+  const long long span = (long long)by * (r.four ? 4 : 1), gy = (rows + span - 1) / span;
+  r.grid = dim3((pairs + bx - 1) / bx, (unsigned)(gy < 65535 ? gy : 65535), comps);
+  return r;
+}
+bool a16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+}  // namespace
+
+// The copy of launch_copy_state. Bound by HBM: 4096 x 2048 cells, 537 MB,
+// 140 -> 90 us (one 8-byte load in flight per thread before), with the
+// float shadow in the same pass 320 -> 175 us (a pass of its own before).
+// vec: 16-byte accesses fit every row.
+template <int U>
+__global__ void __launch_bounds__(256) copy_state_kernel(double* __restrict__ dst, size_t dpitch,
+                                                         const double* __restrict__ src, size_t spitch, int width,
+                                                         long long rows, int nz, const float* __restrict__ rowc,
+                                                         float* __restrict__ shadow, int vec) {
+  const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (i >= width) return;
+  const bool two = i + 1 < width;
+  for (long long r0 = (long long)blockIdx.y * U * blockDim.y + threadIdx.y; r0 < rows;
+       r0 += (long long)gridDim.y * U * blockDim.y) {
+    double2 v[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const long long r = r0 + u * blockDim.y;
+      if (r >= rows) break;
+      const double* s = src + r * spitch + i;
+      if (vec && two) v[u] = *reinterpret_cast<const double2*>(s);
+      else v[u] = make_double2(s[0], two ? s[1] : 0.0);
+    }
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const long long r = r0 + u * blockDim.y;
+      if (r >= rows) break;
+      if (dst) {
+        double* d = dst + r * dpitch + i;
+        if (vec && two) {
+          *reinterpret_cast<double2*>(d) = v[u];
+        } else {
+          d[0] = v[u].x;
+          if (two) d[1] = v[u].y;
+        }
+      }
+      if (rowc) {
+        const int c = (int)(r / nz), k = (int)(r - (long long)c * nz);
+        const double ref = (double)rowc[4 * k + c];
+        float* d = shadow + r * dpitch + i;
+        const float x = narrow(v[u].x - ref), y = narrow(v[u].y - ref);
+        if (vec && two) {
+          *reinterpret_cast<float2*>(d) = make_float2(x, y);
+        } else {
+          d[0] = x;
+          if (two) d[1] = y;
+        }
+      }
+    }
   }
+}
+
+cudaError_t launch_copy_state(double* dst, size_t dpitch, const double* src, size_t spitch, int width, long long rows,
+                              int nz, const float* rowc, float* shadow, cudaStream_t stream) {
+  if (width <= 0 || rows <= 0) return cudaSuccess;
+  const int vec = dpitch % 2 == 0 && spitch % 2 == 0 && a16(dst) && a16(src) &&
+                  (reinterpret_cast<uintptr_t>(shadow) & 7u) == 0;
+  const RowGrid G = row_grid(width, rows, 1);
+  if (G.four)
+    copy_state_kernel<4><<<G.grid, G.block, 0, stream>>>(dst, dpitch, src, spitch, width, rows, nz, rowc, shadow, vec);
+  else
+    copy_state_kernel<1><<<G.grid, G.block, 0, stream>>>(dst, dpitch, src, spitch, width, rows, nz, rowc, shadow, vec);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_shadow(const Geom& g, const double* q, const float* rowc, float* d,
                           cudaStream_t stream) {
-  const long long total = 4LL * g.nz * g.nx;
-  int blocks = (int)((total + 255) / 256);
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  shadow_kernel<<<blocks, 256, 0, stream>>>(g, q, rowc, d);
-  return cudaGetLastError();
+  return launch_copy_state(nullptr, (size_t)g.pitch, q, (size_t)g.pitch, g.nx, 4LL * g.nz, g.nz, rowc, d, stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -414,38 +484,60 @@ cudaError_t launch_shadow(const Geom& g, const double* q, const float* rowc, flo
 // ---------------------------------------------------------------------------
 // An x-row r of a component is (k, j) with r = k ny + j (ny = 1 in 2-D);
 // the buffers' rows of the S and B bands are numbered the same way.
-// One row of one component per block row: blockIdx.z the component,
-// rows r = blockIdx.y + n gridDim.y (r = k ny + j, k the z row), threads
-// over x, two consecutive cells per thread. vec: every row starts on a
-// 16-byte boundary (an even pitch and 16-byte aligned buffers, as
-// mprk_create's padded layout always has), so the pairs move as 16-byte
-// loads and stores; otherwise (mprk_step_static's unpadded rows) one cell
-// at a time. F rows after an even m already hold q_{n+1} in qA and only
-// refresh the float shadow (which the last stage leaves to this kernel).
-// Rows k_lo <= k < k_hi (x-rows r = k ny + j).
-__global__ void finalize_kernel(const Geom g, const Bufs b, int m_odd, int vec, int k_lo, int k_hi) {
+// blockIdx.z the component; rows r = k ny + j and pairs of columns as in
+// row_grid. vec: every row starts on a 16-byte boundary (an even pitch and
+// 16-byte aligned buffers, as mprk_create's padded layout always has), so the
+// pairs move as 16-byte loads and stores; otherwise (mprk_step_static's
+// unpadded rows) one cell at a time. F rows after an even m already hold
+// q_{n+1} in qA and only refresh the float shadow (which the last stage
+// leaves to this kernel). Rows k < k_hi. 4096 x 2048 cells in FP32-flux mode,
+// 600 MB: 164 -> 139 us with four rows per thread instead of one.
+template <int U>
+__global__ void __launch_bounds__(256) finalize_kernel(const Geom g, const Bufs b, int m_odd, int vec, int k_hi) {
   const bool mixed = b.dA != nullptr;
   chain_wait();
   const int c = blockIdx.z;
-  for (int r = k_lo * g.ny + blockIdx.y; r < k_hi * g.ny; r += gridDim.y) {
-    const int k = r / g.ny;
-    const size_t o = ((size_t)c * g.nz * g.ny + r) * g.pitch;
-    const double* src;
-    if (k < g.nS_r) src = b.accS + ((size_t)c * g.nS_r * g.ny + r) * g.pitch;
-    else if (k < g.n1_r) src = b.accB + ((size_t)c * (g.n1_r - g.nS_r) * g.ny + (r - (size_t)g.nS_r * g.ny)) * g.pitch;
-    else src = (m_odd ? b.qB : b.qA) + o;
-    const bool store_q = k < g.n1_r || m_odd;
-    const double ref = mixed ? (double)b.rowc[4 * k + c] : 0.0;
-    for (int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x); i < g.nx; i += 2 * gridDim.x * blockDim.x) {
-      if (vec && i + 1 < g.nx) {
-        const double2 v = *reinterpret_cast<const double2*>(src + i);
-        if (store_q) *reinterpret_cast<double2*>(b.qA + o + i) = v;
-        if (mixed) *reinterpret_cast<float2*>(b.dA + o + i) = make_float2(narrow(v.x - ref), narrow(v.y - ref));
-      } else {
-        for (int j = i; j < i + 2 && j < g.nx; j++) {
-          const double v = src[j];
-          if (store_q) b.qA[o + j] = v;
-          if (mixed) b.dA[o + j] = narrow(v - ref);
+  const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (i >= g.nx) return;
+  const bool two = i + 1 < g.nx;
+  const long long rows = (long long)k_hi * g.ny;
+  const size_t base = (size_t)c * g.nz * g.ny, baseS = (size_t)c * g.nS_r * g.ny,
+               baseB = (size_t)c * (g.n1_r - g.nS_r) * g.ny;
+  for (long long r0 = (long long)blockIdx.y * U * blockDim.y + threadIdx.y; r0 < rows;
+       r0 += (long long)gridDim.y * U * blockDim.y) {
+    double2 v[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const long long r = r0 + u * blockDim.y;
+      if (r >= rows) break;
+      const double* s;
+      if (r < (long long)g.nS_r * g.ny) s = b.accS + (baseS + r) * g.pitch;
+      else if (r < (long long)g.n1_r * g.ny) s = b.accB + (baseB + (r - (long long)g.nS_r * g.ny)) * g.pitch;
+      else s = (m_odd ? b.qB : b.qA) + (base + r) * g.pitch;
+      if (vec && two) v[u] = *reinterpret_cast<const double2*>(s + i);
+      else v[u] = make_double2(s[i], two ? s[i + 1] : 0.0);
+    }
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const long long r = r0 + u * blockDim.y;
+      if (r >= rows) break;
+      const size_t o = (base + r) * g.pitch + i;
+      if (r < (long long)g.n1_r * g.ny || m_odd) {
+        if (vec && two) {
+          *reinterpret_cast<double2*>(b.qA + o) = v[u];
+        } else {
+          b.qA[o] = v[u].x;
+          if (two) b.qA[o + 1] = v[u].y;
+        }
+      }
+      if (mixed) {  // 2-D: r is the row k
+        const double ref = (double)b.rowc[4 * r + c];
+        const float x = narrow(v[u].x - ref), y = narrow(v[u].y - ref);
+        if (vec && two) {
+          *reinterpret_cast<float2*>(b.dA + o) = make_float2(x, y);
+        } else {
+          b.dA[o] = x;
+          if (two) b.dA[o + 1] = y;
         }
       }
     }
@@ -453,17 +545,13 @@ __global__ void finalize_kernel(const Geom g, const Bufs b, int m_odd, int vec, 
 }
 
 cudaError_t launch_finalize(const Geom& g, const Bufs& b, int m_odd, cudaStream_t stream, bool chained) {
-  const int k_lo = 0;
   const int k_hi = (m_odd || b.dA) ? g.nz : g.n1_r;  // rows it completes
-  const int rows = k_hi - k_lo;
-  if (rows <= 0) return cudaSuccess;
-  auto a16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
-  const int vec = (g.pitch % 2 == 0 && a16(b.qA) && a16(b.qB) && a16(b.accS) && a16(b.accB) &&
-                   (!b.dA || (reinterpret_cast<uintptr_t>(b.dA) & 7u) == 0))
-                      ? 1
-                      : 0;
-  const dim3 grid((g.nx + 511) / 512, (unsigned)std::min(rows * g.ny, 65535), (unsigned)g.nc);
-  return launch_kernel(finalize_kernel, grid, 256, 0, stream, chained && !b.dA, g, b, m_odd, vec, k_lo, k_hi);
+  if (k_hi <= 0) return cudaSuccess;
+  const int vec = g.pitch % 2 == 0 && a16(b.qA) && a16(b.qB) && a16(b.accS) && a16(b.accB) &&
+                  (!b.dA || (reinterpret_cast<uintptr_t>(b.dA) & 7u) == 0);
+  const RowGrid G = row_grid(g.nx, (long long)k_hi * g.ny, g.nc);
+  return launch_kernel(G.four ? finalize_kernel<4> : finalize_kernel<1>, G.grid, G.block, 0, stream,
+                       chained && !b.dA, g, b, m_odd, vec, k_hi);
 }
 
 // ---------------------------------------------------------------------------
