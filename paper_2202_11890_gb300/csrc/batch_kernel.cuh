@@ -68,7 +68,7 @@ constexpr int BATCH_ARGS_BYTES = (int)((sizeof(StageArgs) + 127) / 128 * 128);
 template <bool GEN, int ROWS>
 __device__ __noinline__ void batch_tile_fp64(int tile) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  stage_tile<GEN, NTHREADS, ROWS>(*reinterpret_cast<const StageArgs*>(smem_raw), tile,
+  stage_tile<GEN, FP64_THREADS, ROWS>(*reinterpret_cast<const StageArgs*>(smem_raw), tile,
                                   *reinterpret_cast<TileSmem<ROWS>*>(smem_raw + BATCH_ARGS_BYTES));
 }
 

@@ -65,7 +65,7 @@ struct StageWork {
 };
 
 // block size of the batch kernel per precision (the tile's own block size)
-constexpr int batch_threads(int prec) { return prec == 0 ? NTHREADS : MIXED_THREADS; }
+constexpr int batch_threads(int prec) { return prec == 0 ? FP64_THREADS : MIXED_THREADS; }
 
 // The persistent kernel of a precision and FP64 tile rows (mprk_kernels.cu,
 // the translation unit of the single-instance stage kernels, so that both

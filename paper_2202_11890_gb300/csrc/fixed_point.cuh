@@ -159,5 +159,12 @@ __host__ __device__ __forceinline__ i64 from_double(i64 bits, int s) {
   return (v ^ n) - n;
 }
 
+// The same of a positive double.
+__host__ __device__ __forceinline__ i64 from_positive(i64 bits, int s) {
+  const u64 m = (u64)bits << 10 | 1ull << 62;
+  const int sh = 1085 - s - (int)((u64)bits >> 52);
+  return (i64)((m & 0x7fffffffffffffffull) >> (sh & 63));
+}
+
 }  // namespace fx
 }  // namespace mprk

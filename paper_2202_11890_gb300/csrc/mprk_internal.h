@@ -28,6 +28,9 @@ namespace mprk {
 constexpr int TX = 32;
 constexpr int TZ = 8;
 constexpr int NTHREADS = TX * TZ;
+// Threads of the FP64 tile of TZ rows: nine warps, two face jobs each
+// (stage_tile.cuh).
+constexpr int FP64_THREADS = NTHREADS + TX;
 // The FP32-flux kernel's tile is TX x 2*TZ cells; each thread of its fast
 // path carries two cells of one column, rows k and k + TZ.
 constexpr int MTZ = 2 * TZ;

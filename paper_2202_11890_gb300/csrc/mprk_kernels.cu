@@ -23,12 +23,12 @@
 namespace mprk {
 
 // GEN: the general s-stage base (RK3, RK4) in place of Heun's low-storage
-// combination. TZR: tile rows (TZ; 4 or 2 for launches of few tiles). One
-// thread per cell: 80 registers, a few spilled in the tile (three 32 x 8
-// CTAs per SM). NT = 2 TX TZR: two threads per cell for launches with no
-// more tiles than SMs.
-template <bool GEN = false, int NT = NTHREADS, int TZR = TZ>
-__global__ void __launch_bounds__(NT, NT == TX * TZR ? 3 * NTHREADS / NT : 1)
+// combination. TZR: tile rows (TZ; 4 or 2 for launches of few tiles). NT:
+// TZR + 1 warps, up to 27 of them per SM (72 registers); twice that for
+// launches with no more tiles than SMs.
+constexpr int fp64_ctas(int rows) { return rows == TZ ? 3 : rows == TZ / 2 ? 5 : 9; }
+template <bool GEN = false, int NT = FP64_THREADS, int TZR = TZ>
+__global__ void __launch_bounds__(NT, NT == TX * (TZR + 1) ? fp64_ctas(TZR) : 1)
     stage_kernel(const __grid_constant__ StageArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   TileSmem<TZR>& S = *reinterpret_cast<TileSmem<TZR>*>(smem_raw);
@@ -104,10 +104,10 @@ cudaError_t prepare_kernels() {
   e = cudaFuncSetAttribute(stage_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)sizeof(TileSmem<>));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(stage_kernel<false, 2 * NTHREADS>,
+  e = cudaFuncSetAttribute(stage_kernel<false, 2 * FP64_THREADS>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem<>));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(stage_kernel<true, 2 * NTHREADS>,
+  e = cudaFuncSetAttribute(stage_kernel<true, 2 * FP64_THREADS>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem<>));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(yface3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(YfaceSmem));
@@ -182,7 +182,7 @@ namespace {
 // One FP64 stage launch with TZR-row tiles; wide: two threads per cell.
 template <int TZR>
 cudaError_t launch_fp64(const StageArgs& a, int n_tiles, bool wide, cudaStream_t stream, bool chained) {
-  constexpr int NT1 = TX * TZR, NT2 = 2 * TX * TZR;
+  constexpr int NT1 = TX * (TZR + 1), NT2 = 2 * NT1;
   const size_t smem = sizeof(TileSmem<TZR>);
   if (wide && a.g.gen) return launch_kernel(stage_kernel<true, NT2, TZR>, n_tiles, NT2, smem, stream, chained, a);
   if (wide) return launch_kernel(stage_kernel<false, NT2, TZR>, n_tiles, NT2, smem, stream, chained, a);

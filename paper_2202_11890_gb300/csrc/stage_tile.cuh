@@ -5,26 +5,28 @@
 // launches of few tiles). It
 //   1. stages the stage state of the tile plus a two-cell halo in shared
 //      memory (x periodic; stage values q + h R_a rebuilt on the fly in
-//      double), as doubles and as 64-bit fixed point,
-//   2. computes u, w and e = T / (gamma (gamma - 1)) on the tile plus a
-//      one-cell ring, and the interface state (bulk fluxes and wall states of
-//      App. B) when the tile touches it,
-//   3. computes the central differences of u, w along the faces (tangential
-//      viscous gradients), with wall-state ghosts beyond walls and the
-//      interface,
-//   4. computes every x and z face flux of the tile once (Lax–Friedrichs
+//      double), as doubles and as 64-bit fixed point, and computes u, w and
+//      e = T / (gamma (gamma - 1)) on the tile plus a one-cell ring,
+//   2. computes the interface state (bulk fluxes and wall states of App. B)
+//      when the tile touches it,
+//   3. computes every x and z face flux of the tile once (Lax–Friedrichs
 //      inviscid flux of Sec. 2.1 on the linear reconstruction of the
 //      conserved variables, minus the common-value viscous flux of App. B),
-//      in one direction-generic routine written in the face frame,
-//   5. forms R = -div F* + s per cell and applies the partition's stage
+//      in one direction-generic routine written in the face frame, with
+//      mirror or wall-state ghosts beyond walls and the interface,
+//   4. forms R = -div F* + s per cell and applies the partition's stage
 //      combination (Eq. MRK2 in low-storage form) in double precision.
+// Only two barriers separate them: 1 and 2 from 3, and 3 from 4 (with phases
+// of their own for the ring and the tangential differences, and faces dealt to
+// threads in three uneven rounds, the step above took 2.39 ms).
 //
-// Phases 2 to 4 run in 64-bit fixed point (fixed_point.cuh): as double
+// Velocities, differences and fluxes run in 64-bit fixed point (fixed_point.cuh): as double
 // arithmetic they were 300 of the tile's 309 operations per cell on a pipe
 // that completes two per clock and SM, which bound every FP64 launch: the
 // pipe was 86 % busy. Measured: a slow step of 2048 x 1024 cells with m = 8
-// 11.74 -> 2.36 ms (B and F rows of one stage 649 -> 129 to 141 us), 64 x 64
-// with m = 4 165 -> 86 us. Errors of the right-hand side against 80-bit
+// 11.7 -> 2.11 ms (B and F rows of one stage 649 -> 118 to 129 us), 64 x 64
+// with m = 4 167 -> 76 us; now 2320 instructions per cell and warp, 57 % of
+// the integer pipe and 60 % of the issue slots busy. Errors of the right-hand side against 80-bit
 // arithmetic fell from 3e-16..1e-15 to 2e-17..5e-16 (rms per component; rest
 // state with 1 % bumps to 25 % cell noise). A face
 // with a state outside the fixed-point range takes the same formulas in
@@ -40,12 +42,9 @@ namespace mprk {
 
 template <int TZR = TZ>
 struct TileSmem {
-  static constexpr int NZF = (TZR + 1) * TX, NXF = TZR * (TX + 1);  // z and x faces
   double q[4][TZR + 4][TX + 4];  // stage state, rows k0-2.., cols i0-2..
   i64 qi[4][TZR + 4][TX + 4];    // the same: rho, rho E .58, momenta .60
   i64 v[3][TZR + 2][TX + 2];     // u, w, e (.59), rows k0-1.., cols i0-1..
-  i64 tz[2][TZR][TX + 2];        // central z differences of u, w (tangential at x faces)
-  i64 tx[2][TZR + 2][TX];        // central x differences of u, w (tangential at z faces)
   // face fluxes over half the divergence factor (.57; a slow face's as the
   // bits of a double)
   i64 fx[4][TZR][TX + 1];  // face f between cols f-1, f
@@ -55,7 +54,7 @@ struct TileSmem {
   i64 gam_fx[3][TX + 2];   // 2 u_w .59, 2 sigma_xz .57, 2 (u_w sigma_xz - Pi_z) .57
   double fc[2][2][FXC_N];  // viscous coefficients of the double pass
   unsigned char gam_ok[TX + 2];
-  unsigned char slow[NZF + NXF + TX];  // per face: z, x, interface from below
+  unsigned char slow[(2 * TZR + 3) * TX];  // per face: its job and lane (face_id)
 };
 
 // Lax–Friedrichs flux in the face frame, in double (faces outside the
@@ -200,97 +199,63 @@ struct Arith<double> {
   }
 };
 
-// ---- phase 2: u, w, e on the one-cell ring ---------------------------------
-template <typename T, int NT, int TZR>
-__device__ __forceinline__ void ring_phase(const Geom& g, TileSmem<TZR>& S, int k0, int i0) {
-  T* v = reinterpret_cast<T*>(&S.v[0][0][0]);
-  const T* q = Arith<T>::q(S);
-  constexpr int QP = (TZR + 4) * (TX + 4), VP = (TZR + 2) * (TX + 2);
-  for (int e = threadIdx.x; e < VP; e += NT) {
-    const int rr = e / (TX + 2), cc = e - rr * (TX + 2);
-    const int k = k0 - 1 + rr;
-    if (k < 0 || k >= g.nz) continue;
-    const T* p = q + (rr + 1) * (TX + 4) + cc + 1;
-    T o[3];
-    Arith<T>::prims(p[0], p[QP], p[2 * QP], p[3 * QP], o);
-    v[e] = o[0];
-    // the mirror state's u is already flipped; a no-slip x wall flips w too
-    v[VP + e] = (x_ghost(i0 - 1 + cc, g.nx, g.xwall) && g.wall == 0) ? -o[1] : o[1];
-    v[2 * VP + e] = o[2];
-  }
+// u, w, e of the cell of halo row rr, column cc into the ring (phase 1).
+template <typename T, int TZR>
+__device__ __forceinline__ void ring_cell(const Geom& g, TileSmem<TZR>& S, int rr, int cc, int i0, T r, T mu, T mw, T E) {
+  constexpr int VP = (TZR + 2) * (TX + 2);
+  if (rr < 1 || rr > TZR + 2 || cc < 1 || cc > TX + 2) return;
+  T* v = reinterpret_cast<T*>(&S.v[0][0][0]) + (rr - 1) * (TX + 2) + cc - 1;
+  T o[3];
+  Arith<T>::prims(r, mu, mw, E, o);
+  v[0] = o[0];
+  // the mirror state's u is already flipped; a no-slip x wall flips w too
+  v[VP] = (x_ghost(i0 - 2 + cc, g.nx, g.xwall) && g.wall == 0) ? -o[1] : o[1];
+  v[2 * VP] = o[2];
 }
 
-// ---- phase 3: central differences of u, w along the faces ------------------
+// 2 u_w of the interface state in T.
 template <typename T>
-__device__ __forceinline__ T lid_u2(double uw, i64 uw_fx);  // 2 u_w
+__device__ __forceinline__ T lid_u2(double uw, i64 uw_fx);
 template <>
 __device__ __forceinline__ i64 lid_u2<i64>(double, i64 uw_fx) { return uw_fx; }
 template <>
 __device__ __forceinline__ double lid_u2<double>(double uw, i64) { return __dmul_rn(2.0, uw); }
 
-template <typename T, int NT, int TZR>
-__device__ __forceinline__ void diff_phase(const Geom& g, TileSmem<TZR>& S, int k0, int row_hi) {
-  const T* v = reinterpret_cast<const T*>(&S.v[0][0][0]);
-  T* tz = reinterpret_cast<T*>(&S.tz[0][0][0]);
-  T* tx = reinterpret_cast<T*>(&S.tx[0][0][0]);
-  constexpr int VP = (TZR + 2) * (TX + 2), ZP = TZR * (TX + 2), XP = (TZR + 2) * TX;
-  for (int e = threadIdx.x; e < ZP + XP; e += NT) {
-    if (e < ZP) {
-      const int rr = e / (TX + 2), cc = e - rr * (TX + 2), k = k0 + rr;
-      if (k >= row_hi) continue;
-      const T* p = v + (rr + 1) * (TX + 2) + cc;
-      const T u = p[0], w = p[VP];
-      T uu, wu, ud, wd;  // values above and below, or their ghosts
-      if (k + 1 == g.nz) { uu = g.wall ? u : -u; wu = -w; }
-      else if (k + 1 == g.n1) { uu = lid_u2<T>(S.gam[2][cc], S.gam_fx[0][cc]) - u; wu = -w; }
-      else { uu = p[TX + 2]; wu = p[VP + TX + 2]; }
-      if (k == 0) { ud = g.wall ? u : -u; wd = -w; }
-      else if (k == g.n1) { ud = lid_u2<T>(S.gam[2][cc], S.gam_fx[0][cc]) - u; wd = -w; }
-      else { ud = p[-(TX + 2)]; wd = p[VP - (TX + 2)]; }
-      tz[e] = uu - ud;
-      tz[ZP + e] = wu - wd;
-    } else {
-      const int x = e - ZP, rr = x / TX, cc = x - rr * TX, k = k0 - 1 + rr;
-      if (k < 0 || k >= g.nz) continue;
-      const T* p = v + rr * (TX + 2) + cc;
-      tx[x] = p[2] - p[0];
-      tx[XP + x] = p[VP + 2] - p[VP];
-    }
-  }
-}
-
-// ---- phase 4: face fluxes ---------------------------------------------------
-// Face e of the tile: z faces by rows, then x faces by rows, then the
-// interface seen from below. False if no cell of the tile needs it.
+// ---- phase 3: face fluxes ---------------------------------------------------
+// The faces of the tile as jobs of one warp each: TZR rows of z faces, TZR
+// rows of x faces (columns 0 to TX - 1), the z faces above the last row, the
+// x faces right of the last column (one lane per row), and in a tile at the
+// interface its faces seen from below. With TZR + 1 warps these are two jobs
+// per warp, with twice that one: no round leaves warps waiting for a few last
+// faces.
 struct FaceId {
   int isx, f, c;  // z: face row f, column c; x: tile row f, face column c
   int ku;         // row above a z face, or the row of an x face
   int below;      // the interface from fluid 1
 };
+// Face of a job and lane; false if no cell of the tile needs it.
 template <int TZR>
-__device__ __forceinline__ bool face_id(const Geom& g, int e, int k0, int row_hi, FaceId* id) {
-  constexpr int NZF = TileSmem<TZR>::NZF, NXF = TileSmem<TZR>::NXF;
+__device__ __forceinline__ bool face_id(const Geom& g, int job, int lane, int k0, int row_hi, FaceId* id) {
   id->below = 0;
-  if (e < NZF) {
+  id->c = lane;
+  if (job < TZR || job == 2 * TZR) {
     id->isx = 0;
-    id->f = e / TX;
-    id->c = e - id->f * TX;
+    id->f = job < TZR ? job : TZR;
     id->ku = k0 + id->f;
     // needed by the cell below (f >= 1) or above (f < TZR); at the interface
     // this is the side of fluid 2
     return id->ku - 1 < row_hi && !(id->f == TZR && id->ku == g.n1);
   }
-  if (e < NZF + NXF) {
-    const int x = e - NZF;
+  if (job <= 2 * TZR + 1) {
+    const bool edge = job > 2 * TZR;
     id->isx = 1;
-    id->f = x / (TX + 1);
-    id->c = x - id->f * (TX + 1);
+    id->f = edge ? lane : job - TZR;
+    id->c = edge ? TX : lane;
     id->ku = k0 + id->f;
-    return id->ku < row_hi;
+    return id->ku < row_hi && id->f < TZR;
   }
   id->isx = 0;
   id->f = g.n1 - k0;
-  id->c = e - NZF - NXF;
   id->ku = g.n1;
   id->below = 1;
   return id->f >= 1 && id->f <= TZR && g.n1 - 1 < row_hi;
@@ -305,7 +270,7 @@ __device__ __forceinline__ bool face_id(const Geom& g, int e, int k0, int row_hi
 template <typename T, int TZR>
 __device__ __forceinline__ int face_sides(const Geom& g, const TileSmem<TZR>& S, const FaceId& id, T L[4], T R[4],
                                           T vL[5], T vR[5]) {
-  constexpr int QP = (TZR + 4) * (TX + 4), VP = (TZR + 2) * (TX + 2), ZP = TZR * (TX + 2), XP = (TZR + 2) * TX;
+  constexpr int QP = (TZR + 4) * (TX + 4), VP = (TZR + 2) * (TX + 2);
   const int n1 = g.n1, nz = g.nz, ku = id.ku, kd = ku - 1;
   // first of the four cells, their stride, and the planes of m_n, m_t
   const int qs = id.isx ? 1 : TX + 4;
@@ -315,39 +280,80 @@ __device__ __forceinline__ int face_sides(const Geom& g, const TileSmem<TZR>& S,
   const bool from_above = ku == 0 || (lid && !id.below);  // of a boundary face: the inner cell is the upper one
   const bool mir0 = !id.isx && (kd == 0 || kd == n1), mir3 = !id.isx && (ku == nz - 1 || ku == n1 - 1);
   const T* q = Arith<T>::q(S) + q0;
-  auto comp = [&](int plane, bool odd, T& l, T& r) {
-    const T* p = q + plane;
-    T a0 = p[0], a1 = p[qs], a2 = p[2 * qs], a3 = p[3 * qs];
-    if (!id.isx) {  // mirror ghosts beyond a wall or the interface: rho w odd
+  const int planes[4] = {0, pn, pt, 3 * QP};
+  if (wall || lid || mir0 || mir3) {
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const bool odd = c == 1;  // mirror ghosts beyond a wall or the interface: rho w odd
+      const T* p = q + planes[c];
+      T a0 = p[0], a1 = p[qs], a2 = p[2 * qs], a3 = p[3 * qs];
       if (wall || lid) {
         if (from_above) a1 = odd ? -a2 : a2;
         else a2 = odd ? -a1 : a1;
       }
       if (mir0) a0 = odd ? -a1 : a1;
       if (mir3) a3 = odd ? -a2 : a2;
+      L[c] = Arith<T>::rec(a1, a2, a0);
+      R[c] = Arith<T>::rec(a2, a1, a3);
+      if (wall || lid) {
+        if (from_above) L[c] = odd ? -R[c] : R[c];
+        else R[c] = odd ? -L[c] : L[c];
+      }
     }
-    l = Arith<T>::rec(a1, a2, a0);
-    r = Arith<T>::rec(a2, a1, a3);
-    if (wall || lid) {
-      if (from_above) l = odd ? -r : r;
-      else r = odd ? -l : l;
+  } else {
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const T* p = q + planes[c];
+      const T a0 = p[0], a1 = p[qs], a2 = p[2 * qs], a3 = p[3 * qs];
+      L[c] = Arith<T>::rec(a1, a2, a0);
+      R[c] = Arith<T>::rec(a2, a1, a3);
     }
-  };
-  comp(0, false, L[0], R[0]);
-  comp(pn, true, L[1], R[1]);
-  comp(pt, false, L[2], R[2]);
-  comp(3 * QP, false, L[3], R[3]);
+  }
   if (lid) return id.below ? 2 : 3;
-  // velocities, e and tangential differences of the cells at the face
+  // velocities, e and tangential central differences of the cells at the face
   const T* v = reinterpret_cast<const T*>(&S.v[0][0][0]);
-  const int vo = id.isx ? (id.f + 1) * (TX + 2) + id.c : id.f * (TX + 2) + id.c + 1, vs = id.isx ? 1 : TX + 2;
-  const int vn = id.isx ? 0 : VP, vt = VP - vn;
-  const T* t = id.isx ? reinterpret_cast<const T*>(&S.tz[0][0][0]) + id.f * (TX + 2) + id.c
-                      : reinterpret_cast<const T*>(&S.tx[0][0][0]) + id.f * TX + id.c;
-  const int ts = id.isx ? 1 : TX, tn = id.isx ? 0 : XP, tt = id.isx ? ZP : 0;
-  vL[0] = v[vo + vn], vL[1] = v[vo + vt], vL[2] = v[vo + 2 * VP], vL[3] = t[tn], vL[4] = t[tt];
-  vR[0] = v[vo + vs + vn], vR[1] = v[vo + vs + vt], vR[2] = v[vo + vs + 2 * VP], vR[3] = t[ts + tn],
-  vR[4] = t[ts + tt];
+  if (id.isx) {
+    const T* p = v + (id.f + 1) * (TX + 2) + id.c;
+    const bool top = ku + 1 == nz || ku + 1 == n1, bot = ku == 0 || ku == n1;
+#pragma unroll
+    for (int s = 0; s < 2; s++, p++) {
+      T* o = s ? vR : vL;
+      const T u = p[0], w = p[VP];
+      o[0] = u;
+      o[1] = w;
+      o[2] = p[2 * VP];
+      // z differences of u, w, with the ghost 2 (wall state) - cell beyond a
+      // wall or the interface
+      T uu, wu, ud, wd;
+      if (top) {
+        uu = ku + 1 == nz ? (g.wall ? u : -u) : lid_u2<T>(S.gam[2][id.c + s], S.gam_fx[0][id.c + s]) - u;
+        wu = -w;
+      } else {
+        uu = p[TX + 2];
+        wu = p[VP + TX + 2];
+      }
+      if (bot) {
+        ud = ku == 0 ? (g.wall ? u : -u) : lid_u2<T>(S.gam[2][id.c + s], S.gam_fx[0][id.c + s]) - u;
+        wd = -w;
+      } else {
+        ud = p[-(TX + 2)];
+        wd = p[VP - (TX + 2)];
+      }
+      o[3] = uu - ud;
+      o[4] = wu - wd;
+    }
+    return ku >= n1;
+  }
+  const T* p = v + id.f * (TX + 2) + id.c + 1;
+#pragma unroll
+  for (int s = 0; s < 2; s++, p += TX + 2) {
+    T* o = s ? vR : vL;
+    o[0] = p[VP];
+    o[1] = p[0];
+    o[2] = p[2 * VP];
+    o[3] = p[VP + 1] - p[VP - 1];
+    o[4] = p[1] - p[-1];
+  }
   if (wall) {
     const T* c = from_above ? vR : vL;
     T* o = from_above ? vL : vR;
@@ -357,7 +363,7 @@ __device__ __forceinline__ int face_sides(const Geom& g, const TileSmem<TZR>& S,
     o[3] = -c[3];
     o[4] = g.wall ? c[4] : -c[4];
   }
-  return (id.isx ? ku : (ku == 0 ? 0 : kd)) >= n1;
+  return (ku == 0 ? 0 : kd) >= n1;
 }
 
 // The viscous flux over half the divergence factor from the common values of
@@ -424,24 +430,26 @@ __device__ __noinline__ bool face_in_range(const Geom& g, const TileSmem<TZR>& S
   return ok;
 }
 
-// The faces marked slow (all: every face), in double: phases 2 and 3 again as
+// The faces marked slow (all: every face), in double: the ring again as
 // doubles (in the same storage), then their fluxes. Ends with the tile's
-// barrier. A grid wholly outside the range runs about as fast as the tile
-// that did everything in double (2048 x 1024, m = 8: 12.0 ms per step
-// against 11.7).
+// barrier. A grid wholly outside the range runs as fast as the tile that did
+// everything in double (2048 x 1024, m = 8: 11.5 ms per step against 11.7).
 template <int NT, int TZR>
 __device__ __noinline__ void slow_faces(const Geom& g, TileSmem<TZR>& S, int k0, int i0, int row_hi, bool all) {
-  ring_phase<double, NT, TZR>(g, S, k0, i0);
+  for (int e = threadIdx.x; e < (TZR + 2) * (TX + 2); e += NT) {
+    const int rr = e / (TX + 2) + 1, cc = e % (TX + 2) + 1, k = k0 - 2 + rr;
+    if (k >= 0 && k < g.nz)
+      ring_cell<double, TZR>(g, S, rr, cc, i0, S.q[0][rr][cc], S.q[1][rr][cc], S.q[2][rr][cc], S.q[3][rr][cc]);
+  }
   if (threadIdx.x < 4 * FXC_N) {
     const int j = threadIdx.x % FXC_N, f = threadIdx.x / FXC_N;
     S.fc[f >> 1][f & 1][j] = visc_coef(g, f >> 1, f & 1, j);
   }
   __syncthreads();
-  diff_phase<double, NT, TZR>(g, S, k0, row_hi);
-  __syncthreads();
-  for (int e = threadIdx.x; e < TileSmem<TZR>::NZF + TileSmem<TZR>::NXF + TX; e += NT) {
+  for (int job = threadIdx.x / 32; job < 2 * TZR + 3; job += NT / 32) {
+    const int lane = threadIdx.x % 32, e = job * TX + lane;
     FaceId id;
-    if (!face_id<TZR>(g, e, k0, row_hi, &id) || !(all || S.slow[e])) continue;
+    if (!face_id<TZR>(g, job, lane, k0, row_hi, &id) || !(all || S.slow[e])) continue;
     if (all) S.slow[e] = 1;
     double L[4], R[4], vL[5], vR[5], V[3], F[4];
     const int fl = face_sides<double, TZR>(g, S, id, L, R, vL, vR);
@@ -471,12 +479,12 @@ __device__ __noinline__ void slow_faces(const Geom& g, TileSmem<TZR>& S, int k0,
 // GEN selects the general s-stage base method (Sec. 3 remark) in place of
 // Heun's low-storage path: s R_a slots, the stage values of the region
 // tableaus built from the base, and its weights b in the combinations.
-// NT: threads of the CTA. TX x TZR gives one thread per cell; launches with
-// fewer tiles than the GPU has SMs take twice that, so that each SM holds
-// more warps of the few tiles there are: every phase but the last spreads
-// its work over all threads, and the last (one cell per thread) uses the
-// first TX x TZR. TZR: tile rows.
-template <bool GEN = false, int NT = NTHREADS, int TZR = TZ>
+// NT: threads of the CTA. TZR + 1 warps make two rounds of face jobs;
+// launches with fewer tiles than the GPU has SMs take twice that, one round,
+// so that each SM holds more warps of the few tiles there are. Every phase
+// but the last spreads its work over all threads, and the last (one cell per
+// thread) uses the first TX x TZR. TZR: tile rows.
+template <bool GEN = false, int NT = FP64_THREADS, int TZR = TZ>
 __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSmem<TZR>& S) {
   const Geom& g = a.g;
   const int tid = threadIdx.x;
@@ -502,43 +510,48 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
     return odd_stage ? __fma_rn(h, Ra[off], base[off]) : base[off];
   };
 
-  // ---- 1. stage state of the tile and its halo --------------------------
+  // ---- 1. stage state of the tile and its halo; u, w, e on the ring ------
   bool bad = !a.fx.on, good = false;  // some cell outside, inside the fixed-point range
   for (int e = tid; e < (TZR + 4) * (TX + 4); e += NT) {
     const int rr = e / (TX + 4), cc = e - rr * (TX + 4);
     const int k = k0 - 2 + rr;
-    double val[4] = {0.0, 0.0, 0.0, 0.0};
-    if (k >= 0 && k < nz) {
-      bool gh;
-      const int i = halo_col(i0 - 2 + cc, nx, g.xwall, &gh);
+    if (k < 0 || k >= nz) {
+      // read by faces next to a wall, which replace it by the mirror cell
 #pragma unroll
-      for (int c = 0; c < 4; c++) val[c] = stage_value(c, k, i);
-      if (gh) val[1] = -val[1];  // mirror state beyond an x wall
-      const bool in = cell_in_range(val[0], val[1], val[2], val[3]);
-      bad |= !in;
-      good |= in;
+      for (int c = 0; c < 4; c++) {
+        S.q[c][rr][cc] = 0.0;
+        S.qi[c][rr][cc] = 0;
+      }
+      continue;
     }
+    bool gh;
+    const int i = halo_col(i0 - 2 + cc, nx, g.xwall, &gh);
+    double val[4];
+#pragma unroll
+    for (int c = 0; c < 4; c++) val[c] = stage_value(c, k, i);
+    if (gh) val[1] = -val[1];  // mirror state beyond an x wall
+    const bool in = cell_in_range(val[0], val[1], val[2], val[3]);
+    bad |= !in;
+    good |= in;
+    i64 t[4];
 #pragma unroll
     for (int c = 0; c < 4; c++) {
       S.q[c][rr][cc] = val[c];
-      S.qi[c][rr][cc] =
-          fx::from_double(__double_as_longlong(val[c]), c == 1 || c == 2 ? fx::S_MOM - 2 : fx::S_RHO - 2);
+      t[c] = c == 1 || c == 2 ? fx::from_double(__double_as_longlong(val[c]), fx::S_MOM - 2)
+                              : fx::from_positive(__double_as_longlong(val[c]), fx::S_RHO - 2);
+      S.qi[c][rr][cc] = t[c];
     }
+    ring_cell<i64, TZR>(g, S, rr, cc, i0, t[0], t[1], t[2], t[3]);
   }
   const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZR);
-  bad = __syncthreads_or(bad);
-  bool none = false;  // no cell inside: every face in double
-  if (bad) none = !a.fx.on || !__syncthreads_or(good);
-
-  // ---- 2. u, w, e on the one-cell ring; interface state ------------------
-  if (!none) ring_phase<i64, NT, TZR>(g, S, k0, i0);
+  // ---- 2. interface state -------------------------------------------------
+  // of column i0-1+j in double precision from the two cells touching Gamma
+  // (App. B, Eq. bulk-flux and the wall states), by the last threads, which
+  // staged fewer cells
   if (has_gamma) {
-    bool lid_bad = false;
-    if (tid < TX + 2) {
-      // Interface state of column i0-1+tid in double precision from the two
-      // cells touching Gamma (App. B, Eq. bulk-flux and the wall states).
+    for (int j = NT - 1 - tid; j < TX + 2; j += NT) {
       bool gh;
-      const int i = halo_col(i0 - 1 + tid, nx, g.xwall, &gh);
+      const int i = halo_col(i0 - 1 + j, nx, g.xwall, &gh);
       double u[2], T[2];
 #pragma unroll
       for (int s = 0; s < 2; s++) {
@@ -556,34 +569,29 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
       const double sig = __dmul_rn(g.bu, __dsub_rn(u[1], u[0]));
       const double Pi = __dmul_rn(-g.bT, __dsub_rn(T[1], T[0]));
       const double uw = __fma_rn(sig, g.cu1, u[0]), En = __fma_rn(uw, sig, -Pi);
-      S.gam[0][tid] = sig;
-      S.gam[1][tid] = Pi;
-      S.gam[2][tid] = uw;
+      S.gam[0][j] = sig;
+      S.gam[1][j] = Pi;
+      S.gam[2][j] = uw;
       const bool ok = fabs(uw) < 1.9 && fabs(sig) < 2.0 && fabs(En) < 2.0;  // false for NaN
-      S.gam_ok[tid] = ok;
-      lid_bad = !ok;
-      S.gam_fx[0][tid] = __double2ll_rn(ok ? uw * (double)(2ll << fx::S_VEL) : 0.0);
-      S.gam_fx[1][tid] = __double2ll_rn(ok ? sig * (double)(2ll << fx::S_FLUX) : 0.0);
-      S.gam_fx[2][tid] = __double2ll_rn(ok ? En * (double)(2ll << fx::S_FLUX) : 0.0);
+      S.gam_ok[j] = ok;
+      bad |= !ok;
+      S.gam_fx[0][j] = __double2ll_rn(ok ? __dmul_rn(uw, (double)(2ll << fx::S_VEL)) : 0.0);
+      S.gam_fx[1][j] = __double2ll_rn(ok ? __dmul_rn(sig, (double)(2ll << fx::S_FLUX)) : 0.0);
+      S.gam_fx[2][j] = __double2ll_rn(ok ? __dmul_rn(En, (double)(2ll << fx::S_FLUX)) : 0.0);
     }
-    bad |= __syncthreads_or(lid_bad) != 0;
-  } else {
-    __syncthreads();
   }
+  bad = __syncthreads_or(bad);
+  bool none = false;  // no cell inside: every face in double
+  if (bad) none = !a.fx.on || !__syncthreads_or(good);
 
-  // ---- 3. tangential differences ------------------------------------------
-  if (!none) {
-    diff_phase<i64, NT, TZR>(g, S, k0, row_hi);
-    __syncthreads();
-  }
-
-  // ---- 4. face fluxes ----------------------------------------------------
-  constexpr int NZF = TileSmem<TZR>::NZF, NXF = TileSmem<TZR>::NXF;
+  // ---- 3. face fluxes ----------------------------------------------------
+  static_assert(TX == 32 && NT % 32 == 0, "a job is one warp wide");
   bool slow = false;
-  const int n_faces = NZF + NXF + (has_gamma ? TX : 0);
-  for (int e = none ? n_faces : tid; e < n_faces; e += NT) {
+  const int jobs = none ? 0 : 2 * TZR + 2 + has_gamma;
+  const int warp = __shfl_sync(0xffffffffu, tid / 32, 0), lane = tid % 32;
+  for (int job = warp; job < jobs; job += NT / 32) {
     FaceId id;
-    if (!face_id<TZR>(g, e, k0, row_hi, &id)) continue;
+    if (!face_id<TZR>(g, job, lane, k0, row_hi, &id)) continue;
     bool ok = !bad || face_in_range<TZR>(g, S, id, k0);
     if (ok) {
       i64 L[4], R[4], vL[5], vR[5], V[3], F[4];
@@ -598,13 +606,13 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
       ok = fx_flux<2>(g, a.fx, L, R, V, F);
       if (ok) store_flux(S, id, F);
     }
-    S.slow[e] = !ok;
+    S.slow[job * TX + lane] = !ok;
     slow |= !ok;
   }
   slow = none || __syncthreads_or(slow);
   if (slow) slow_faces<NT, TZR>(g, S, k0, i0, row_hi, none);
 
-  // ---- 5. R = -div F* + s and the stage combination ----------------------
+  // ---- 4. R = -div F* + s and the stage combination ----------------------
   {
     const int rr = tid / TX, cc = tid - rr * TX;
     const int k = k0 + rr, i = i0 + cc;
@@ -615,10 +623,10 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
     double R[4];
     bool s0 = false, s1 = false, s2 = false, s3 = false;  // slow faces of the cell: left, right, lower, upper
     if (slow) {
-      s0 = S.slow[NZF + rr * (TX + 1) + cc];
-      s1 = S.slow[NZF + rr * (TX + 1) + cc + 1];
+      s0 = S.slow[(TZR + rr) * TX + cc];
+      s1 = S.slow[cc < TX - 1 ? (TZR + rr) * TX + cc + 1 : (2 * TZR + 1) * TX + rr];
       s2 = S.slow[rr * TX + cc];
-      s3 = S.slow[under_gamma ? NZF + NXF + cc : (rr + 1) * TX + cc];
+      s3 = S.slow[(under_gamma ? 2 * TZR + 2 : rr + 1 < TZR ? rr + 1 : 2 * TZR) * TX + cc];
     }
     if (s0 && s1 && s2 && s3) {
 #pragma unroll
