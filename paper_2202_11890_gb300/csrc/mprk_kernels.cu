@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(MIXED_THREADS, 3)
 // 3-D stage (App. B in full): the y faces of a plane pair, then the x and z
 // faces, the divergence and the combination of a plane; one CTA per TX x TZ
 // tile of an x-z plane, blockIdx = (tile column, tile row, plane).
-// Three CTAs per SM in both (80 registers; 52 and 72 KB of shared memory).
+// Three CTAs per SM in both (80 and 72 registers; 52 and 58 KB of shared memory).
 __global__ void __launch_bounds__(NTHREADS, 3)
     yface3_kernel(const __grid_constant__ StageArgs a, const __grid_constant__ Fx3Const C) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(NTHREADS, 3)
   yface_tile(a, C, a.row0 + blockIdx.y * TZ, blockIdx.x * TX, blockIdx.z, *reinterpret_cast<YfaceSmem*>(smem_raw));
 }
 
-__global__ void __launch_bounds__(NTHREADS, 3)
+__global__ void __launch_bounds__(TILE3_THREADS, 3)
     stage3_kernel(const __grid_constant__ StageArgs a, const __grid_constant__ Fx3Const C) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   chain_wait();
@@ -89,7 +89,7 @@ cudaError_t launch_stage3(const StageArgs& a, cudaStream_t stream, bool chained)
   fixed_point_const3(a.g, &C);
   cudaError_t e = launch_kernel(yface3_kernel, grid, NTHREADS, sizeof(YfaceSmem), stream, chained, a, C);
   if (e != cudaSuccess) return e;
-  return launch_kernel(stage3_kernel, grid, NTHREADS, sizeof(Tile3Smem), stream, true, a, C);
+  return launch_kernel(stage3_kernel, grid, TILE3_THREADS, sizeof(Tile3Smem), stream, true, a, C);
 }
 
 size_t stage_smem_bytes(int precision) {

@@ -18,7 +18,7 @@
 // As in the 2-D tile, velocities, differences and fluxes run in 64-bit fixed
 // point (fixed_point.cuh), because the double pipe bound both kernels (80 to
 // 86 % busy with 125 + 238 operations per cell). Measured: a slow step of
-// 512 x 64 x 200 cells with m = 4 44.1 -> 9.7 ms. A face whose own cells leave
+// 512 x 64 x 200 cells with m = 4 44.1 -> 9.3 ms. A face whose own cells leave
 // the range is evaluated in double by a second pass over the tile; which form
 // a face takes depends on its cells alone, so neighbouring tiles agree on the
 // faces they share. Fluxes come over half the divergence factor of their
@@ -28,6 +28,7 @@
 #include "fixed_flux.cuh"
 #include "fp64_recip.cuh"
 #include "mprk_internal.h"
+#include "stage_tile.cuh"
 
 namespace mprk {
 
@@ -438,13 +439,11 @@ __device__ __forceinline__ void yface_tile(const StageArgs& a, const Fx3Const& C
 
 // ---- x and z faces, divergence and stage combination ----------------------
 
+constexpr int TILE3_THREADS = FP64_THREADS;  // nine warps, two face jobs each (face_id in stage_tile.cuh)
 struct Tile3Smem {
-  static constexpr int NZF = (TZ + 1) * TX, NXF = TZ * (TX + 1);
   i64 q[5][TZ + 4][TX + 4];   // plane j, rows k0-2.., cols i0-2..
   i64 v[4][TZ + 2][TX + 2];   // u, v, w, e on the ring
   i64 vy[3][TZ + 2][TX + 2];  // central y differences of u, v, w on the ring
-  i64 tz[2][TZ][TX + 2];      // central z differences of u, w at x-face cells
-  i64 tx[2][TZ + 2][TX];      // central x differences of u, w at z-face cells
   i64 fx[5][TZ][TX + 1];      // x face fluxes, face f between cols f-1, f
   i64 fz[5][TZ + 1][TX];      // z face fluxes seen from above
   i64 fg[5][TX];              // interface flux seen from fluid 1
@@ -452,29 +451,26 @@ struct Tile3Smem {
   unsigned char ok[TZ + 4][TX + 4];
   unsigned char oky[TZ + 2][TX + 2];  // the cells in planes j-1 and j+1
   unsigned char lid_ok[TX + 2];
-  unsigned char slow[NZF + NXF + TX];  // per face: z, x, interface from below
+  unsigned char slow[(2 * TZ + 3) * TX];  // per face: its job and lane
 };
 
-// Phases 1 to 3 in T: stage state, velocities, y differences, interface
-// state, then the tangential differences. Returns (T = i64) 0, or 1 where
+// Phases 1 and 2 in T: stage state, velocities and their y differences, and
+// the interface state. Returns (T = i64) 0, or 1 where
 // some cell or interface state leaves the fixed-point range, or 2 where every
 // cell does. Ends with a barrier.
 template <typename T>
-__device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, int k0, int i0, int j, int row_hi,
-                                            Tile3Smem& S) {
+__device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, int k0, int i0, int j, Tile3Smem& S) {
   constexpr bool FX = (T)0.5 == (T)0;
   const Geom& g = a.g;
   const int tid = threadIdx.x, nz = g.nz, n1 = g.n1;
   const int jm = wrap3(j - 1, g.ny), jp = wrap3(j + 1, g.ny);
-  constexpr int QP = (TZ + 4) * (TX + 4), ZP = TZ * (TX + 2), XP = (TZ + 2) * TX;
+  constexpr int QP = (TZ + 4) * (TX + 4);
   T* q = reinterpret_cast<T*>(&S.q[0][0][0]);
   T* v = reinterpret_cast<T*>(&S.v[0][0][0]);
   T* vy = reinterpret_cast<T*>(&S.vy[0][0][0]);
-  T* tz = reinterpret_cast<T*>(&S.tz[0][0][0]);
-  T* tx = reinterpret_cast<T*>(&S.tx[0][0][0]);
   T* lid = reinterpret_cast<T*>(&S.lid[0][0]);
   bool bad = false, good = false;
-  for (int e = tid; e < QP; e += NTHREADS) {
+  for (int e = tid; e < QP; e += TILE3_THREADS) {
     const int rr = e / (TX + 4), cc = e - rr * (TX + 4);
     const int k = k0 - 2 + rr;
     if (k < 0 || k >= nz) {
@@ -506,7 +502,7 @@ __device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, in
       for (int c = 0; c < 4; c++) v[c * RING3 + (rr - 1) * (TX + 2) + cc - 1] = o[c];
     }
   }
-  for (int e = tid; e < RING3; e += NTHREADS) {
+  for (int e = tid; e < RING3; e += TILE3_THREADS) {
     const int rr = e / (TX + 2), cc = e - rr * (TX + 2);
     const int k = k0 - 1 + rr;
     if (k < 0 || k >= nz) continue;
@@ -532,68 +528,24 @@ __device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, in
     for (int c = 0; c < 3; c++) vy[c * RING3 + e] = up[c] - dn[c];
   }
   const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZ);
-  if (has_gamma && tid < TX + 2) {
-    double st[L3_N];
-    interface3(a, G, j, wrap3(i0 - 1 + tid, g.nx), st);
-    const bool ok = store_lid<T>(st, lid + tid, TX + 2);
-    if (FX) S.lid_ok[tid] = ok;
-    bad |= !ok;
-  }
-  if (FX) {
-    bad = __syncthreads_or(bad);
-    if (bad && !__syncthreads_or(good)) return 2;
-  } else {
-    __syncthreads();
-  }
-  for (int e = tid; e < ZP + XP; e += NTHREADS) {
-    if (e < ZP) {
-      const int rr = e / (TX + 2), cc = e - rr * (TX + 2), k = k0 + rr;
-      if (k >= row_hi) continue;
-      const T* p = v + (rr + 1) * (TX + 2) + cc;
-      tz[e] = dz_vel(g, k, 0, p, TX + 2, lid + cc, TX + 2);
-      tz[ZP + e] = dz_vel(g, k, 2, p + 2 * RING3, TX + 2, lid + cc, TX + 2);
-    } else {
-      const int x = e - ZP, rr = x / TX, cc = x - rr * TX, k = k0 - 1 + rr;
-      if (k < 0 || k >= nz) continue;
-      const T* p = v + rr * (TX + 2) + cc;
-      tx[x] = p[2] - p[0];
-      tx[XP + x] = p[2 * RING3 + 2] - p[2 * RING3];
+  if (has_gamma) {
+    // by the last threads, which staged fewer cells
+    const int e = TILE3_THREADS - 1 - tid;
+    if (e < TX + 2) {
+      double st[L3_N];
+      interface3(a, G, j, wrap3(i0 - 1 + e, g.nx), st);
+      const bool ok = store_lid<T>(st, lid + e, TX + 2);
+      if (FX) S.lid_ok[e] = ok;
+      bad |= !ok;
     }
   }
-  __syncthreads();
+  if (!FX) {
+    __syncthreads();
+    return 0;
+  }
+  bad = __syncthreads_or(bad);
+  if (bad && !__syncthreads_or(good)) return 2;
   return bad;
-}
-
-// Face e of the tile, numbered and placed as in the 2-D tile.
-struct Face3 {
-  int isx, f, c;  // z: face row f, column c; x: tile row f, face column c
-  int ku;         // row above a z face, or the row of an x face
-  int below;      // the interface from fluid 1
-};
-__device__ __forceinline__ bool face3_id(const Geom& g, int e, int k0, int row_hi, Face3* id) {
-  constexpr int NZF = Tile3Smem::NZF, NXF = Tile3Smem::NXF;
-  id->below = 0;
-  if (e < NZF) {
-    id->isx = 0;
-    id->f = e / TX;
-    id->c = e - id->f * TX;
-    id->ku = k0 + id->f;
-    return id->ku - 1 < row_hi && !(id->f == TZ && id->ku == g.n1);
-  }
-  if (e < NZF + NXF) {
-    const int x = e - NZF;
-    id->isx = 1;
-    id->f = x / (TX + 1);
-    id->c = x - id->f * (TX + 1);
-    id->ku = k0 + id->f;
-    return id->ku < row_hi;
-  }
-  id->isx = 0;
-  id->f = g.n1 - k0;
-  id->c = e - NZF - NXF;
-  id->ku = g.n1;
-  id->below = 1;
-  return id->f >= 1 && id->f <= TZ && g.n1 - 1 < row_hi;
 }
 
 // The flux of face id in T, stored; false where it leaves the range. A
@@ -601,8 +553,8 @@ __device__ __forceinline__ bool face3_id(const Geom& g, int e, int k0, int row_h
 // state on one side and its mirror on the other; an outer wall's viscous
 // ghost is 2 wall state - cell.
 template <typename T>
-__device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Smem& S, const Face3& id) {
-  constexpr int QP = (TZ + 4) * (TX + 4), ZP = TZ * (TX + 2), XP = (TZ + 2) * TX;
+__device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Smem& S, const FaceId& id) {
+  constexpr int QP = (TZ + 4) * (TX + 4);
   const int n1 = g.n1, nz = g.nz, ku = id.ku, kd = ku - 1;
   const int qs = id.isx ? 1 : TX + 4;
   const int q0 = id.isx ? (id.f + 2) * (TX + 4) + id.c : id.f * (TX + 4) + id.c + 2;
@@ -613,24 +565,6 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
   const bool mir0 = !id.isx && (kd == 0 || kd == n1), mir3 = !id.isx && (ku == nz - 1 || ku == n1 - 1);
   const T* q = reinterpret_cast<const T*>(&S.q[0][0][0]) + q0;
   T L[5], R[5], V[4];
-  auto comp = [&](int plane, bool odd, T& l, T& r) {
-    const T* p = q + plane * QP;
-    T a0 = p[0], a1 = p[qs], a2 = p[2 * qs], a3 = p[3 * qs];
-    if (!id.isx) {
-      if (wall || lidf) {
-        if (from_above) a1 = odd ? -a2 : a2;
-        else a2 = odd ? -a1 : a1;
-      }
-      if (mir0) a0 = odd ? -a1 : a1;
-      if (mir3) a3 = odd ? -a2 : a2;
-    }
-    l = Arith3<T>::rec(a1, a2, a0);
-    r = Arith3<T>::rec(a2, a1, a3);
-    if (wall || lidf) {
-      if (from_above) l = odd ? -r : r;
-      else r = odd ? -l : l;
-    }
-  };
   if (lidf) {
     const T* lid = reinterpret_cast<const T*>(&S.lid[0][0]) + id.c + 1;
     V[0] = 0;
@@ -641,15 +575,12 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
     const T* v = reinterpret_cast<const T*>(&S.v[0][0][0]);
     const T* vy = reinterpret_cast<const T*>(&S.vy[0][0][0]);
     const int vo = id.isx ? (id.f + 1) * (TX + 2) + id.c : id.f * (TX + 2) + id.c + 1, vs = id.isx ? 1 : TX + 2;
-    const T* t = id.isx ? reinterpret_cast<const T*>(&S.tz[0][0][0]) + id.f * (TX + 2) + id.c
-                        : reinterpret_cast<const T*>(&S.tx[0][0][0]) + id.f * TX + id.c;
-    const int ts = id.isx ? 1 : TX;
+    const T* lid = reinterpret_cast<const T*>(&S.lid[0][0]) + id.c;
     VSide<T> s[2];
 #pragma unroll
     for (int side = 0; side < 2; side++) {
       const T* p = v + vo + side * vs;
       const T* y = vy + vo + side * vs;
-      const T* d = t + side * ts;
       s[side].u[0] = p[(pn - 1) * RING3];
       s[side].u[1] = p[(p1 - 1) * RING3];
       s[side].u[2] = p[(p2 - 1) * RING3];
@@ -657,11 +588,11 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
       if (id.isx) {  // t1 = y: du, dv; t2 = z: du, dw
         s[side].g1[0] = y[0];
         s[side].g1[1] = y[RING3];
-        s[side].g2[0] = d[0];
-        s[side].g2[1] = d[ZP];
+        s[side].g2[0] = dz_vel(g, ku, 0, p, TX + 2, lid + side, TX + 2);
+        s[side].g2[1] = dz_vel(g, ku, 2, p + 2 * RING3, TX + 2, lid + side, TX + 2);
       } else {  // t1 = x: dw, du; t2 = y: dw, dv
-        s[side].g1[0] = d[XP];
-        s[side].g1[1] = d[0];
+        s[side].g1[0] = p[2 * RING3 + 1] - p[2 * RING3 - 1];
+        s[side].g1[1] = p[1] - p[-1];
         s[side].g2[0] = y[2 * RING3];
         s[side].g2[1] = y[RING3];
       }
@@ -682,11 +613,35 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
     }
     visc3(C, id.isx ? 0 : 2, (id.isx ? ku : (ku == 0 ? 0 : kd)) >= n1, s[0], s[1], V);
   }
-  comp(0, false, L[0], R[0]);
-  comp(pn, true, L[1], R[1]);
-  comp(p1, false, L[2], R[2]);
-  comp(p2, false, L[3], R[3]);
-  comp(4, false, L[4], R[4]);
+  const int planes[5] = {0, pn * QP, p1 * QP, p2 * QP, 4 * QP};
+  if (wall || lidf || mir0 || mir3) {
+#pragma unroll
+    for (int c = 0; c < 5; c++) {
+      const bool odd = c == 1;  // mirror ghosts beyond a wall or the interface: rho w odd
+      const T* p = q + planes[c];
+      T a0 = p[0], a1 = p[qs], a2 = p[2 * qs], a3 = p[3 * qs];
+      if (wall || lidf) {
+        if (from_above) a1 = odd ? -a2 : a2;
+        else a2 = odd ? -a1 : a1;
+      }
+      if (mir0) a0 = odd ? -a1 : a1;
+      if (mir3) a3 = odd ? -a2 : a2;
+      L[c] = Arith3<T>::rec(a1, a2, a0);
+      R[c] = Arith3<T>::rec(a2, a1, a3);
+      if (wall || lidf) {
+        if (from_above) L[c] = odd ? -R[c] : R[c];
+        else R[c] = odd ? -L[c] : L[c];
+      }
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 5; c++) {
+      const T* p = q + planes[c];
+      const T a0 = p[0], a1 = p[qs], a2 = p[2 * qs], a3 = p[3 * qs];
+      L[c] = Arith3<T>::rec(a1, a2, a0);
+      R[c] = Arith3<T>::rec(a2, a1, a3);
+    }
+  }
   i64 F[5];
   if (!flux3(g, C, L, R, V, F)) return false;
   i64* o;
@@ -709,7 +664,7 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
 // Do the cells that face id reads lie in the range? The four across it, the
 // y neighbours and the third-direction neighbours of the two at it, and the
 // interface states. Asked only in tiles where some cell does not.
-__device__ __noinline__ bool face3_in_range(const Geom& g, const Tile3Smem& S, const Face3 id, int k0) {
+__device__ __noinline__ bool face3_in_range(const Geom& g, const Tile3Smem& S, const FaceId id, int k0) {
   auto cell = [&](int r, int c) {  // halo row and column
     const int k = k0 - 2 + r;
     return k < 0 || k >= g.nz || S.ok[r][c];
@@ -737,10 +692,11 @@ __device__ __noinline__ bool face3_in_range(const Geom& g, const Tile3Smem& S, c
 // restaged as doubles.
 __device__ __noinline__ void slow_faces3(const StageArgs& a, const Fx3Const& C, int k0, int i0, int j, int row_hi,
                                          Tile3Smem& S, bool all) {
-  tile3_cells<double>(a, geo3(a.g), k0, i0, j, row_hi, S);
-  for (int e = threadIdx.x; e < Tile3Smem::NZF + Tile3Smem::NXF + TX; e += NTHREADS) {
-    Face3 id;
-    if (face3_id(a.g, e, k0, row_hi, &id) && (all || S.slow[e])) face3<double>(a.g, C, S, id);
+  tile3_cells<double>(a, geo3(a.g), k0, i0, j, S);
+  for (int job = threadIdx.x / 32; job < 2 * TZ + 3; job += TILE3_THREADS / 32) {
+    const int lane = threadIdx.x % 32;
+    FaceId id;
+    if (face_id<TZ>(a.g, job, lane, k0, row_hi, &id) && (all || S.slow[job * TX + lane])) face3<double>(a.g, C, S, id);
   }
   __syncthreads();
 }
@@ -753,27 +709,28 @@ __device__ __forceinline__ void stage_tile3(const StageArgs& a, const Fx3Const& 
   const int nz = g.nz, nx = g.nx, ny = g.ny, n1 = g.n1;
   const int row_hi = a.rhs_only ? a.rhs_hi : nz;
 
-  // ---- 1-3. stage state, velocities, tangential differences -----------------
-  const int out = C.k.on ? tile3_cells<i64>(a, G, k0, i0, j, row_hi, S) : 2;
+  // ---- 1-2. stage state, velocities, interface state -------------------------
+  const int out = C.k.on ? tile3_cells<i64>(a, G, k0, i0, j, S) : 2;
 
-  // ---- 4. face fluxes -----------------------------------------------------
+  // ---- 3. face fluxes -----------------------------------------------------
   const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZ);
-  const int n_faces = Tile3Smem::NZF + Tile3Smem::NXF + (has_gamma ? TX : 0);
+  const int jobs = out == 2 ? 0 : 2 * TZ + 2 + has_gamma;
+  const int warp = __shfl_sync(0xffffffffu, tid / 32, 0), lane = tid % 32;
   bool slow = false;
-  for (int e = out == 2 ? n_faces : tid; e < n_faces; e += NTHREADS) {
-    Face3 id;
-    if (!face3_id(g, e, k0, row_hi, &id)) continue;
+  for (int job = warp; job < jobs; job += TILE3_THREADS / 32) {
+    FaceId id;
+    if (!face_id<TZ>(g, job, lane, k0, row_hi, &id)) continue;
     const bool ok = (out == 0 || face3_in_range(g, S, id, k0)) && face3<i64>(g, C, S, id);
-    S.slow[e] = !ok;
+    S.slow[job * TX + lane] = !ok;
     slow |= !ok;
   }
   slow = out == 2 || __syncthreads_or(slow);
   if (slow) slow_faces3(a, C, k0, i0, j, row_hi, S, out == 2);
 
-  // ---- 5. R = -div F* + s and the stage combination -------------------------
+  // ---- 4. R = -div F* + s and the stage combination -------------------------
   const int rr = tid / TX, cc = tid - rr * TX;
   const int k = k0 + rr, i = i0 + cc;
-  if (k >= row_hi || i >= nx) return;
+  if (rr >= TZ || k >= row_hi || i >= nx) return;
   const bool under_gamma = (k == n1 - 1);
   const size_t row = (size_t)(k * ny + j) * g.pitch + i;  // offset within a component
   const size_t plane = G.plane;
@@ -794,9 +751,9 @@ __device__ __forceinline__ void stage_tile3(const StageArgs& a, const Fx3Const& 
   bool dbl = any >= 0x10000000;  // some y flux is a double
   if (out == 2) dbl = true;
   else if (slow)
-    dbl = dbl || S.slow[Tile3Smem::NZF + rr * (TX + 1) + cc] || S.slow[Tile3Smem::NZF + rr * (TX + 1) + cc + 1] ||
-          S.slow[rr * TX + cc] ||
-          S.slow[under_gamma ? Tile3Smem::NZF + Tile3Smem::NXF + cc : (rr + 1) * TX + cc];
+    dbl = dbl || S.slow[(TZ + rr) * TX + cc] ||
+          S.slow[cc < TX - 1 ? (TZ + rr) * TX + cc + 1 : (2 * TZ + 1) * TX + rr] || S.slow[rr * TX + cc] ||
+          S.slow[(under_gamma ? 2 * TZ + 2 : rr + 1 < TZ ? rr + 1 : 2 * TZ) * TX + cc];
   if (dbl) {
 #pragma unroll
     for (int c = 0; c < 5; c++) {
