@@ -60,6 +60,17 @@ enum {
   FXC_N
 };
 
+// Interface: the wall velocity u_w = u_1 + LID_1 (u_2 - u_1) = u_2 - LID_2
+// (u_2 - u_1), so that the ghost 2 u_w - u of either fluid is u + 2 LID_f
+// (other fluid's u - u).
+enum {
+  LID_S,  // 2 b_u: twice the shear stress from u_2 - u_1
+  LID_1,  // b_u dz1 / (2 mu1)
+  LID_2,  // b_u dz2 / (2 mu2) = 1 - LID_1
+  LID_T,  // 2 b_T gamma (gamma - 1): twice -Pi_z from e_2 - e_1
+  LID_N
+};
+
 // Fixed-point constants of the FP64 tile's face fluxes (fixed_point.cuh).
 struct FxConst {
   int on;              // every factor below fits its scale: the fluxes run in fixed point
@@ -67,6 +78,7 @@ struct FxConst {
   double scale;        // their factor: 2^-57 of half of 1/dx
   FxW gm1;             // (gamma - 1).61
   FxW gg;              // gamma (gamma - 1).62
+  FxW lid[LID_N];      // interface, .62
   FxW fc[2][2][FXC_N]; // viscous coefficients per direction (x, z) and fluid, .62
 };
 
@@ -171,6 +183,14 @@ __host__ __device__ inline double visc_coef(const Geom& g, int dir, int fl, int 
     case FXC_C: return 2.0 * mu * in;
     case FXC_D: return 0.5 * mu * it;
     default: return 2.0 * (fl ? g.kap2 : g.kap1) * g.gamma * g.gm1 * in;
+  }
+}
+__host__ __device__ inline double lid_coef(const Geom& g, int j) {
+  switch (j) {
+    case LID_S: return 2.0 * g.bu;
+    case LID_1: return g.bu * g.cu1;
+    case LID_2: return g.bu * g.cu2;
+    default: return 2.0 * g.bT * g.gamma * g.gm1;
   }
 }
 // Fills the fixed-point constants of a geometry (mprk_runtime.cu).

@@ -24,7 +24,7 @@ namespace mprk {
 
 // GEN: the general s-stage base (RK3, RK4) in place of Heun's low-storage
 // combination. TZR: tile rows (TZ; 4 or 2 for launches of few tiles). NT:
-// TZR + 1 warps, up to 27 of them per SM (72 registers); twice that for
+// TZR + 1 warps, up to 27 of them per SM (72 registers); 2 TZR + 3 for
 // launches with no more tiles than SMs.
 constexpr int fp64_ctas(int rows) { return rows == TZ ? 3 : rows == TZ / 2 ? 5 : 9; }
 template <bool GEN = false, int NT = FP64_THREADS, int TZR = TZ>
@@ -104,10 +104,10 @@ cudaError_t prepare_kernels() {
   e = cudaFuncSetAttribute(stage_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)sizeof(TileSmem<>));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(stage_kernel<false, 2 * FP64_THREADS>,
+  e = cudaFuncSetAttribute(stage_kernel<false, TX * (2 * TZ + 3)>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem<>));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(stage_kernel<true, 2 * FP64_THREADS>,
+  e = cudaFuncSetAttribute(stage_kernel<true, TX * (2 * TZ + 3)>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem<>));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(yface3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(YfaceSmem));
@@ -182,7 +182,7 @@ namespace {
 // One FP64 stage launch with TZR-row tiles; wide: two threads per cell.
 template <int TZR>
 cudaError_t launch_fp64(const StageArgs& a, int n_tiles, bool wide, cudaStream_t stream, bool chained) {
-  constexpr int NT1 = TX * (TZR + 1), NT2 = 2 * NT1;
+  constexpr int NT1 = TX * (TZR + 1), NT2 = TX * (2 * TZR + 3);
   const size_t smem = sizeof(TileSmem<TZR>);
   if (wide && a.g.gen) return launch_kernel(stage_kernel<true, NT2, TZR>, n_tiles, NT2, smem, stream, chained, a);
   if (wide) return launch_kernel(stage_kernel<false, NT2, TZR>, n_tiles, NT2, smem, stream, chained, a);

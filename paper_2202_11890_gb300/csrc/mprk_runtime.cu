@@ -323,6 +323,12 @@ static bool fx_gas(const Geom& g, FxConst* out) {
   if (!(gg < 1.9)) return false;
   out->gm1 = fx_factor(g.gm1, 61);
   out->gg = fx_factor(gg, 62);
+  for (int j = 0; j < LID_N; j++) {
+    // harmonic means of the fluids' coefficients below: under 1 with them
+    const double x = lid_coef(g, j);
+    if (!(x < 1.0)) return false;
+    out->lid[j] = fx_factor(x, 62);
+  }
   return true;
 }
 

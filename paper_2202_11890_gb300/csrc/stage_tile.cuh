@@ -7,25 +7,24 @@
 //      memory (x periodic; stage values q + h R_a rebuilt on the fly in
 //      double), as doubles and as 64-bit fixed point, and computes u, w and
 //      e = T / (gamma (gamma - 1)) on the tile plus a one-cell ring,
-//   2. computes the interface state (bulk fluxes and wall states of App. B)
-//      when the tile touches it,
-//   3. computes every x and z face flux of the tile once (Lax–Friedrichs
+//   2. computes every x and z face flux of the tile once (Lax–Friedrichs
 //      inviscid flux of Sec. 2.1 on the linear reconstruction of the
 //      conserved variables, minus the common-value viscous flux of App. B),
 //      in one direction-generic routine written in the face frame, with
-//      mirror or wall-state ghosts beyond walls and the interface,
-//   4. forms R = -div F* + s per cell and applies the partition's stage
+//      mirror or wall-state ghosts beyond walls and the interface and the
+//      interface's bulk fluxes and wall states (App. B),
+//   3. forms R = -div F* + s per cell and applies the partition's stage
 //      combination (Eq. MRK2 in low-storage form) in double precision.
-// Only two barriers separate them: 1 and 2 from 3, and 3 from 4 (with phases
-// of their own for the ring and the tangential differences, and faces dealt to
-// threads in three uneven rounds, the step above took 2.39 ms).
+// Only two barriers separate them (with phases of their own for the ring, the
+// tangential differences and the interface state, and faces dealt to threads
+// in three uneven rounds, the step below took 2.39 ms).
 //
 // Velocities, differences and fluxes run in 64-bit fixed point (fixed_point.cuh): as double
 // arithmetic they were 300 of the tile's 309 operations per cell on a pipe
 // that completes two per clock and SM, which bound every FP64 launch: the
 // pipe was 86 % busy. Measured: a slow step of 2048 x 1024 cells with m = 8
-// 11.7 -> 2.11 ms (B and F rows of one stage 649 -> 118 to 129 us), 64 x 64
-// with m = 4 167 -> 76 us; now 2320 instructions per cell and warp, 57 % of
+// 11.7 -> 2.08 ms (B and F rows of one stage 649 -> 116 to 127 us), 64 x 64
+// with m = 4 167 -> 55 us; now 2320 instructions per cell and warp, 57 % of
 // the integer pipe and 60 % of the issue slots busy. Errors of the right-hand side against 80-bit
 // arithmetic fell from 3e-16..1e-15 to 2e-17..5e-16 (rms per component; rest
 // state with 1 % bumps to 25 % cell noise). A face
@@ -50,10 +49,7 @@ struct TileSmem {
   i64 fx[4][TZR][TX + 1];  // face f between cols f-1, f
   i64 fz[4][TZR + 1][TX];  // seen from above at the interface
   i64 fg[4][TX];           // the interface seen from fluid 1 (below)
-  double gam[3][TX + 2];   // sigma_xz, Pi_z, u_w per column i0-1..
-  i64 gam_fx[3][TX + 2];   // 2 u_w .59, 2 sigma_xz .57, 2 (u_w sigma_xz - Pi_z) .57
   double fc[2][2][FXC_N];  // viscous coefficients of the double pass
-  unsigned char gam_ok[TX + 2];
   unsigned char slow[(2 * TZR + 3) * TX];  // per face: its job and lane (face_id)
 };
 
@@ -213,20 +209,36 @@ __device__ __forceinline__ void ring_cell(const Geom& g, TileSmem<TZR>& S, int r
   v[2 * VP] = o[2];
 }
 
-// 2 u_w of the interface state in T.
-template <typename T>
-__device__ __forceinline__ T lid_u2(double uw, i64 uw_fx);
-template <>
-__device__ __forceinline__ i64 lid_u2<i64>(double, i64 uw_fx) { return uw_fx; }
-template <>
-__device__ __forceinline__ double lid_u2<double>(double uw, i64) { return __dmul_rn(2.0, uw); }
+// Interface (App. B, Eq. bulk-flux and the wall states after it), from the
+// velocities and e of the two cells touching it: the ghost velocity 2 u_w - u
+// of the cell `own` in fluid f + 1, and twice (sigma, u_w sigma - Pi), the
+// flux both fluids share. In double from the state, by 34 threads of the tile
+// before its faces, these took the launch of 64 x 64 cells a quarter of its
+// time: a warp's double operation occupies its scheduler for 64 clocks.
+__device__ __forceinline__ i64 lid_ghost(const Geom&, const FxConst& k, int f, i64 own, i64 other) {
+  return own + (fx::mul(fx::split((other - own) << 2), k.lid[LID_1 + f]) << 1);
+}
+__device__ __forceinline__ double lid_ghost(const Geom& g, const FxConst&, int f, double own, double other) {
+  return __fma_rn(__dmul_rn(2.0, lid_coef(g, LID_1 + f)), __dsub_rn(other, own), own);
+}
+__device__ __forceinline__ void lid_flux(const Geom&, const FxConst& k, i64 u1, i64 u2, i64 e1, i64 e2, i64 V[2]) {
+  const i64 du = u2 - u1, uw = u1 + fx::mul(fx::split(du << 2), k.lid[LID_1]);
+  V[0] = fx::mul(fx::split(du), k.lid[LID_S]);                                        // .57
+  V[1] = (fx::mul(fx::split(uw << 3), fx::split(V[0])) << 2) + fx::mul(fx::split(e2 - e1), k.lid[LID_T]);
+}
+__device__ __forceinline__ void lid_flux(const Geom& g, const FxConst&, double u1, double u2, double e1, double e2,
+                                         double V[2]) {
+  const double du = __dsub_rn(u2, u1), uw = __fma_rn(lid_coef(g, LID_1), du, u1);
+  V[0] = __dmul_rn(lid_coef(g, LID_S), du);
+  V[1] = __fma_rn(uw, V[0], __dmul_rn(lid_coef(g, LID_T), __dsub_rn(e2, e1)));
+}
 
-// ---- phase 3: face fluxes ---------------------------------------------------
+// ---- phase 2: face fluxes ---------------------------------------------------
 // The faces of the tile as jobs of one warp each: TZR rows of z faces, TZR
 // rows of x faces (columns 0 to TX - 1), the z faces above the last row, the
 // x faces right of the last column (one lane per row), and in a tile at the
 // interface its faces seen from below. With TZR + 1 warps these are two jobs
-// per warp, with twice that one: no round leaves warps waiting for a few last
+// per warp, with 2 TZR + 3 one: no round leaves warps waiting for a few last
 // faces.
 struct FaceId {
   int isx, f, c;  // z: face row f, column c; x: tile row f, face column c
@@ -265,11 +277,12 @@ __device__ __forceinline__ bool face_id(const Geom& g, int job, int lane, int k0
 // reconstructed from the four cells across it, and the two cells' velocities,
 // e and tangential differences (un, ut, e, gn, gt). A boundary face (outer
 // wall or interface) has the inner cell's state on one side and its mirror
-// on the other; an outer wall's viscous ghost is 2 wall state - cell. Returns
-// the fluid of the face's coefficients, 2 + fluid at the interface.
+// on the other; an outer wall's viscous ghost is 2 wall state - cell, and the
+// interface has its own viscous flux VI (sigma, energy). Returns the fluid of
+// the face's coefficients, 2 at the interface.
 template <typename T, int TZR>
-__device__ __forceinline__ int face_sides(const Geom& g, const TileSmem<TZR>& S, const FaceId& id, T L[4], T R[4],
-                                          T vL[5], T vR[5]) {
+__device__ __forceinline__ int face_sides(const Geom& g, const FxConst& fk, const TileSmem<TZR>& S, const FaceId& id,
+                                          T L[4], T R[4], T vL[5], T vR[5], T VI[2]) {
   constexpr int QP = (TZR + 4) * (TX + 4), VP = (TZR + 2) * (TX + 2);
   const int n1 = g.n1, nz = g.nz, ku = id.ku, kd = ku - 1;
   // first of the four cells, their stride, and the planes of m_n, m_t
@@ -309,9 +322,13 @@ __device__ __forceinline__ int face_sides(const Geom& g, const TileSmem<TZR>& S,
       R[c] = Arith<T>::rec(a2, a1, a3);
     }
   }
-  if (lid) return id.below ? 2 : 3;
   // velocities, e and tangential central differences of the cells at the face
   const T* v = reinterpret_cast<const T*>(&S.v[0][0][0]);
+  if (lid) {
+    const T* p = v + id.f * (TX + 2) + id.c + 1;
+    lid_flux(g, fk, p[0], p[TX + 2], p[2 * VP], p[2 * VP + TX + 2], VI);
+    return 2;
+  }
   if (id.isx) {
     const T* p = v + (id.f + 1) * (TX + 2) + id.c;
     const bool top = ku + 1 == nz || ku + 1 == n1, bot = ku == 0 || ku == n1;
@@ -326,14 +343,14 @@ __device__ __forceinline__ int face_sides(const Geom& g, const TileSmem<TZR>& S,
       // wall or the interface
       T uu, wu, ud, wd;
       if (top) {
-        uu = ku + 1 == nz ? (g.wall ? u : -u) : lid_u2<T>(S.gam[2][id.c + s], S.gam_fx[0][id.c + s]) - u;
+        uu = ku + 1 == nz ? (g.wall ? u : -u) : lid_ghost(g, fk, 0, u, p[TX + 2]);
         wu = -w;
       } else {
         uu = p[TX + 2];
         wu = p[VP + TX + 2];
       }
       if (bot) {
-        ud = ku == 0 ? (g.wall ? u : -u) : lid_u2<T>(S.gam[2][id.c + s], S.gam_fx[0][id.c + s]) - u;
+        ud = ku == 0 ? (g.wall ? u : -u) : lid_ghost(g, fk, 1, u, p[-(TX + 2)]);
         wd = -w;
       } else {
         ud = p[-(TX + 2)];
@@ -409,8 +426,7 @@ __device__ __forceinline__ void store_flux(TileSmem<TZR>& S, const FaceId& id, c
 }
 
 // Do the cells that face id reads (four across it, and the tangential
-// neighbours of the two at it), and the interface states if it reads any,
-// lie in the fixed-point range? Asked only in tiles where some cell does not.
+// neighbours of the two at it) lie in the fixed-point range? Asked only in tiles where some cell does not.
 template <int TZR>
 __device__ __noinline__ bool face_in_range(const Geom& g, const TileSmem<TZR>& S, const FaceId id, int k0) {
   auto cell = [&](int r, int c) {  // halo row and column
@@ -421,11 +437,9 @@ __device__ __noinline__ bool face_in_range(const Geom& g, const TileSmem<TZR>& S
   if (id.isx) {
     for (int j = 0; j < 4; j++) ok = ok && cell(id.f + 2, id.c + j);
     for (int j = 0; j < 4; j++) ok = ok && cell(id.f + 1 + 2 * (j >> 1), id.c + 1 + (j & 1));
-    if (id.ku == g.n1 || id.ku == g.n1 - 1) ok = ok && S.gam_ok[id.c] && S.gam_ok[id.c + 1];
   } else {
     for (int j = 0; j < 4; j++) ok = ok && cell(id.f + j, id.c + 2);
     for (int j = 0; j < 4; j++) ok = ok && cell(id.f + 1 + (j >> 1), id.c + 1 + 2 * (j & 1));
-    if (id.ku == g.n1) ok = ok && S.gam_ok[id.c + 1];
   }
   return ok;
 }
@@ -435,7 +449,7 @@ __device__ __noinline__ bool face_in_range(const Geom& g, const TileSmem<TZR>& S
 // barrier. A grid wholly outside the range runs as fast as the tile that did
 // everything in double (2048 x 1024, m = 8: 11.5 ms per step against 11.7).
 template <int NT, int TZR>
-__device__ __noinline__ void slow_faces(const Geom& g, TileSmem<TZR>& S, int k0, int i0, int row_hi, bool all) {
+__device__ __noinline__ void slow_faces(const Geom& g, const FxConst& fk, TileSmem<TZR>& S, int k0, int i0, int row_hi, bool all) {
   for (int e = threadIdx.x; e < (TZR + 2) * (TX + 2); e += NT) {
     const int rr = e / (TX + 2) + 1, cc = e % (TX + 2) + 1, k = k0 - 2 + rr;
     if (k >= 0 && k < g.nz)
@@ -452,12 +466,9 @@ __device__ __noinline__ void slow_faces(const Geom& g, TileSmem<TZR>& S, int k0,
     if (!face_id<TZR>(g, job, lane, k0, row_hi, &id) || !(all || S.slow[e])) continue;
     if (all) S.slow[e] = 1;
     double L[4], R[4], vL[5], vR[5], V[3], F[4];
-    const int fl = face_sides<double, TZR>(g, S, id, L, R, vL, vR);
-    if (fl >= 2) {
-      V[0] = 0.0;
-      V[1] = 2.0 * S.gam[0][id.c + 1];
-      V[2] = 2.0 * __fma_rn(S.gam[2][id.c + 1], S.gam[0][id.c + 1], -S.gam[1][id.c + 1]);
-    } else {
+    V[0] = 0.0;
+    const int fl = face_sides<double, TZR>(g, fk, S, id, L, R, vL, vR, V + 1);
+    if (fl < 2) {
       double_visc(S.fc[id.isx ? 0 : 1][fl], vL, vR, V);
     }
     double_flux(g, L, R, V, F);
@@ -480,7 +491,7 @@ __device__ __noinline__ void slow_faces(const Geom& g, TileSmem<TZR>& S, int k0,
 // Heun's low-storage path: s R_a slots, the stage values of the region
 // tableaus built from the base, and its weights b in the combinations.
 // NT: threads of the CTA. TZR + 1 warps make two rounds of face jobs;
-// launches with fewer tiles than the GPU has SMs take twice that, one round,
+// launches with fewer tiles than the GPU has SMs take 2 TZR + 3, one round,
 // so that each SM holds more warps of the few tiles there are. Every phase
 // but the last spreads its work over all threads, and the last (one cell per
 // thread) uses the first TX x TZR. TZR: tile rows.
@@ -544,47 +555,11 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
     ring_cell<i64, TZR>(g, S, rr, cc, i0, t[0], t[1], t[2], t[3]);
   }
   const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZR);
-  // ---- 2. interface state -------------------------------------------------
-  // of column i0-1+j in double precision from the two cells touching Gamma
-  // (App. B, Eq. bulk-flux and the wall states), by the last threads, which
-  // staged fewer cells
-  if (has_gamma) {
-    for (int j = NT - 1 - tid; j < TX + 2; j += NT) {
-      bool gh;
-      const int i = halo_col(i0 - 1 + j, nx, g.xwall, &gh);
-      double u[2], T[2];
-#pragma unroll
-      for (int s = 0; s < 2; s++) {
-        double qq[4];
-#pragma unroll
-        for (int c = 0; c < 4; c++) qq[c] = stage_value(c, n1 - 1 + s, i);
-        if (gh) qq[1] = -qq[1];  // mirror state beyond an x wall
-        const double inv = 1.0 / qq[0];
-        u[s] = __dmul_rn(qq[1], inv);
-        const double w = __dmul_rn(qq[2], inv);
-        const double k = __fma_rn(qq[2], w, __dmul_rn(qq[1], u[s]));
-        const double p = __dmul_rn(g.gm1, __fma_rn(-0.5, k, qq[3]));
-        T[s] = __dmul_rn(__dmul_rn(g.gamma, p), inv);
-      }
-      const double sig = __dmul_rn(g.bu, __dsub_rn(u[1], u[0]));
-      const double Pi = __dmul_rn(-g.bT, __dsub_rn(T[1], T[0]));
-      const double uw = __fma_rn(sig, g.cu1, u[0]), En = __fma_rn(uw, sig, -Pi);
-      S.gam[0][j] = sig;
-      S.gam[1][j] = Pi;
-      S.gam[2][j] = uw;
-      const bool ok = fabs(uw) < 1.9 && fabs(sig) < 2.0 && fabs(En) < 2.0;  // false for NaN
-      S.gam_ok[j] = ok;
-      bad |= !ok;
-      S.gam_fx[0][j] = __double2ll_rn(ok ? __dmul_rn(uw, (double)(2ll << fx::S_VEL)) : 0.0);
-      S.gam_fx[1][j] = __double2ll_rn(ok ? __dmul_rn(sig, (double)(2ll << fx::S_FLUX)) : 0.0);
-      S.gam_fx[2][j] = __double2ll_rn(ok ? __dmul_rn(En, (double)(2ll << fx::S_FLUX)) : 0.0);
-    }
-  }
   bad = __syncthreads_or(bad);
   bool none = false;  // no cell inside: every face in double
   if (bad) none = !a.fx.on || !__syncthreads_or(good);
 
-  // ---- 3. face fluxes ----------------------------------------------------
+  // ---- 2. face fluxes ----------------------------------------------------
   static_assert(TX == 32 && NT % 32 == 0, "a job is one warp wide");
   bool slow = false;
   const int jobs = none ? 0 : 2 * TZR + 2 + has_gamma;
@@ -595,12 +570,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
     bool ok = !bad || face_in_range<TZR>(g, S, id, k0);
     if (ok) {
       i64 L[4], R[4], vL[5], vR[5], V[3], F[4];
-      const int fl = face_sides<i64, TZR>(g, S, id, L, R, vL, vR);
-      if (fl >= 2) {
-        V[0] = 0;
-        V[1] = S.gam_fx[1][id.c + 1];
-        V[2] = S.gam_fx[2][id.c + 1];
-      } else {
+      V[0] = 0;
+      const int fl = face_sides<i64, TZR>(g, a.fx, S, id, L, R, vL, vR, V + 1);
+      if (fl < 2) {
         fx_visc(a.fx.fc[id.isx ? 0 : 1][fl], vL, vR, V);
       }
       ok = fx_flux<2>(g, a.fx, L, R, V, F);
@@ -610,9 +582,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
     slow |= !ok;
   }
   slow = none || __syncthreads_or(slow);
-  if (slow) slow_faces<NT, TZR>(g, S, k0, i0, row_hi, none);
+  if (slow) slow_faces<NT, TZR>(g, a.fx, S, k0, i0, row_hi, none);
 
-  // ---- 4. R = -div F* + s and the stage combination ----------------------
+  // ---- 3. R = -div F* + s and the stage combination ----------------------
   {
     const int rr = tid / TX, cc = tid - rr * TX;
     const int k = k0 + rr, i = i0 + cc;

@@ -18,7 +18,7 @@
 // As in the 2-D tile, velocities, differences and fluxes run in 64-bit fixed
 // point (fixed_point.cuh), because the double pipe bound both kernels (80 to
 // 86 % busy with 125 + 238 operations per cell). Measured: a slow step of
-// 512 x 64 x 200 cells with m = 4 44.1 -> 9.3 ms. A face whose own cells leave
+// 512 x 64 x 200 cells with m = 4 44.1 -> 8.8 ms. A face whose own cells leave
 // the range is evaluated in double by a second pass over the tile; which form
 // a face takes depends on its cells alone, so neighbouring tiles agree on the
 // faces they share. Fluxes come over half the divergence factor of their
@@ -188,68 +188,19 @@ __device__ __forceinline__ double flux_value(i64 f) {
   return __dmul_rn((double)f, 1.0 / (double)(1ll << fx::S_FLUX));
 }
 
-// Interface state of column (i, j) (App. B, Eq. bulk-flux and the wall
-// states after it), doubled: 2 u_w, 2 v_w of fluid 1 and of fluid 2, each
-// with its own formula, 2 sigma_xz, 2 sigma_yz, and 2 (u_w sigma_xz + v_w
-// sigma_yz - Pi_z) of each fluid.
-enum { L3_U1, L3_V1, L3_U2, L3_V2, L3_SX, L3_SY, L3_E1, L3_E2, L3_N };
-__device__ __forceinline__ void interface3(const StageArgs& a, const Geo3& G, int j, int i, double out[L3_N]) {
-  const Geom& g = a.g;
-  double v1[4], v2[4], q[5];
-  stage_val3(a, G, G.n1 - 1, j, i, q);
-  Arith3<double>::prims(q, v1);
-  stage_val3(a, G, G.n1, j, i, q);
-  Arith3<double>::prims(q, v2);
-  const double sxz = __dmul_rn(g.bu, __dsub_rn(v2[0], v1[0]));
-  const double syz = __dmul_rn(g.bu, __dsub_rn(v2[1], v1[1]));  // b_v = b_u
-  const double gg = __dmul_rn(g.gamma, g.gm1);                  // T / e
-  const double Pi = __dmul_rn(__dmul_rn(-g.bT, gg), __dsub_rn(v2[3], v1[3]));
-  const double u1 = __fma_rn(sxz, g.cu1, v1[0]), w1 = __fma_rn(syz, g.cu1, v1[1]);
-  const double u2 = __fma_rn(-sxz, g.cu2, v2[0]), w2 = __fma_rn(-syz, g.cu2, v2[1]);
-  out[L3_U1] = 2.0 * u1;
-  out[L3_V1] = 2.0 * w1;
-  out[L3_U2] = 2.0 * u2;
-  out[L3_V2] = 2.0 * w2;
-  out[L3_SX] = 2.0 * sxz;
-  out[L3_SY] = 2.0 * syz;
-  out[L3_E1] = 2.0 * __fma_rn(u1, sxz, __fma_rn(w1, syz, -Pi));
-  out[L3_E2] = 2.0 * __fma_rn(u2, sxz, __fma_rn(w2, syz, -Pi));
-}
-// The same as T into column cc of L (row stride ls); false where a value
-// leaves the fixed-point range.
+// Central z difference (unscaled) of velocity component comp at row k from
+// the cell and its neighbours above and below (v, rows of stride vr), with
+// the ghost 2 (wall state) - cell beyond a wall or Gamma; component 2 (w) is
+// normal there.
 template <typename T>
-__device__ __forceinline__ bool store_lid(const double s[L3_N], T* L, int ls);
-template <>
-__device__ __forceinline__ bool store_lid<double>(const double s[L3_N], double* L, int ls) {
-#pragma unroll
-  for (int q = 0; q < L3_N; q++) L[q * ls] = s[q];
-  return true;
-}
-template <>
-__device__ __forceinline__ bool store_lid<i64>(const double s[L3_N], i64* L, int ls) {
-  bool ok = true;
-#pragma unroll
-  for (int q = 0; q < L3_N; q++) ok = ok && fabs(s[q]) < 3.8;  // false for NaN
-#pragma unroll
-  for (int q = 0; q < L3_N; q++)
-    L[q * ls] = __double2ll_rn(ok ? __dmul_rn(s[q], (double)(1ll << (q < L3_SX ? fx::S_VEL : fx::S_FLUX))) : 0.0);
-  return ok;
-}
-
-// Central z differences (unscaled) of the velocities A and B at row k from
-// the cell and its neighbours above and below, with the ghost 2 (wall state)
-// - interior beyond a wall or Gamma; component 2 (w) is normal there. v: the
-// cell's u in a plane of stride vp, rows of stride vr; lid: the column's
-// interface state.
-template <typename T>
-__device__ __forceinline__ T dz_vel(const Geom& g, int k, int comp, const T* v, int vr, const T* lid, int ls) {
-  const T c = v[0];
+__device__ __forceinline__ T dz_vel(const Geom& g, const FxConst& c, int k, int comp, const T* v, int vr) {
+  const T u = v[0];
   T up, dn;
-  if (k + 1 == g.nz) up = (comp == 2 || !g.wall) ? -c : c;
-  else if (k + 1 == g.n1) up = comp == 2 ? -c : lid[(L3_U1 + comp) * ls] - c;  // fluid 1's top row
+  if (k + 1 == g.nz) up = (comp == 2 || !g.wall) ? -u : u;
+  else if (k + 1 == g.n1) up = comp == 2 ? -u : lid_ghost(g, c, 0, u, v[vr]);  // fluid 1's top row
   else up = v[vr];
-  if (k == 0) dn = (comp == 2 || !g.wall) ? -c : c;
-  else if (k == g.n1) dn = comp == 2 ? -c : lid[(L3_U2 + comp) * ls] - c;  // fluid 2's bottom row
+  if (k == 0) dn = (comp == 2 || !g.wall) ? -u : u;
+  else if (k == g.n1) dn = comp == 2 ? -u : lid_ghost(g, c, 1, u, v[-vr]);  // fluid 2's bottom row
   else dn = v[-vr];
   return up - dn;
 }
@@ -303,9 +254,7 @@ constexpr int RING3 = (TZ + 2) * (TX + 2);  // tile plus a one-cell ring
 struct YfaceSmem {
   i64 q[2][5][TZ + 2][TX + 2];   // planes j and j+1, rows k0-1.., cols i0-1..
   i64 v[2][4][TZ + 2][TX + 2];   // u, v, w, e on the ring
-  i64 lid[2][L3_N][TX];          // interface state of the tile columns
   unsigned char ok[2][TZ + 2][TX + 2];
-  unsigned char lid_ok[2][TX];
 };
 
 // The y face between planes j and j+1 of the thread's cell (k, i), in T, from
@@ -324,7 +273,6 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
   const int j1 = wrap3(j + 1, g.ny);
   T* Sq = reinterpret_cast<T*>(&S.q[0][0][0][0]);
   T* Sv = reinterpret_cast<T*>(&S.v[0][0][0][0]);
-  T* Sl = reinterpret_cast<T*>(&S.lid[0][0][0]);
   bool bad = false;
   for (int e = tid; e < 2 * RING3; e += NTHREADS) {
     const int side = e >= RING3, rem = e - side * RING3;
@@ -350,15 +298,6 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
 #pragma unroll
     for (int c = 0; c < 4; c++) Sv[(side * 4 + c) * RING3 + rem] = v[c];
   }
-  const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZ);
-  if (has_gamma && tid < 2 * TX) {
-    const int side = tid / TX, cc = tid - side * TX;
-    double st[L3_N];
-    interface3(a, G, side ? j1 : j, wrap3(i0 + cc, g.nx), st);
-    const bool ok = store_lid<T>(st, Sl + side * L3_N * TX + cc, TX);
-    if (FX) S.lid_ok[side][cc] = ok;
-    bad |= !ok;
-  }
   const int rr = tid / TX, cc = tid - rr * TX;
   const int k = k0 + rr, i = i0 + cc;
   const bool mine = k < row_hi && i < g.nx;
@@ -382,12 +321,11 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
   if (FX) {
     if (bad) {
       // the face's own cells: the four across it and the x and z neighbours
-      // of the two at it (inside the grid), and the interface states it reads
+      // of the two at it (inside the grid)
       for (int s = 0; s < 2; s++) {
         out_ok = out_ok && S.ok[s][rr + 1][cc + 1] && S.ok[s][rr + 1][cc] && S.ok[s][rr + 1][cc + 2];
         if (k > 0) out_ok = out_ok && S.ok[s][rr][cc + 1];
         if (k + 1 < nz) out_ok = out_ok && S.ok[s][rr + 2][cc + 1];
-        if (k == n1 || k == n1 - 1) out_ok = out_ok && S.lid_ok[s][cc];
       }
     }
     if (!out_ok) return false;
@@ -406,15 +344,14 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
 #pragma unroll
   for (int side = 0; side < 2; side++) {
     const T* V = Sv + side * 4 * RING3 + at;
-    const T* lid = Sl + side * L3_N * TX + cc;
     s[side].u[0] = V[RING3];
     s[side].u[1] = V[0];
     s[side].u[2] = V[2 * RING3];
     s[side].e = V[3 * RING3];
     s[side].g1[0] = V[RING3 + 1] - V[RING3 - 1];  // x differences of v, u
     s[side].g1[1] = V[1] - V[-1];
-    s[side].g2[0] = dz_vel(g, k, 1, V + RING3, TX + 2, lid, TX);  // z differences of v, w
-    s[side].g2[1] = dz_vel(g, k, 2, V + 2 * RING3, TX + 2, lid, TX);
+    s[side].g2[0] = dz_vel(g, C.k, k, 1, V + RING3, TX + 2);  // z differences of v, w
+    s[side].g2[1] = dz_vel(g, C.k, k, 2, V + 2 * RING3, TX + 2);
   }
   T V[4];
   visc3(C, 1, k >= n1, s[0], s[1], V);
@@ -447,16 +384,13 @@ struct Tile3Smem {
   i64 fx[5][TZ][TX + 1];      // x face fluxes, face f between cols f-1, f
   i64 fz[5][TZ + 1][TX];      // z face fluxes seen from above
   i64 fg[5][TX];              // interface flux seen from fluid 1
-  i64 lid[L3_N][TX + 2];      // interface state per ring column
   unsigned char ok[TZ + 4][TX + 4];
   unsigned char oky[TZ + 2][TX + 2];  // the cells in planes j-1 and j+1
-  unsigned char lid_ok[TX + 2];
   unsigned char slow[(2 * TZ + 3) * TX];  // per face: its job and lane
 };
 
-// Phases 1 and 2 in T: stage state, velocities and their y differences, and
-// the interface state. Returns (T = i64) 0, or 1 where
-// some cell or interface state leaves the fixed-point range, or 2 where every
+// Phase 1 in T: stage state, velocities and their y differences. Returns
+// (T = i64) 0, or 1 where some cell leaves the fixed-point range, or 2 where every
 // cell does. Ends with a barrier.
 template <typename T>
 __device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, int k0, int i0, int j, Tile3Smem& S) {
@@ -468,7 +402,6 @@ __device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, in
   T* q = reinterpret_cast<T*>(&S.q[0][0][0]);
   T* v = reinterpret_cast<T*>(&S.v[0][0][0]);
   T* vy = reinterpret_cast<T*>(&S.vy[0][0][0]);
-  T* lid = reinterpret_cast<T*>(&S.lid[0][0]);
   bool bad = false, good = false;
   for (int e = tid; e < QP; e += TILE3_THREADS) {
     const int rr = e / (TX + 4), cc = e - rr * (TX + 4);
@@ -527,18 +460,6 @@ __device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, in
 #pragma unroll
     for (int c = 0; c < 3; c++) vy[c * RING3 + e] = up[c] - dn[c];
   }
-  const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZ);
-  if (has_gamma) {
-    // by the last threads, which staged fewer cells
-    const int e = TILE3_THREADS - 1 - tid;
-    if (e < TX + 2) {
-      double st[L3_N];
-      interface3(a, G, j, wrap3(i0 - 1 + e, g.nx), st);
-      const bool ok = store_lid<T>(st, lid + e, TX + 2);
-      if (FX) S.lid_ok[e] = ok;
-      bad |= !ok;
-    }
-  }
   if (!FX) {
     __syncthreads();
     return 0;
@@ -566,16 +487,20 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
   const T* q = reinterpret_cast<const T*>(&S.q[0][0][0]) + q0;
   T L[5], R[5], V[4];
   if (lidf) {
-    const T* lid = reinterpret_cast<const T*>(&S.lid[0][0]) + id.c + 1;
+    // the bulk fluxes, with the wall velocities (one value for both fluids)
+    const T* p = reinterpret_cast<const T*>(&S.v[0][0][0]) + id.f * (TX + 2) + id.c + 1;
     V[0] = 0;
-    V[1] = lid[L3_SX * (TX + 2)];
-    V[2] = lid[L3_SY * (TX + 2)];
-    V[3] = lid[(id.below ? L3_E1 : L3_E2) * (TX + 2)];
+    T e2[2];  // each with its part of the energy: the heat flux once
+    lid_flux(g, C.k, p[0], p[TX + 2], p[3 * RING3], p[3 * RING3 + TX + 2], e2);
+    V[1] = e2[0];
+    V[3] = e2[1];
+    lid_flux(g, C.k, p[RING3], p[RING3 + TX + 2], T(0), T(0), e2);
+    V[2] = e2[0];
+    V[3] = V[3] + e2[1];
   } else {
     const T* v = reinterpret_cast<const T*>(&S.v[0][0][0]);
     const T* vy = reinterpret_cast<const T*>(&S.vy[0][0][0]);
     const int vo = id.isx ? (id.f + 1) * (TX + 2) + id.c : id.f * (TX + 2) + id.c + 1, vs = id.isx ? 1 : TX + 2;
-    const T* lid = reinterpret_cast<const T*>(&S.lid[0][0]) + id.c;
     VSide<T> s[2];
 #pragma unroll
     for (int side = 0; side < 2; side++) {
@@ -588,8 +513,8 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
       if (id.isx) {  // t1 = y: du, dv; t2 = z: du, dw
         s[side].g1[0] = y[0];
         s[side].g1[1] = y[RING3];
-        s[side].g2[0] = dz_vel(g, ku, 0, p, TX + 2, lid + side, TX + 2);
-        s[side].g2[1] = dz_vel(g, ku, 2, p + 2 * RING3, TX + 2, lid + side, TX + 2);
+        s[side].g2[0] = dz_vel(g, C.k, ku, 0, p, TX + 2);
+        s[side].g2[1] = dz_vel(g, C.k, ku, 2, p + 2 * RING3, TX + 2);
       } else {  // t1 = x: dw, du; t2 = y: dw, dv
         s[side].g1[0] = p[2 * RING3 + 1] - p[2 * RING3 - 1];
         s[side].g1[1] = p[1] - p[-1];
@@ -662,8 +587,7 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
 }
 
 // Do the cells that face id reads lie in the range? The four across it, the
-// y neighbours and the third-direction neighbours of the two at it, and the
-// interface states. Asked only in tiles where some cell does not.
+// y neighbours and the third-direction neighbours of the two at it. Asked only in tiles where some cell does not.
 __device__ __noinline__ bool face3_in_range(const Geom& g, const Tile3Smem& S, const FaceId id, int k0) {
   auto cell = [&](int r, int c) {  // halo row and column
     const int k = k0 - 2 + r;
@@ -678,12 +602,10 @@ __device__ __noinline__ bool face3_in_range(const Geom& g, const Tile3Smem& S, c
     for (int s = 0; s < 4; s++) ok = ok && cell(id.f + 2, id.c + s);
     for (int s = 0; s < 2; s++)
       ok = ok && cell(id.f + 1, id.c + 1 + s) && cell(id.f + 3, id.c + 1 + s) && celly(id.f + 1, id.c + s);
-    if (id.ku == g.n1 || id.ku == g.n1 - 1) ok = ok && S.lid_ok[id.c] && S.lid_ok[id.c + 1];
   } else {
     for (int s = 0; s < 4; s++) ok = ok && cell(id.f + s, id.c + 2);
     for (int s = 0; s < 2; s++)
       ok = ok && cell(id.f + 1 + s, id.c + 1) && cell(id.f + 1 + s, id.c + 3) && celly(id.f + s, id.c + 1);
-    if (id.ku == g.n1) ok = ok && S.lid_ok[id.c + 1];
   }
   return ok;
 }
@@ -709,10 +631,10 @@ __device__ __forceinline__ void stage_tile3(const StageArgs& a, const Fx3Const& 
   const int nz = g.nz, nx = g.nx, ny = g.ny, n1 = g.n1;
   const int row_hi = a.rhs_only ? a.rhs_hi : nz;
 
-  // ---- 1-2. stage state, velocities, interface state -------------------------
+  // ---- 1. stage state, velocities -------------------------
   const int out = C.k.on ? tile3_cells<i64>(a, G, k0, i0, j, S) : 2;
 
-  // ---- 3. face fluxes -----------------------------------------------------
+  // ---- 2. face fluxes -----------------------------------------------------
   const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZ);
   const int jobs = out == 2 ? 0 : 2 * TZ + 2 + has_gamma;
   const int warp = __shfl_sync(0xffffffffu, tid / 32, 0), lane = tid % 32;
@@ -727,7 +649,7 @@ __device__ __forceinline__ void stage_tile3(const StageArgs& a, const Fx3Const& 
   slow = out == 2 || __syncthreads_or(slow);
   if (slow) slow_faces3(a, C, k0, i0, j, row_hi, S, out == 2);
 
-  // ---- 4. R = -div F* + s and the stage combination -------------------------
+  // ---- 3. R = -div F* + s and the stage combination -------------------------
   const int rr = tid / TX, cc = tid - rr * TX;
   const int k = k0 + rr, i = i0 + cc;
   if (rr >= TZ || k >= row_hi || i >= nx) return;
