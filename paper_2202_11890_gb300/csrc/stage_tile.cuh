@@ -383,6 +383,57 @@ __device__ __forceinline__ int face_sides(const Geom& g, const FxConst& fk, cons
   return (ku == 0 ? 0 : kd) >= n1;
 }
 
+// A tile none of whose faces lies at, or next to, a wall or the interface, and
+// none beyond the launch's rows: its faces need no ghosts and no row tests.
+template <int TZR>
+__device__ __forceinline__ bool tile_plain(const Geom& g, int k0, int row_hi) {
+  return k0 >= 2 && k0 + TZR <= g.nz - 2 && k0 + TZR <= row_hi && (g.n1 < k0 - 1 || g.n1 > k0 + TZR + 1);
+}
+// face_id and face_sides of such a tile, per direction: every cell at a fixed
+// offset from the face's first one. Without the row tests and the addresses
+// by direction 2048 x 1024 cells, m = 8, went from 2.118 to 2.058 ms per step,
+// 1024 x 512 with the RK4 base from 1.049 to 1.030 ms.
+// The general form stays for the tiles at the walls and the interface and
+// those with a cell outside the fixed-point range.
+template <int TZR>
+__device__ __forceinline__ bool face_id_plain(int job, int lane, int k0, FaceId* id) {
+  const bool edge = job == 2 * TZR + 1;
+  id->below = 0;
+  id->isx = job >= TZR && job != 2 * TZR;
+  id->f = edge ? lane : job < TZR ? job : job - TZR;
+  id->c = edge ? TX : lane;
+  id->ku = k0 + id->f;
+  return !edge || lane < TZR;
+}
+template <bool X, int TZR>
+__device__ __forceinline__ void face_sides_plain(const TileSmem<TZR>& S, const FaceId& id, i64 L[4], i64 R[4], i64 vL[5],
+                                                 i64 vR[5]) {
+  constexpr int QP = (TZR + 4) * (TX + 4), VP = (TZR + 2) * (TX + 2), VW = TX + 2;
+  constexpr int qs = X ? 1 : TX + 4, vs = X ? 1 : VW, vt = X ? VW : 1;  // along the normal; across it
+  constexpr int pn = X ? 1 : 2, pt = 3 - pn;
+  const i64* q = &S.qi[0][X ? id.f + 2 : id.f][X ? id.c : id.c + 2];
+  constexpr int planes[4] = {0, pn * QP, pt * QP, 3 * QP};
+#pragma unroll
+  for (int c = 0; c < 4; c++) {
+    const i64* p = q + planes[c];
+    const i64 a0 = p[0], a1 = p[qs], a2 = p[2 * qs], a3 = p[3 * qs];
+    L[c] = Arith<i64>::rec(a1, a2, a0);
+    R[c] = Arith<i64>::rec(a2, a1, a3);
+  }
+  const i64* v = &S.v[0][X ? id.f + 1 : id.f][X ? id.c : id.c + 1];
+  constexpr int vn = (pn - 1) * VP, vu = (pt - 1) * VP;
+#pragma unroll
+  for (int s = 0; s < 2; s++) {
+    const i64* p = v + s * vs;
+    i64* o = s ? vR : vL;
+    o[0] = p[vn];
+    o[1] = p[vu];
+    o[2] = p[2 * VP];
+    o[3] = p[vn + vt] - p[vn - vt];
+    o[4] = p[vu + vt] - p[vu - vt];
+  }
+}
+
 // The viscous flux over half the divergence factor from the common values of
 // App. B: (sigma_nn, sigma_nt, u . sigma_n + kappa dT/dn), .57.
 __device__ __forceinline__ void fx_visc(const FxW* fc, const i64 vL[5], const i64 vR[5], i64 V[3]) {
@@ -564,14 +615,24 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
   bool slow = false;
   const int jobs = none ? 0 : 2 * TZR + 2 + has_gamma;
   const int warp = __shfl_sync(0xffffffffu, tid / 32, 0), lane = tid % 32;
+  const bool plain = !bad && tile_plain<TZR>(g, k0, row_hi);
   for (int job = warp; job < jobs; job += NT / 32) {
     FaceId id;
-    if (!face_id<TZR>(g, job, lane, k0, row_hi, &id)) continue;
-    bool ok = !bad || face_in_range<TZR>(g, S, id, k0);
+    i64 L[4], R[4], vL[5], vR[5], V[3], F[4];
+    V[0] = 0;
+    int fl;
+    bool ok = true;
+    if (plain) {
+      if (!face_id_plain<TZR>(job, lane, k0, &id)) continue;
+      if (id.isx) face_sides_plain<true, TZR>(S, id, L, R, vL, vR);
+      else face_sides_plain<false, TZR>(S, id, L, R, vL, vR);
+      fl = k0 >= n1;
+    } else {
+      if (!face_id<TZR>(g, job, lane, k0, row_hi, &id)) continue;
+      ok = !bad || face_in_range<TZR>(g, S, id, k0);
+      if (ok) fl = face_sides<i64, TZR>(g, a.fx, S, id, L, R, vL, vR, V + 1);
+    }
     if (ok) {
-      i64 L[4], R[4], vL[5], vR[5], V[3], F[4];
-      V[0] = 0;
-      const int fl = face_sides<i64, TZR>(g, a.fx, S, id, L, R, vL, vR, V + 1);
       if (fl < 2) {
         fx_visc(a.fx.fc[id.isx ? 0 : 1][fl], vL, vR, V);
       }

@@ -140,3 +140,30 @@ def test_same_bits_in_every_tile_shape_and_in_a_batch(kind, tmp_path):
     assert np.isfinite(results[0]).all()
     for r in results[1:]:
         assert np.array_equal(results[0], r)
+
+
+@pytest.mark.parametrize("n1", range(5, 27))
+def test_same_bits_wherever_the_interface_meets_a_tile(n1, tmp_path):
+    """Tiles away from walls and the interface read their faces without ghosts;
+    every distance of the interface (row n1 of 34) from the edges of 8-, 4- and
+    2-row tiles gives the same bits, and the oracle's right-hand side."""
+    from paper_2202_11890_gb300 import mprk as M
+    grid = W.Grid(41, n1 - 4, 4, 34 - n1)
+    rng = np.random.default_rng(47)
+    rho, p = W.rest_primitives(grid)
+    r = [0.02 * rng.uniform(-1, 1, rho.shape) for _ in range(4)]
+    q = W.conserved(rho * (1 + r[0]), r[2], r[3], p * (1 + r[1]))
+    cfg, P, _ = pair(grid, 2, dt=0.001)
+    assert np.all(rel_err(gpu_rhs(cfg, q), O.rhs(P, q)) < 1e-12)
+    results = []
+    try:
+        for sh in SHAPES:
+            load_table(tmp_path, M, launch_buckets(grid, 2), sh)
+            with M.Instance(cfg, q) as inst:
+                inst.step(1)
+                results.append(inst.state())
+    finally:
+        M.mprk_tune_clear()
+    assert np.isfinite(results[0]).all()
+    for r in results[1:]:
+        assert np.array_equal(results[0], r)
