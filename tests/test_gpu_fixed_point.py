@@ -142,7 +142,7 @@ def test_same_bits_in_every_tile_shape_and_in_a_batch(kind, tmp_path):
         assert np.array_equal(results[0], r)
 
 
-@pytest.mark.parametrize("n1", range(5, 27))
+@pytest.mark.parametrize("n1", range(6, 27))
 def test_same_bits_wherever_the_interface_meets_a_tile(n1, tmp_path):
     """Tiles away from walls and the interface read their faces without ghosts;
     every distance of the interface (row n1 of 34) from the edges of 8-, 4- and
