@@ -270,8 +270,8 @@ TileShape default_tile_shape(const StageArgs& a);
 // Launchers (mprk_kernels.cu). All enqueue on `stream` and return the launch error.
 // chained: the launch before it on the stream is one of the same slow step
 // (or of the step before), so the two may overlap at their ends: the kernel
-// is launched as soon as every CTA of the one before has started, and its
-// CTAs wait for that one's completion before they touch memory (chain_wait).
+// is launched as soon as every CTA of the one before allows it (chain_next), and
+// its CTAs wait for that one's completion before they touch memory (chain_wait).
 // FP64 launches only: the FP32-flux launches ran 3 to 7 % slower chained
 // (4096 x 2048: 5.04 -> 5.24 ms for two steps), and ignore it.
 // maps (FP32-flux only, may be null) enables the staged tiles. shape (FP64
@@ -302,17 +302,22 @@ cudaError_t prepare_kernels();  // one-time attribute setup (dynamic shared memo
 size_t stage_smem_bytes(int precision);
 
 #ifdef __CUDACC__
-// Overlap of consecutive launches (programmatic dependent launch): lets the
-// next launch's CTAs start where this one leaves room, and waits until the
-// launch before this one has completed and its writes are visible. Every
-// thread calls it before its first access to the step's buffers, so a
-// launch's completion implies that of all before it. Without a chained
-// launch both are no-ops. A slow step of 64 x 64 cells, launched on a stream,
-// 105.6 -> 94.3 us (nine launches); as a graph 85.7 -> 84.6 us.
-__device__ __forceinline__ void chain_wait() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+// Overlap of consecutive launches (programmatic dependent launch).
+// chain_wait waits until the launch before this one has completed and its
+// writes are visible; every thread calls it before its first access to the
+// step's buffers, so a launch's completion implies that of all before it.
+// chain_next lets the next launch's CTAs start, once every CTA of this one has
+// called it. Without a chained launch both are no-ops. A slow step of 64 x 64
+// cells, launched on a stream, 105.6 -> 94.3 us (nine launches); as a graph
+// 85.7 -> 84.6 us. chain_next stands behind the faces: called as the kernel
+// starts, the next launch's CTAs fill the SMs that have room first, two or
+// three on some while others stay empty (321 x 273 cells, m = 4, 166 against
+// 131 us per step; 128 x 128 61.5 against 57.2). Kernels that fill an SM with
+// one CTA, and the 3-D ones, whose launches are many waves long, call it first
+// (100 x 300 cells 955 against 970 us for ten steps, 512 x 64 x 200 8.88
+// against 8.91 ms).
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // One launch, chained to the one before it on the stream or not.
 template <typename... P, typename... A>

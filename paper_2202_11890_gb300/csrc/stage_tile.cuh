@@ -667,6 +667,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
   slow = none || __syncthreads_or(slow);
   if (slow) slow_faces<NT, TZR>(g, a.fx, S, k0, i0, row_hi, none);
 
+  chain_next();
+
   // ---- 3. R = -div F* + s and the stage combination ----------------------
   {
     const int rr = tid / TX, cc = tid - rr * TX;
