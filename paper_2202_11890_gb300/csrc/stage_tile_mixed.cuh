@@ -330,7 +330,7 @@ __device__ __forceinline__ bool odd_mode(const StageArgs& a) {
 }
 
 // The general path on the TX x TZ cells from row k0, column i0.
-template <int PAR>
+template <int PAR, bool CHAIN = false>
 __device__ __forceinline__ void mixed_subtile(const StageArgs& a, int k0, int i0, MixedSmem& S) {
   const Geom& g = a.g;
   const int tid = threadIdx.x;
@@ -464,6 +464,7 @@ __device__ __forceinline__ void mixed_subtile(const StageArgs& a, int k0, int i0
   __syncthreads();
   if (tx == TX - 1 && ty < TZ) fxr = S.fxr[ty];
 
+  if (CHAIN) chain_next();
   // ---- 3. R (float) and the stage combination (double) -------------------
   const int i = i0 + tx;
   if (!live || i >= nx) return;
@@ -628,6 +629,8 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
+// Orders ordinary accesses visible to this thread before its later bulk copies.
+__device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 // One 3D tensor copy (tile mode) of the box at (x, y, z) of tmap into dst.
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tmap, int x, int y, int z,
                                             unsigned long long* bar) {
@@ -848,7 +851,7 @@ __device__ __forceinline__ void prefetch_combination(const StageArgs& a, int k0,
 // The pair path on the TX x MTZ interior tile from row k0, column i0. stg,
 // when not null, receives the tile's float planes by tensor copies that
 // complete on bar (phase 0). Returns false if the wait for them gave up.
-template <int PAR>
+template <int PAR, bool CHAIN = false>
 __device__ __forceinline__ bool pair_tile(const StageArgs& a, int k0, int i0, PairSmem& S, const Stage* stg,
                                           unsigned long long* bar) {
   const Geom& g = a.g;
@@ -998,6 +1001,7 @@ __device__ __forceinline__ bool pair_tile(const StageArgs& a, int k0, int i0, Pa
     }
   }
   __syncthreads();
+  if (CHAIN) chain_next();
   if (!own) return true;
   if (tx == TX - 1) {
     const float4 ea = S.fxa[p], eb = S.fxb[p];
@@ -1090,14 +1094,14 @@ union MixedTileSmem {
 // half: a tile on the general path runs as two TX x TZ halves one after the
 // other (-1), or as two CTAs, each with one half (0 and 1; half 1 of a pair
 // tile has nothing to do).
-template <int PAR>
+template <int PAR, bool CHAIN = false>
 __device__ __forceinline__ bool stage_tile_mixed(const StageArgs& a, int k0, int i0, MixedTileSmem& S,
                                                  const Stage* stg, unsigned long long* bar, int half = -1) {
-  if (pair_interior(a, k0, i0)) return half > 0 || pair_tile<PAR>(a, k0, i0, S.pair, stg, bar);
+  if (pair_interior(a, k0, i0)) return half > 0 || pair_tile<PAR, CHAIN>(a, k0, i0, S.pair, stg, bar);
   const int hi = rhs_mode<PAR>(a) ? a.rhs_hi : a.g.nz;
   for (int h = max(half, 0); h < (half < 0 ? 2 : half + 1) && k0 + h * TZ < hi; h++) {
     if (half < 0 && h > 0) __syncthreads();  // the first half's phase 3 reads shared memory
-    mixed_subtile<PAR>(a, k0 + h * TZ, i0, S.gen);
+    mixed_subtile<PAR, CHAIN>(a, k0 + h * TZ, i0, S.gen);
   }
   return true;
 }
