@@ -72,10 +72,9 @@ __device__ __noinline__ void batch_tile_fp64(int tile) {
                                   *reinterpret_cast<TileSmem<ROWS>*>(smem_raw + BATCH_ARGS_BYTES));
 }
 
-// three CTAs per SM in both precisions (80 and 72 registers; the FP32-flux
-// form spills some, and still runs faster than at two CTAs). ROWS: rows of
-// the FP64 tile, TZ (one thread per cell) or TZ / 2 (two threads per cell);
-// the block size stays the same.
+// three CTAs per SM in both precisions (72 registers; both spill some, and
+// the FP32-flux form still runs faster than at two CTAs). ROWS: rows of the
+// FP64 tile, TZ or TZ / 2; the block size stays the same.
 template <int PREC, int ROWS = TZ>
 __global__ void __launch_bounds__(batch_threads(PREC), 3) batch_kernel(const BatchArgs A) {
   extern __shared__ __align__(128) unsigned char smem_raw[];

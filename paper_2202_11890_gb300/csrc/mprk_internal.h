@@ -263,8 +263,8 @@ inline bool tile_shape_valid(const TileShape& t) {
 // when the tuning table has one for their size bucket (mprk_batch.cu).
 bool tuned_tile_shape(long long cells, TileShape* out);
 // The shape launch_stage takes without a tuned one: the shortest tile whose
-// launch fits in one wave (n tiles <= SMs), with two threads per cell; a
-// launch that does not fit even with TZ rows keeps them, one thread per cell.
+// launch fits in one wave (n tiles <= SMs), with a warp per face job; a
+// launch that does not fit even with TZ rows keeps them, two jobs per warp.
 TileShape default_tile_shape(const StageArgs& a);
 
 // Launchers (mprk_kernels.cu). All enqueue on `stream` and return the launch error.
@@ -272,8 +272,8 @@ TileShape default_tile_shape(const StageArgs& a);
 // (or of the step before), so the two may overlap at their ends: the kernel
 // is launched as soon as every CTA of the one before allows it (chain_next), and
 // its CTAs wait for that one's completion before they touch memory (chain_wait).
-// FP64 launches only: the FP32-flux launches ran 3 to 7 % slower chained
-// (4096 x 2048: 5.04 -> 5.24 ms for two steps), and ignore it.
+// FP32-flux launches are chained only within one wave (launch_stage): longer
+// ones ran 3 to 7 % slower (4096 x 2048: 5.04 -> 5.24 ms for two steps).
 // maps (FP32-flux only, may be null) enables the staged tiles. shape (FP64
 // only, may be null) overrides the tuned and the default tile shape.
 cudaError_t launch_stage(const StageArgs& a, int precision, int n_tiles, cudaStream_t stream,

@@ -1,7 +1,7 @@
 // mprk_kernels.cu — CUDA kernels of one MPRK2 slow step for sm_103a:
 //   stage_kernel        FP64 fused RHS + stage combination over the rows of
-//                       one stage (one thread per cell, or two in launches
-//                       with fewer tiles than SMs; Heun or a general base)
+//                       one stage (a warp per face job in launches with fewer
+//                       tiles than SMs, else per two; Heun or a general base)
 //   stage_kernel_mixed  the FP32-flux form, one instantiation per stage parity
 //   yface3_kernel, stage3_kernel  the 3-D model (App. B)
 //   finalize_kernel     moves q_{n+1} of the S and B rows (and of F rows after
@@ -187,7 +187,8 @@ int sm_count() {
 }  // namespace
 
 namespace {
-// One FP64 stage launch with TZR-row tiles; wide: two threads per cell.
+// One FP64 stage launch with TZR-row tiles; wide: a warp per face job instead of
+// one per two.
 template <int TZR>
 cudaError_t launch_fp64(const StageArgs& a, int n_tiles, bool wide, cudaStream_t stream, bool chained) {
   constexpr int NT1 = TX * (TZR + 1), NT2 = TX * (2 * TZR + 3);
