@@ -23,8 +23,8 @@
 // arithmetic they were 300 of the tile's 309 operations per cell on a pipe
 // that completes two per clock and SM, which bound every FP64 launch: the
 // pipe was 86 % busy. Measured: a slow step of 2048 x 1024 cells with m = 8
-// 11.7 -> 2.08 ms (B and F rows of one stage 649 -> 116 to 127 us), 64 x 64
-// with m = 4 167 -> 55 us; now 2320 instructions per cell and warp, 57 % of
+// 11.7 -> 2.06 ms (B and F rows of one stage 649 -> 114 us), 64 x 64
+// with m = 4 167 -> 55 us; 2300 instructions per cell, 57 % of
 // the integer pipe and 60 % of the issue slots busy. Errors of the right-hand side against 80-bit
 // arithmetic fell from 3e-16..1e-15 to 2e-17..5e-16 (rms per component; rest
 // state with 1 % bumps to 25 % cell noise). A face
