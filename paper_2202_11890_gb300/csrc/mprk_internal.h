@@ -313,9 +313,9 @@ size_t stage_smem_bytes(int precision);
 // starts, the next launch's CTAs fill the SMs that have room first, two or
 // three on some while others stay empty (321 x 273 cells, m = 4, 166 against
 // 131 us per step; 128 x 128 61.5 against 57.2). Kernels that fill an SM with
-// one CTA, and the 3-D ones, whose launches are many waves long, call it first
-// (100 x 300 cells 955 against 970 us for ten steps, 512 x 64 x 200 8.88
-// against 8.91 ms).
+// one CTA call it first (100 x 300 cells 63.0 against 63.7 us per step), and
+// so do the 3-D ones, whose launches are many waves long (the same within
+// 0.5 %).
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -251,9 +251,9 @@ cudaError_t launch_stage(const StageArgs& a, int precision, int n_tiles, cudaStr
     const bool one_wave = 2 * n_tiles <= 3 * sm_count();
     const dim3 grid(a.tiles_x, n_tiles / a.tiles_x, one_wave ? 2 : 1);
     const size_t smem = mixed_kernel_smem(a.stage & 1);
-    // chained in launches of one wave that use every SM: 200 x 200 cells 65.8 ->
-    // 61.7 us per step (m = 4), 321 x 273 72.2 -> 69.0; 64 x 64 59.5 -> 61.5,
-    // 4096 x 2048 1.96 -> 2.02 ms
+    // chained in launches of one wave that use every SM: 321 x 273 cells 70.2 ->
+    // 68.3 us per step (m = 4), 200 x 200 the same; chained everywhere, 64 x 64
+    // took 61.5 us instead of 59.5 and 4096 x 2048 2.02 ms instead of 1.96
     if (chained && one_wave && 2 * n_tiles >= sm_count() && !a.rhs_only) {
       auto* k = a.stage & 1 ? stage_kernel_mixed<1, true> : stage_kernel_mixed<0, true>;
       return launch_kernel(k, grid, MIXED_THREADS, smem, stream, true, s, sb, f, ra);
@@ -506,7 +506,6 @@ cudaError_t launch_shadow(const Geom& g, const double* q, const float* rowc, flo
 template <int U>
 __global__ void __launch_bounds__(256) finalize_kernel(const Geom g, const Bufs b, int m_odd, int vec, int k_hi) {
   const bool mixed = b.dA != nullptr;
-  if (mixed) chain_next();  // FP64: 55.6 against 53.7 us per step of 64 x 64; FP32 flux: 63.9 against 65.8 of 200 x 200
   chain_wait();
   const int c = blockIdx.z;
   const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
