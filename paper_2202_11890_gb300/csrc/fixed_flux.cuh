@@ -69,13 +69,30 @@ __device__ __noinline__ i64 fx_roe_speed(i64 rL, i64 rR, i64 unL, i64 unR, i64 d
   return __double2ll_rn(__dmul_rn(__dadd_rn(fabs(un), sqrt_f64(c2)), (double)(1ll << fx::S_VEL)));
 }
 
-// The face flux over half the divergence factor (.57), or false where a
-// state leaves the range: F = f(q_L) + f(q_R) + lambda (q_L - q_R) - V,
-// lambda the largest |u_n| + a over the left, right and Roe-averaged states.
-// V: the viscous (or interface) part of the momenta and the energy.
+// The flux of the tangential momentum in double, from the four cells across
+// the face (L1, R1 those at it) or a boundary face's one state. Unlike the
+// other components it has no term of the size of density or pressure, so its
+// rounding has to follow the momenta themselves, however small. f(q_L) +
+// f(q_R) + lambda (q_L - q_R) regrouped as L (u_L + u_R) + (L - R) (lambda -
+// u_R), whose velocity sums are exact integers.
+struct FxTan {
+  double us, lr;  // u_nL + u_nR, lambda - u_nR
+};
+__device__ __forceinline__ double tan_flux(const FxTan& t, double L, double R, double V) {
+  return __fma_rn(__dsub_rn(L, R), t.lr, __fma_rn(L, t.us, -V));
+}
+__device__ __forceinline__ double tan_flux(const FxTan& t, double L2, double L1, double R1, double R2, double V) {
+  return tan_flux(t, __fma_rn(0.25, __dsub_rn(R1, L2), L1), __fma_rn(0.25, __dsub_rn(L1, R2), R1), V);
+}
+
+// The fluxes of mass, normal momentum and energy over half the divergence
+// factor (.57), or false where a state leaves the range: F = f(q_L) + f(q_R) +
+// lambda (q_L - q_R) - V, lambda the largest |u_n| + a over the left, right
+// and Roe-averaged states. Vn, VE: the viscous (or interface) part of the
+// normal momentum and the energy. t: the factors of the tangential momenta.
 template <int ND>
 __device__ __forceinline__ bool fx_flux(const Geom& g, const FxConst& k, const i64 L[ND + 2], const i64 R[ND + 2],
-                                        const i64 V[ND + 1], i64 F[ND + 2]) {
+                                        i64 Vn, i64 VE, i64 F[3], FxTan* t) {
   constexpr int E = ND + 1;
   FxSide<ND> l, r;
   fx_side<ND>(k, L, &l);
@@ -108,16 +125,15 @@ __device__ __forceinline__ bool fx_flux(const Geom& g, const FxConst& k, const i
   }
   const FxW lam59 = fx::split(lam), lam61 = fx::split(lam << 2);
   F[0] = (L[1] >> 5) + (R[1] >> 5) + fx::mul(fx::split(L[0] - R[0]), lam61);
-  F[1] = (l.mu + l.p) + (r.mu + r.p) + fx::mul(fx::split(L[1] - R[1]), lam59) - V[0];
-#pragma unroll
-  for (int t = 0; t < ND - 1; t++)
-    F[2 + t] = fx::mul2(l.mt[t], l.un, r.mt[t], r.un) + fx::mul(fx::split(L[2 + t] - R[2 + t]), lam59) - V[1 + t];
-  F[E] = fx::mul(fx::split(l.eh), fx::split(l.un_ << 3)) + fx::mul(fx::split(r.eh), fx::split(r.un_ << 3)) +
-         fx::mul(fx::split(L[E] - R[E]), lam61) - V[ND];
+  F[1] = (l.mu + l.p) + (r.mu + r.p) + fx::mul(fx::split(L[1] - R[1]), lam59) - Vn;
+  F[2] = fx::mul(fx::split(l.eh), fx::split(l.un_ << 3)) + fx::mul(fx::split(r.eh), fx::split(r.un_ << 3)) +
+         fx::mul(fx::split(L[E] - R[E]), lam61) - VE;
+  t->us = __longlong_as_double(fx::to_double(l.un_ + r.un_, fx::S_VEL));
+  t->lr = __longlong_as_double(fx::to_double(lam - r.un_, fx::S_VEL));
   // room for the sums of the divergence: |F| < 8
   int top = 0;
 #pragma unroll
-  for (int c = 0; c < ND + 2; c++) {
+  for (int c = 0; c < 3; c++) {
     const int h = (int)(F[c] >> 32);
     top |= h ^ (h >> 31);
   }

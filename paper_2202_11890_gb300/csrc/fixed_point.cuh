@@ -7,7 +7,8 @@
 // one, and a 64 x 64-bit product taken to its upper half about four. The
 // face fluxes of the FP64 tile run here: states, speeds and fluxes of a
 // nondimensional flow (density, sound speed and pressure near one) as 64-bit
-// integers in units of 2^-57 to 2^-62. Their rounding errors are below 2^-56
+// integers in units of 2^-57 to 2^-62, except the flux of the tangential
+// momentum (fixed_flux.cuh). Their rounding errors are below 2^-56
 // absolute, an eighth of the rounding of a double near one; a face whose
 // states leave the representable range is evaluated in double instead
 // (stage_tile.cuh).
@@ -147,6 +148,22 @@ __host__ __device__ __forceinline__ i64 sqroot(i64 x) {
   const int e50 = (int)(e >> 7);
   const i64 g = (e << 6) + ((3 * mulhi32(e50, e50)) >> 7);  // (e/2 + 3 e^2 / 8).64
   return t + mul(split(t), split(g));
+}
+
+// x.s as a double, rounded to nearest (halves away from zero): the mantissa
+// shifted to bit 62, whose leading one raises the exponent field by one, as
+// does a carry of the rounding. On the integer pipes: a conversion
+// instruction runs at the double pipe's rate.
+__host__ __device__ __forceinline__ i64 to_double(i64 x, int s) {
+  const u64 a = x < 0 ? 0ull - (u64)x : (u64)x;
+  if (a == 0) return 0;
+#ifdef __CUDA_ARCH__
+  const int z = __clzll((i64)a);
+#else
+  const int z = __builtin_clzll(a);
+#endif
+  const u64 m = ((a << z >> 10) + 1) >> 1;
+  return (i64)(((u64)(1085 - s - z) << 52) + m) | (x & (i64)(1ull << 63));
 }
 
 // A double of a cell state within the bounds above, as an integer of scale

@@ -76,10 +76,13 @@ struct FxConst {
   int on;              // every factor below fits its scale: the fluxes run in fixed point
   int square;          // dx = dz1 = dz2: x and z differences add before the scaling
   double scale;        // their factor: 2^-57 of half of 1/dx
+  double scale_z[2];   // 2^-57 of half of 1/dz per fluid
   FxW gm1;             // (gamma - 1).61
   FxW gg;              // gamma (gamma - 1).62
   FxW lid[LID_N];      // interface, .62
   FxW fc[2][2][FXC_N]; // viscous coefficients per direction (x, z) and fluid, .62
+  double tc[2][2][2];  // of them C and D in double, for the tangential momentum
+  double tlid[LID_N];  // the interface's factors in double, LID_1 and LID_2 doubled
 };
 
 // The same of the 3-D tiles: directions x (tangents y, z), y (x, z) and z
@@ -95,9 +98,10 @@ enum {
   F3_N
 };
 struct Fx3Const {
-  FxConst k;  // its fc unused; square: dx = dy = dz1 = dz2
+  FxConst k;  // its fc and tc unused; square: dx = dy = dz1 = dz2
   FxW fc[3][2][F3_N];
   double fd[3][2][F3_N];
+  double scale_y;  // 2^-57 of half of 1/dy
 };
 
 // Physics and grid of one instance, constant over its life.

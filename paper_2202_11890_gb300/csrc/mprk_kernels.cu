@@ -79,24 +79,23 @@ __global__ void __launch_bounds__(NTHREADS, 3)
   yface_tile(a, C, a.row0 + blockIdx.y * TZ, blockIdx.x * TX, blockIdx.z, *reinterpret_cast<YfaceSmem*>(smem_raw));
 }
 
-__global__ void __launch_bounds__(TILE3_THREADS, 3)
+__global__ void __launch_bounds__(TILE3_THREADS, 2)
     stage3_kernel(const __grid_constant__ StageArgs a, const __grid_constant__ Fx3Const C) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   chain_next();
   chain_wait();
-  stage_tile3(a, C, a.row0 + blockIdx.y * TZ, blockIdx.x * TX, blockIdx.z, *reinterpret_cast<Tile3Smem*>(smem_raw));
+  stage_tile3(a, C, a.row0 + blockIdx.y * TZ3, blockIdx.x * TX, blockIdx.z, *reinterpret_cast<Tile3Smem*>(smem_raw));
 }
 
 cudaError_t launch_stage3(const StageArgs& a, cudaStream_t stream, bool chained) {
   const int hi = a.rhs_only ? a.rhs_hi : a.g.nz;
-  const int tz = (hi - a.row0 + TZ - 1) / TZ;
-  if (tz <= 0) return cudaSuccess;
-  const dim3 grid(a.tiles_x, tz, a.g.ny);
+  const int rows = hi - a.row0;
+  if (rows <= 0) return cudaSuccess;
   Fx3Const C;
   fixed_point_const3(a.g, &C);
-  cudaError_t e = launch_kernel(yface3_kernel, grid, NTHREADS, sizeof(YfaceSmem), stream, chained, a, C);
+  cudaError_t e = launch_kernel(yface3_kernel, dim3(a.tiles_x, (rows + TZ - 1) / TZ, a.g.ny), NTHREADS, sizeof(YfaceSmem), stream, chained, a, C);
   if (e != cudaSuccess) return e;
-  return launch_kernel(stage3_kernel, grid, TILE3_THREADS, sizeof(Tile3Smem), stream, true, a, C);
+  return launch_kernel(stage3_kernel, dim3(a.tiles_x, (rows + TZ3 - 1) / TZ3, a.g.ny), TILE3_THREADS, sizeof(Tile3Smem), stream, true, a, C);
 }
 
 size_t stage_smem_bytes(int precision) {

@@ -319,16 +319,20 @@ static FxW fx_factor(double x, int digits) {
 static bool fx_gas(const Geom& g, FxConst* out) {
   *out = FxConst{};
   out->scale = ldexp(0.5 * g.inv_dx, -57);
+  out->scale_z[0] = ldexp(0.5 * g.inv_dz1, -57);
+  out->scale_z[1] = ldexp(0.5 * g.inv_dz2, -57);
   const double gg = g.gamma * g.gm1;
-  if (!(gg < 1.9)) return false;
-  out->gm1 = fx_factor(g.gm1, 61);
-  out->gg = fx_factor(gg, 62);
+  bool ok = gg < 1.9;
   for (int j = 0; j < LID_N; j++) {
     // harmonic means of the fluids' coefficients below: under 1 with them
     const double x = lid_coef(g, j);
-    if (!(x < 1.0)) return false;
-    out->lid[j] = fx_factor(x, 62);
+    out->tlid[j] = j == LID_1 || j == LID_2 ? 2.0 * x : x;
+    ok = ok && x < 1.0;  // false for NaN
+    if (ok) out->lid[j] = fx_factor(x, 62);
   }
+  if (!ok) return false;
+  out->gm1 = fx_factor(g.gm1, 61);
+  out->gg = fx_factor(gg, 62);
   return true;
 }
 
@@ -346,6 +350,7 @@ void mprk::fixed_point_const(const Geom& g, FxConst* out) {
         const double x = visc_coef(g, dir, fl, j);
         ok = ok && std::fabs(x) < 1.0;  // false for NaN
         if (ok) f.fc[dir][fl][j] = fx_factor(x, 62);
+        if (j == FXC_C || j == FXC_D) f.tc[dir][fl][j - FXC_C] = x;
       }
   f.on = ok;
 }
@@ -353,6 +358,7 @@ void mprk::fixed_point_const(const Geom& g, FxConst* out) {
 void mprk::fixed_point_const3(const Geom& g, Fx3Const* out) {
   Fx3Const& f = *out;
   bool ok = fx_gas(g, &f.k);
+  f.scale_y = ldexp(0.5 * g.inv_dy, -57);
   f.k.square = g.inv_dx == g.inv_dy && g.inv_dx == g.inv_dz1 && g.inv_dx == g.inv_dz2;
   for (int dir = 0; dir < 3; dir++)
     for (int fl = 0; fl < 2; fl++) {

@@ -19,18 +19,18 @@
 // tangential differences and the interface state, and faces dealt to threads
 // in three uneven rounds, the step below took 2.39 ms).
 //
-// Velocities, differences and fluxes run in 64-bit fixed point (fixed_point.cuh): as double
-// arithmetic they were 300 of the tile's 309 operations per cell on a pipe
-// that completes two per clock and SM, which bound every FP64 launch: the
-// pipe was 86 % busy. Measured: a slow step of 2048 x 1024 cells with m = 8
-// 11.7 -> 2.06 ms (B and F rows of one stage 649 -> 114 us), 64 x 64
-// with m = 4 167 -> 55 us; 2300 instructions per cell, 57 % of
-// the integer pipe and 60 % of the issue slots busy. Errors of the right-hand side against 80-bit
-// arithmetic fell from 3e-16..1e-15 to 2e-17..5e-16 (rms per component; rest
-// state with 1 % bumps to 25 % cell noise). A face
-// with a state outside the fixed-point range takes the same formulas in
-// double (slow_faces); which form a face takes depends on its own cells
-// alone, so results do not depend on the tile shape or the launch.
+// The fluxes of mass, normal momentum and energy run in 64-bit fixed point
+// (fixed_point.cuh): as double arithmetic the faces were 300 of the tile's 309
+// operations per cell on a pipe that completes two per clock and SM, which
+// bound every FP64 launch: the pipe was 86 % busy. The flux of the tangential
+// momentum stays in double, because nothing in it is as large as density or
+// pressure: in fixed point a shear of 1e-6 in a flow uniform along x had 3e4
+// times the double form's error. Measured: a slow step of 2048 x 1024 cells
+// with m = 8 11.7 -> 2.84 ms (2.06 with that flux in fixed point too), 64 x 64
+// with m = 4 167 -> 62 us (55). A face with a state outside the fixed-point
+// range takes the same formulas in double (slow_faces); which form a face
+// takes depends on its own cells alone, so results do not depend on the tile
+// shape or the launch.
 #pragma once
 
 #include "fixed_flux.cuh"
@@ -44,8 +44,9 @@ struct TileSmem {
   double q[4][TZR + 4][TX + 4];  // stage state, rows k0-2.., cols i0-2..
   i64 qi[4][TZR + 4][TX + 4];    // the same: rho, rho E .58, momenta .60
   i64 v[3][TZR + 2][TX + 2];     // u, w, e (.59), rows k0-1.., cols i0-1..
-  // face fluxes over half the divergence factor (.57; a slow face's as the
-  // bits of a double)
+  double vd[2][TZR + 2][TX + 2];  // u, w
+  // face fluxes over half the divergence factor (.57; the tangential momentum
+  // and every component of a slow face as the bits of a double)
   i64 fx[4][TZR][TX + 1];  // face f between cols f-1, f
   i64 fz[4][TZR + 1][TX];  // seen from above at the interface
   i64 fg[4][TX];           // the interface seen from fluid 1 (below)
@@ -187,14 +188,16 @@ struct Arith<i64> {
   static __device__ __forceinline__ const i64* q(const TileSmem<TZR>& S) { return &S.qi[0][0][0]; }
   // q + (upper - lower neighbour) / 4
   static __device__ __forceinline__ i64 rec(i64 a, i64 up, i64 dn) { return (a << 2) + (up - dn); }
-  // u, w, e of a cell
-  static __device__ __forceinline__ void prims(i64 r, i64 mu, i64 mw, i64 E, i64 out[3]) {
-    const FxW inv = fx::split(fx::recip(r << 2));
+  // u, w, e of a cell; 1/rho .61
+  static __device__ __forceinline__ i64 prims(i64 r, i64 mu, i64 mw, i64 E, i64 out[3]) {
+    const i64 inv_ = fx::recip(r << 2);
+    const FxW inv = fx::split(inv_);
     const FxW m1 = fx::split(mu << 2), m2 = fx::split(mw << 2);
     out[0] = fx::mul(m1, inv);
     out[1] = fx::mul(m2, inv);
     const i64 k = fx::mul(m1, fx::split(out[0])) + fx::mul(m2, fx::split(out[1]));  // .57; k/2 is .58
     out[2] = fx::mul(fx::split((E - k) << 2), inv) << 2;
+    return inv_;
   }
 };
 template <>
@@ -203,50 +206,63 @@ struct Arith<double> {
   static __device__ __forceinline__ const double* q(const TileSmem<TZR>& S) { return &S.q[0][0][0]; }
   static __device__ __forceinline__ double rec(double a, double up, double dn) { return __fma_rn(0.25, __dsub_rn(up, dn), a);
   }
-  static __device__ __forceinline__ void prims(double r, double mu, double mw, double E, double out[3]) {
+  static __device__ __forceinline__ double prims(double r, double mu, double mw, double E, double out[3]) {
     const double inv = recip_f64(r);
     out[0] = __dmul_rn(mu, inv);
     out[1] = __dmul_rn(mw, inv);
     out[2] = __dmul_rn(__fma_rn(-0.5, __fma_rn(mw, out[1], __dmul_rn(mu, out[0])), E), inv);
+    return inv;
   }
 };
 
-// u, w, e of the cell of halo row rr, column cc into the ring (phase 1).
+// u, w, e of the cell of halo row rr, column cc into the ring (phase 1); in
+// fixed point also u and w in double (q: the state).
 template <typename T, int TZR>
-__device__ __forceinline__ void ring_cell(const Geom& g, TileSmem<TZR>& S, int rr, int cc, int i0, T r, T mu, T mw, T E) {
+__device__ __forceinline__ void ring_cell(const Geom& g, TileSmem<TZR>& S, int rr, int cc, int i0, T r, T mu, T mw, T E,
+                                          const double* q = nullptr) {
   constexpr int VP = (TZR + 2) * (TX + 2);
   if (rr < 1 || rr > TZR + 2 || cc < 1 || cc > TX + 2) return;
   T* v = reinterpret_cast<T*>(&S.v[0][0][0]) + (rr - 1) * (TX + 2) + cc - 1;
   T o[3];
-  Arith<T>::prims(r, mu, mw, E, o);
-  v[0] = o[0];
+  const T inv = Arith<T>::prims(r, mu, mw, E, o);
   // the mirror state's u is already flipped; a no-slip x wall flips w too
-  v[VP] = (x_ghost(i0 - 2 + cc, g.nx, g.xwall) && g.wall == 0) ? -o[1] : o[1];
+  const bool flip = x_ghost(i0 - 2 + cc, g.nx, g.xwall) && g.wall == 0;
+  v[0] = o[0];
+  v[VP] = flip ? -o[1] : o[1];
   v[2 * VP] = o[2];
+  if (q) {
+    const double id = __longlong_as_double(fx::to_double((i64)inv, 61)), w = __dmul_rn(q[2], id);
+    S.vd[0][rr - 1][cc - 1] = __dmul_rn(q[1], id);
+    S.vd[1][rr - 1][cc - 1] = flip ? -w : w;
+  }
 }
 
 // Interface (App. B, Eq. bulk-flux and the wall states after it), from the
 // velocities and e of the two cells touching it: the ghost velocity 2 u_w - u
-// of the cell `own` in fluid f + 1, and twice (sigma, u_w sigma - Pi), the
-// flux both fluids share. In double from the state, by 34 threads of the tile
+// of the cell `own` in fluid f + 1, and twice u_w sigma and -Pi, which with
+// twice sigma make the flux both fluids share. In double from the state, by 34 threads of the tile
 // before its faces, these took the launch of 64 x 64 cells a quarter of its
 // time: a warp's double operation occupies its scheduler for 64 clocks.
 __device__ __forceinline__ i64 lid_ghost(const Geom&, const FxConst& k, int f, i64 own, i64 other) {
   return own + (fx::mul(fx::split((other - own) << 2), k.lid[LID_1 + f]) << 1);
 }
-__device__ __forceinline__ double lid_ghost(const Geom& g, const FxConst&, int f, double own, double other) {
-  return __fma_rn(__dmul_rn(2.0, lid_coef(g, LID_1 + f)), __dsub_rn(other, own), own);
+__device__ __forceinline__ double lid_ghost(const Geom&, const FxConst& k, int f, double own, double other) {
+  return __fma_rn(k.tlid[LID_1 + f], __dsub_rn(other, own), own);
 }
-__device__ __forceinline__ void lid_flux(const Geom&, const FxConst& k, i64 u1, i64 u2, i64 e1, i64 e2, i64 V[2]) {
-  const i64 du = u2 - u1, uw = u1 + fx::mul(fx::split(du << 2), k.lid[LID_1]);
-  V[0] = fx::mul(fx::split(du), k.lid[LID_S]);                                        // .57
-  V[1] = (fx::mul(fx::split(uw << 3), fx::split(V[0])) << 2) + fx::mul(fx::split(e2 - e1), k.lid[LID_T]);
+// The energy's part of one wall velocity component (sig: its sigma .59); the
+// heat flux.
+__device__ __forceinline__ i64 lid_work(const FxConst& k, i64 u1, i64 u2, i64 sig) {
+  const i64 uw = u1 + fx::mul(fx::split((u2 - u1) << 2), k.lid[LID_1]);
+  return fx::mul(fx::split(uw << 3), fx::split(sig));
 }
-__device__ __forceinline__ void lid_flux(const Geom& g, const FxConst&, double u1, double u2, double e1, double e2,
-                                         double V[2]) {
-  const double du = __dsub_rn(u2, u1), uw = __fma_rn(lid_coef(g, LID_1), du, u1);
-  V[0] = __dmul_rn(lid_coef(g, LID_S), du);
-  V[1] = __fma_rn(uw, V[0], __dmul_rn(lid_coef(g, LID_T), __dsub_rn(e2, e1)));
+__device__ __forceinline__ i64 lid_heat(const FxConst& k, i64 e1, i64 e2) {
+  return fx::mul(fx::split(e2 - e1), k.lid[LID_T]);
+}
+__device__ __forceinline__ double lid_work(const FxConst& k, double u1, double u2, double sig) {
+  return __dmul_rn(__fma_rn(__dmul_rn(0.5, k.tlid[LID_1]), __dsub_rn(u2, u1), u1), sig);
+}
+__device__ __forceinline__ double lid_heat(const FxConst& k, double e1, double e2) {
+  return __dmul_rn(k.tlid[LID_T], __dsub_rn(e2, e1));
 }
 
 // ---- phase 2: face fluxes ---------------------------------------------------
@@ -293,12 +309,12 @@ __device__ __forceinline__ bool face_id(const Geom& g, int job, int lane, int k0
 // reconstructed from the four cells across it, and the two cells' velocities,
 // e and tangential differences (un, ut, e, gn, gt). A boundary face (outer
 // wall or interface) has the inner cell's state on one side and its mirror
-// on the other; an outer wall's viscous ghost is 2 wall state - cell, and the
-// interface has its own viscous flux VI (sigma, energy). Returns the fluid of
-// the face's coefficients, 2 at the interface.
+// on the other; an outer wall's viscous ghost is 2 wall state - cell, and at
+// the interface only (ut, e) are set. Returns the fluid of the face's
+// coefficients, 2 at the interface.
 template <typename T, int TZR>
 __device__ __forceinline__ int face_sides(const Geom& g, const FxConst& fk, const TileSmem<TZR>& S, const FaceId& id,
-                                          T L[4], T R[4], T vL[5], T vR[5], T VI[2]) {
+                                          T L[4], T R[4], T vL[5], T vR[5]) {
   constexpr int QP = (TZR + 4) * (TX + 4), VP = (TZR + 2) * (TX + 2);
   const int n1 = g.n1, nz = g.nz, ku = id.ku, kd = ku - 1;
   // first of the four cells, their stride, and the planes of m_n, m_t
@@ -342,7 +358,10 @@ __device__ __forceinline__ int face_sides(const Geom& g, const FxConst& fk, cons
   const T* v = reinterpret_cast<const T*>(&S.v[0][0][0]);
   if (lid) {
     const T* p = v + id.f * (TX + 2) + id.c + 1;
-    lid_flux(g, fk, p[0], p[TX + 2], p[2 * VP], p[2 * VP + TX + 2], VI);
+    vL[1] = p[0];
+    vR[1] = p[TX + 2];
+    vL[2] = p[2 * VP];
+    vR[2] = p[2 * VP + TX + 2];
     return 2;
   }
   if (id.isx) {
@@ -445,21 +464,18 @@ __device__ __forceinline__ void face_sides_plain(const TileSmem<TZR>& S, const F
     o[0] = p[vn];
     o[1] = p[vu];
     o[2] = p[2 * VP];
-    o[3] = p[vn + vt] - p[vn - vt];
     o[4] = p[vu + vt] - p[vu - vt];
   }
 }
 
-// The viscous flux over half the divergence factor from the common values of
-// App. B: (sigma_nn, sigma_nt, u . sigma_n + kappa dT/dn), .57.
-__device__ __forceinline__ void fx_visc(const FxW* fc, const i64 vL[5], const i64 vR[5], i64 V[3]) {
-  const FxW du = fx::split(vR[0] - vL[0]), dt = fx::split(vR[1] - vL[1]);
-  V[0] = fx::mul2(fc[FXC_A], du, fc[FXC_B], fx::split(vL[4] + vR[4]));
-  V[1] = fx::mul2(fc[FXC_C], dt, fc[FXC_D], fx::split(vL[3] + vR[3]));
-  // (u_L + u_R) / 2 . sigma: .61 x .57 -> .54, half of it at .55
-  const i64 us = fx::mul2(fx::split((vL[0] + vR[0]) << 2), fx::split(V[0]), fx::split((vL[1] + vR[1]) << 2),
-                          fx::split(V[1]));
-  V[2] = (us << 2) + fx::mul(fc[FXC_K], fx::split(vR[2] - vL[2]));
+// The viscous flux of the normal momentum and the energy over half the
+// divergence factor from the common values of App. B: sigma_nn and u .
+// sigma_n + kappa dT/dn, .57; snt: sigma_nt .59.
+__device__ __forceinline__ void fx_visc(const FxW* fc, const i64 vL[5], const i64 vR[5], i64 snt, i64* Vn, i64* VE) {
+  *Vn = fx::mul2(fc[FXC_A], fx::split(vR[0] - vL[0]), fc[FXC_B], fx::split(vL[4] + vR[4]));
+  // (u_L + u_R) . sigma: .61 x .59 -> .56, half of it at .57
+  *VE = fx::mul2(fx::split((vL[0] + vR[0]) << 2), fx::split(*Vn << 2), fx::split((vL[1] + vR[1]) << 2), fx::split(snt)) +
+        fx::mul(fc[FXC_K], fx::split(vR[2] - vL[2]));
 }
 
 // The same flux in double.
@@ -474,7 +490,74 @@ __device__ __forceinline__ void double_visc(const double* fc, const double vL[5]
   V[2] = __fma_rn(0.5, us, __dmul_rn(fc[FXC_K], __dsub_rn(vR[2], vL[2])));
 }
 
-// Fluxes to shared memory, back in (rho, rho u, rho w, rho E) order.
+// The tangential viscous flux sigma_nt over half the divergence factor, in
+// double, of face id in fluid fl (2: the interface), with the ghosts of
+// face_sides; and the flux of the tangential momentum (tan_flux) from it.
+template <int TZR>
+__device__ __forceinline__ double visc_tan(const Geom& g, const FxConst& fk, const TileSmem<TZR>& S, const FaceId& id,
+                                           int fl) {
+  constexpr int VS = TX + 2;
+  const int ku = id.ku;
+  const double* u = &S.vd[0][id.isx ? id.f + 1 : id.f][id.isx ? id.c : id.c + 1];
+  const double* w = u + (TZR + 2) * VS;
+  if (id.isx) {
+    const bool top = ku + 1 == g.nz || ku + 1 == g.n1, bot = ku == 0 || ku == g.n1;
+    double gn = 0.0;
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+      const double c = u[s];
+      double up = u[s + VS], dn = u[s - VS];
+      if (top) up = ku + 1 == g.nz ? (g.wall ? c : -c) : lid_ghost(g, fk, 0, c, up);
+      if (bot) dn = ku == 0 ? (g.wall ? c : -c) : lid_ghost(g, fk, 1, c, dn);
+      gn = s ? __dadd_rn(gn, __dsub_rn(up, dn)) : __dsub_rn(up, dn);
+    }
+    return __fma_rn(fk.tc[0][fl][0], __dsub_rn(w[1], w[0]), __dmul_rn(fk.tc[0][fl][1], gn));
+  }
+  if (fl == 2) return __dmul_rn(fk.tlid[LID_S], __dsub_rn(u[VS], u[0]));
+  if (ku == 0 || ku == g.nz)  // the ghost's u is +-u and its difference of w the opposite
+    return g.wall ? 0.0 : __dmul_rn(fk.tc[1][fl][0], ku == 0 ? __dmul_rn(2.0, u[VS]) : __dmul_rn(-2.0, u[0]));
+  return __fma_rn(fk.tc[1][fl][0], __dsub_rn(u[VS], u[0]),
+                  __dmul_rn(fk.tc[1][fl][1], __dadd_rn(__dsub_rn(w[1], w[-1]), __dsub_rn(w[VS + 1], w[VS - 1]))));
+}
+template <int TZR>
+__device__ __forceinline__ double face_tan(const Geom& g, const TileSmem<TZR>& S, const FaceId& id, const FxTan& t,
+                                           double V) {
+  constexpr int QS = TX + 4;
+  const int n1 = g.n1, nz = g.nz, ku = id.ku;
+  if (id.isx) {
+    const double* q = &S.q[2][id.f + 2][id.c];
+    return tan_flux(t, q[0], q[1], q[2], q[3], V);
+  }
+  const double* q = &S.q[1][id.f][id.c + 2];
+  const bool edge = ku == 0 || ku == nz || ku == n1, from_above = ku == 0 || (ku == n1 && !id.below);
+  double a0 = q[0], a1 = q[QS], a2 = q[2 * QS], a3 = q[3 * QS];
+  if (edge) {
+    if (from_above) a1 = a2;
+    else a2 = a1;
+  }
+  if (ku == 1 || ku == n1 + 1) a0 = a1;
+  if (ku == nz - 1 || ku == n1 - 1) a3 = a2;
+  if (!edge) return tan_flux(t, a0, a1, a2, a3, V);
+  const double m = from_above ? __fma_rn(0.25, __dsub_rn(a1, a3), a2) : __fma_rn(0.25, __dsub_rn(a2, a0), a1);
+  return tan_flux(t, m, m, V);
+}
+template <bool X, int TZR>
+__device__ __forceinline__ double visc_tan_plain(const FxConst& fk, const TileSmem<TZR>& S, const FaceId& id, int fl) {
+  constexpr int vs = X ? 1 : TX + 2, vt = X ? TX + 2 : 1;
+  const double* un = &S.vd[X ? 0 : 1][X ? id.f + 1 : id.f][X ? id.c : id.c + 1];
+  const double* ut = &S.vd[X ? 1 : 0][X ? id.f + 1 : id.f][X ? id.c : id.c + 1];
+  const double gn = __dadd_rn(__dsub_rn(un[vt], un[-vt]), __dsub_rn(un[vs + vt], un[vs - vt]));
+  return __fma_rn(fk.tc[X ? 0 : 1][fl][0], __dsub_rn(ut[vs], ut[0]), __dmul_rn(fk.tc[X ? 0 : 1][fl][1], gn));
+}
+template <bool X, int TZR>
+__device__ __forceinline__ double face_tan_plain(const TileSmem<TZR>& S, const FaceId& id, const FxTan& t, double V) {
+  constexpr int qs = X ? 1 : TX + 4;
+  const double* q = &S.q[X ? 2 : 1][X ? id.f + 2 : id.f][X ? id.c : id.c + 2];
+  return tan_flux(t, q[0], q[qs], q[2 * qs], q[3 * qs], V);
+}
+
+// Fluxes (mass, normal and tangential momentum, energy) to shared memory, back
+// in (rho, rho u, rho w, rho E) order.
 template <int TZR>
 __device__ __forceinline__ void store_flux(TileSmem<TZR>& S, const FaceId& id, const i64 F[4]) {
   i64* p;
@@ -533,10 +616,13 @@ __device__ __noinline__ void slow_faces(const Geom& g, const FxConst& fk, TileSm
     if (!face_id<TZR>(g, job, lane, k0, row_hi, &id) || !(all || S.slow[e])) continue;
     if (all) S.slow[e] = 1;
     double L[4], R[4], vL[5], vR[5], V[3], F[4];
-    V[0] = 0.0;
-    const int fl = face_sides<double, TZR>(g, fk, S, id, L, R, vL, vR, V + 1);
+    const int fl = face_sides<double, TZR>(g, fk, S, id, L, R, vL, vR);
     if (fl < 2) {
       double_visc(S.fc[id.isx ? 0 : 1][fl], vL, vR, V);
+    } else {
+      V[0] = 0.0;
+      V[1] = __dmul_rn(fk.tlid[LID_S], __dsub_rn(vR[1], vL[1]));
+      V[2] = __dadd_rn(lid_work(fk, vL[1], vR[1], V[1]), lid_heat(fk, vL[2], vR[2]));
     }
     double_flux(g, L, R, V, F);
     i64 o[4];
@@ -625,7 +711,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
                               : fx::from_positive(__double_as_longlong(val[c]), fx::S_RHO - 2);
       S.qi[c][rr][cc] = t[c];
     }
-    ring_cell<i64, TZR>(g, S, rr, cc, i0, t[0], t[1], t[2], t[3]);
+    ring_cell<i64, TZR>(g, S, rr, cc, i0, t[0], t[1], t[2], t[3], val);
   }
   const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZR);
   bad = __syncthreads_or(bad);
@@ -640,26 +726,41 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
   const bool plain = !bad && tile_plain<TZR>(g, k0, row_hi);
   for (int job = warp; job < jobs; job += NT / 32) {
     FaceId id;
-    i64 L[4], R[4], vL[5], vR[5], V[3], F[4];
-    V[0] = 0;
+    i64 L[4], R[4], vL[5], vR[5], Vn = 0, VE, F[4];
     int fl;
     bool ok = true;
+    double Vt;
     if (plain) {
       if (!face_id_plain<TZR>(job, lane, k0, &id)) continue;
-      if (id.isx) face_sides_plain<true, TZR>(S, id, L, R, vL, vR);
-      else face_sides_plain<false, TZR>(S, id, L, R, vL, vR);
       fl = k0 >= n1;
+      if (id.isx) {
+        face_sides_plain<true, TZR>(S, id, L, R, vL, vR);
+        Vt = visc_tan_plain<true, TZR>(a.fx, S, id, fl);
+      } else {
+        face_sides_plain<false, TZR>(S, id, L, R, vL, vR);
+        Vt = visc_tan_plain<false, TZR>(a.fx, S, id, fl);
+      }
     } else {
       if (!face_id<TZR>(g, job, lane, k0, row_hi, &id)) continue;
       ok = !bad || face_in_range<TZR>(g, S, id, k0);
-      if (ok) fl = face_sides<i64, TZR>(g, a.fx, S, id, L, R, vL, vR, V + 1);
+      if (ok) {
+        fl = face_sides<i64, TZR>(g, a.fx, S, id, L, R, vL, vR);
+        Vt = visc_tan<TZR>(g, a.fx, S, id, fl);
+      }
     }
     if (ok) {
-      if (fl < 2) {
-        fx_visc(a.fx.fc[id.isx ? 0 : 1][fl], vL, vR, V);
+      const i64 snt = fx::from_double(__double_as_longlong(Vt), fx::S_VEL);
+      if (fl < 2) fx_visc(a.fx.fc[id.isx ? 0 : 1][fl], vL, vR, snt, &Vn, &VE);
+      else VE = lid_work(a.fx, vL[1], vR[1], snt) + lid_heat(a.fx, vL[2], vR[2]);
+      FxTan t;
+      ok = fx_flux<2>(g, a.fx, L, R, Vn, VE, F, &t);
+      if (ok) {
+        F[3] = F[2];
+        F[2] = __double_as_longlong(!plain    ? face_tan<TZR>(g, S, id, t, Vt)
+                                    : id.isx ? face_tan_plain<true, TZR>(S, id, t, Vt)
+                                             : face_tan_plain<false, TZR>(S, id, t, Vt));
+        store_flux(S, id, F);
       }
-      ok = fx_flux<2>(g, a.fx, L, R, V, F);
-      if (ok) store_flux(S, id, F);
     }
     S.slow[job * TX + lane] = !ok;
     slow |= !ok;
@@ -697,18 +798,23 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
 #pragma unroll
       for (int c = 0; c < 4; c++) {
         auto val = [&](i64 f, bool sl) { return sl ? __longlong_as_double(f) : __dmul_rn((double)f, s57); };
-        const double dx = __dsub_rn(val(S.fx[c][rr][cc], s0), val(S.fx[c][rr][cc + 1], s1));
-        const double dz = __dsub_rn(val(S.fz[c][rr][cc], s2),
-                                    val(under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc], s3));
+        const bool tx = c == 2, tz = c == 1;  // the tangential momentum of x and z faces
+        const double dx = __dsub_rn(val(S.fx[c][rr][cc], s0 || tx), val(S.fx[c][rr][cc + 1], s1 || tx));
+        const double dz = __dsub_rn(val(S.fz[c][rr][cc], s2 || tz),
+                                    val(under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc], s3 || tz));
         R[c] = __fma_rn(hx, dx, __dmul_rn(hz, dz));
       }
     } else {
+      const double sz = a.fx.scale_z[k >= n1];
 #pragma unroll
       for (int c = 0; c < 4; c++) {
-        const i64 dx = S.fx[c][rr][cc] - S.fx[c][rr][cc + 1];
-        const i64 dz = S.fz[c][rr][cc] - (under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc]);
-        R[c] = a.fx.square ? __dmul_rn(a.fx.scale, (double)(dx + dz))
-                           : __fma_rn(a.fx.scale, (double)dx, __dmul_rn(__dmul_rn(hz, s57), (double)dz));
+        const i64 x0 = S.fx[c][rr][cc], x1 = S.fx[c][rr][cc + 1];
+        const i64 z0 = S.fz[c][rr][cc], z1 = under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc];
+        auto diff = [&](i64 f, i64 h) { return __dsub_rn(__longlong_as_double(f), __longlong_as_double(h)); };
+        if (c == 1) R[c] = __fma_rn(a.fx.scale, (double)(x0 - x1), __dmul_rn(hz, diff(z0, z1)));
+        else if (c == 2) R[c] = __fma_rn(sz, (double)(z0 - z1), __dmul_rn(hx, diff(x0, x1)));
+        else if (a.fx.square) R[c] = __dmul_rn(a.fx.scale, (double)((x0 - x1) + (z0 - z1)));
+        else R[c] = __fma_rn(a.fx.scale, (double)(x0 - x1), __dmul_rn(sz, (double)(z0 - z1)));
       }
     }
     R[2] = __fma_rn(-g.G, S.q[0][rr + 2][cc + 2], R[2]);

@@ -15,10 +15,11 @@
 // derivatives averaged from the two cells' central differences, sigma =
 // mu (grad u + grad u^T - 2/3 div u I), heat flux -kappa grad T.
 //
-// As in the 2-D tile, velocities, differences and fluxes run in 64-bit fixed
-// point (fixed_point.cuh), because the double pipe bound both kernels (80 to
-// 86 % busy with 125 + 238 operations per cell). Measured: a slow step of
-// 512 x 64 x 200 cells with m = 4 44.1 -> 8.8 ms. A face whose own cells leave
+// As in the 2-D tile, the fluxes of mass, normal momentum and energy run in
+// 64-bit fixed point (fixed_point.cuh), because the double pipe bound both
+// kernels (80 to 86 % busy with 125 + 238 operations per cell), and those of
+// the tangential momenta in double. Measured: a slow step of 512 x 64 x 200
+// cells with m = 4 44.1 -> 14.9 ms. A face whose own cells leave
 // the range is evaluated in double by a second pass over the tile; which form
 // a face takes depends on its cells alone, so neighbouring tiles agree on the
 // faces they share. Fluxes come over half the divergence factor of their
@@ -69,7 +70,8 @@ __device__ __forceinline__ void lf_face5(const double l[5], const double r[5], d
 
 // One side of a face in its frame: velocity (u_n, u_t1, u_t2), e = T / (gamma
 // (gamma - 1)), and the cell's central differences (unscaled) of u_n and u_t1
-// along t1 (g1) and of u_n and u_t2 along t2 (g2).
+// along t1 (g1) and of u_n and u_t2 along t2 (g2). The fixed-point form uses
+// neither difference of u_n.
 template <typename T>
 struct VSide {
   T u[3], e, g1[2], g2[2];
@@ -131,13 +133,10 @@ struct Arith3<i64> {
     return fx::from_double(__double_as_longlong(q), c == 0 || c == 4 ? fx::S_RHO - 2 : fx::S_MOM - 2);
   }
   static __device__ __forceinline__ i64 rec(i64 a, i64 up, i64 dn) { return (a << 2) + (up - dn); }
-  static __device__ __forceinline__ void vel(const i64 q[4], i64 v[3]) {
-    const FxW inv = fx::split(fx::recip(q[0] << 2));
-#pragma unroll
-    for (int c = 0; c < 3; c++) v[c] = fx::mul(fx::split(q[c + 1] << 2), inv);
-  }
-  static __device__ __forceinline__ void prims(const i64 q[5], i64 v[4]) {
-    const FxW inv = fx::split(fx::recip(q[0] << 2));
+  // u, v, w, e of a cell; 1/rho in double
+  static __device__ __forceinline__ double prims(const i64 q[5], i64 v[4]) {
+    const i64 inv_ = fx::recip(q[0] << 2);
+    const FxW inv = fx::split(inv_);
     i64 k = 0;
 #pragma unroll
     for (int c = 0; c < 3; c++) {
@@ -146,6 +145,7 @@ struct Arith3<i64> {
       k += fx::mul(m, fx::split(v[c]));
     }
     v[3] = fx::mul(fx::split((q[4] - k) << 2), inv) << 2;  // k .57: k/2 .58
+    return __longlong_as_double(fx::to_double(inv_, 61));
   }
 };
 template <>
@@ -154,12 +154,7 @@ struct Arith3<double> {
   static __device__ __forceinline__ double rec(double a, double up, double dn) {
     return __fma_rn(0.25, __dsub_rn(up, dn), a);
   }
-  static __device__ __forceinline__ void vel(const double q[4], double v[3]) {
-    const double inv = recip_f64(q[0]);
-#pragma unroll
-    for (int c = 0; c < 3; c++) v[c] = __dmul_rn(q[c + 1], inv);
-  }
-  static __device__ __forceinline__ void prims(const double q[5], double v[4]) {
+  static __device__ __forceinline__ double prims(const double q[5], double v[4]) {
     const double inv = recip_f64(q[0]);
     double k = 0.0;
 #pragma unroll
@@ -168,13 +163,14 @@ struct Arith3<double> {
       k = __fma_rn(q[c + 1], v[c], k);
     }
     v[3] = __dmul_rn(__fma_rn(-0.5, k, q[4]), inv);
+    return inv;
   }
 };
 
-// A stored flux: the .57 integer itself (|F| < 8, so its top four bits agree)
-// or the bits of a double, whose top four bits differ for 2^-511 <= |F| <
-// 2^513. Smaller doubles store as zero, larger ones and NaN as the positive
-// NaN.
+// A stored flux of mass, normal momentum or energy: the .57 integer itself
+// (|F| < 8, so its top four bits agree) or the bits of a double, whose top
+// four bits differ for 2^-511 <= |F| < 2^513. Smaller doubles store as zero,
+// larger ones and NaN as the positive NaN. Tangential momenta are doubles.
 __device__ __forceinline__ bool flux_is_double(i64 f) {
   return (unsigned)((int)(f >> 32) + 0x10000000) >= 0x20000000u;
 }
@@ -209,17 +205,19 @@ __device__ __forceinline__ T dz_vel(const Geom& g, const FxConst& c, int k, int 
 // sigma_nt1, sigma_nt2, u^.sigma_n + kappa dT/dn). With G[a][b] = d u_a /
 // d x_b (b = normal, t1, t2): sigma_nn = mu (4/3 G00 - 2/3 (G11 + G22)),
 // sigma_nt = mu (G_t0 + G_0t); the derivative factors sit in the coefficients.
+// In fixed point only sigma_nn and the energy, from the other two as doubles.
 __device__ __forceinline__ void visc3(const Fx3Const& c, int dir, int fl, const VSide<i64>& L, const VSide<i64>& R,
-                                      i64 V[4]) {
+                                      const double s[2], i64* Vn, i64* VE) {
   const FxW* f = c.fc[dir][fl];
-  V[0] = fx::mul2(f[F3_A], fx::split(R.u[0] - L.u[0]), f[F3_B1], fx::split(L.g1[1] + R.g1[1])) +
-         fx::mul(fx::split(L.g2[1] + R.g2[1]), f[F3_B2]);
-  V[1] = fx::mul2(f[F3_C], fx::split(R.u[1] - L.u[1]), f[F3_D1], fx::split(L.g1[0] + R.g1[0]));
-  V[2] = fx::mul2(f[F3_C], fx::split(R.u[2] - L.u[2]), f[F3_D2], fx::split(L.g2[0] + R.g2[0]));
-  i64 us = 0;  // (u_L + u_R) . sigma .54
+  *Vn = fx::mul2(f[F3_A], fx::split(R.u[0] - L.u[0]), f[F3_B1], fx::split(L.g1[1] + R.g1[1])) +
+        fx::mul(fx::split(L.g2[1] + R.g2[1]), f[F3_B2]);
+  // (u_L + u_R) . sigma: .61 x .59 -> .56, half of it at .57
+  i64 us = fx::mul(fx::split((L.u[0] + R.u[0]) << 2), fx::split(*Vn << 2));
 #pragma unroll
-  for (int q = 0; q < 3; q++) us += fx::mul(fx::split((L.u[q] + R.u[q]) << 2), fx::split(V[q]));
-  V[3] = (us << 2) + fx::mul(fx::split(R.e - L.e), f[F3_K]);
+  for (int t = 0; t < 2; t++)
+    us += fx::mul(fx::split((L.u[1 + t] + R.u[1 + t]) << 2),
+                  fx::split(fx::from_double(__double_as_longlong(s[t]), fx::S_VEL)));
+  *VE = us + fx::mul(fx::split(R.e - L.e), f[F3_K]);
 }
 __device__ __forceinline__ void visc3(const Fx3Const& c, int dir, int fl, const VSide<double>& L,
                                       const VSide<double>& R, double V[4]) {
@@ -234,26 +232,23 @@ __device__ __forceinline__ void visc3(const Fx3Const& c, int dir, int fl, const 
   V[3] = __fma_rn(0.5, us, __dmul_rn(f[F3_K], __dsub_rn(R.e, L.e)));
 }
 
-// The face flux, as stored; false where it leaves the fixed-point range.
-__device__ __forceinline__ bool flux3(const Geom& g, const Fx3Const& c, const i64 L[5], const i64 R[5], const i64 V[4],
-                                      i64 F[5]) {
-  return fx_flux<3>(g, c.k, L, R, V, F);
-}
-__device__ __forceinline__ bool flux3(const Geom& g, const Fx3Const&, const double L[5], const double R[5],
-                                      const double V[4], i64 F[5]) {
+// The face flux in double: the tangential momenta as they are, the others
+// tagged.
+__device__ __forceinline__ void flux3(const Geom& g, const double L[5], const double R[5], const double V[4], i64 F[5]) {
   double o[5];
   lf_face5(L, R, g.gamma, g.gm1, V, o);
 #pragma unroll
-  for (int q = 0; q < 5; q++) F[q] = flux_tag(o[q]);
-  return true;
+  for (int q = 0; q < 5; q++) F[q] = q == 2 || q == 3 ? __double_as_longlong(o[q]) : flux_tag(o[q]);
 }
 
 // ---- y faces ------------------------------------------------------------------
 
 constexpr int RING3 = (TZ + 2) * (TX + 2);  // tile plus a one-cell ring
 struct YfaceSmem {
-  i64 q[2][5][TZ + 2][TX + 2];   // planes j and j+1, rows k0-1.., cols i0-1..
-  i64 v[2][4][TZ + 2][TX + 2];   // u, v, w, e on the ring
+  i64 q[2][5][TZ + 2][TX + 2];    // planes j and j+1, rows k0-1.., cols i0-1..
+  i64 v[2][4][TZ + 2][TX + 2];    // u, v, w, e on the ring
+  double vd[2][3][TZ + 2][TX + 2];  // u, v, w
+  double qd[2][2][TZ][TX];        // rho u, rho w of the tile's cells
   unsigned char ok[2][TZ + 2][TX + 2];
 };
 
@@ -273,6 +268,7 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
   const int j1 = wrap3(j + 1, g.ny);
   T* Sq = reinterpret_cast<T*>(&S.q[0][0][0][0]);
   T* Sv = reinterpret_cast<T*>(&S.v[0][0][0][0]);
+  double* Sd = &S.vd[0][0][0][0];
   bool bad = false;
   for (int e = tid; e < 2 * RING3; e += NTHREADS) {
     const int side = e >= RING3, rem = e - side * RING3;
@@ -294,24 +290,35 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
       t[c] = Arith3<T>::cell(q[c], c);
       Sq[(side * 5 + c) * RING3 + rem] = t[c];
     }
-    Arith3<T>::prims(t, v);
+    const double inv = Arith3<T>::prims(t, v);
 #pragma unroll
     for (int c = 0; c < 4; c++) Sv[(side * 4 + c) * RING3 + rem] = v[c];
+    if (FX) {
+#pragma unroll
+      for (int c = 0; c < 3; c++) Sd[(side * 3 + c) * RING3 + rem] = __dmul_rn(q[c + 1], inv);
+      if (rr >= 1 && rr <= TZ && cc >= 1 && cc <= TX) {
+        S.qd[side][0][rr - 1][cc - 1] = q[1];
+        S.qd[side][1][rr - 1][cc - 1] = q[3];
+      }
+    }
   }
   const int rr = tid / TX, cc = tid - rr * TX;
   const int k = k0 + rr, i = i0 + cc;
   const bool mine = k < row_hi && i < g.nx;
   // the outer two of the four cells across the face
   T am[5], ap[5];
+  double dm[2], dp[2];  // their rho u, rho w
   bool out_ok = true;
   if (mine && want) {
     double q[5];
     stage_val3(a, G, k, wrap3(j - 1, g.ny), i, q);
     out_ok = cell_in_range3(q);
+    dm[0] = q[1], dm[1] = q[3];
 #pragma unroll
     for (int c = 0; c < 5; c++) am[c] = Arith3<T>::cell(q[c], c);
     stage_val3(a, G, k, wrap3(j + 2, g.ny), i, q);
     out_ok = out_ok && cell_in_range3(q);
+    dp[0] = q[1], dp[1] = q[3];
 #pragma unroll
     for (int c = 0; c < 5; c++) ap[c] = Arith3<T>::cell(q[c], c);
   }
@@ -348,15 +355,40 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
     s[side].u[1] = V[0];
     s[side].u[2] = V[2 * RING3];
     s[side].e = V[3 * RING3];
-    s[side].g1[0] = V[RING3 + 1] - V[RING3 - 1];  // x differences of v, u
-    s[side].g1[1] = V[1] - V[-1];
-    s[side].g2[0] = dz_vel(g, C.k, k, 1, V + RING3, TX + 2);  // z differences of v, w
-    s[side].g2[1] = dz_vel(g, C.k, k, 2, V + 2 * RING3, TX + 2);
+    if (!FX) {
+      s[side].g1[0] = V[RING3 + 1] - V[RING3 - 1];             // x and z differences of v
+      s[side].g2[0] = dz_vel(g, C.k, k, 1, V + RING3, TX + 2);
+    }
+    s[side].g1[1] = V[1] - V[-1];                              // x difference of u
+    s[side].g2[1] = dz_vel(g, C.k, k, 2, V + 2 * RING3, TX + 2);  // z difference of w
   }
-  T V[4];
-  visc3(C, 1, k >= n1, s[0], s[1], V);
   i64 F[5];
-  if (!flux3(g, C, L, R, V, F)) return false;
+  if constexpr (FX) {
+    const double* d = Sd + at;  // plane j; the next plane 3 RING3 behind
+    const double* f = C.fd[1][k >= n1];
+    double gx = 0.0, gz = 0.0, sig[2];
+#pragma unroll
+    for (int side = 0; side < 2; side++) {
+      const double* v = d + (3 * side + 1) * RING3;
+      const double x = __dsub_rn(v[1], v[-1]), z = dz_vel(g, C.k, k, 1, v, TX + 2);
+      gx = side ? __dadd_rn(gx, x) : x;
+      gz = side ? __dadd_rn(gz, z) : z;
+    }
+    sig[0] = __fma_rn(f[F3_C], __dsub_rn(d[3 * RING3], d[0]), __dmul_rn(f[F3_D1], gx));
+    sig[1] = __fma_rn(f[F3_C], __dsub_rn(d[5 * RING3], d[2 * RING3]), __dmul_rn(f[F3_D2], gz));
+    i64 Vn, VE, o[3];
+    FxTan t;
+    visc3(C, 1, k >= n1, s[0], s[1], sig, &Vn, &VE);
+    if (!fx_flux<3>(g, C.k, L, R, Vn, VE, o, &t)) return false;
+    F[0] = o[0], F[1] = o[1], F[4] = o[2];
+#pragma unroll
+    for (int c = 0; c < 2; c++)
+      F[2 + c] = __double_as_longlong(tan_flux(t, dm[c], S.qd[0][c][rr][cc], S.qd[1][c][rr][cc], dp[c], sig[c]));
+  } else {
+    T V[4];
+    visc3(C, 1, k >= n1, s[0], s[1], V);
+    flux3(g, L, R, V, F);
+  }
 #pragma unroll
   for (int c = 0; c < 5; c++) {
     const int f = c == 1 ? 2 : (c == 2 ? 1 : c);
@@ -376,17 +408,25 @@ __device__ __forceinline__ void yface_tile(const StageArgs& a, const Fx3Const& C
 
 // ---- x and z faces, divergence and stage combination ----------------------
 
-constexpr int TILE3_THREADS = FP64_THREADS;  // nine warps, two face jobs each (face_id in stage_tile.cuh)
+// TX x TZ3 cells: 13 warps, two face jobs each (face_id in stage_tile.cuh). 110
+// KB of shared memory, two CTAs (26 warps) per SM; as TX x 8 tiles the doubles
+// of the tangential momenta would not leave room for three.
+constexpr int TZ3 = 12;
+constexpr int TILE3_THREADS = TX * (TZ3 + 1);
+constexpr int RINGS = (TZ3 + 2) * (TX + 2);
 struct Tile3Smem {
-  i64 q[5][TZ + 4][TX + 4];   // plane j, rows k0-2.., cols i0-2..
-  i64 v[4][TZ + 2][TX + 2];   // u, v, w, e on the ring
-  i64 vy[3][TZ + 2][TX + 2];  // central y differences of u, v, w on the ring
-  i64 fx[5][TZ][TX + 1];      // x face fluxes, face f between cols f-1, f
-  i64 fz[5][TZ + 1][TX];      // z face fluxes seen from above
-  i64 fg[5][TX];              // interface flux seen from fluid 1
-  unsigned char ok[TZ + 4][TX + 4];
-  unsigned char oky[TZ + 2][TX + 2];  // the cells in planes j-1 and j+1
-  unsigned char slow[(2 * TZ + 3) * TX];  // per face: its job and lane
+  i64 q[5][TZ3 + 4][TX + 4];       // plane j, rows k0-2.., cols i0-2..
+  double qd[3][TZ3 + 4][TX + 4];   // rho u, rho v, rho w
+  i64 v[4][TZ3 + 2][TX + 2];       // u, v, w, e on the ring
+  double vd[3][TZ3 + 2][TX + 2];   // u, v, w
+  i64 vy[3][TZ3 + 2][TX + 2];      // central y differences of u, v, w on the ring: u and w as doubles
+  // fluxes: the tangential momenta as doubles, the others tagged
+  i64 fx[5][TZ3][TX + 1];          // x face f between cols f-1, f
+  i64 fz[5][TZ3 + 1][TX];          // z faces seen from above
+  i64 fg[5][TX];                   // interface flux seen from fluid 1
+  unsigned char ok[TZ3 + 4][TX + 4];
+  unsigned char oky[TZ3 + 2][TX + 2];  // the cells in planes j-1 and j+1
+  unsigned char slow[(2 * TZ3 + 3) * TX];  // per face: its job and lane
 };
 
 // Phase 1 in T: stage state, velocities and their y differences. Returns
@@ -398,10 +438,9 @@ __device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, in
   const Geom& g = a.g;
   const int tid = threadIdx.x, nz = g.nz, n1 = g.n1;
   const int jm = wrap3(j - 1, g.ny), jp = wrap3(j + 1, g.ny);
-  constexpr int QP = (TZ + 4) * (TX + 4);
+  constexpr int QP = (TZ3 + 4) * (TX + 4);
   T* q = reinterpret_cast<T*>(&S.q[0][0][0]);
   T* v = reinterpret_cast<T*>(&S.v[0][0][0]);
-  T* vy = reinterpret_cast<T*>(&S.vy[0][0][0]);
   bool bad = false, good = false;
   for (int e = tid; e < QP; e += TILE3_THREADS) {
     const int rr = e / (TX + 4), cc = e - rr * (TX + 4);
@@ -410,6 +449,9 @@ __device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, in
       // read by the faces next to a wall, which replace it by the mirror cell
 #pragma unroll
       for (int c = 0; c < 5; c++) q[c * QP + e] = (T)0;
+      if (FX)
+#pragma unroll
+        for (int c = 0; c < 3; c++) (&S.qd[0][0][0])[c * QP + e] = 0.0;
       continue;
     }
     double x[5];
@@ -427,38 +469,56 @@ __device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, in
       t[c] = Arith3<T>::cell(x[c], c);
       q[c * QP + e] = t[c];
     }
-    // velocities on the one-cell ring
-    if (rr >= 1 && rr <= TZ + 2 && cc >= 1 && cc <= TX + 2) {
-      T o[4];
-      Arith3<T>::prims(t, o);
+    if (FX)
 #pragma unroll
-      for (int c = 0; c < 4; c++) v[c * RING3 + (rr - 1) * (TX + 2) + cc - 1] = o[c];
+      for (int c = 0; c < 3; c++) (&S.qd[0][0][0])[c * QP + e] = x[c + 1];
+    // velocities on the one-cell ring
+    if (rr >= 1 && rr <= TZ3 + 2 && cc >= 1 && cc <= TX + 2) {
+      T o[4];
+      const double inv = Arith3<T>::prims(t, o);
+      const int at = (rr - 1) * (TX + 2) + cc - 1;
+#pragma unroll
+      for (int c = 0; c < 4; c++) v[c * RINGS + at] = o[c];
+      if (FX)
+#pragma unroll
+        for (int c = 0; c < 3; c++) (&S.vd[0][0][0])[c * RINGS + at] = __dmul_rn(x[c + 1], inv);
     }
   }
-  for (int e = tid; e < RING3; e += TILE3_THREADS) {
+  for (int e = tid; e < RINGS; e += TILE3_THREADS) {
     const int rr = e / (TX + 2), cc = e - rr * (TX + 2);
     const int k = k0 - 1 + rr;
     if (k < 0 || k >= nz) continue;
     const int i = wrap3(i0 - 1 + cc, g.nx);
-    double x[5];
-    T t[4], up[3], dn[3];
+    double x[5], d[3];
+    T dv = 0;
     bool in = true;
 #pragma unroll
     for (int s = 0; s < 2; s++) {
       stage_val3(a, G, k, s ? jm : jp, i, x);
       if (FX) in = in && cell_in_range3(x);
       if (!in) break;
+      double inv;
+      if constexpr (FX) {
+        const i64 inv_ = fx::recip(Arith3<i64>::cell(x[0], 0) << 2);
+        const i64 v_ = fx::mul(fx::split(Arith3<i64>::cell(x[2], 2) << 2), fx::split(inv_));
+        dv = s ? dv - v_ : v_;
+        inv = __longlong_as_double(fx::to_double(inv_, 61));
+      } else {
+        inv = recip_f64(x[0]);
+      }
 #pragma unroll
-      for (int c = 0; c < 4; c++) t[c] = Arith3<T>::cell(x[c], c);
-      Arith3<T>::vel(t, s ? dn : up);
+      for (int c = 0; c < 3; c++)
+        if (!FX || c != 1) d[c] = s ? __dsub_rn(d[c], __dmul_rn(x[c + 1], inv)) : __dmul_rn(x[c + 1], inv);
     }
     if (FX) {
       S.oky[rr][cc] = in;
       bad |= !in;
     }
     if (!in) continue;
-#pragma unroll
-    for (int c = 0; c < 3; c++) vy[c * RING3 + e] = up[c] - dn[c];
+    if constexpr (!FX) dv = d[1];
+    (&S.vy[0][0][0])[e] = __double_as_longlong(d[0]);
+    reinterpret_cast<T*>(&S.vy[1][0][0])[e] = dv;
+    (&S.vy[2][0][0])[e] = __double_as_longlong(d[2]);
   }
   if (!FX) {
     __syncthreads();
@@ -475,7 +535,8 @@ __device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, in
 // ghost is 2 wall state - cell.
 template <typename T>
 __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Smem& S, const FaceId& id) {
-  constexpr int QP = (TZ + 4) * (TX + 4);
+  constexpr bool FX = (T)0.5 == (T)0;
+  constexpr int QP = (TZ3 + 4) * (TX + 4), VW = TX + 2;
   const int n1 = g.n1, nz = g.nz, ku = id.ku, kd = ku - 1;
   const int qs = id.isx ? 1 : TX + 4;
   const int q0 = id.isx ? (id.f + 2) * (TX + 4) + id.c : id.f * (TX + 4) + id.c + 2;
@@ -484,42 +545,73 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
   const bool wall = !id.isx && (ku == 0 || ku == nz), lidf = !id.isx && ku == n1;
   const bool from_above = ku == 0 || (lidf && !id.below);
   const bool mir0 = !id.isx && (kd == 0 || kd == n1), mir3 = !id.isx && (ku == nz - 1 || ku == n1 - 1);
+  const int dir = id.isx ? 0 : 2, fl = (id.isx ? ku : (ku == 0 ? 0 : kd)) >= n1;
+  // the first cell at the face on the ring; in double its velocity planes
+  const int vo = id.isx ? (id.f + 1) * VW + id.c : id.f * VW + id.c + 1, vs = id.isx ? 1 : VW;
   const T* q = reinterpret_cast<const T*>(&S.q[0][0][0]) + q0;
-  T L[5], R[5], V[4];
+  const T* v = reinterpret_cast<const T*>(&S.v[0][0][0]) + vo;
+  const T* vy1 = reinterpret_cast<const T*>(&S.vy[1][0][0]) + vo;
+  T L[5], R[5], V[4];  // FX: V[0] and V[3] only
+  double sig[2];       // FX: the tangential stresses
+  if (FX) {
+    const double* d = reinterpret_cast<const double*>(FX ? (const void*)&S.vd[0][0][0] : (const void*)v) + (FX ? vo : 0);
+    const double* d1 = d + (p1 - 1) * RINGS;
+    const double* d2 = d + (p2 - 1) * RINGS;
+    const double t1 = __dsub_rn(d1[vs], d1[0]), t2 = __dsub_rn(d2[vs], d2[0]);
+    if (lidf) {
+      sig[0] = __dmul_rn(C.k.tlid[LID_S], t1);
+      sig[1] = __dmul_rn(C.k.tlid[LID_S], t2);
+    } else if (wall) {  // the ghosts' velocities are +-those of the cell, their differences of w the opposite
+      const double cw = g.wall ? 0.0 : ku == 0 ? 2.0 : -2.0;
+      const int o = ku == 0 ? vs : 0;
+      sig[0] = __dmul_rn(C.fd[2][fl][F3_C], __dmul_rn(cw, d1[o]));
+      sig[1] = __dmul_rn(C.fd[2][fl][F3_C], __dmul_rn(cw, d2[o]));
+    } else {
+      const double* f = C.fd[dir][fl];
+      const double* n = d + (pn - 1) * RINGS;
+      const double* y = reinterpret_cast<const double*>(&S.vy[pn - 1][0][0]) + vo;
+      // differences of u_n along y and along the third direction, of both cells
+      const double gy = __dadd_rn(y[0], y[vs]);
+      const double gt = id.isx ? __dadd_rn(dz_vel(g, C.k, ku, 0, n, VW), dz_vel(g, C.k, ku, 0, n + 1, VW))
+                               : __dadd_rn(__dsub_rn(n[1], n[-1]), __dsub_rn(n[VW + 1], n[VW - 1]));
+      sig[0] = __fma_rn(f[F3_C], t1, __dmul_rn(f[F3_D1], id.isx ? gy : gt));
+      sig[1] = __fma_rn(f[F3_C], t2, __dmul_rn(f[F3_D2], id.isx ? gt : gy));
+    }
+  }
   if (lidf) {
     // the bulk fluxes, with the wall velocities (one value for both fluids)
-    const T* p = reinterpret_cast<const T*>(&S.v[0][0][0]) + id.f * (TX + 2) + id.c + 1;
     V[0] = 0;
-    T e2[2];  // each with its part of the energy: the heat flux once
-    lid_flux(g, C.k, p[0], p[TX + 2], p[3 * RING3], p[3 * RING3 + TX + 2], e2);
-    V[1] = e2[0];
-    V[3] = e2[1];
-    lid_flux(g, C.k, p[RING3], p[RING3 + TX + 2], T(0), T(0), e2);
-    V[2] = e2[0];
-    V[3] = V[3] + e2[1];
+    V[3] = lid_heat(C.k, v[3 * RINGS], v[3 * RINGS + VW]);
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+      const T u1 = v[c * RINGS], u2 = v[c * RINGS + VW];
+      if constexpr (FX) {
+        V[3] += lid_work(C.k, u1, u2, fx::from_double(__double_as_longlong(sig[c]), fx::S_VEL));
+      } else {
+        V[1 + c] = __dmul_rn(C.k.tlid[LID_S], __dsub_rn(u2, u1));
+        V[3] = __dadd_rn(V[3], lid_work(C.k, u1, u2, V[1 + c]));
+      }
+    }
   } else {
-    const T* v = reinterpret_cast<const T*>(&S.v[0][0][0]);
-    const T* vy = reinterpret_cast<const T*>(&S.vy[0][0][0]);
-    const int vo = id.isx ? (id.f + 1) * (TX + 2) + id.c : id.f * (TX + 2) + id.c + 1, vs = id.isx ? 1 : TX + 2;
     VSide<T> s[2];
 #pragma unroll
     for (int side = 0; side < 2; side++) {
-      const T* p = v + vo + side * vs;
-      const T* y = vy + vo + side * vs;
-      s[side].u[0] = p[(pn - 1) * RING3];
-      s[side].u[1] = p[(p1 - 1) * RING3];
-      s[side].u[2] = p[(p2 - 1) * RING3];
-      s[side].e = p[3 * RING3];
+      const T* p = v + side * vs;
+      const T* y = vy1 + side * vs;
+      s[side].u[0] = p[(pn - 1) * RINGS];
+      s[side].u[1] = p[(p1 - 1) * RINGS];
+      s[side].u[2] = p[(p2 - 1) * RINGS];
+      s[side].e = p[3 * RINGS];
       if (id.isx) {  // t1 = y: du, dv; t2 = z: du, dw
-        s[side].g1[0] = y[0];
-        s[side].g1[1] = y[RING3];
-        s[side].g2[0] = dz_vel(g, C.k, ku, 0, p, TX + 2);
-        s[side].g2[1] = dz_vel(g, C.k, ku, 2, p + 2 * RING3, TX + 2);
+        s[side].g1[0] = y[-RINGS];
+        s[side].g1[1] = y[0];
+        if (!FX) s[side].g2[0] = dz_vel(g, C.k, ku, 0, p, VW);
+        s[side].g2[1] = dz_vel(g, C.k, ku, 2, p + 2 * RINGS, VW);
       } else {  // t1 = x: dw, du; t2 = y: dw, dv
-        s[side].g1[0] = p[2 * RING3 + 1] - p[2 * RING3 - 1];
+        s[side].g1[0] = p[2 * RINGS + 1] - p[2 * RINGS - 1];
         s[side].g1[1] = p[1] - p[-1];
-        s[side].g2[0] = y[2 * RING3];
-        s[side].g2[1] = y[RING3];
+        s[side].g2[0] = y[RINGS];
+        s[side].g2[1] = y[0];
       }
     }
     if (wall) {
@@ -536,16 +628,18 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
       if (from_above) s[0] = o;
       else s[1] = o;
     }
-    visc3(C, id.isx ? 0 : 2, (id.isx ? ku : (ku == 0 ? 0 : kd)) >= n1, s[0], s[1], V);
+    if constexpr (FX) visc3(C, dir, fl, s[0], s[1], sig, V, V + 3);
+    else visc3(C, dir, fl, s[0], s[1], V);
   }
   const int planes[5] = {0, pn * QP, p1 * QP, p2 * QP, 4 * QP};
-  if (wall || lidf || mir0 || mir3) {
+  const bool edge = wall || lidf;
+  if (edge || mir0 || mir3) {
 #pragma unroll
     for (int c = 0; c < 5; c++) {
       const bool odd = c == 1;  // mirror ghosts beyond a wall or the interface: rho w odd
       const T* p = q + planes[c];
       T a0 = p[0], a1 = p[qs], a2 = p[2 * qs], a3 = p[3 * qs];
-      if (wall || lidf) {
+      if (edge) {
         if (from_above) a1 = odd ? -a2 : a2;
         else a2 = odd ? -a1 : a1;
       }
@@ -553,7 +647,7 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
       if (mir3) a3 = odd ? -a2 : a2;
       L[c] = Arith3<T>::rec(a1, a2, a0);
       R[c] = Arith3<T>::rec(a2, a1, a3);
-      if (wall || lidf) {
+      if (edge) {
         if (from_above) L[c] = odd ? -R[c] : R[c];
         else R[c] = odd ? -L[c] : L[c];
       }
@@ -568,15 +662,40 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
     }
   }
   i64 F[5];
-  if (!flux3(g, C, L, R, V, F)) return false;
+  if constexpr (FX) {
+    i64 m[3];
+    FxTan t;
+    if (!fx_flux<3>(g, C.k, L, R, V[0], V[3], m, &t)) return false;
+    F[0] = m[0], F[1] = m[1], F[4] = m[2];
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+      const double* p = &S.qd[0][0][0] + q0 + ((c ? p2 : p1) - 1) * QP;
+      double a0 = p[0], a1 = p[qs], a2 = p[2 * qs], a3 = p[3 * qs], f;
+      if (edge) {
+        if (from_above) a1 = a2;
+        else a2 = a1;
+      }
+      if (mir0) a0 = a1;
+      if (mir3) a3 = a2;
+      if (edge) {
+        const double b = from_above ? __fma_rn(0.25, __dsub_rn(a1, a3), a2) : __fma_rn(0.25, __dsub_rn(a2, a0), a1);
+        f = tan_flux(t, b, b, sig[c]);
+      } else {
+        f = tan_flux(t, a0, a1, a2, a3, sig[c]);
+      }
+      F[2 + c] = __double_as_longlong(f);
+    }
+  } else {
+    flux3(g, L, R, V, F);
+  }
   i64* o;
   int plane;
   if (id.isx) {
-    o = &S.fx[0][id.f][id.c], plane = TZ * (TX + 1);
+    o = &S.fx[0][id.f][id.c], plane = TZ3 * (TX + 1);
   } else if (id.below) {
     o = &S.fg[0][id.c], plane = TX;
   } else {
-    o = &S.fz[0][id.f][id.c], plane = (TZ + 1) * TX;
+    o = &S.fz[0][id.f][id.c], plane = (TZ3 + 1) * TX;
   }
   o[0] = F[0];
   o[pn * plane] = F[1];
@@ -615,10 +734,10 @@ __device__ __noinline__ bool face3_in_range(const Geom& g, const Tile3Smem& S, c
 __device__ __noinline__ void slow_faces3(const StageArgs& a, const Fx3Const& C, int k0, int i0, int j, int row_hi,
                                          Tile3Smem& S, bool all) {
   tile3_cells<double>(a, geo3(a.g), k0, i0, j, S);
-  for (int job = threadIdx.x / 32; job < 2 * TZ + 3; job += TILE3_THREADS / 32) {
+  for (int job = threadIdx.x / 32; job < 2 * TZ3 + 3; job += TILE3_THREADS / 32) {
     const int lane = threadIdx.x % 32;
     FaceId id;
-    if (face_id<TZ>(a.g, job, lane, k0, row_hi, &id) && (all || S.slow[job * TX + lane])) face3<double>(a.g, C, S, id);
+    if (face_id<TZ3>(a.g, job, lane, k0, row_hi, &id) && (all || S.slow[job * TX + lane])) face3<double>(a.g, C, S, id);
   }
   __syncthreads();
 }
@@ -635,13 +754,13 @@ __device__ __forceinline__ void stage_tile3(const StageArgs& a, const Fx3Const& 
   const int out = C.k.on ? tile3_cells<i64>(a, G, k0, i0, j, S) : 2;
 
   // ---- 2. face fluxes -----------------------------------------------------
-  const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZ);
-  const int jobs = out == 2 ? 0 : 2 * TZ + 2 + has_gamma;
+  const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZ3);
+  const int jobs = out == 2 ? 0 : 2 * TZ3 + 2 + has_gamma;
   const int warp = __shfl_sync(0xffffffffu, tid / 32, 0), lane = tid % 32;
   bool slow = false;
   for (int job = warp; job < jobs; job += TILE3_THREADS / 32) {
     FaceId id;
-    if (!face_id<TZ>(g, job, lane, k0, row_hi, &id)) continue;
+    if (!face_id<TZ3>(g, job, lane, k0, row_hi, &id)) continue;
     const bool ok = (out == 0 || face3_in_range(g, S, id, k0)) && face3<i64>(g, C, S, id);
     S.slow[job * TX + lane] = !ok;
     slow |= !ok;
@@ -652,14 +771,14 @@ __device__ __forceinline__ void stage_tile3(const StageArgs& a, const Fx3Const& 
   // ---- 3. R = -div F* + s and the stage combination -------------------------
   const int rr = tid / TX, cc = tid - rr * TX;
   const int k = k0 + rr, i = i0 + cc;
-  if (rr >= TZ || k >= row_hi || i >= nx) return;
+  if (rr >= TZ3 || k >= row_hi || i >= nx) return;
   const bool under_gamma = (k == n1 - 1);
   const size_t row = (size_t)(k * ny + j) * g.pitch + i;  // offset within a component
   const size_t plane = G.plane;
   const int jm = wrap3(j - 1, ny);
   const i64* gy = reinterpret_cast<const i64*>(a.gy);
   const double hx = 0.5 * g.inv_dx, hy = 0.5 * g.inv_dy, hz = 0.5 * (k < n1 ? g.inv_dz1 : g.inv_dz2);
-  const double s57 = 1.0 / (double)(1ll << fx::S_FLUX);
+  const double sz = C.k.scale_z[k >= n1];
   double R[5];
   i64 y0[5], y1[5];
   int any = 0;
@@ -667,33 +786,45 @@ __device__ __forceinline__ void stage_tile3(const StageArgs& a, const Fx3Const& 
   for (int c = 0; c < 5; c++) {
     y0[c] = gy[G.at(c, k, jm, i)];
     y1[c] = gy[G.at(c, k, j, i)];
+    if (c == 1 || c == 3) continue;  // the tangential momenta
     const int h0 = (int)(y0[c] >> 32), h1 = (int)(y1[c] >> 32);
     any |= (h0 ^ (h0 >> 31)) | (h1 ^ (h1 >> 31));
   }
   bool dbl = any >= 0x10000000;  // some y flux is a double
   if (out == 2) dbl = true;
   else if (slow)
-    dbl = dbl || S.slow[(TZ + rr) * TX + cc] ||
-          S.slow[cc < TX - 1 ? (TZ + rr) * TX + cc + 1 : (2 * TZ + 1) * TX + rr] || S.slow[rr * TX + cc] ||
-          S.slow[(under_gamma ? 2 * TZ + 2 : rr + 1 < TZ ? rr + 1 : 2 * TZ) * TX + cc];
+    dbl = dbl || S.slow[(TZ3 + rr) * TX + cc] ||
+          S.slow[cc < TX - 1 ? (TZ3 + rr) * TX + cc + 1 : (2 * TZ3 + 1) * TX + rr] || S.slow[rr * TX + cc] ||
+          S.slow[(under_gamma ? 2 * TZ3 + 2 : rr + 1 < TZ3 ? rr + 1 : 2 * TZ3) * TX + cc];
   if (dbl) {
 #pragma unroll
     for (int c = 0; c < 5; c++) {
-      const double dx = __dsub_rn(flux_value(S.fx[c][rr][cc]), flux_value(S.fx[c][rr][cc + 1]));
-      const double dz = __dsub_rn(flux_value(S.fz[c][rr][cc]),
-                                  flux_value(under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc]));
-      const double dy = __dsub_rn(flux_value(y0[c]), flux_value(y1[c]));
+      auto diff = [&](i64 f, i64 h, bool tangential) {
+        return tangential ? __dsub_rn(__longlong_as_double(f), __longlong_as_double(h))
+                          : __dsub_rn(flux_value(f), flux_value(h));
+      };
+      const double dx = diff(S.fx[c][rr][cc], S.fx[c][rr][cc + 1], c == 2 || c == 3);
+      const double dz = diff(S.fz[c][rr][cc], under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc], c == 1 || c == 2);
+      const double dy = diff(y0[c], y1[c], c == 1 || c == 3);
       R[c] = __fma_rn(hx, dx, __fma_rn(hy, dy, __dmul_rn(hz, dz)));
     }
   } else {
 #pragma unroll
     for (int c = 0; c < 5; c++) {
-      const i64 dx = S.fx[c][rr][cc] - S.fx[c][rr][cc + 1];
-      const i64 dz = S.fz[c][rr][cc] - (under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc]);
-      const i64 dy = y0[c] - y1[c];
-      R[c] = C.k.square ? __dmul_rn(C.k.scale, (double)(dx + dy + dz))
-                        : __fma_rn(C.k.scale, (double)dx,
-                                   __fma_rn(__dmul_rn(hy, s57), (double)dy, __dmul_rn(__dmul_rn(hz, s57), (double)dz)));
+      const i64 x0 = S.fx[c][rr][cc], x1 = S.fx[c][rr][cc + 1];
+      const i64 z0 = S.fz[c][rr][cc], z1 = under_gamma ? S.fg[c][cc] : S.fz[c][rr + 1][cc];
+      auto sum = [&](double sn, i64 n, double ha, i64 a0, i64 a1, double hb, i64 b0, i64 b1) {
+        const double da = __dsub_rn(__longlong_as_double(a0), __longlong_as_double(a1));
+        const double db = __dsub_rn(__longlong_as_double(b0), __longlong_as_double(b1));
+        return __fma_rn(sn, (double)n, __fma_rn(ha, da, __dmul_rn(hb, db)));
+      };
+      if (c == 1) R[c] = sum(C.k.scale, x0 - x1, hy, y0[c], y1[c], hz, z0, z1);
+      else if (c == 2) R[c] = sum(C.scale_y, y0[c] - y1[c], hx, x0, x1, hz, z0, z1);
+      else if (c == 3) R[c] = sum(sz, z0 - z1, hx, x0, x1, hy, y0[c], y1[c]);
+      else if (C.k.square) R[c] = __dmul_rn(C.k.scale, (double)((x0 - x1) + (y0[c] - y1[c]) + (z0 - z1)));
+      else
+        R[c] = __fma_rn(C.k.scale, (double)(x0 - x1),
+                        __fma_rn(C.scale_y, (double)(y0[c] - y1[c]), __dmul_rn(sz, (double)(z0 - z1))));
     }
   }
   {
