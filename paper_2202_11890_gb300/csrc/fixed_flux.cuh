@@ -124,7 +124,8 @@ __device__ __forceinline__ bool fx_flux(const Geom& g, const FxConst& k, const i
     }
   }
   const FxW lam59 = fx::split(lam), lam61 = fx::split(lam << 2);
-  F[0] = (L[1] >> 5) + (R[1] >> 5) + fx::mul(fx::split(L[0] - R[0]), lam61);
+  // one rounding of the sum: exactly zero at a wall, where m_nR = -m_nL
+  F[0] = ((L[1] + R[1] + 16) >> 5) + fx::mul(fx::split(L[0] - R[0]), lam61);
   F[1] = (l.mu + l.p) + (r.mu + r.p) + fx::mul(fx::split(L[1] - R[1]), lam59) - Vn;
   F[2] = fx::mul(fx::split(l.eh), fx::split(l.un_ << 3)) + fx::mul(fx::split(r.eh), fx::split(r.un_ << 3)) +
          fx::mul(fx::split(L[E] - R[E]), lam61) - VE;

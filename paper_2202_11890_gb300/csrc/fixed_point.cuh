@@ -8,10 +8,17 @@
 // face fluxes of the FP64 tile run here: states, speeds and fluxes of a
 // nondimensional flow (density, sound speed and pressure near one) as 64-bit
 // integers in units of 2^-57 to 2^-62, except the flux of the tangential
-// momentum (fixed_flux.cuh). Their rounding errors are below 2^-56
-// absolute, an eighth of the rounding of a double near one; a face whose
-// states leave the representable range is evaluated in double instead
-// (stage_tile.cuh).
+// momentum (fixed_flux.cuh). A face whose states leave the representable
+// range is evaluated in double instead (stage_tile.cuh).
+//
+// Errors are absolute. A product errs by at most 3/4 of its unit (mul), a pair
+// of products by one (mul2). A flux in units of 2^-57 sums its products: 1.25
+// units for mass, 3.75 for the normal momentum (and 1 to 1.75 for sigma_nn),
+// 2.25 for the energy, whose viscous part adds up to 3.5 units in 2-D and 6 in 3-D
+// (fx_visc, visc3; 2.5 and 4 at the interface; tests/test_fixed_flux.py), plus
+// the errors of its factors, of units up to 2^-57. Over the states tested the
+// right-hand side errs by 3 to 14 % of the double form's in mass, normal
+// momentum and energy (root mean square, tests/test_gpu_flux_precision.py).
 //
 // Notation: x.s means the integer x * 2^s. Products drop 64 bits, so
 // a.s * b.t gives (a b).(s + t - 64).

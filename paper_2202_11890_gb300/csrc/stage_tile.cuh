@@ -251,11 +251,11 @@ __device__ __forceinline__ double lid_ghost(const Geom&, const FxConst& k, int f
 }
 // The energy's part of one wall velocity component (sig: its sigma .59); the
 // heat flux.
-__device__ __forceinline__ i64 lid_work(const FxConst& k, i64 u1, i64 u2, i64 sig) {
+__host__ __device__ __forceinline__ i64 lid_work(const FxConst& k, i64 u1, i64 u2, i64 sig) {
   const i64 uw = u1 + fx::mul(fx::split((u2 - u1) << 2), k.lid[LID_1]);
   return fx::mul(fx::split(uw << 3), fx::split(sig));
 }
-__device__ __forceinline__ i64 lid_heat(const FxConst& k, i64 e1, i64 e2) {
+__host__ __device__ __forceinline__ i64 lid_heat(const FxConst& k, i64 e1, i64 e2) {
   return fx::mul(fx::split(e2 - e1), k.lid[LID_T]);
 }
 __device__ __forceinline__ double lid_work(const FxConst& k, double u1, double u2, double sig) {
@@ -471,7 +471,7 @@ __device__ __forceinline__ void face_sides_plain(const TileSmem<TZR>& S, const F
 // The viscous flux of the normal momentum and the energy over half the
 // divergence factor from the common values of App. B: sigma_nn and u .
 // sigma_n + kappa dT/dn, .57; snt: sigma_nt .59.
-__device__ __forceinline__ void fx_visc(const FxW* fc, const i64 vL[5], const i64 vR[5], i64 snt, i64* Vn, i64* VE) {
+__host__ __device__ __forceinline__ void fx_visc(const FxW* fc, const i64 vL[5], const i64 vR[5], i64 snt, i64* Vn, i64* VE) {
   *Vn = fx::mul2(fc[FXC_A], fx::split(vR[0] - vL[0]), fc[FXC_B], fx::split(vL[4] + vR[4]));
   // (u_L + u_R) . sigma: .61 x .59 -> .56, half of it at .57
   *VE = fx::mul2(fx::split((vL[0] + vR[0]) << 2), fx::split(*Vn << 2), fx::split((vL[1] + vR[1]) << 2), fx::split(snt)) +

@@ -205,18 +205,15 @@ __device__ __forceinline__ T dz_vel(const Geom& g, const FxConst& c, int k, int 
 // sigma_nt1, sigma_nt2, u^.sigma_n + kappa dT/dn). With G[a][b] = d u_a /
 // d x_b (b = normal, t1, t2): sigma_nn = mu (4/3 G00 - 2/3 (G11 + G22)),
 // sigma_nt = mu (G_t0 + G_0t); the derivative factors sit in the coefficients.
-// In fixed point only sigma_nn and the energy, from the other two as doubles.
-__device__ __forceinline__ void visc3(const Fx3Const& c, int dir, int fl, const VSide<i64>& L, const VSide<i64>& R,
-                                      const double s[2], i64* Vn, i64* VE) {
-  const FxW* f = c.fc[dir][fl];
+// In fixed point only sigma_nn and the energy, with the other two (snt) .59.
+__host__ __device__ __forceinline__ void visc3(const FxW* f, const VSide<i64>& L, const VSide<i64>& R, const i64 snt[2],
+                                               i64* Vn, i64* VE) {
   *Vn = fx::mul2(f[F3_A], fx::split(R.u[0] - L.u[0]), f[F3_B1], fx::split(L.g1[1] + R.g1[1])) +
         fx::mul(fx::split(L.g2[1] + R.g2[1]), f[F3_B2]);
   // (u_L + u_R) . sigma: .61 x .59 -> .56, half of it at .57
   i64 us = fx::mul(fx::split((L.u[0] + R.u[0]) << 2), fx::split(*Vn << 2));
 #pragma unroll
-  for (int t = 0; t < 2; t++)
-    us += fx::mul(fx::split((L.u[1 + t] + R.u[1 + t]) << 2),
-                  fx::split(fx::from_double(__double_as_longlong(s[t]), fx::S_VEL)));
+  for (int t = 0; t < 2; t++) us += fx::mul(fx::split((L.u[1 + t] + R.u[1 + t]) << 2), fx::split(snt[t]));
   *VE = us + fx::mul(fx::split(R.e - L.e), f[F3_K]);
 }
 __device__ __forceinline__ void visc3(const Fx3Const& c, int dir, int fl, const VSide<double>& L,
@@ -378,7 +375,9 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
     sig[1] = __fma_rn(f[F3_C], __dsub_rn(d[5 * RING3], d[2 * RING3]), __dmul_rn(f[F3_D2], gz));
     i64 Vn, VE, o[3];
     FxTan t;
-    visc3(C, 1, k >= n1, s[0], s[1], sig, &Vn, &VE);
+    const i64 snt[2] = {fx::from_double(__double_as_longlong(sig[0]), fx::S_VEL),
+                        fx::from_double(__double_as_longlong(sig[1]), fx::S_VEL)};
+    visc3(C.fc[1][k >= n1], s[0], s[1], snt, &Vn, &VE);
     if (!fx_flux<3>(g, C.k, L, R, Vn, VE, o, &t)) return false;
     F[0] = o[0], F[1] = o[1], F[4] = o[2];
 #pragma unroll
@@ -553,6 +552,7 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
   const T* vy1 = reinterpret_cast<const T*>(&S.vy[1][0][0]) + vo;
   T L[5], R[5], V[4];  // FX: V[0] and V[3] only
   double sig[2];       // FX: the tangential stresses
+  i64 snt[2];          // the same .59
   if (FX) {
     const double* d = reinterpret_cast<const double*>(FX ? (const void*)&S.vd[0][0][0] : (const void*)v) + (FX ? vo : 0);
     const double* d1 = d + (p1 - 1) * RINGS;
@@ -577,6 +577,8 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
       sig[0] = __fma_rn(f[F3_C], t1, __dmul_rn(f[F3_D1], id.isx ? gy : gt));
       sig[1] = __fma_rn(f[F3_C], t2, __dmul_rn(f[F3_D2], id.isx ? gt : gy));
     }
+#pragma unroll
+    for (int c = 0; c < 2; c++) snt[c] = fx::from_double(__double_as_longlong(sig[c]), fx::S_VEL);
   }
   if (lidf) {
     // the bulk fluxes, with the wall velocities (one value for both fluids)
@@ -586,7 +588,7 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
     for (int c = 0; c < 2; c++) {
       const T u1 = v[c * RINGS], u2 = v[c * RINGS + VW];
       if constexpr (FX) {
-        V[3] += lid_work(C.k, u1, u2, fx::from_double(__double_as_longlong(sig[c]), fx::S_VEL));
+        V[3] += lid_work(C.k, u1, u2, snt[c]);
       } else {
         V[1 + c] = __dmul_rn(C.k.tlid[LID_S], __dsub_rn(u2, u1));
         V[3] = __dadd_rn(V[3], lid_work(C.k, u1, u2, V[1 + c]));
@@ -628,7 +630,7 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
       if (from_above) s[0] = o;
       else s[1] = o;
     }
-    if constexpr (FX) visc3(C, dir, fl, s[0], s[1], sig, V, V + 3);
+    if constexpr (FX) visc3(C.fc[dir][fl], s[0], s[1], snt, V, V + 3);
     else visc3(C, dir, fl, s[0], s[1], V);
   }
   const int planes[5] = {0, pn * QP, p1 * QP, p2 * QP, 4 * QP};

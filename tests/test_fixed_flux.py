@@ -1,0 +1,169 @@
+"""The 64-bit fixed-point arithmetic of the FP64 faces, compiled for the host,
+against exact rational numbers: the products, reciprocal, square root and
+conversions, and the viscous part of the normal momentum and the energy in 2-D,
+in 3-D and at the interface.
+
+Bounds, in units of the result's last digit. A product drops the low 32 x 32
+bits (at most 1/4) and rounds the cross products (1/2): 3/4 alone, 1 for two
+that share a rounding. With velocities |u| <= 1.32 and stresses taken .57
+(sigma_nn) or truncated to .59 (sigma_nt), the viscous energy errs by its own
+products, by 1.32 times the error of sigma_nn and by 1.32 / 4 per sigma_nt:
+2-D 1 + 3/4 + 1.32 (1 + 1/4), 3-D 4 (3/4) + 1.32 (7/4 + 2/4), the interface per
+component 3/4 + 1.32 / 4 + |sigma| (3/4)(1/4) and 3/4 for the heat."""
+import ctypes as C
+import random
+import subprocess
+from fractions import Fraction as Fr
+
+import numpy as np
+import pytest
+
+from paper_2202_11890_gb300 import build
+
+SHIM = r"""
+#include <cuda_runtime.h>
+#include <cstring>
+#include "mprk_internal.h"
+#include "stage_tile.cuh"
+#include "stage_tile3d.cuh"
+using namespace mprk;
+extern "C" {
+void prim(const i64* in, i64* o) {  // in: a, b, c, d; rho .60; x .61; the bits of a double
+  const FxW a = fx::split(in[0]), b = fx::split(in[1]), c = fx::split(in[2]), d = fx::split(in[3]);
+  o[0] = fx::mul(a, b);
+  o[1] = fx::mul2(a, b, c, d);
+  o[2] = fx::recip(in[4]);
+  o[3] = fx::sqroot(in[5]);
+  o[4] = fx::from_double(in[6], 60);
+  o[5] = fx::to_double(in[0], 59);
+}
+void visc2(const i64* f, const i64* v, i64* o) {  // f: coefficients; v: L, R of five, snt
+  FxW fc[FXC_N];
+  for (int j = 0; j < FXC_N; j++) fc[j] = fx::split(f[j]);
+  fx_visc(fc, v, v + 5, v[10], o, o + 1);
+}
+void visc3d(const i64* f, const i64* v, i64* o) {  // v: L, R of (u[3], e, g1, g2), snt[2]
+  FxW fc[F3_N];
+  for (int j = 0; j < F3_N; j++) fc[j] = fx::split(f[j]);
+  VSide<i64> s[2];
+  for (int k = 0; k < 2; k++) {
+    for (int j = 0; j < 3; j++) s[k].u[j] = v[6 * k + j];
+    s[k].e = v[6 * k + 3];
+    s[k].g1[1] = v[6 * k + 4];
+    s[k].g2[1] = v[6 * k + 5];
+  }
+  visc3(fc, s[0], s[1], v + 12, o, o + 1);
+}
+void lid(const i64* f, const i64* v, i64* o) {  // u1, u2, e1, e2, snt
+  FxConst k;
+  for (int j = 0; j < LID_N; j++) k.lid[j] = fx::split(f[j]);
+  o[0] = lid_work(k, v[0], v[1], v[4]) + lid_heat(k, v[2], v[3]);
+}
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("fx")
+    (d / "fx.cu").write_text(SHIM)
+    out = str(d / "fx.so")
+    r = subprocess.run([build.nvcc(), *build.ARCH, *build.FLAGS, "-shared", "-o", out, str(d / "fx.cu")],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return C.CDLL(out)
+
+
+def call(fn, *args, n):
+    out = (C.c_longlong * n)()
+    fn(*[(C.c_longlong * len(a))(*a) for a in args], out)
+    return list(out)
+
+
+def bits(x):
+    return int(np.float64(x).view(np.int64))
+
+
+def value(b):
+    return Fr(float(np.int64(b).view(np.float64)))
+
+
+def test_primitives_within_their_bounds(lib):
+    rng = random.Random(3)
+    one = Fr(2) ** 64
+    for _ in range(4000):
+        a, b, c, d = (int(rng.uniform(-1, 1) * 2 ** rng.uniform(30, 61.5)) for _ in range(4))
+        rho, x = int(rng.uniform(0.3, 4.9) * 2 ** 60), int(rng.uniform(0.26, 3.9) * 2 ** 61)
+        y = rng.uniform(-1, 1) * 2.0 ** rng.uniform(-70, 1)
+        o = call(lib.prim, [a, b, c, d, rho, x, bits(y)], n=6)
+        assert abs(o[0] - Fr(a) * b / one) <= Fr(3, 4)
+        assert abs(o[1] - (Fr(a) * b + Fr(c) * d) / one) <= 1
+        # one third-order step from a seed of 2^-19: a rest of 2^-57, and roundings
+        # of the last two products relative to results of at least 2^58
+        assert abs(Fr(o[2]) * rho / Fr(2) ** 121 - 1) <= Fr(2) ** -56
+        assert abs(Fr(o[3]) ** 2 / (Fr(x) / Fr(2) ** 61 * Fr(2) ** 118) - 1) <= Fr(2) ** -55
+        exact = Fr(y) * 2 ** 60
+        assert abs(o[4]) <= abs(exact) < abs(o[4]) + 1 and (o[4] == 0 or (o[4] > 0) == (y > 0))
+        assert value(o[5]) == Fr(a / 2 ** 59) or abs(value(o[5]) - Fr(a) / 2 ** 59) <= abs(Fr(a)) / 2 ** 112
+    for a in (0, 1, -1, 2 ** 53 + 1, 2 ** 62 - 1, -(2 ** 62) + 1, 2 ** 63 - 1, -(2 ** 63)):
+        o = call(lib.prim, [a, 1, 1, 1, 2 ** 60, 2 ** 60, 0], n=6)
+        assert abs(value(o[5]) * 2 ** 59 - a) <= abs(Fr(a)) / 2 ** 53
+
+
+U, E, N = 1.32, 4.8, 59  # cell velocities and e as the range bounds them, .59
+
+
+def coefficients(rng, n):
+    """(8/3) mu / d and the rest below one, as the launch constants allow."""
+    f = [rng.uniform(0, 1), -rng.uniform(0, 0.125), -rng.uniform(0, 0.125), rng.uniform(0, 1), 0, 0, rng.uniform(0, 1)]
+    f = f if n == 7 else [f[0], f[1], 0, 0, f[6]]
+    return [int(x * 2 ** 62) for x in f]
+
+
+def scaled(rng):
+    """Factors for velocities and their differences, from the range's ends to weak flows."""
+    return rng.choice([1.0, 1.0, 2.0 ** -rng.uniform(0, 40)])
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_viscous_energy_within_its_bound(lib, dim):
+    rng = random.Random(dim)
+    for _ in range(6000):
+        s = scaled(rng)
+        r = lambda m: int(rng.choice([rng.uniform(-m, m), m, -m]) * s * 2 ** N)  # noqa: E731
+        f = coefficients(rng, 5 if dim == 2 else 7)
+        exact = rng.uniform(-2, 2) * s, rng.uniform(-2, 2) * s  # the double stresses
+        snt = [int(x * 2 ** N) for x in exact]  # truncated toward zero
+        if dim == 2:
+            v = [[r(U), r(U), r(E), 0, r(5.25)] for _ in range(2)]
+            Vn, VE = call(lib.visc2, f, v[0] + v[1] + snt[:1], n=2)
+            L, R = v
+            sn = Fr(f[0]) * (R[0] - L[0]) + Fr(f[1]) * (L[4] + R[4])
+            sums, heat, kap, bn, be = [L[0] + R[0], L[1] + R[1]], R[2] - L[2], f[4], 1, 1.75 + U * 1.25
+        else:
+            v = [[r(U), r(U), r(U), r(E), r(2.64), r(5.25)] for _ in range(2)]
+            Vn, VE = call(lib.visc3d, f, v[0] + v[1] + snt, n=2)
+            L, R = v
+            sn = Fr(f[0]) * (R[0] - L[0]) + Fr(f[1]) * (L[4] + R[4]) + Fr(f[2]) * (L[5] + R[5])
+            sums = [L[j] + R[j] for j in range(3)]
+            heat, kap, bn, be = R[3] - L[3], f[6], 1.75, 3.0 + U * 2.25
+        sn = sn / Fr(2) ** 64  # .57
+        assert abs(Vn - sn) <= bn
+        work = Fr(sums[0], 2) * sn / Fr(2) ** N
+        for t, x in zip(sums[1:], exact):
+            work += Fr(t, 2) * Fr(x) * Fr(2) ** 57 / Fr(2) ** N
+        assert abs(VE - (work + Fr(kap) * heat / Fr(2) ** 64)) <= be, (s, float(VE - work))
+
+
+def test_interface_energy_within_its_bound(lib):
+    rng = random.Random(5)
+    for _ in range(6000):
+        s = scaled(rng)
+        r = lambda m: int(rng.choice([rng.uniform(-m, m), m, -m]) * s * 2 ** N)  # noqa: E731
+        f = [0] + [int(rng.uniform(0, 1) * 2 ** 62) for _ in range(3)]
+        u1, u2, e1, e2 = r(U), r(U), r(E), r(E)
+        sig = rng.uniform(-2.6, 2.6) * s
+        out, = call(lib.lid, f, [u1, u2, e1, e2, int(sig * 2 ** N)], n=1)
+        uw = u1 + Fr(f[1]) * (u2 - u1) / Fr(2) ** 62
+        exact = uw * Fr(sig) / Fr(4) + Fr(f[3]) * (e2 - e1) / Fr(2) ** 64
+        assert abs(out - exact) <= 1.5 + U / 4 + 2.6 * 0.75 / 4
