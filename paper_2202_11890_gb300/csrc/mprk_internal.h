@@ -316,10 +316,8 @@ size_t stage_smem_bytes(int precision);
 // 85.7 -> 84.6 us. chain_next stands behind the faces: called as the kernel
 // starts, the next launch's CTAs fill the SMs that have room first, two or
 // three on some while others stay empty (321 x 273 cells, m = 4, 166 against
-// 131 us per step; 128 x 128 61.5 against 57.2). Kernels that fill an SM with
-// one CTA call it first (100 x 300 cells 63.0 against 63.7 us per step), and
-// so do the 3-D ones, whose launches are many waves long (the same within
-// 0.5 %).
+// 131 us per step; 128 x 128 61.5 against 57.2). The 3-D ones, whose launches
+// are many waves long, call it first (the same within 0.5 %).
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -32,7 +32,6 @@ __global__ void __launch_bounds__(NT, NT == TX * (TZR + 1) ? fp64_ctas(TZR) : 1)
     stage_kernel(const __grid_constant__ StageArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   TileSmem<TZR>& S = *reinterpret_cast<TileSmem<TZR>*>(smem_raw);
-  if (NT > 512) chain_next();  // one CTA per SM: the next launch's cannot gather on some
   chain_wait();
   stage_tile<GEN, NT, TZR>(a, blockIdx.x, S);
 }
@@ -250,9 +249,11 @@ cudaError_t launch_stage(const StageArgs& a, int precision, int n_tiles, cudaStr
     const bool one_wave = 2 * n_tiles <= 3 * sm_count();
     const dim3 grid(a.tiles_x, n_tiles / a.tiles_x, one_wave ? 2 : 1);
     const size_t smem = mixed_kernel_smem(a.stage & 1);
-    // chained in launches of one wave that use every SM: 321 x 273 cells 70.2 ->
-    // 68.3 us per step (m = 4), 200 x 200 the same; chained everywhere, 64 x 64
-    // took 61.5 us instead of 59.5 and 4096 x 2048 2.02 ms instead of 1.96
+    // chained in launches of one wave that use every SM, us per step (m = 4, as
+    // a graph) of steps whose first launches have 198, 216, 247 and 256 tiles:
+    // 73.05 -> 69.77, 69.77 -> 66.8, 77.3 -> 75.95, 77.95 -> 76.0; with 84 to
+    // 99 tiles the same; chained everywhere, 64 x 64 (8 tiles) took 61.5 us
+    // instead of 59.5 and 4096 x 2048 2.02 ms instead of 1.96
     if (chained && one_wave && 2 * n_tiles >= sm_count() && !a.rhs_only) {
       auto* k = a.stage & 1 ? stage_kernel_mixed<1, true> : stage_kernel_mixed<0, true>;
       return launch_kernel(k, grid, MIXED_THREADS, smem, stream, true, s, sb, f, ra);
