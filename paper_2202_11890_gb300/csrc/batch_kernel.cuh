@@ -142,13 +142,11 @@ __global__ void __launch_bounds__(batch_threads(PREC), 3) batch_kernel(const Bat
 // waits. With no persistent loop around it, the FP32-flux tile fits its
 // registers without spilling while it reads its arguments from the table in
 // global memory.
-// single >= 0: every CTA of the launch takes stage arguments `single` and
-// tile blockIdx.x (a launch over one instance: no work-list load).
 template <int PAR>
 __global__ void __launch_bounds__(MIXED_THREADS, 3)
-    wave_stage_mixed(const StageArgs* __restrict__ tab, const StageWork* __restrict__ work, int single) {
+    wave_stage_mixed(const StageArgs* __restrict__ tab, const StageWork* __restrict__ work) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  const StageWork w = single >= 0 ? StageWork{single, 3 * (int)blockIdx.x} : work[blockIdx.x];
+  const StageWork w = work[blockIdx.x];
   const StageArgs& a = tab[w.args];
   const int t = w.tile / 3, half = w.tile - 3 * t - 1;
   const int tzi = t / a.tiles_x, txi = t - tzi * a.tiles_x;

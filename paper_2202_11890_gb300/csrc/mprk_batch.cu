@@ -313,7 +313,7 @@ void build_wave(const std::vector<BatchInst>& hinst, int groups, std::vector<Sta
         only = bi.args_base + st;
       }
       off[g].push_back((int)work.size());
-      single[g].push_back(n_in == 1 ? only : -1);  // a launch over one instance reads no work list
+      single[g].push_back(n_in == 1 ? only : -1);  // a launch over one instance: launch_stage
     }
     for (int j : members[g]) {
       // bands of rows of one component (finalize_rows in batch_kernel.cuh)
@@ -365,7 +365,7 @@ void wave_step(const WaveLaunches& L, const BatchInst* d_insts, const StageArgs*
       if (one >= 0)
         launch_stage(L.h_args[one], 1, stage_tiles(L.h_args[one]), st, &L.h_maps[L.args_inst[one]]);
       else
-        wave_launch_stage(k & 1, o[k + 1] - o[k], d_args, d_work + o[k], -1, st);
+        wave_launch_stage(k & 1, o[k + 1] - o[k], d_args, d_work + o[k], st);
     }
     wave_launch_finalize(o[launches] - o[launches - 1], d_insts, d_work + o[launches - 1], st);
   }
