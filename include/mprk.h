@@ -173,13 +173,13 @@ int mprk_step_batch(mprk_instance* const* insts, int count, int n_slow_steps);
  * items), the CTAs per SM (1 to 3; with the per-stage form, the number of
  * instance groups, 1, 2 or 4, whose launches run on streams of their own so
  * that one group's launch tail overlaps another's work), and in FP64 the
- * shape of the stage
- * tile of the 256-thread CTA: 32 x 8 cells with one thread per cell or
- * 32 x 4 with two (the FP32-flux tile is 32 x 16). Single-instance FP64
- * stage launches (mprk_step) choose among six tile shapes: 32 x 8, 32 x 4
- * or 32 x 2 cells, with one or two threads per cell. Every shape evaluates
- * the same arithmetic in the same order (Sec. 2.1, App. B), so results are
- * bitwise the same whatever is chosen.
+ * shape of the stage tile: 32 x 8 or 32 x 4 cells, in a CTA of nine warps
+ * (the FP32-flux tile is 32 x 16). Single-instance FP64 stage launches
+ * (mprk_step) choose among six tile shapes: 32 x 8, 32 x 4 or 32 x 2 cells,
+ * with two rows of faces per warp (rows + 1 warps; threads_per_cell 1) or one
+ * (2 rows + 3 warps; threads_per_cell 2). Every shape evaluates the same arithmetic
+ * in the same order (Sec. 2.1, App. B), so results are bitwise the same
+ * whatever is chosen.
  * A process-wide table keeps the fastest choices measured:
  *  - batches: per precision and size bucket (floor(log2) of the mean cells
  *    per instance); without an entry, in FP64 2 tiles per item, every CTA
@@ -187,8 +187,8 @@ int mprk_step_batch(mprk_instance* const* insts, int count, int n_slow_steps);
  *    instance groups;
  *  - single-instance FP64 stage launches: per size bucket (floor(log2) of
  *    the cells of the launch); without an entry, the shortest tile whose
- *    launch fits in one wave of the GPU's SMs, with two threads per cell,
- *    or 32 x 8 with one thread per cell when none fits.
+ *    launch fits in one wave of the GPU's SMs, with 2 rows + 3 warps, or
+ *    32 x 8 with nine warps when none fits.
  * mprk_step_batch, the server and the FP64 stage launches (including graphs
  * captured afterwards by mprk_create) read the table. */
 
@@ -204,8 +204,7 @@ int mprk_batch_tune(mprk_instance* const* insts, int count, int reps, double out
  * cells: writes it and returns 1, or writes the defaults (ctas_per_sm 0:
  * every CTA that fits, or two instance groups; group 0 in FP32 flux: the
  * per-stage form) and
- * returns 0. tile_rows: 8 or 4 in FP64 (one or two threads per cell), 16 in
- * FP32 flux. Needs no device. */
+ * returns 0. tile_rows: 8 or 4 in FP64, 16 in FP32 flux. Needs no device. */
 int mprk_tune_lookup(int precision, double mean_cells, int* group, int* ctas_per_sm, int* tile_rows);
 
 /* Time the six tile shapes of single-instance FP64 stage launches on these
@@ -221,8 +220,8 @@ int mprk_tune_lookup(int precision, double mean_cells, int* group, int* ctas_per
 int mprk_tile_tune(mprk_instance* const* insts, int count, int reps, int* entries);
 
 /* The table's tile shape for a single-instance FP64 stage launch of `cells`
- * cells: writes it (tile rows 8, 4 or 2; threads per cell 1 or 2) and
- * returns 1, or returns 0 when the table has none (the default rule
+ * cells: writes it (tile rows 8, 4 or 2; threads_per_cell 1 for rows + 1
+ * warps, 2 for 2 rows + 3) and returns 1, or returns 0 when the table has none (the default rule
  * applies). Needs no device. */
 int mprk_tile_lookup(double cells, int* tile_rows, int* threads_per_cell);
 
@@ -297,9 +296,12 @@ int mprk_info(const mprk_instance* inst, double* dt, long long* cell_stages_per_
  * rows of R outside [k_lo, k_hi) are left untouched. Asynchronous. */
 int mprk_rhs(mprk_instance* inst, const double* W_dev, double* R_dev, int k_lo, int k_hi);
 
-/* Timing hook: run one slow step (it advances the state) as a CUDA graph
- * captured like the one mprk_step replays, with an event record node before
- * the first launch and after every launch, on the instance stream.
+/* Timing hook: run one slow step (it advances the state) as a CUDA graph of
+ * the launches that mprk_step replays, with an event record node before the
+ * first launch and after every launch, on the instance stream. Each launch
+ * starts when the one before has completed, while mprk_step's overlap at
+ * their ends (and FP32-flux launches of one wave are compiled apart for
+ * that), so the durations add up to more than a step.
  * launch_ms[j] receives the duration of launch j and launch_cells[j] the
  * cell right-hand-side evaluations it made (0 for the step completion); the
  * launches are the s*m stages in order (s = 2 for the Heun base), then the

@@ -67,10 +67,8 @@ struct StageWork {
 // block size of the batch kernel per precision (the tile's own block size)
 constexpr int batch_threads(int prec) { return prec == 0 ? FP64_THREADS : MIXED_THREADS; }
 
-// The persistent kernel of a precision and FP64 tile rows (mprk_kernels.cu,
-// the translation unit of the single-instance stage kernels, so that both
-// kernels call one compiled copy of each FP64 tile body): its shared-memory
-// limit and CTAs per SM, and its launch.
+// The persistent kernel of a precision and FP64 tile rows (mprk_kernels.cu):
+// its shared-memory limit and CTAs per SM, and its launch.
 cudaError_t batch_prepare(int prec, int rows, size_t smem, int* per_sm);
 void batch_launch(int prec, int rows, int grid, size_t smem, cudaStream_t s, const BatchArgs& A);
 // The per-stage form (FP32 flux): one stage launch of `grid` CTAs of stage

@@ -15,7 +15,8 @@
 // stream order (captured in one graph per slow step by mprk_step_batch).
 // This file builds the work lists, plans and tuning; the kernel itself is
 // compiled with the single-instance stage kernels (batch_kernel.cuh, included
-// by mprk_kernels.cu), so that both call one compiled copy of the FP64 tile.
+// by mprk_kernels.cu). Both inline the FP64 tile, whose operations name their
+// rounding, so an instance's results are bitwise the same in either.
 // Since items are taken in list order, every item an item waits on was taken
 // earlier by a CTA that is already running, so the waits always end. Waits
 // are bounded all the same: after a fixed number of clock cycles a CTA sets
@@ -97,7 +98,7 @@ struct Plan {
   int precision = 0;
   int bucket = 0;      // size bucket of the instance set (tuning key)
   int group = 0;       // tiles per work item
-  int rows = TZ;       // FP64 tile rows (TZ, or TZ / 2 with two threads per cell)
+  int rows = TZ;       // FP64 tile rows (TZ or TZ / 2)
   int per_sm = 0;      // CTAs per SM of the persistent launch
   int per_sm_req = 0;  // CTAs per SM asked for (0: as many as fit)
   int n_items = 0;

@@ -24,7 +24,7 @@
 
 namespace mprk {
 
-// Tile of the stage kernel: TX columns by TZ rows, one thread per cell.
+// Tile of the stage kernels: TX columns by TZ rows.
 constexpr int TX = 32;
 constexpr int TZ = 8;
 constexpr int NTHREADS = TX * TZ;
@@ -255,7 +255,8 @@ struct StageMaps {
 cudaError_t make_stage_maps(const Geom& g, const Bufs& b, StageMaps* out);
 
 // Shape of the FP64 stage tile: rows per tile (TZ, TZ/2 or TZ/4, with TX
-// columns) and threads per cell (1 or 2). Every shape computes the same
+// columns) and tpc: 1 for two face jobs per warp (rows + 1 warps), 2 for one (2
+// rows + 3; the tables' "threads per cell"). Every shape computes the same
 // arithmetic in the same order, so results do not depend on it.
 struct TileShape {
   int rows, tpc;

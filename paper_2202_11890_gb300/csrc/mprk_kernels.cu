@@ -199,8 +199,9 @@ cudaError_t launch_fp64(const StageArgs& a, int n_tiles, bool wide, cudaStream_t
 }  // namespace
 
 TileShape default_tile_shape(const StageArgs& a) {
-  // One SM completes two FP64 operations per clock, so a launch of fewer
-  // tiles than SMs is bound by the FP64 work of one tile.
+  // A launch of fewer tiles than SMs takes as long as one tile: its chain of
+  // staging, faces and combination, shortest with few rows and a warp per
+  // face job.
   const int sms = sm_count();
   StageArgs s = a;
   int n = 0;

@@ -828,10 +828,9 @@ int mprk_profile_step(mprk_instance* I, double* launch_ms, long long* launch_cel
   if (!I) return fail(MPRK_EINVAL, "instance is NULL");
   const Geom& g = I->g;
   const int n = g.s * g.m + 1;
-  // The step is captured exactly as the one mprk_step replays, with an
-  // event record node before the first launch and after
-  // each launch on the instance stream, and runs as a graph: each duration
-  // is then the kernel as the step graph runs it.
+  // The launches of the step that mprk_step replays, with an event record
+  // node before the first and after each on the instance stream, run as a
+  // graph. Not chained: the events stand between them.
   cudaEvent_t ev[4 * 64 + 2];
   int made = 0;
   int rc = MPRK_OK;

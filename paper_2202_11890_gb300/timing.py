@@ -40,10 +40,10 @@ def stage_kernel_times(h: int, stream_ptr: int, reps: int = 3):
     """(ms, cell-stages, share): the summed duration of the stage-kernel
     launches of one slow step, the cell-stages they computed, and their
     share of the step's launches, medians over `reps` slow steps run as a
-    graph with an event node after every launch. The event nodes add a gap
-    before each launch, so the durations run a little long; their share
-    scaled by the plain graph's step time bounds the kernel's own time
-    (see kernel_ms_per_step)."""
+    graph with an event node after every launch. The launches run one after
+    another there, while mprk_step's overlap at their ends, so the durations
+    run a little long; their share scaled by the plain graph's step time
+    bounds the kernel's own time (see kernel_ms_per_step)."""
     tot, share, cells = [], [], None
     for _ in range(reps):
         ms, c = M.mprk_profile_step(h)
@@ -57,6 +57,7 @@ def stage_kernel_times(h: int, stream_ptr: int, reps: int = 3):
 def kernel_ms_per_step(step_ms: float, share: float) -> float:
     """The stage kernel's time per slow step inside the step graph: its share
     of the launches (event-timed) times the plain graph's step time. It
-    counts the gaps between launches to the kernels in proportion, so it is
-    an upper bound of their busy time, and never exceeds the step."""
+    counts the gaps between launches to the kernels in proportion, and takes
+    the share from launches that do not overlap, so it is an upper bound of
+    their busy time, and never exceeds the step."""
     return step_ms * share
