@@ -54,13 +54,14 @@ extern "C" {
 #define MPRK_ENOTFOUND (-9)  /* unknown ticket                             */
 
 /* ---- enumerations ------------------------------------------------------ */
-#define MPRK_FP64 0     /* state, stage values, combinations and the fluxes of
-                           the tangential momenta in double; the fluxes of mass,
-                           normal momentum and energy in 64-bit fixed point with
-                           an absolute rounding of a few 2^-57 where a face's
+#define MPRK_FP64 0     /* state, stage values and combinations in double. The
+                           face fluxes in double too, except where a face's
                            states are near one (density in [0.5, 4), |momentum|
                            < 0.656, energy in [1/16, 4), sound speed squared in
-                           [0.26, 3.9]), in double elsewhere                   */
+                           [0.26, 3.9]): there in 64-bit integers, those of mass,
+                           normal momentum and energy with an absolute rounding
+                           of a few 2^-57, those of the tangential momenta with
+                           one of 2^-55 of the momenta themselves              */
 #define MPRK_FP32FLUX 1 /* fluxes and RHS in float; stage values, the buffer
                            accumulation and all stage combinations in double  */
 

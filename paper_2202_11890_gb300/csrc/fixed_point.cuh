@@ -170,8 +170,26 @@ __host__ __device__ __forceinline__ i64 to_double(i64 x, int s) {
   const int z = __builtin_clzll(a);
 #endif
   const u64 m = ((a << z >> 10) + 1) >> 1;
-  return (i64)(((u64)(1085 - s - z) << 52) + m) | (x & (i64)(1ull << 63));
+  const int e = 1085 - s - z;
+  if (e <= 0) return 0;  // below the normal doubles
+  return (i64)(((u64)e << 52) + m) | (x & (i64)(1ull << 63));
 }
+
+// A double below one in magnitude as a signed 53-bit mantissa, its leading one
+// at bit 62, over its 10-bit exponent field (subnormals as zero); and such a
+// mantissa with its leading one at bit 58 for the exponent field e, its own or
+// a larger one.
+__host__ __device__ __forceinline__ i64 pack(i64 bits) {
+  const int e = (int)((u64)bits >> 52 & 0x7ff);
+  const i64 m = (i64)(((u64)bits << 10 & 0x3fffffffffffffffull) | 1ull << 62), n = bits >> 63;
+  return e == 0 ? 0 : ((m ^ n) - n) | e;
+}
+__host__ __device__ __forceinline__ int pack_exp(i64 w) { return (int)w & 1023; }
+__host__ __device__ __forceinline__ i64 shr(i64 x, int s) { return x >> (s < 63 ? s : 63); }
+__host__ __device__ __forceinline__ i64 unpack(i64 w, int e) { return shr(w & ~1023ll, 4 + e - pack_exp(w)); }
+// The velocity of a cell, .59 of 2^(its momentum's exponent - 1023), from the
+// packed momentum and 1/rho .61.
+__host__ __device__ __forceinline__ i64 packed_velocity(i64 w, FxW inv) { return mul(split(w & ~1023ll), inv); }
 
 // A double of a cell state within the bounds above, as an integer of scale
 // s (truncated toward zero; exact when its last bit is at least 2^-s).

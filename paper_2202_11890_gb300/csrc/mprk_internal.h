@@ -50,6 +50,11 @@ constexpr unsigned ST_TIMEOUT = 4u;
 struct FxW {
   int lo, hi;
 };
+// A factor in (0, 1) scaled to [1/2, 1): f 2^-62 2^-s.
+struct FxN {
+  FxW f;
+  int s;
+};
 // Coefficients of the viscous face flux over half the divergence factor.
 enum {
   FXC_A,  // (8/3) mu / d_n: sigma_nn from the normal difference of u_n
@@ -81,7 +86,8 @@ struct FxConst {
   FxW gg;              // gamma (gamma - 1).62
   FxW lid[LID_N];      // interface, .62
   FxW fc[2][2][FXC_N]; // viscous coefficients per direction (x, z) and fluid, .62
-  double tc[2][2][2];  // of them C and D in double, for the tangential momentum
+  FxN tc[2][2][2];     // of them C and D for the tangential stress
+  FxN ts;              // LID_S likewise
   double tlid[LID_N];  // the interface's factors in double, LID_1 and LID_2 doubled
 };
 
@@ -101,6 +107,7 @@ struct Fx3Const {
   FxConst k;  // its fc and tc unused; square: dx = dy = dz1 = dz2
   FxW fc[3][2][F3_N];
   double fd[3][2][F3_N];
+  FxN tc[3][2][3];  // C, D1, D2 for the tangential stresses
   double scale_y;  // 2^-57 of half of 1/dy
 };
 

@@ -314,6 +314,11 @@ static FxW fx_factor(double x, int digits) {
   w.hi = (int)((v - w.lo) >> 32);
   return w;
 }
+static FxN fx_scaled(double x) {
+  int e = 0;
+  const double m = frexp(x, &e);  // x in (0, 1): e <= 0
+  return FxN{fx_factor(m, 62), -e};
+}
 // The constants shared by 2-D and 3-D, with `on` and `square` clear; false
 // where gamma does not fit.
 static bool fx_gas(const Geom& g, FxConst* out) {
@@ -331,6 +336,7 @@ static bool fx_gas(const Geom& g, FxConst* out) {
     if (ok) out->lid[j] = fx_factor(x, 62);
   }
   if (!ok) return false;
+  out->ts = fx_scaled(out->tlid[LID_S]);
   out->gm1 = fx_factor(g.gm1, 61);
   out->gg = fx_factor(gg, 62);
   return true;
@@ -350,7 +356,7 @@ void mprk::fixed_point_const(const Geom& g, FxConst* out) {
         const double x = visc_coef(g, dir, fl, j);
         ok = ok && std::fabs(x) < 1.0;  // false for NaN
         if (ok) f.fc[dir][fl][j] = fx_factor(x, 62);
-        if (j == FXC_C || j == FXC_D) f.tc[dir][fl][j - FXC_C] = x;
+        if (ok && (j == FXC_C || j == FXC_D)) f.tc[dir][fl][j - FXC_C] = fx_scaled(x);
       }
   f.on = ok;
 }
@@ -372,6 +378,7 @@ void mprk::fixed_point_const3(const Geom& g, Fx3Const* out) {
         f.fc[dir][fl][j] = FxW{};
         ok = ok && std::fabs(v[j]) < 1.0;
         if (ok) f.fc[dir][fl][j] = fx_factor(v[j], 62);
+        if (ok && j >= F3_C && j <= F3_D2) f.tc[dir][fl][j - F3_C] = fx_scaled(v[j]);
       }
     }
   f.k.on = ok;

@@ -23,11 +23,11 @@
 // (fixed_point.cuh): as double arithmetic the faces were 300 of the tile's 309
 // operations per cell on a pipe that completes two per clock and SM, which
 // bound every FP64 launch: the pipe was 86 % busy. The flux of the tangential
-// momentum stays in double, because nothing in it is as large as density or
-// pressure: in fixed point a shear of 1e-6 in a flow uniform along x had 3e4
-// times the double form's error. Measured: a slow step of 2048 x 1024 cells
-// with m = 8 11.7 -> 2.84 ms (2.06 with that flux in fixed point too), 64 x 64
-// with m = 4 167 -> 62 us (55). A face with a state outside the fixed-point
+// momentum has no term as large as density or pressure (in fixed point a shear
+// of 1e-6 in a flow uniform along x had 3e4 times the double form's error), so
+// its integers carry an exponent (fixed_flux.cuh). Measured: a slow step of
+// 2048 x 1024 cells with m = 8 11.7 -> 2.37 ms (2.06 with that flux in fixed
+// point too), 64 x 64 with m = 4 185 -> 63.5 us (58.4). A face with a state outside the fixed-point
 // range takes the same formulas in double (slow_faces); which form a face
 // takes depends on its own cells alone, so results do not depend on the tile
 // shape or the launch.
@@ -44,8 +44,9 @@ struct TileSmem {
   double q[4][TZR + 4][TX + 4];  // stage state, rows k0-2.., cols i0-2..
   i64 qi[4][TZR + 4][TX + 4];    // the same: rho, rho E .58, momenta .60
   i64 v[3][TZR + 2][TX + 2];     // u, w, e (.59), rows k0-1.., cols i0-1..
-  double vd[2][TZR + 2][TX + 2];  // u, w
-  // face fluxes over half the divergence factor (.57; the tangential momentum
+  i64 qw[2][TZR + 4][TX + 4];     // rho u, rho w packed (fixed_point.cuh)
+  i64 vp[2][TZR + 2][TX + 2];     // u, w under the exponents of qw
+  // face fluxes over half the divergence factor (.57; the tangential momentum's
   // and every component of a slow face as the bits of a double)
   i64 fx[4][TZR][TX + 1];  // face f between cols f-1, f
   i64 fz[4][TZR + 1][TX];  // seen from above at the interface
@@ -216,10 +217,9 @@ struct Arith<double> {
 };
 
 // u, w, e of the cell of halo row rr, column cc into the ring (phase 1); in
-// fixed point also u and w in double (q: the state).
+// fixed point also u and w from the packed momenta.
 template <typename T, int TZR>
-__device__ __forceinline__ void ring_cell(const Geom& g, TileSmem<TZR>& S, int rr, int cc, int i0, T r, T mu, T mw, T E,
-                                          const double* q = nullptr) {
+__device__ __forceinline__ void ring_cell(const Geom& g, TileSmem<TZR>& S, int rr, int cc, int i0, T r, T mu, T mw, T E) {
   constexpr int VP = (TZR + 2) * (TX + 2);
   if (rr < 1 || rr > TZR + 2 || cc < 1 || cc > TX + 2) return;
   T* v = reinterpret_cast<T*>(&S.v[0][0][0]) + (rr - 1) * (TX + 2) + cc - 1;
@@ -230,10 +230,11 @@ __device__ __forceinline__ void ring_cell(const Geom& g, TileSmem<TZR>& S, int r
   v[0] = o[0];
   v[VP] = flip ? -o[1] : o[1];
   v[2 * VP] = o[2];
-  if (q) {
-    const double id = __longlong_as_double(fx::to_double((i64)inv, 61)), w = __dmul_rn(q[2], id);
-    S.vd[0][rr - 1][cc - 1] = __dmul_rn(q[1], id);
-    S.vd[1][rr - 1][cc - 1] = flip ? -w : w;
+  if constexpr (sizeof(inv) == 8 && (T)0.5 == (T)0) {
+    const FxW iw = fx::split(inv);
+    const i64 w = fx::packed_velocity(S.qw[1][rr][cc], iw);
+    S.vp[0][rr - 1][cc - 1] = fx::packed_velocity(S.qw[0][rr][cc], iw);
+    S.vp[1][rr - 1][cc - 1] = flip ? -w : w;
   }
 }
 
@@ -263,6 +264,45 @@ __device__ __forceinline__ double lid_work(const FxConst& k, double u1, double u
 }
 __device__ __forceinline__ double lid_heat(const FxConst& k, double e1, double e2) {
   return __dmul_rn(k.tlid[LID_T], __dsub_rn(e2, e1));
+}
+
+// ---- aligned velocity differences of the tangential stresses ----------------
+// u: a cell's velocity under its momentum's exponent, w: the packed momentum
+// or that exponent; vs, qs (vt, qt): the strides of either along the face normal (across it).
+// The two cells at the face are at 0 and vs.
+__device__ __forceinline__ FxA vel_diff(const i64* u, const i64* w, int vs, int qs) {
+  const int a = fx::pack_exp(w[0]), b = fx::pack_exp(w[qs]), e = max(a, b);
+  return FxA{vel_at(u[vs], b, e) - vel_at(u[0], a, e), e};
+}
+// The sum of both cells' central differences across the normal.
+template <typename W>
+__device__ __forceinline__ FxA vel_cross(const i64* u, const W* w, int vs, int qs, int vt, int qt) {
+  const int a = fx::pack_exp(w[-qt]), b = fx::pack_exp(w[qt]), c = fx::pack_exp(w[qs - qt]), d = fx::pack_exp(w[qs + qt]);
+  const int e = max(max(a, b), max(c, d));
+  return FxA{(vel_at(u[vt], b, e) - vel_at(u[-vt], a, e)) + (vel_at(u[vs + vt], d, e) - vel_at(u[vs - vt], c, e)), e};
+}
+// The same along z for a component tangential to walls and interface, of the
+// cells ua and ub of row k, with the ghosts 2 (wall state) - cell beyond them.
+template <typename W>
+__device__ __forceinline__ FxA dz_pair(const Geom& g, const FxConst& c, int k, const i64* ua, const i64* ub, int vr,
+                                       const W* wa, const W* wb, int qr) {
+  const bool top = k + 1 == g.nz || k + 1 == g.n1, bot = k == 0 || k == g.n1;
+  int e = max(max(fx::pack_exp(wa[-qr]), fx::pack_exp(wa[qr])), max(fx::pack_exp(wb[-qr]), fx::pack_exp(wb[qr])));
+  if (top || bot) e = max(e, max(fx::pack_exp(wa[0]), fx::pack_exp(wb[0])));
+  i64 sum = 0;
+#pragma unroll
+  for (int s = 0; s < 2; s++) {
+    const i64* u = s ? ub : ua;
+    const W* w = s ? wb : wa;
+    i64 up = vel_at(u[vr], fx::pack_exp(w[qr]), e), dn = vel_at(u[-vr], fx::pack_exp(w[-qr]), e);
+    if (top || bot) {
+      const i64 own = vel_at(u[0], fx::pack_exp(w[0]), e);
+      if (top) up = k + 1 == g.nz ? (g.wall ? own : -own) : lid_ghost(g, c, 0, own, up);
+      if (bot) dn = k == 0 ? (g.wall ? own : -own) : lid_ghost(g, c, 1, own, dn);
+    }
+    sum += up - dn;
+  }
+  return FxA{sum, e};
 }
 
 // ---- phase 2: face fluxes ---------------------------------------------------
@@ -490,69 +530,57 @@ __device__ __forceinline__ void double_visc(const double* fc, const double vL[5]
   V[2] = __fma_rn(0.5, us, __dmul_rn(fc[FXC_K], __dsub_rn(vR[2], vL[2])));
 }
 
-// The tangential viscous flux sigma_nt over half the divergence factor, in
-// double, of face id in fluid fl (2: the interface), with the ghosts of
-// face_sides; and the flux of the tangential momentum (tan_flux) from it.
+// The tangential stress of face id in fluid fl (2: the interface), with the
+// ghosts of face_sides; and the flux of the tangential momentum from it.
 template <int TZR>
-__device__ __forceinline__ double visc_tan(const Geom& g, const FxConst& fk, const TileSmem<TZR>& S, const FaceId& id,
-                                           int fl) {
-  constexpr int VS = TX + 2;
-  const int ku = id.ku;
-  const double* u = &S.vd[0][id.isx ? id.f + 1 : id.f][id.isx ? id.c : id.c + 1];
-  const double* w = u + (TZR + 2) * VS;
-  if (id.isx) {
-    const bool top = ku + 1 == g.nz || ku + 1 == g.n1, bot = ku == 0 || ku == g.n1;
-    double gn = 0.0;
-#pragma unroll
-    for (int s = 0; s < 2; s++) {
-      const double c = u[s];
-      double up = u[s + VS], dn = u[s - VS];
-      if (top) up = ku + 1 == g.nz ? (g.wall ? c : -c) : lid_ghost(g, fk, 0, c, up);
-      if (bot) dn = ku == 0 ? (g.wall ? c : -c) : lid_ghost(g, fk, 1, c, dn);
-      gn = s ? __dadd_rn(gn, __dsub_rn(up, dn)) : __dsub_rn(up, dn);
-    }
-    return __fma_rn(fk.tc[0][fl][0], __dsub_rn(w[1], w[0]), __dmul_rn(fk.tc[0][fl][1], gn));
+__device__ __forceinline__ FxStress visc_tan(const Geom& g, const FxConst& fk, const TileSmem<TZR>& S, const FaceId& id,
+                                             int fl) {
+  constexpr int VS = TX + 2, QS = TX + 4;
+  const int ku = id.ku, r = id.isx ? id.f + 1 : id.f, c = id.isx ? id.c : id.c + 1;
+  const i64* u = &S.vp[0][r][c];  // of the first cell at the face
+  const i64* w = &S.vp[1][r][c];
+  const i64* mu = &S.qw[0][r + 1][c + 1];
+  const i64* mw = &S.qw[1][r + 1][c + 1];
+  if (id.isx)
+    return tan_stress(fk.tc[0][fl][0], vel_diff(w, mw, 1, 1), fk.tc[0][fl][1],
+                      dz_pair(g, fk, ku, u, u + 1, VS, mu, mu + 1, QS));
+  if (ku == 0 || ku == g.nz) {  // the ghost's u is +-u and its difference of w the opposite
+    if (g.wall) return FxStress{0, 0};
+    const int e = fx::pack_exp(ku == 0 ? mu[QS] : mu[0]);
+    const i64 x = vel_at(ku == 0 ? u[VS] : u[0], e, e) << 1;
+    return tan_stress(fk.tc[1][fl][0], FxA{ku == 0 ? x : -x, e});
   }
-  if (fl == 2) return __dmul_rn(fk.tlid[LID_S], __dsub_rn(u[VS], u[0]));
-  if (ku == 0 || ku == g.nz)  // the ghost's u is +-u and its difference of w the opposite
-    return g.wall ? 0.0 : __dmul_rn(fk.tc[1][fl][0], ku == 0 ? __dmul_rn(2.0, u[VS]) : __dmul_rn(-2.0, u[0]));
-  return __fma_rn(fk.tc[1][fl][0], __dsub_rn(u[VS], u[0]),
-                  __dmul_rn(fk.tc[1][fl][1], __dadd_rn(__dsub_rn(w[1], w[-1]), __dsub_rn(w[VS + 1], w[VS - 1]))));
+  const FxA du = vel_diff(u, mu, VS, QS);
+  if (fl == 2) return tan_stress(fk.ts, du);
+  return tan_stress(fk.tc[1][fl][0], du, fk.tc[1][fl][1], vel_cross(w, mw, VS, QS, 1, 1));
 }
 template <int TZR>
-__device__ __forceinline__ double face_tan(const Geom& g, const TileSmem<TZR>& S, const FaceId& id, const FxTan& t,
-                                           double V) {
+__device__ __forceinline__ i64 face_tan(const Geom& g, const TileSmem<TZR>& S, const FaceId& id, const FxTan& t,
+                                        FxStress V) {
   constexpr int QS = TX + 4;
   const int n1 = g.n1, nz = g.nz, ku = id.ku;
   if (id.isx) {
-    const double* q = &S.q[2][id.f + 2][id.c];
+    const i64* q = &S.qw[1][id.f + 2][id.c];
     return tan_flux(t, q[0], q[1], q[2], q[3], V);
   }
-  const double* q = &S.q[1][id.f][id.c + 2];
-  const bool edge = ku == 0 || ku == nz || ku == n1, from_above = ku == 0 || (ku == n1 && !id.below);
-  double a0 = q[0], a1 = q[QS], a2 = q[2 * QS], a3 = q[3 * QS];
-  if (edge) {
-    if (from_above) a1 = a2;
-    else a2 = a1;
-  }
-  if (ku == 1 || ku == n1 + 1) a0 = a1;
-  if (ku == nz - 1 || ku == n1 - 1) a3 = a2;
-  if (!edge) return tan_flux(t, a0, a1, a2, a3, V);
-  const double m = from_above ? __fma_rn(0.25, __dsub_rn(a1, a3), a2) : __fma_rn(0.25, __dsub_rn(a2, a0), a1);
-  return tan_flux(t, m, m, V);
+  const i64* q = &S.qw[0][id.f][id.c + 2];
+  const i64 a1 = q[QS], a2 = q[2 * QS];
+  if (ku == 0 || ku == nz || ku == n1) return tan_flux(t, 0, 0, 0, 0, V);  // nothing flows through
+  return tan_flux(t, ku == 1 || ku == n1 + 1 ? a1 : q[0], a1, a2, ku == nz - 1 || ku == n1 - 1 ? a2 : q[3 * QS], V);
 }
 template <bool X, int TZR>
-__device__ __forceinline__ double visc_tan_plain(const FxConst& fk, const TileSmem<TZR>& S, const FaceId& id, int fl) {
-  constexpr int vs = X ? 1 : TX + 2, vt = X ? TX + 2 : 1;
-  const double* un = &S.vd[X ? 0 : 1][X ? id.f + 1 : id.f][X ? id.c : id.c + 1];
-  const double* ut = &S.vd[X ? 1 : 0][X ? id.f + 1 : id.f][X ? id.c : id.c + 1];
-  const double gn = __dadd_rn(__dsub_rn(un[vt], un[-vt]), __dsub_rn(un[vs + vt], un[vs - vt]));
-  return __fma_rn(fk.tc[X ? 0 : 1][fl][0], __dsub_rn(ut[vs], ut[0]), __dmul_rn(fk.tc[X ? 0 : 1][fl][1], gn));
+__device__ __forceinline__ FxStress visc_tan_plain(const FxConst& fk, const TileSmem<TZR>& S, const FaceId& id, int fl) {
+  constexpr int VS = TX + 2, QS = TX + 4;
+  const int r = X ? id.f + 1 : id.f, c = X ? id.c : id.c + 1;
+  constexpr int n = X ? 0 : 1, t = 1 - n;  // planes of the normal and the tangential component
+  return tan_stress(fk.tc[t ? 0 : 1][fl][0], vel_diff(&S.vp[t][r][c], &S.qw[t][r + 1][c + 1], X ? 1 : VS, X ? 1 : QS),
+                    fk.tc[t ? 0 : 1][fl][1],
+                    vel_cross(&S.vp[n][r][c], &S.qw[n][r + 1][c + 1], X ? 1 : VS, X ? 1 : QS, X ? VS : 1, X ? QS : 1));
 }
 template <bool X, int TZR>
-__device__ __forceinline__ double face_tan_plain(const TileSmem<TZR>& S, const FaceId& id, const FxTan& t, double V) {
+__device__ __forceinline__ i64 face_tan_plain(const TileSmem<TZR>& S, const FaceId& id, const FxTan& t, FxStress V) {
   constexpr int qs = X ? 1 : TX + 4;
-  const double* q = &S.q[X ? 2 : 1][X ? id.f + 2 : id.f][X ? id.c : id.c + 2];
+  const i64* q = &S.qw[X ? 1 : 0][X ? id.f + 2 : id.f][X ? id.c : id.c + 2];
   return tan_flux(t, q[0], q[qs], q[2 * qs], q[3 * qs], V);
 }
 
@@ -685,6 +713,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
         S.q[c][rr][cc] = 0.0;
         S.qi[c][rr][cc] = 0;
       }
+      S.qw[0][rr][cc] = S.qw[1][rr][cc] = 0;
       continue;
     }
     bool gh;
@@ -710,8 +739,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
       t[c] = c == 1 || c == 2 ? fx::from_double(__double_as_longlong(val[c]), fx::S_MOM - 2)
                               : fx::from_positive(__double_as_longlong(val[c]), fx::S_RHO - 2);
       S.qi[c][rr][cc] = t[c];
+      if (c == 1 || c == 2) S.qw[c - 1][rr][cc] = fx::pack(__double_as_longlong(val[c]));
     }
-    ring_cell<i64, TZR>(g, S, rr, cc, i0, t[0], t[1], t[2], t[3], val);
+    ring_cell<i64, TZR>(g, S, rr, cc, i0, t[0], t[1], t[2], t[3]);
   }
   const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZR);
   bad = __syncthreads_or(bad);
@@ -729,7 +759,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
     i64 L[4], R[4], vL[5], vR[5], Vn = 0, VE, F[4];
     int fl;
     bool ok = true;
-    double Vt;
+    FxStress Vt;
     if (plain) {
       if (!face_id_plain<TZR>(job, lane, k0, &id)) continue;
       fl = k0 >= n1;
@@ -749,16 +779,16 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
       }
     }
     if (ok) {
-      const i64 snt = fx::from_double(__double_as_longlong(Vt), fx::S_VEL);
+      const i64 snt = stress59(Vt);
       if (fl < 2) fx_visc(a.fx.fc[id.isx ? 0 : 1][fl], vL, vR, snt, &Vn, &VE);
       else VE = lid_work(a.fx, vL[1], vR[1], snt) + lid_heat(a.fx, vL[2], vR[2]);
       FxTan t;
       ok = fx_flux<2>(g, a.fx, L, R, Vn, VE, F, &t);
       if (ok) {
         F[3] = F[2];
-        F[2] = __double_as_longlong(!plain    ? face_tan<TZR>(g, S, id, t, Vt)
-                                    : id.isx ? face_tan_plain<true, TZR>(S, id, t, Vt)
-                                             : face_tan_plain<false, TZR>(S, id, t, Vt));
+        F[2] = !plain   ? face_tan<TZR>(g, S, id, t, Vt)
+               : id.isx ? face_tan_plain<true, TZR>(S, id, t, Vt)
+                        : face_tan_plain<false, TZR>(S, id, t, Vt);
         store_flux(S, id, F);
       }
     }

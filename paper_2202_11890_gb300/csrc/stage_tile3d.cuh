@@ -18,8 +18,8 @@
 // As in the 2-D tile, the fluxes of mass, normal momentum and energy run in
 // 64-bit fixed point (fixed_point.cuh), because the double pipe bound both
 // kernels (80 to 86 % busy with 125 + 238 operations per cell), and those of
-// the tangential momenta in double. Measured: a slow step of 512 x 64 x 200
-// cells with m = 4 44.1 -> 14.9 ms. A face whose own cells leave
+// the tangential momenta in integers with an exponent. Measured: a slow step
+// of 512 x 64 x 200 cells with m = 4 44.1 -> 11.3 ms. A face whose own cells leave
 // the range is evaluated in double by a second pass over the tile; which form
 // a face takes depends on its cells alone, so neighbouring tiles agree on the
 // faces they share. Fluxes come over half the divergence factor of their
@@ -133,8 +133,8 @@ struct Arith3<i64> {
     return fx::from_double(__double_as_longlong(q), c == 0 || c == 4 ? fx::S_RHO - 2 : fx::S_MOM - 2);
   }
   static __device__ __forceinline__ i64 rec(i64 a, i64 up, i64 dn) { return (a << 2) + (up - dn); }
-  // u, v, w, e of a cell; 1/rho in double
-  static __device__ __forceinline__ double prims(const i64 q[5], i64 v[4]) {
+  // u, v, w, e of a cell; 1/rho .61
+  static __device__ __forceinline__ i64 prims(const i64 q[5], i64 v[4]) {
     const i64 inv_ = fx::recip(q[0] << 2);
     const FxW inv = fx::split(inv_);
     i64 k = 0;
@@ -145,7 +145,7 @@ struct Arith3<i64> {
       k += fx::mul(m, fx::split(v[c]));
     }
     v[3] = fx::mul(fx::split((q[4] - k) << 2), inv) << 2;  // k .57: k/2 .58
-    return __longlong_as_double(fx::to_double(inv_, 61));
+    return inv_;
   }
 };
 template <>
@@ -244,8 +244,11 @@ constexpr int RING3 = (TZ + 2) * (TX + 2);  // tile plus a one-cell ring
 struct YfaceSmem {
   i64 q[2][5][TZ + 2][TX + 2];    // planes j and j+1, rows k0-1.., cols i0-1..
   i64 v[2][4][TZ + 2][TX + 2];    // u, v, w, e on the ring
-  double vd[2][3][TZ + 2][TX + 2];  // u, v, w
-  double qd[2][2][TZ][TX];        // rho u, rho w of the tile's cells
+  // packed momenta (fixed_point.cuh) and velocities under their exponents: u
+  // and w in the tile's cells, v on the ring with its exponents alone
+  i64 vn[2][TZ + 2][TX + 2];
+  short wn[2][TZ + 2][TX + 2];
+  i64 wt[2][2][TZ][TX], vt[2][2][TZ][TX];
   unsigned char ok[2][TZ + 2][TX + 2];
 };
 
@@ -265,13 +268,15 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
   const int j1 = wrap3(j + 1, g.ny);
   T* Sq = reinterpret_cast<T*>(&S.q[0][0][0][0]);
   T* Sv = reinterpret_cast<T*>(&S.v[0][0][0][0]);
-  double* Sd = &S.vd[0][0][0][0];
   bool bad = false;
   for (int e = tid; e < 2 * RING3; e += NTHREADS) {
     const int side = e >= RING3, rem = e - side * RING3;
     const int rr = rem / (TX + 2), cc = rem - rr * (TX + 2);
     const int k = k0 - 1 + rr;
-    if (k < 0 || k >= nz) continue;
+    if (k < 0 || k >= nz) {
+      if (FX) S.wn[side][rr][cc] = 0;
+      continue;
+    }
     double q[5];
     stage_val3(a, G, k, side ? j1 : j, wrap3(i0 - 1 + cc, g.nx), q);
     bool in = true;
@@ -287,15 +292,21 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
       t[c] = Arith3<T>::cell(q[c], c);
       Sq[(side * 5 + c) * RING3 + rem] = t[c];
     }
-    const double inv = Arith3<T>::prims(t, v);
+    const T inv = Arith3<T>::prims(t, v);
 #pragma unroll
     for (int c = 0; c < 4; c++) Sv[(side * 4 + c) * RING3 + rem] = v[c];
-    if (FX) {
-#pragma unroll
-      for (int c = 0; c < 3; c++) Sd[(side * 3 + c) * RING3 + rem] = __dmul_rn(q[c + 1], inv);
+    if constexpr (FX) {
+      const FxW iw = fx::split(inv);
+      const i64 w = fx::pack(__double_as_longlong(q[2]));
+      S.wn[side][rr][cc] = (short)fx::pack_exp(w);
+      S.vn[side][rr][cc] = fx::packed_velocity(w, iw);
       if (rr >= 1 && rr <= TZ && cc >= 1 && cc <= TX) {
-        S.qd[side][0][rr - 1][cc - 1] = q[1];
-        S.qd[side][1][rr - 1][cc - 1] = q[3];
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+          const i64 m = fx::pack(__double_as_longlong(q[2 * c + 1]));
+          S.wt[side][c][rr - 1][cc - 1] = m;
+          S.vt[side][c][rr - 1][cc - 1] = fx::packed_velocity(m, iw);
+        }
       }
     }
   }
@@ -304,18 +315,18 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
   const bool mine = k < row_hi && i < g.nx;
   // the outer two of the four cells across the face
   T am[5], ap[5];
-  double dm[2], dp[2];  // their rho u, rho w
+  i64 wm[2], wp[2];  // their rho u, rho w packed
   bool out_ok = true;
   if (mine && want) {
     double q[5];
     stage_val3(a, G, k, wrap3(j - 1, g.ny), i, q);
     out_ok = cell_in_range3(q);
-    dm[0] = q[1], dm[1] = q[3];
+    if (FX) wm[0] = fx::pack(__double_as_longlong(q[1])), wm[1] = fx::pack(__double_as_longlong(q[3]));
 #pragma unroll
     for (int c = 0; c < 5; c++) am[c] = Arith3<T>::cell(q[c], c);
     stage_val3(a, G, k, wrap3(j + 2, g.ny), i, q);
     out_ok = out_ok && cell_in_range3(q);
-    dp[0] = q[1], dp[1] = q[3];
+    if (FX) wp[0] = fx::pack(__double_as_longlong(q[1])), wp[1] = fx::pack(__double_as_longlong(q[3]));
 #pragma unroll
     for (int c = 0; c < 5; c++) ap[c] = Arith3<T>::cell(q[c], c);
   }
@@ -361,28 +372,25 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
   }
   i64 F[5];
   if constexpr (FX) {
-    const double* d = Sd + at;  // plane j; the next plane 3 RING3 behind
-    const double* f = C.fd[1][k >= n1];
-    double gx = 0.0, gz = 0.0, sig[2];
-#pragma unroll
-    for (int side = 0; side < 2; side++) {
-      const double* v = d + (3 * side + 1) * RING3;
-      const double x = __dsub_rn(v[1], v[-1]), z = dz_vel(g, C.k, k, 1, v, TX + 2);
-      gx = side ? __dadd_rn(gx, x) : x;
-      gz = side ? __dadd_rn(gz, z) : z;
-    }
-    sig[0] = __fma_rn(f[F3_C], __dsub_rn(d[3 * RING3], d[0]), __dmul_rn(f[F3_D1], gx));
-    sig[1] = __fma_rn(f[F3_C], __dsub_rn(d[5 * RING3], d[2 * RING3]), __dmul_rn(f[F3_D2], gz));
+    const FxN* tc = C.tc[1][k >= n1];
+    const i64* vn = &S.vn[0][rr + 1][cc + 1];
+    const short* wn = &S.wn[0][rr + 1][cc + 1];
+    const i64* vt = &S.vt[0][0][rr][cc];
+    const i64* wt = &S.wt[0][0][rr][cc];
+    constexpr int CELLS = TZ * TX;
+    const FxStress sig[2] = {
+        tan_stress(tc[0], vel_diff(vt, wt, 2 * CELLS, 2 * CELLS), tc[1], vel_cross(vn, wn, RING3, RING3, 1, 1)),
+        tan_stress(tc[0], vel_diff(vt + CELLS, wt + CELLS, 2 * CELLS, 2 * CELLS), tc[2],
+                   dz_pair(g, C.k, k, vn, vn + RING3, TX + 2, wn, wn + RING3, TX + 2))};
     i64 Vn, VE, o[3];
     FxTan t;
-    const i64 snt[2] = {fx::from_double(__double_as_longlong(sig[0]), fx::S_VEL),
-                        fx::from_double(__double_as_longlong(sig[1]), fx::S_VEL)};
+    const i64 snt[2] = {stress59(sig[0]), stress59(sig[1])};
     visc3(C.fc[1][k >= n1], s[0], s[1], snt, &Vn, &VE);
     if (!fx_flux<3>(g, C.k, L, R, Vn, VE, o, &t)) return false;
     F[0] = o[0], F[1] = o[1], F[4] = o[2];
 #pragma unroll
     for (int c = 0; c < 2; c++)
-      F[2 + c] = __double_as_longlong(tan_flux(t, dm[c], S.qd[0][c][rr][cc], S.qd[1][c][rr][cc], dp[c], sig[c]));
+      F[2 + c] = tan_flux(t, wm[c], wt[c * CELLS], wt[(2 + c) * CELLS], wp[c], sig[c]);
   } else {
     T V[4];
     visc3(C, 1, k >= n1, s[0], s[1], V);
@@ -408,17 +416,20 @@ __device__ __forceinline__ void yface_tile(const StageArgs& a, const Fx3Const& C
 // ---- x and z faces, divergence and stage combination ----------------------
 
 // TX x TZ3 cells: 13 warps, two face jobs each (face_id in stage_tile.cuh). 110
-// KB of shared memory, two CTAs (26 warps) per SM; as TX x 8 tiles the doubles
-// of the tangential momenta would not leave room for three.
+// KB of shared memory, two CTAs (26 warps) per SM; as TX x 8 tiles the packed
+// momenta and their velocities would not leave room for three.
 constexpr int TZ3 = 12;
 constexpr int TILE3_THREADS = TX * (TZ3 + 1);
 constexpr int RINGS = (TZ3 + 2) * (TX + 2);
 struct Tile3Smem {
   i64 q[5][TZ3 + 4][TX + 4];       // plane j, rows k0-2.., cols i0-2..
-  double qd[3][TZ3 + 4][TX + 4];   // rho u, rho v, rho w
+  i64 qw[3][TZ3 + 4][TX + 4];      // rho u, rho v, rho w packed (fixed_point.cuh)
   i64 v[4][TZ3 + 2][TX + 2];       // u, v, w, e on the ring
-  double vd[3][TZ3 + 2][TX + 2];   // u, v, w
-  i64 vy[3][TZ3 + 2][TX + 2];      // central y differences of u, v, w on the ring: u and w as doubles
+  i64 vp[3][TZ3 + 2][TX + 2];      // u, v, w under the exponents of qw
+  // central y differences of u, v, w on the ring: in fixed point v .59, u and w
+  // .57 under the exponents ye
+  i64 vy[3][TZ3 + 2][TX + 2];
+  short ye[2][TZ3 + 2][TX + 2];
   // fluxes: the tangential momenta as doubles, the others tagged
   i64 fx[5][TZ3][TX + 1];          // x face f between cols f-1, f
   i64 fz[5][TZ3 + 1][TX];          // z faces seen from above
@@ -450,7 +461,7 @@ __device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, in
       for (int c = 0; c < 5; c++) q[c * QP + e] = (T)0;
       if (FX)
 #pragma unroll
-        for (int c = 0; c < 3; c++) (&S.qd[0][0][0])[c * QP + e] = 0.0;
+        for (int c = 0; c < 3; c++) (&S.qw[0][0][0])[c * QP + e] = 0;
       continue;
     }
     double x[5];
@@ -470,17 +481,20 @@ __device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, in
     }
     if (FX)
 #pragma unroll
-      for (int c = 0; c < 3; c++) (&S.qd[0][0][0])[c * QP + e] = x[c + 1];
+      for (int c = 0; c < 3; c++) (&S.qw[0][0][0])[c * QP + e] = fx::pack(__double_as_longlong(x[c + 1]));
     // velocities on the one-cell ring
     if (rr >= 1 && rr <= TZ3 + 2 && cc >= 1 && cc <= TX + 2) {
       T o[4];
-      const double inv = Arith3<T>::prims(t, o);
+      const T inv = Arith3<T>::prims(t, o);
       const int at = (rr - 1) * (TX + 2) + cc - 1;
 #pragma unroll
       for (int c = 0; c < 4; c++) v[c * RINGS + at] = o[c];
-      if (FX)
+      if constexpr (FX) {
+        const FxW iw = fx::split(inv);
 #pragma unroll
-        for (int c = 0; c < 3; c++) (&S.vd[0][0][0])[c * RINGS + at] = __dmul_rn(x[c + 1], inv);
+        for (int c = 0; c < 3; c++)
+          (&S.vp[0][0][0])[c * RINGS + at] = fx::packed_velocity((&S.qw[0][0][0])[c * QP + e], iw);
+      }
     }
   }
   for (int e = tid; e < RINGS; e += TILE3_THREADS) {
@@ -488,36 +502,45 @@ __device__ __forceinline__ int tile3_cells(const StageArgs& a, const Geo3& G, in
     const int k = k0 - 1 + rr;
     if (k < 0 || k >= nz) continue;
     const int i = wrap3(i0 - 1 + cc, g.nx);
-    double x[5], d[3];
-    T dv = 0;
+    double x[5];
+    T d[3], u[2];
+    int ex[2];
     bool in = true;
 #pragma unroll
     for (int s = 0; s < 2; s++) {
       stage_val3(a, G, k, s ? jm : jp, i, x);
       if (FX) in = in && cell_in_range3(x);
       if (!in) break;
-      double inv;
       if constexpr (FX) {
-        const i64 inv_ = fx::recip(Arith3<i64>::cell(x[0], 0) << 2);
-        const i64 v_ = fx::mul(fx::split(Arith3<i64>::cell(x[2], 2) << 2), fx::split(inv_));
-        dv = s ? dv - v_ : v_;
-        inv = __longlong_as_double(fx::to_double(inv_, 61));
-      } else {
-        inv = recip_f64(x[0]);
-      }
+        const FxW inv = fx::split(fx::recip(Arith3<i64>::cell(x[0], 0) << 2));
+        const i64 v_ = fx::mul(fx::split(Arith3<i64>::cell(x[2], 2) << 2), inv);
+        d[1] = s ? d[1] - v_ : v_;
 #pragma unroll
-      for (int c = 0; c < 3; c++)
-        if (!FX || c != 1) d[c] = s ? __dsub_rn(d[c], __dmul_rn(x[c + 1], inv)) : __dmul_rn(x[c + 1], inv);
+        for (int c = 0; c < 2; c++) {
+          const i64 w = fx::pack(__double_as_longlong(x[2 * c + 1])), p = fx::packed_velocity(w, inv);
+          const int ew = fx::pack_exp(w);
+          if (s) {
+            const int em = max(ew, ex[c]);
+            d[2 * c] = vel_at(u[c], ex[c], em) - vel_at(p, ew, em);
+            S.ye[c][rr][cc] = (short)em;
+          } else {
+            u[c] = p;
+            ex[c] = ew;
+          }
+        }
+      } else {
+        const double inv = recip_f64(x[0]);
+#pragma unroll
+        for (int c = 0; c < 3; c++) d[c] = s ? __dsub_rn(d[c], __dmul_rn(x[c + 1], inv)) : __dmul_rn(x[c + 1], inv);
+      }
     }
     if (FX) {
       S.oky[rr][cc] = in;
       bad |= !in;
     }
     if (!in) continue;
-    if constexpr (!FX) dv = d[1];
-    (&S.vy[0][0][0])[e] = __double_as_longlong(d[0]);
-    reinterpret_cast<T*>(&S.vy[1][0][0])[e] = dv;
-    (&S.vy[2][0][0])[e] = __double_as_longlong(d[2]);
+#pragma unroll
+    for (int c = 0; c < 3; c++) reinterpret_cast<T*>(&S.vy[0][0][0])[c * RINGS + e] = d[c];
   }
   if (!FX) {
     __syncthreads();
@@ -551,34 +574,44 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
   const T* v = reinterpret_cast<const T*>(&S.v[0][0][0]) + vo;
   const T* vy1 = reinterpret_cast<const T*>(&S.vy[1][0][0]) + vo;
   T L[5], R[5], V[4];  // FX: V[0] and V[3] only
-  double sig[2];       // FX: the tangential stresses
+  FxStress sig[2];     // FX: the tangential stresses
   i64 snt[2];          // the same .59
   if (FX) {
-    const double* d = reinterpret_cast<const double*>(FX ? (const void*)&S.vd[0][0][0] : (const void*)v) + (FX ? vo : 0);
-    const double* d1 = d + (p1 - 1) * RINGS;
-    const double* d2 = d + (p2 - 1) * RINGS;
-    const double t1 = __dsub_rn(d1[vs], d1[0]), t2 = __dsub_rn(d2[vs], d2[0]);
-    if (lidf) {
-      sig[0] = __dmul_rn(C.k.tlid[LID_S], t1);
-      sig[1] = __dmul_rn(C.k.tlid[LID_S], t2);
-    } else if (wall) {  // the ghosts' velocities are +-those of the cell, their differences of w the opposite
-      const double cw = g.wall ? 0.0 : ku == 0 ? 2.0 : -2.0;
-      const int o = ku == 0 ? vs : 0;
-      sig[0] = __dmul_rn(C.fd[2][fl][F3_C], __dmul_rn(cw, d1[o]));
-      sig[1] = __dmul_rn(C.fd[2][fl][F3_C], __dmul_rn(cw, d2[o]));
+    const i64* p = &S.vp[0][0][0] + vo;
+    const i64* m = &S.qw[0][0][0] + q0 + qs;  // the same cell
+    const int o1 = (p1 - 1) * RINGS, o2 = (p2 - 1) * RINGS, m1 = (p1 - 1) * QP, m2 = (p2 - 1) * QP;
+    if (wall) {  // the ghosts' velocities are +-those of the cell, their differences of w the opposite
+      sig[0] = sig[1] = FxStress{0, 0};
+      if (!g.wall) {
+        const int ov = ku == 0 ? vs : 0, om = ku == 0 ? qs : 0;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+          const int e = fx::pack_exp(m[(c ? m2 : m1) + om]);
+          const i64 x = vel_at(p[(c ? o2 : o1) + ov], e, e) << 1;
+          sig[c] = tan_stress(C.tc[2][fl][0], FxA{ku == 0 ? x : -x, e});
+        }
+      }
     } else {
-      const double* f = C.fd[dir][fl];
-      const double* n = d + (pn - 1) * RINGS;
-      const double* y = reinterpret_cast<const double*>(&S.vy[pn - 1][0][0]) + vo;
-      // differences of u_n along y and along the third direction, of both cells
-      const double gy = __dadd_rn(y[0], y[vs]);
-      const double gt = id.isx ? __dadd_rn(dz_vel(g, C.k, ku, 0, n, VW), dz_vel(g, C.k, ku, 0, n + 1, VW))
-                               : __dadd_rn(__dsub_rn(n[1], n[-1]), __dsub_rn(n[VW + 1], n[VW - 1]));
-      sig[0] = __fma_rn(f[F3_C], t1, __dmul_rn(f[F3_D1], id.isx ? gy : gt));
-      sig[1] = __fma_rn(f[F3_C], t2, __dmul_rn(f[F3_D2], id.isx ? gt : gy));
+      const FxA t1 = vel_diff(p + o1, m + m1, vs, qs), t2 = vel_diff(p + o2, m + m2, vs, qs);
+      if (lidf) {
+        sig[0] = tan_stress(C.k.ts, t1);
+        sig[1] = tan_stress(C.k.ts, t2);
+      } else {
+        const FxN* tc = C.tc[dir][fl];
+        const i64* n = p + (pn - 1) * RINGS;
+        const i64* mn = m + (pn - 1) * QP;
+        // differences of u_n along y and along the third direction, of both cells
+        const i64* y = &S.vy[pn - 1][0][0] + vo;
+        const short* ye = &S.ye[id.isx ? 0 : 1][0][0] + vo;
+        const int ey = max(ye[0], ye[vs]);
+        const FxA gy = {fx::shr(y[0], ey - ye[0]) + fx::shr(y[vs], ey - ye[vs]), ey};
+        const FxA gt = id.isx ? dz_pair(g, C.k, ku, n, n + 1, VW, mn, mn + 1, TX + 4) : vel_cross(n, mn, vs, qs, 1, 1);
+        sig[0] = tan_stress(tc[0], t1, tc[1], id.isx ? gy : gt);
+        sig[1] = tan_stress(tc[0], t2, tc[2], id.isx ? gt : gy);
+      }
     }
 #pragma unroll
-    for (int c = 0; c < 2; c++) snt[c] = fx::from_double(__double_as_longlong(sig[c]), fx::S_VEL);
+    for (int c = 0; c < 2; c++) snt[c] = stress59(sig[c]);
   }
   if (lidf) {
     // the bulk fluxes, with the wall velocities (one value for both fluids)
@@ -671,21 +704,10 @@ __device__ __forceinline__ bool face3(const Geom& g, const Fx3Const& C, Tile3Sme
     F[0] = m[0], F[1] = m[1], F[4] = m[2];
 #pragma unroll
     for (int c = 0; c < 2; c++) {
-      const double* p = &S.qd[0][0][0] + q0 + ((c ? p2 : p1) - 1) * QP;
-      double a0 = p[0], a1 = p[qs], a2 = p[2 * qs], a3 = p[3 * qs], f;
-      if (edge) {
-        if (from_above) a1 = a2;
-        else a2 = a1;
-      }
-      if (mir0) a0 = a1;
-      if (mir3) a3 = a2;
-      if (edge) {
-        const double b = from_above ? __fma_rn(0.25, __dsub_rn(a1, a3), a2) : __fma_rn(0.25, __dsub_rn(a2, a0), a1);
-        f = tan_flux(t, b, b, sig[c]);
-      } else {
-        f = tan_flux(t, a0, a1, a2, a3, sig[c]);
-      }
-      F[2 + c] = __double_as_longlong(f);
+      const i64* p = &S.qw[0][0][0] + q0 + ((c ? p2 : p1) - 1) * QP;
+      const i64 a1 = p[qs], a2 = p[2 * qs];
+      F[2 + c] = edge ? tan_flux(t, 0, 0, 0, 0, sig[c])  // nothing flows through
+                      : tan_flux(t, mir0 ? a1 : p[0], a1, a2, mir3 ? a2 : p[3 * qs], sig[c]);
     }
   } else {
     flux3(g, L, R, V, F);

@@ -37,6 +37,16 @@ void prim(const i64* in, i64* o) {  // in: a, b, c, d; rho .60; x .61; the bits 
   o[4] = fx::from_double(in[6], 60);
   o[5] = fx::to_double(in[0], 59);
 }
+void tangent(const i64* in, i64* o) {  // in: bits of L2, L1, R1, R2; us, lr; V, its e; C, its shift; x, its e
+  i64 w[4];
+  for (int j = 0; j < 4; j++) w[j] = fx::pack(in[j]);
+  o[0] = tan_flux(FxTan{in[4], in[5]}, w[0], w[1], w[2], w[3], FxStress{in[6], (int)in[7]});
+  const FxN c = {fx::split(in[8]), (int)in[9]};
+  const FxStress s = tan_stress(c, FxA{in[10], (int)in[11]}, c, FxA{in[10] / 3, (int)in[11] - 9});
+  o[1] = s.v;
+  o[2] = s.e;
+  o[3] = stress59(s);
+}
 void visc2(const i64* f, const i64* v, i64* o) {  // f: coefficients; v: L, R of five, snt
   FxW fc[FXC_N];
   for (int j = 0; j < FXC_N; j++) fc[j] = fx::split(f[j]);
@@ -108,6 +118,37 @@ def test_primitives_within_their_bounds(lib):
     for a in (0, 1, -1, 2 ** 53 + 1, 2 ** 62 - 1, -(2 ** 62) + 1, 2 ** 63 - 1, -(2 ** 63)):
         o = call(lib.prim, [a, 1, 1, 1, 2 ** 60, 2 ** 60, 0], n=6)
         assert abs(value(o[5]) * 2 ** 59 - a) <= abs(Fr(a)) / 2 ** 53
+
+
+def test_tangential_flux_follows_the_momenta(lib):
+    """Momenta of every size down to 1e-300, zeros and neighbours of other sizes
+    among them. Units of 2^-55 of the largest one's power of two: the pair of
+    products 1; each momentum cut at 2^-58 with weights up to 3/2 of u_L + u_R
+    (3.66) and 2 of lambda - u_R (5.64), (5.49 + 11.28) / 8; the two parts
+    aligned, 1 each at the larger exponent; and the double's rounding."""
+    rng = random.Random(11)
+    for _ in range(6000):
+        scale = 2.0 ** -rng.choice([0, 1, 7, 20, 33, 60, 200, 900])
+        m = [rng.choice([rng.uniform(-0.65, 0.65), rng.uniform(-0.65, 0.65) * 2.0 ** -rng.randint(0, 70), 0.0]) * scale
+             for _ in range(4)]
+        us, lr = int(rng.uniform(-3.66, 3.66) * 2 ** 59), int(rng.uniform(0.5, 5.64) * 2 ** 59)
+        big = max(map(abs, m))
+        em = max((bits(abs(x)) >> 52) for x in m)
+        v, ev = int(rng.uniform(-1, 1) * 2 ** 58), max(em + rng.randint(-70, 3), -40)
+        fac, sh, x = int(rng.uniform(0.5, 1) * 2 ** 62), rng.randint(0, 30), int(rng.uniform(-1, 1) * 2 ** 60)
+        ex = rng.randint(1, 1022)
+        o = call(lib.tangent, [bits(t) for t in m] + [us, lr, v, ev, fac, sh, x, ex], n=4)
+        a0, a1, a2, a3 = map(Fr, m)
+        L, R = a1 + (a2 - a0) / 4, a2 + (a1 - a3) / 4
+        exact = (L * us + (L - R) * lr) / Fr(2) ** 59 - Fr(v) * Fr(2) ** (ev - 1023 - 55)
+        unit = lambda e: Fr(2) ** (e - 1023 - 55)  # noqa: E731
+        bound = (1 + Fr(17, 8)) * unit(em) + 2 * unit(max(em, ev)) + abs(exact) / 2 ** 53 + Fr(2) ** -1022
+        assert abs(value(o[0]) - exact) <= bound, (m, big)
+        # the stress from two differences: 3/4 each, 1 for the alignment
+        e = ex - sh
+        s = Fr(x) * fac / Fr(2) ** 64 * unit(e) + int(Fr(x, 3)) * fac / Fr(2) ** 64 * unit(e - 9)
+        assert o[2] == e and abs(o[1] * unit(e) - s) <= Fr(11, 4) * unit(e)
+        assert abs(Fr(o[3]) - o[1] * unit(e) * Fr(2) ** 59) < 1
 
 
 U, E, N = 1.32, 4.8, 59  # cell velocities and e as the range bounds them, .59
