@@ -86,6 +86,7 @@ struct FxConst {
   FxW gg;              // gamma (gamma - 1).62
   FxW lid[LID_N];      // interface, .62
   FxW fc[2][2][FXC_N]; // viscous coefficients per direction (x, z) and fluid, .62
+  double fd[2][2][FXC_N];  // the same in double, of the double pass
   FxN tc[2][2][2];     // of them C and D for the tangential stress
   FxN ts;              // LID_S likewise
   double tlid[LID_N];  // the interface's factors in double, LID_1 and LID_2 doubled
@@ -104,7 +105,7 @@ enum {
   F3_N
 };
 struct Fx3Const {
-  FxConst k;  // its fc and tc unused; square: dx = dy = dz1 = dz2
+  FxConst k;  // its fc, fd and tc unused; square: dx = dy = dz1 = dz2
   FxW fc[3][2][F3_N];
   double fd[3][2][F3_N];
   FxN tc[3][2][3];  // C, D1, D2 for the tangential stresses

@@ -353,7 +353,7 @@ void mprk::fixed_point_const(const Geom& g, FxConst* out) {
   for (int dir = 0; dir < 2; dir++)
     for (int fl = 0; fl < 2; fl++)
       for (int j = 0; j < FXC_N; j++) {
-        const double x = visc_coef(g, dir, fl, j);
+        const double x = f.fd[dir][fl][j] = visc_coef(g, dir, fl, j);
         ok = ok && std::fabs(x) < 1.0;  // false for NaN
         if (ok) f.fc[dir][fl][j] = fx_factor(x, 62);
         if (ok && (j == FXC_C || j == FXC_D)) f.tc[dir][fl][j - FXC_C] = fx_scaled(x);

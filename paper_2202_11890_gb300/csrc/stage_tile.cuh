@@ -51,7 +51,6 @@ struct TileSmem {
   i64 fx[4][TZR][TX + 1];  // face f between cols f-1, f
   i64 fz[4][TZR + 1][TX];  // seen from above at the interface
   i64 fg[4][TX];           // the interface seen from fluid 1 (below)
-  double fc[2][2][FXC_N];  // viscous coefficients of the double pass
   unsigned char slow[(2 * TZR + 3) * TX];  // per face: its job and lane (face_id)
 };
 
@@ -60,26 +59,18 @@ struct TileSmem {
 // along the face normal, m_t along the face. Output is f(q_L) + f(q_R) +
 // lambda (q_L - q_R) - V: V the viscous or interface part of (m_n, m_t, rho E).
 // lambda is the largest |u_n| + a over the left, right and Roe-averaged
-// states (Sec. 2.1); the Roe weights sqrt(rho)/(sqrt(rho_L) + sqrt(rho_R))
-// times the enthalpy H = (rho E + p)/rho are formed as (rho E + p)/sqrt(rho).
-__device__ __forceinline__ void lf_face(double lr, double lmn, double lmt, double lE, double rr, double rmn, double rmt,
-                                        double rE, double gamma, double gm1, const double V[3], double out[4]) {
-  const double rsL = rsqrt_f64(lr), rsR = rsqrt_f64(rr);
-  const double invL = __dmul_rn(rsL, rsL), invR = __dmul_rn(rsR, rsR);
-  const double sL = __dmul_rn(lr, rsL), sR = __dmul_rn(rr, rsR);  // sqrt(rho)
+// states (Sec. 2.1).
+__device__ __forceinline__ void lf_face(const Geom& g, const double L[4], const double R[4], const double V[3],
+                                        double out[4]) {
+  const double lr = L[0], lmn = L[1], lmt = L[2], lE = L[3], rr = R[0], rmn = R[1], rmt = R[2], rE = R[3];
+  const double invL = recip_f64(lr), invR = recip_f64(rr);
   const double unL = __dmul_rn(lmn, invL), utL = __dmul_rn(lmt, invL);
   const double unR = __dmul_rn(rmn, invR), utR = __dmul_rn(rmt, invR);
   const double kL = __fma_rn(lmt, utL, __dmul_rn(lmn, unL)), kR = __fma_rn(rmt, utR, __dmul_rn(rmn, unR));
-  const double pL = __dmul_rn(gm1, __fma_rn(-0.5, kL, lE)), pR = __dmul_rn(gm1, __fma_rn(-0.5, kR, rE));
-  const double cL = sqrt_f64(__dmul_rn(__dmul_rn(gamma, pL), invL));
-  const double cR = sqrt_f64(__dmul_rn(__dmul_rn(gamma, pR), invR));
+  const double pL = __dmul_rn(g.gm1, __fma_rn(-0.5, kL, lE)), pR = __dmul_rn(g.gm1, __fma_rn(-0.5, kR, rE));
   const double eL = __dadd_rn(lE, pL), eR = __dadd_rn(rE, pR);
-  const double den = recip_f64(__dadd_rn(sL, sR));
-  const double un = __dmul_rn(__fma_rn(sR, unR, __dmul_rn(sL, unL)), den);
-  const double ut = __dmul_rn(__fma_rn(sR, utR, __dmul_rn(sL, utL)), den);
-  const double H = __dmul_rn(__fma_rn(eR, rsR, __dmul_rn(eL, rsL)), den);
-  const double c = sqrt_f64(__dmul_rn(gm1, __fma_rn(-0.5, __fma_rn(ut, ut, __dmul_rn(un, un)), H)));
-  const double lam = max_speed(max_speed(__dadd_rn(fabs(unL), cL), __dadd_rn(fabs(unR), cR)), __dadd_rn(fabs(un), c));
+  const double lam = face_speed(g, lr, rr, unL, unR, __dsub_rn(utR, utL), 0.0, __dmul_rn(__dmul_rn(g.gamma, pL), invL),
+                                __dmul_rn(__dmul_rn(g.gamma, pR), invR));
   out[0] = __fma_rn(lam, __dsub_rn(lr, rr), __dadd_rn(lmn, rmn));
   const double f1 = __dsub_rn(__dadd_rn(__fma_rn(lmn, unL, pL), __fma_rn(rmn, unR, pR)), V[0]);
   out[1] = __fma_rn(lam, __dsub_rn(lmn, rmn), f1);
@@ -519,10 +510,6 @@ __host__ __device__ __forceinline__ void fx_visc(const FxW* fc, const i64 vL[5],
 }
 
 // The same flux in double.
-__device__ __forceinline__ void double_flux(const Geom& g, const double L[4], const double R[4], const double V[3],
-                                            double F[4]) {
-  lf_face(L[0], L[1], L[2], L[3], R[0], R[1], R[2], R[3], g.gamma, g.gm1, V, F);
-}
 __device__ __forceinline__ void double_visc(const double* fc, const double vL[5], const double vR[5], double V[3]) {
   V[0] = __fma_rn(fc[FXC_A], __dsub_rn(vR[0], vL[0]), __dmul_rn(fc[FXC_B], __dadd_rn(vL[4], vR[4])));
   V[1] = __fma_rn(fc[FXC_C], __dsub_rn(vR[1], vL[1]), __dmul_rn(fc[FXC_D], __dadd_rn(vL[3], vR[3])));
@@ -622,20 +609,29 @@ __device__ __noinline__ bool face_in_range(const Geom& g, const TileSmem<TZR>& S
   return ok;
 }
 
+// Is the face of this lane evaluated in fixed point (out: its own cells are
+// not in range)? The double pass runs a job's 32 faces together, so one of them
+// outside takes the whole row of faces there, and the fixed-point pass is spared
+// (30 % of the cells outside: 512 x 256, m = 4, 618 -> 579 us). An x face that two tiles
+// evaluate, on a tile's edge or the wrap, asks its own cells alone.
+__device__ __forceinline__ bool row_in_range(const FaceId& id, int i0, int nx, bool out) {
+  const bool alone = id.isx && (id.c == 0 || id.c == TX || i0 + id.c == nx);
+  const bool any = __any_sync(0xffffffffu, out && !alone);
+  return !(out || (any && !alone));
+}
+
 // The faces marked slow (all: every face), in double: the ring again as
 // doubles (in the same storage), then their fluxes. Ends with the tile's
-// barrier. A grid wholly outside the range runs as fast as the tile that did
-// everything in double (2048 x 1024, m = 8: 11.5 ms per step against 11.7).
+// barrier. Against the tile that did everything in double, us per step: 2048 x
+// 1024, m = 8, wholly outside 9378 (11683), 30 % of the cells outside 9957
+// (11690); 512 x 256, m = 4, 442 (519) and 490 (519); with the Roe speed of
+// every face and coefficients computed per tile 11556, 11979, 552 and 579.
 template <int NT, int TZR>
 __device__ __noinline__ void slow_faces(const Geom& g, const FxConst& fk, TileSmem<TZR>& S, int k0, int i0, int row_hi, bool all) {
   for (int e = threadIdx.x; e < (TZR + 2) * (TX + 2); e += NT) {
     const int rr = e / (TX + 2) + 1, cc = e % (TX + 2) + 1, k = k0 - 2 + rr;
     if (k >= 0 && k < g.nz)
       ring_cell<double, TZR>(g, S, rr, cc, i0, S.q[0][rr][cc], S.q[1][rr][cc], S.q[2][rr][cc], S.q[3][rr][cc]);
-  }
-  if (threadIdx.x < 4 * FXC_N) {
-    const int j = threadIdx.x % FXC_N, f = threadIdx.x / FXC_N;
-    S.fc[f >> 1][f & 1][j] = visc_coef(g, f >> 1, f & 1, j);
   }
   __syncthreads();
   for (int job = threadIdx.x / 32; job < 2 * TZR + 3; job += NT / 32) {
@@ -646,13 +642,13 @@ __device__ __noinline__ void slow_faces(const Geom& g, const FxConst& fk, TileSm
     double L[4], R[4], vL[5], vR[5], V[3], F[4];
     const int fl = face_sides<double, TZR>(g, fk, S, id, L, R, vL, vR);
     if (fl < 2) {
-      double_visc(S.fc[id.isx ? 0 : 1][fl], vL, vR, V);
+      double_visc(fk.fd[id.isx ? 0 : 1][fl], vL, vR, V);
     } else {
       V[0] = 0.0;
       V[1] = __dmul_rn(fk.tlid[LID_S], __dsub_rn(vR[1], vL[1]));
       V[2] = __dadd_rn(lid_work(fk, vL[1], vR[1], V[1]), lid_heat(fk, vL[2], vR[2]));
     }
-    double_flux(g, L, R, V, F);
+    lf_face(g, L, R, V, F);
     i64 o[4];
 #pragma unroll
     for (int c = 0; c < 4; c++) o[c] = __double_as_longlong(F[c]);
@@ -702,7 +698,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
   };
 
   // ---- 1. stage state of the tile and its halo; u, w, e on the ring ------
-  bool bad = !a.fx.on, good = false;  // some cell outside, inside the fixed-point range
+  bool bad = false, good = false;  // some cell outside, inside the fixed-point range
   for (int e = tid; e < (TZR + 4) * (TX + 4); e += NT) {
     const int rr = e / (TX + 4), cc = e - rr * (TX + 4);
     const int k = k0 - 2 + rr;
@@ -729,13 +725,15 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
       for (int c = 0; c < 4; c++) val[c] = stage_value(c, k, i);
     }
     if (gh) val[1] = -val[1];  // mirror state beyond an x wall
-    const bool in = cell_in_range(val[0], val[1], val[2], val[3]);
+#pragma unroll
+    for (int c = 0; c < 4; c++) S.q[c][rr][cc] = val[c];
+    const bool in = a.fx.on && cell_in_range(val[0], val[1], val[2], val[3]);
     bad |= !in;
     good |= in;
+    if (!in) continue;  // no face in fixed point reads the cell
     i64 t[4];
 #pragma unroll
     for (int c = 0; c < 4; c++) {
-      S.q[c][rr][cc] = val[c];
       t[c] = c == 1 || c == 2 ? fx::from_double(__double_as_longlong(val[c]), fx::S_MOM - 2)
                               : fx::from_positive(__double_as_longlong(val[c]), fx::S_RHO - 2);
       S.qi[c][rr][cc] = t[c];
@@ -746,7 +744,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
   const bool has_gamma = (n1 >= k0 && n1 <= k0 + TZR);
   bad = __syncthreads_or(bad);
   bool none = false;  // no cell inside: every face in double
-  if (bad) none = !a.fx.on || !__syncthreads_or(good);
+  if (bad) none = !__syncthreads_or(good);
 
   // ---- 2. face fluxes ----------------------------------------------------
   static_assert(TX == 32 && NT % 32 == 0, "a job is one warp wide");
@@ -771,8 +769,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs& a, int tile, TileSme
         Vt = visc_tan_plain<false, TZR>(a.fx, S, id, fl);
       }
     } else {
-      if (!face_id<TZR>(g, job, lane, k0, row_hi, &id)) continue;
-      ok = !bad || face_in_range<TZR>(g, S, id, k0);
+      const bool valid = face_id<TZR>(g, job, lane, k0, row_hi, &id);
+      if (bad) ok = row_in_range(id, i0, nx, valid && !face_in_range<TZR>(g, S, id, k0));
+      if (!valid) continue;
       if (ok) {
         fl = face_sides<i64, TZR>(g, a.fx, S, id, L, R, vL, vR);
         Vt = visc_tan<TZR>(g, a.fx, S, id, fl);

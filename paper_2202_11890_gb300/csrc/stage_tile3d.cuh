@@ -37,29 +37,18 @@ constexpr int NC3 = 5;
 
 // Lax–Friedrichs flux (Sec. 2.1) in a face frame, in double: a state is (rho,
 // m_n, m_t1, m_t2, rho E); lambda is the largest |u_n| + a over the left,
-// right and Roe-averaged states. The Roe weights times the enthalpy
-// (rho E + p)/rho are formed as (rho E + p)/sqrt(rho). V: the viscous part.
-__device__ __forceinline__ void lf_face5(const double l[5], const double r[5], double gamma, double gm1,
-                                         const double V[4], double out[5]) {
-  const double rsL = rsqrt_f64(l[0]), rsR = rsqrt_f64(r[0]);
-  const double invL = __dmul_rn(rsL, rsL), invR = __dmul_rn(rsR, rsR);
-  const double sL = __dmul_rn(l[0], rsL), sR = __dmul_rn(r[0], rsR);  // sqrt(rho)
+// right and Roe-averaged states. V: the viscous part.
+__device__ __forceinline__ void lf_face5(const Geom& g, const double l[5], const double r[5], const double V[4],
+                                         double out[5]) {
+  const double invL = recip_f64(l[0]), invR = recip_f64(r[0]);
   const double unL = __dmul_rn(l[1], invL), t1L = __dmul_rn(l[2], invL), t2L = __dmul_rn(l[3], invL);
   const double unR = __dmul_rn(r[1], invR), t1R = __dmul_rn(r[2], invR), t2R = __dmul_rn(r[3], invR);
   const double kL = __fma_rn(l[3], t2L, __fma_rn(l[2], t1L, __dmul_rn(l[1], unL)));
   const double kR = __fma_rn(r[3], t2R, __fma_rn(r[2], t1R, __dmul_rn(r[1], unR)));
-  const double pL = __dmul_rn(gm1, __fma_rn(-0.5, kL, l[4])), pR = __dmul_rn(gm1, __fma_rn(-0.5, kR, r[4]));
-  const double cL = sqrt_f64(__dmul_rn(__dmul_rn(gamma, pL), invL));
-  const double cR = sqrt_f64(__dmul_rn(__dmul_rn(gamma, pR), invR));
+  const double pL = __dmul_rn(g.gm1, __fma_rn(-0.5, kL, l[4])), pR = __dmul_rn(g.gm1, __fma_rn(-0.5, kR, r[4]));
   const double eL = __dadd_rn(l[4], pL), eR = __dadd_rn(r[4], pR);
-  const double den = recip_f64(__dadd_rn(sL, sR));
-  const double un = __dmul_rn(__fma_rn(sR, unR, __dmul_rn(sL, unL)), den);
-  const double t1 = __dmul_rn(__fma_rn(sR, t1R, __dmul_rn(sL, t1L)), den);
-  const double t2 = __dmul_rn(__fma_rn(sR, t2R, __dmul_rn(sL, t2L)), den);
-  const double H = __dmul_rn(__fma_rn(eR, rsR, __dmul_rn(eL, rsL)), den);
-  const double k = __fma_rn(t2, t2, __fma_rn(t1, t1, __dmul_rn(un, un)));
-  const double c = sqrt_f64(__dmul_rn(gm1, __fma_rn(-0.5, k, H)));
-  const double lam = max_speed(max_speed(__dadd_rn(fabs(unL), cL), __dadd_rn(fabs(unR), cR)), __dadd_rn(fabs(un), c));
+  const double lam = face_speed(g, l[0], r[0], unL, unR, __dsub_rn(t1R, t1L), __dsub_rn(t2R, t2L),
+                                __dmul_rn(__dmul_rn(g.gamma, pL), invL), __dmul_rn(__dmul_rn(g.gamma, pR), invR));
   out[0] = __fma_rn(lam, __dsub_rn(l[0], r[0]), __dadd_rn(l[1], r[1]));
   const double f1 = __dsub_rn(__dadd_rn(__fma_rn(l[1], unL, pL), __fma_rn(r[1], unR, pR)), V[0]);
   out[1] = __fma_rn(lam, __dsub_rn(l[1], r[1]), f1);
@@ -233,7 +222,7 @@ __device__ __forceinline__ void visc3(const Fx3Const& c, int dir, int fl, const 
 // tagged.
 __device__ __forceinline__ void flux3(const Geom& g, const double L[5], const double R[5], const double V[4], i64 F[5]) {
   double o[5];
-  lf_face5(L, R, g.gamma, g.gm1, V, o);
+  lf_face5(g, L, R, V, o);
 #pragma unroll
   for (int q = 0; q < 5; q++) F[q] = q == 2 || q == 3 ? __double_as_longlong(o[q]) : flux_tag(o[q]);
 }
@@ -332,9 +321,8 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
   }
   if (FX) bad = __syncthreads_or(bad);
   else __syncthreads();
-  if (!mine || !want) return true;
   if (FX) {
-    if (bad) {
+    if (bad && mine) {
       // the face's own cells: the four across it and the x and z neighbours
       // of the two at it (inside the grid)
       for (int s = 0; s < 2; s++) {
@@ -343,8 +331,10 @@ __device__ __forceinline__ bool yface_pass(const StageArgs& a, const Fx3Const& C
         if (k + 1 < nz) out_ok = out_ok && S.ok[s][rr + 2][cc + 1];
       }
     }
-    if (!out_ok) return false;
+    // one face outside takes its row to the double pass (row_in_range)
+    if (__any_sync(0xffffffffu, !out_ok)) return !mine;
   }
+  if (!mine || !want) return true;
   // face frame: normal rho v, t1 rho u, t2 rho w
   const int at = (rr + 1) * (TX + 2) + cc + 1;
   T L[5], R[5];
@@ -784,8 +774,11 @@ __device__ __forceinline__ void stage_tile3(const StageArgs& a, const Fx3Const& 
   bool slow = false;
   for (int job = warp; job < jobs; job += TILE3_THREADS / 32) {
     FaceId id;
-    if (!face_id<TZ3>(g, job, lane, k0, row_hi, &id)) continue;
-    const bool ok = (out == 0 || face3_in_range(g, S, id, k0)) && face3<i64>(g, C, S, id);
+    const bool valid = face_id<TZ3>(g, job, lane, k0, row_hi, &id);
+    bool ok = true;
+    if (out) ok = row_in_range(id, i0, nx, valid && !face3_in_range(g, S, id, k0));
+    if (!valid) continue;
+    ok = ok && face3<i64>(g, C, S, id);
     S.slow[job * TX + lane] = !ok;
     slow |= !ok;
   }
