@@ -40,9 +40,8 @@ METRIC = "cell-stage updates/s"
 # the reference/deviation sums: 12 per face.
 FLOPS_PER_CELL_STAGE = {True: 355.7, False: 381.6}
 # Nominal unit counts of the GB300 for context: 152 SMs x 2 DFMA/clk x
-# 2 flop x 2.07 GHz, and 128 FP32 lanes per SM. The FP64 roofline's peak is
-# measured on the box by the library's register-only FMA probe
-# (mprk_probe_fp64), like the HBM peak is a measured copy.
+# 2 flop x 2.07 GHz, and 128 FP32 lanes per SM. The library's register-only FMA
+# probe (mprk_probe_fp64) measures the former on the device.
 FP64_NOMINAL_GFLOPS = 152 * 2 * 2 * 2.07
 FP32_PEAK_GFLOPS = 152 * 128 * 2 * 2.07
 _FP64_PROBE = None
@@ -52,8 +51,7 @@ def fp64_peak():
     """(peak GFLOP/s, source, probe) of the FP64 units: the unit count taken
     from the device (its SM count and peak SM clock) at 2 DFMA per SM clock,
     with the register-only FMA probe's measured rate beside it (run once per
-    process). The unit-count figure is the larger, so fractions against it
-    are the conservative ones."""
+    process)."""
     global _FP64_PROBE
     if _FP64_PROBE is None:
         from paper_2202_11890_gb300 import mprk as M
@@ -73,11 +71,14 @@ def fp64_peak():
 # order, comments and whitespace removed); after any change to that code
 # bench.py reports traffic as null.
 CSRC = os.path.join(ROOT, "paper_2202_11890_gb300", "csrc")
+FP64_FILES = ("stage_tile.cuh", "stage_tile3d.cuh", "fixed_point.cuh", "fixed_flux.cuh", "fp64_recip.cuh",
+              "batch_kernel.cuh", "mprk_internal.h", "mprk_kernels.cu")
+FP64_SHA256 = "499fd84f46e8abc8ea463943444252f01f83eb1976596ec4da1411776be368fc"
 TRAFFIC = {
     "stage_kernel": {
-        "files": ("stage_tile.cuh", "fp64_recip.cuh", "mprk_internal.h", "mprk_kernels.cu"),
-        "sha256": "1cc93c59d4076bfba1a35f3537abd9cf162908f0f45fe50a6fd7e47b9f7c8894",
-        "bytes_per_step": 1170924544,
+        "files": FP64_FILES,
+        "sha256": FP64_SHA256,
+        "bytes_per_step": 1187514112,
     },
     "stage_kernel_mixed": {
         "files": ("stage_tile_mixed.cuh", "mprk_internal.h", "mprk_kernels.cu"),
@@ -108,6 +109,20 @@ def measured_traffic(kernel: str, launches: int):
     if t["bytes_per_step"] is None or t["sha256"] != source_hash(t["files"]):
         return None
     return t["bytes_per_step"] / launches
+
+
+# Instructions per cell-stage (smsp__inst_executed.sum times 32 over the
+# launch's cells) of the FP64 kernels, from captures of the same sources: the
+# stage kernel over a slow step of 2048 x 1024 cells, m = 8; the RK4 form over
+# the four stages of a substep of 1024 x 512; the 3-D pair at 512 x 64 x 200;
+# the batch kernel over 64 uneven instances.
+FP64_INSTRUCTIONS = {"stage_kernel": 2699, "stage_kernel<GEN>": 2941, "yface3_kernel+stage3_kernel": 7064,
+                     "batch_kernel": 3230}
+
+
+def measured_instructions(kernel: str):
+    """Instructions per cell-stage, or None when the sources changed since."""
+    return FP64_INSTRUCTIONS[kernel] if FP64_SHA256 == source_hash(FP64_FILES) else None
 
 
 def algorithmic_bytes(g: W.Grid, m: int, fp64: bool):
@@ -265,22 +280,33 @@ def fp32_accuracy(M, cfg, q0, steps: int) -> dict:
             "mass_drift_fluid1_fluid2": {"fp32flux": drift(d0a, d1a), "fp64": drift(d0b, d1b)}}
 
 
-# The FP64 tiles' face fluxes run in 64-bit fixed point on the integer pipes, so
-# their formulas' operations, counted as written, may exceed the double pipe's peak.
-FP64_NOTE = "face fluxes in 64-bit fixed point on the integer pipes: frac counts the formulas against the double pipe"
+def fp64_roofline(kernel: str, cell_stages: float, ms: float, flops_per_cell_stage: float, traffic=None) -> dict:
+    """The FP64 kernels against the rate at which warp instructions can be
+    issued (four per clock and SM): the face fluxes run in 64-bit integers, so
+    that neither the double pipe nor HBM bounds them. The formulas' operations,
+    counted as written, over the double pipe's peak stand beside it as a ratio
+    (above one: what doing them in double would take at least)."""
+    fp64, psrc, probe = fp64_peak()
+    peak = 4 * probe["sms"] * probe["max_mhz"] / 1e3
+    inst = measured_instructions(kernel)
+    achieved = None if inst is None else cell_stages * inst / 32 / (ms * 1e-3) / 1e9
+    gflops = cell_stages * flops_per_cell_stage / (ms * 1e-3) / 1e9
+    return {"bound": "issue", "achieved": achieved, "peak": peak, "unit": "G warp instructions/s",
+            "frac": None if inst is None else achieved / peak, "traffic": traffic,
+            "instructions_per_cell_stage": inst,
+            "peak_source": f"4 per clock x {probe['sms']} SMs x {probe['max_mhz']:.0f} MHz peak clock",
+            "formula_gflops": gflops, "formula_over_fp64_pipe": gflops / fp64, "fp64_pipe_gflops": fp64,
+            "fp64_pipe_source": psrc, "probe_gflops": probe["gflops"]}
 
 
 def roofline_of(fp64: bool, stage_cells: int, stage_ms: float, stage_bytes: float, traffic):
-    """Both fractions of the stage kernel: the binding one first (FP64 units
-    in the FP64 mode, HBM in the FP32-flux mode), the other beside it."""
+    """Both fractions of the stage kernel: the binding one first (instruction
+    issue in the FP64 mode, HBM in the FP32-flux mode), the other beside it."""
     peaks, src = measured_peaks()
     ach_gflops = stage_cells * FLOPS_PER_CELL_STAGE[fp64] / (stage_ms * 1e-3) / 1e9
     ach_gbs = stage_bytes / (stage_ms * 1e-3) / 1e9
     if fp64:
-        peak, psrc, probe = fp64_peak()
-        return {"bound": "alu", "note": FP64_NOTE, "achieved": ach_gflops, "peak": peak, "unit": "GFLOP/s",
-                "frac": ach_gflops / peak, "traffic": traffic, "peak_source": psrc,
-                "probe_gflops": probe["gflops"], "frac_of_probe": ach_gflops / probe["gflops"],
+        return {**fp64_roofline("stage_kernel", stage_cells, stage_ms, FLOPS_PER_CELL_STAGE[True], traffic),
                 "hbm_achieved_gbs": ach_gbs, "hbm_peak_gbs": peaks["hbm_gbs"],
                 "hbm_frac": ach_gbs / peaks["hbm_gbs"], "hbm_peak_source": src}
     return {"bound": "hbm", "achieved": ach_gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
@@ -536,9 +562,8 @@ def measure_batched(M, T, precision: str, steps: int, warmup: int, count: int = 
     gbs = nbytes * steps / (t_batch * 1e-3) / 1e9
     gflops = cs * FLOPS_PER_CELL_STAGE[fp64] * steps / (t_batch * 1e-3) / 1e9
     if fp64:
-        peak, psrc, probe = fp64_peak()
-        roof = {"bound": "alu", "note": FP64_NOTE, "achieved": gflops, "peak": peak, "unit": "GFLOP/s", "frac": gflops / peak,
-                "traffic": None, "peak_source": psrc, "frac_of_probe": gflops / probe["gflops"], "hbm_achieved_gbs": gbs, "hbm_peak_gbs": peaks["hbm_gbs"],
+        roof = {**fp64_roofline("batch_kernel", cs * steps, t_batch, FLOPS_PER_CELL_STAGE[True]),
+                "hbm_achieved_gbs": gbs, "hbm_peak_gbs": peaks["hbm_gbs"],
                 "hbm_frac": gbs / peaks["hbm_gbs"], "hbm_peak_source": src, "algorithmic_bytes_per_step": nbytes}
     else:
         roof = {"bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
@@ -897,7 +922,6 @@ def run_cube(args):
         M.mprk_step_io(inst.h, [pin_in] * e2e_steps, [pin_out] * e2e_steps)
         e2e_s = time.perf_counter() - t0
     value = cs * steps / (t_ms * 1e-3)
-    ach = stage_cells * FLOPS_PER_CELL_STAGE_3D / (stage_ms * 1e-3) / 1e9
     stage_bytes, fin_bytes = algorithmic_bytes3(g, wl.m)
     peaks, src = measured_peaks()
     out = {"metric": METRIC, "value": value, "unit": "cell-stages/s", "n_gpus": ws, "steps": steps,
@@ -906,9 +930,7 @@ def run_cube(args):
            "config": {"workload": wl.name, "nx": g.nx, "ny": g.ny, "rows_S_B_F": [g.nS, g.nB, g.nF], "m": wl.m,
                       "cell_stages_per_step": cs, "parallelism": f"replicas x{ws}",
                       "l2": "working set > L2 (a state is 262 MB); no flush"},
-           "roofline": {"bound": "alu", "note": FP64_NOTE, "achieved": ach, "peak": fp64_peak()[0], "unit": "GFLOP/s",
-                        "frac": ach / fp64_peak()[0], "traffic": None, "peak_source": fp64_peak()[1],
-                        "frac_of_probe": ach / fp64_peak()[2]["gflops"],
+           "roofline": {**fp64_roofline("yface3_kernel+stage3_kernel", stage_cells, stage_ms, FLOPS_PER_CELL_STAGE_3D),
                         "hbm_achieved_gbs": stage_bytes / (stage_ms * 1e-3) / 1e9,
                         "hbm_peak_gbs": peaks["hbm_gbs"],
                         "hbm_frac": stage_bytes / (stage_ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
@@ -1058,7 +1080,6 @@ def run_base(args):
         _, stage_cells, share = T.stage_kernel_times(inst.h, stream, reps=3)
         stage_ms = T.kernel_ms_per_step(t_ms / steps, share)
     value = cs * steps / (t_ms * 1e-3)
-    ach = stage_cells * FLOPS_PER_CELL_STAGE[True] / (stage_ms * 1e-3) / 1e9
 
     # accuracy: the thermal convection with each base
     cw = W.convection_100()
@@ -1098,9 +1119,7 @@ def run_base(args):
            "config": {"workload": wl.name.replace("_m8", "_m8_rk4base"), "nx": g.nx,
                       "rows_S_B_F": [g.nS, g.nB, g.nF], "m": wl.m, "base": "rk4",
                       "cell_stages_per_step": cs, "l2": "working set > L2; no flush"},
-           "roofline": {"bound": "alu", "note": FP64_NOTE, "achieved": ach, "peak": fp64_peak()[0], "unit": "GFLOP/s",
-                        "frac": ach / fp64_peak()[0], "traffic": None, "peak_source": fp64_peak()[1],
-                        "frac_of_probe": ach / fp64_peak()[2]["gflops"],
+           "roofline": {**fp64_roofline("stage_kernel<GEN>", stage_cells, stage_ms, FLOPS_PER_CELL_STAGE[True]),
                         "flops": "the Heun stage's count; the RK4 stage values and weights add < 2 %"},
            "kernel": {"name": "stage_kernel<GEN>", "ms_per_step": stage_ms,
                       "cell_stages_per_step": stage_cells, "launches_per_step": 4 * wl.m},

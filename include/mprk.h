@@ -312,8 +312,8 @@ int mprk_rhs(mprk_instance* inst, const double* W_dev, double* R_dev, int k_lo, 
 int mprk_profile_step(mprk_instance* inst, double* launch_ms, long long* launch_cells, int cap);
 
 /* Measurement hook: the FP64 fused multiply-add throughput of the current
- * device, the denominator of the FP64 path's arithmetic roofline (the RHS
- * of Sec. 2.1 and App. B is FP64-arithmetic-bound in the FP64 mode).
+ * device, which would bound the RHS of Sec. 2.1 and App. B with every
+ * operation in double (the reason for the integer face fluxes).
  * Register-only kernels run independent FMA chains per thread (16 chains
  * of `iters` steps, or 8 of 2 iters; multiplier and addend in registers or
  * literals; 1 <= iters <= 2^30) on one full wave of 256-thread CTAs (as

@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(MIXED_THREADS, 3)
 
 // 3-D stage (App. B in full): the y faces of a plane pair, then the x and z
 // faces, the divergence and the combination of a plane; one CTA per TX x TZ
-// tile of an x-z plane, blockIdx = (tile column, tile row, plane).
+// (y faces) or TX x TZ3 tile of an x-z plane, blockIdx = (tile column, tile row, plane).
 // Three CTAs of y faces per SM (80 registers, 71 KB of shared memory each), two
 // of the others (72 registers, 110 KB).
 __global__ void __launch_bounds__(NTHREADS, 3)

@@ -27,10 +27,11 @@
 // of 1e-6 in a flow uniform along x had 3e4 times the double form's error), so
 // its integers carry an exponent (fixed_flux.cuh). Measured: a slow step of
 // 2048 x 1024 cells with m = 8 11.7 -> 2.37 ms (2.06 with that flux in fixed
-// point too), 64 x 64 with m = 4 185 -> 63.5 us (58.4). A face with a state outside the fixed-point
-// range takes the same formulas in double (slow_faces); which form a face
-// takes depends on its own cells alone, so results do not depend on the tile
-// shape or the launch.
+// point too), 64 x 64 with m = 4 185 -> 63.5 us (58.4). Faces with
+// a state outside the fixed-point range take the same formulas in double
+// (slow_faces), a row of 32 at a time (row_in_range); which form a face takes
+// depends on its row's cells alone, so results do not depend on the tile shape
+// or the launch.
 #pragma once
 
 #include "fixed_flux.cuh"

@@ -7,7 +7,7 @@
 //  * yface3: one CTA per TX x TZ tile of an x–z plane j computes the y-face
 //    fluxes G* between planes j and j+1 of its cells and stores them (face
 //    j+1/2 at index j) in a state-sized buffer;
-//  * stage3: one CTA per TX x TZ tile of plane j computes its x and z faces
+//  * stage3: one CTA per TX x TZ3 tile of plane j computes its x and z faces
 //    as the 2-D tile does, takes the y divergence from the stored y faces,
 //    adds the source and applies the stage combination.
 // Every face is computed once. Viscous fluxes use the common face values
@@ -19,9 +19,9 @@
 // 64-bit fixed point (fixed_point.cuh), because the double pipe bound both
 // kernels (80 to 86 % busy with 125 + 238 operations per cell), and those of
 // the tangential momenta in integers with an exponent. Measured: a slow step
-// of 512 x 64 x 200 cells with m = 4 44.1 -> 11.3 ms. A face whose own cells leave
-// the range is evaluated in double by a second pass over the tile; which form
-// a face takes depends on its cells alone, so neighbouring tiles agree on the
+// of 512 x 64 x 200 cells with m = 4 44.1 -> 11.3 ms. Faces whose cells leave
+// the range are evaluated in double by a second pass over the tile, a row of 32
+// at a time (row_in_range in stage_tile.cuh), so neighbouring tiles agree on the
 // faces they share. Fluxes come over half the divergence factor of their
 // direction, as .57 integers or as doubles (flux_tag).
 #pragma once
