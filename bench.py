@@ -82,8 +82,8 @@ TRAFFIC = {
     },
     "stage_kernel_mixed": {
         "files": ("stage_tile_mixed.cuh", "mprk_internal.h", "mprk_kernels.cu"),
-        "sha256": "70f97e7c7a75239400053bc9d8f307e748da86b7a75da26c9e9f119fa6b11ae3",
-        "bytes_per_step": 5149178880,
+        "sha256": "7831c00f316be8d503bc92448231e6939eb9df6ba62a2245c11d5a5c25c1704c",
+        "bytes_per_step": 5162544384,
     },
 }
 
@@ -293,7 +293,7 @@ def fp64_roofline(kernel: str, cell_stages: float, ms: float, flops_per_cell_sta
     gflops = cell_stages * flops_per_cell_stage / (ms * 1e-3) / 1e9
     return {"bound": "issue", "achieved": achieved, "peak": peak, "unit": "G warp instructions/s",
             "frac": None if inst is None else achieved / peak, "traffic": traffic,
-            "instructions_per_cell_stage": inst,
+            "instructions_per_cell_stage": inst,  # of 32 x 8 tiles (32 x 12 in 3-D); shorter ones take more
             "peak_source": f"4 per clock x {probe['sms']} SMs x {probe['max_mhz']:.0f} MHz peak clock",
             "formula_gflops": gflops, "formula_over_fp64_pipe": gflops / fp64, "fp64_pipe_gflops": fp64,
             "fp64_pipe_source": psrc, "probe_gflops": probe["gflops"]}

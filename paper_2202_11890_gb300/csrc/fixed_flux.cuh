@@ -124,7 +124,7 @@ struct FxStress {
   int e;
 };
 // A velocity of exponent field ex (packed_velocity) for the exponent field e.
-__host__ __device__ __forceinline__ i64 vel_at(i64 u, int ex, int e) { return fx::shr(u, 2 + e - ex); }
+__host__ __device__ __forceinline__ i64 vel_at(i64 u, int ex, int e) { return fx::shr(u, 1 + e - ex); }
 // From the difference across the face and the two cells' tangential differences.
 __host__ __device__ __forceinline__ FxStress tan_stress(const FxN& C, FxA du, const FxN& D, FxA gn) {
   const int ec = du.e - C.s, ed = gn.e - D.s, e = ec > ed ? ec : ed;

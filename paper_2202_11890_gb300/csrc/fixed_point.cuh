@@ -72,7 +72,7 @@ __host__ __device__ __forceinline__ u32 mulhi_u(u32 a, u32 b) {
 }
 
 // A multiplicand: x = hi 2^32 + lo with lo signed, so that every partial
-// product is one signed 32 x 32 -> 64-bit multiply-add.
+// product is one signed 32 x 32 -> 64-bit multiply-add. x < 2^63 - 2^31.
 __host__ __device__ __forceinline__ FxW split(i64 x) {
   FxW w;
   w.lo = (int)x;
@@ -187,9 +187,10 @@ __host__ __device__ __forceinline__ i64 pack(i64 bits) {
 __host__ __device__ __forceinline__ int pack_exp(i64 w) { return (int)w & 1023; }
 __host__ __device__ __forceinline__ i64 shr(i64 x, int s) { return x >> (s < 63 ? s : 63); }
 __host__ __device__ __forceinline__ i64 unpack(i64 w, int e) { return shr(w & ~1023ll, 4 + e - pack_exp(w)); }
-// The velocity of a cell, .59 of 2^(its momentum's exponent - 1023), from the
-// packed momentum and 1/rho .61.
-__host__ __device__ __forceinline__ i64 packed_velocity(i64 w, FxW inv) { return mul(split(w & ~1023ll), inv); }
+// The velocity of a cell, .58 of 2^(its momentum's exponent - 1023), from the
+// packed momentum and 1/rho .61. Halved, because split's carry needs |x| below
+// 2^63 - 2^31, which a mantissa of 31 leading ones exceeds.
+__host__ __device__ __forceinline__ i64 packed_velocity(i64 w, FxW inv) { return mul(split((w & ~1023ll) >> 1), inv); }
 
 // A double of a cell state within the bounds above, as an integer of scale
 // s (truncated toward zero; exact when its last bit is at least 2^-s).

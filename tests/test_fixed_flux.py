@@ -37,6 +37,10 @@ void prim(const i64* in, i64* o) {  // in: a, b, c, d; rho .60; x .61; the bits 
   o[4] = fx::from_double(in[6], 60);
   o[5] = fx::to_double(in[0], 59);
 }
+void velocity(const i64* in, i64* o) {  // the bits of a momentum, rho .60; for the exponent field in[2]
+  const i64 w = fx::pack(in[0]);
+  o[0] = vel_at(fx::packed_velocity(w, fx::split(fx::recip(in[1]))), fx::pack_exp(w), (int)in[2]);
+}
 void tangent(const i64* in, i64* o) {  // in: bits of L2, L1, R1, R2; us, lr; V, its e; C, its shift; x, its e
   i64 w[4];
   for (int j = 0; j < 4; j++) w[j] = fx::pack(in[j]);
@@ -120,7 +124,32 @@ def test_primitives_within_their_bounds(lib):
         assert abs(value(o[5]) * 2 ** 59 - a) <= abs(Fr(a)) / 2 ** 53
 
 
-def test_tangential_flux_follows_the_momenta(lib):
+# mantissas at the ends of their words: the carries of split, pack and unpack
+ENDS = [0, 1, 2 ** 52 - 1, 2 ** 52 - 2, 2 ** 51, 2 ** 21, 2 ** 21 - 1, 2 ** 20, 2 ** 22 - 1, 2 ** 52 - 2 ** 21,
+        2 ** 52 - 2 ** 20, 2 ** 52 - 2 ** 22, 2 ** 53 - 2 ** 31 & (2 ** 52 - 1)]
+
+
+def from_parts(mantissa, exponent, negative):
+    x = float(np.int64(exponent << 52 | mantissa).view(np.float64))
+    return -x if negative else x
+
+
+@pytest.mark.parametrize("ends", [True, False])
+def test_velocity_of_any_mantissa(lib, ends):
+    """m / rho under m's exponent, .57: the product's 3/4 of a unit at twice that
+    resolution, the cut to .57, and 1/rho within 2^-56."""
+    rng = random.Random(13)
+    for n in range(4000):
+        man = rng.choice(ENDS) if ends else rng.getrandbits(52)
+        e = rng.choice([1, 2, 500, 1000, 1020, 1021, rng.randint(1, 1021)])
+        m, rho = from_parts(man, e, rng.random() < 0.5), int(rng.uniform(0.5, 4.0) * 2 ** 60)
+        o, = call(lib.velocity, [bits(m), rho, e], n=1)
+        exact = Fr(m) / (Fr(rho) / 2 ** 60) * Fr(2) ** (57 - e + 1023)
+        assert abs(o - exact) <= Fr(3, 2) + abs(exact) / 2 ** 56, (m, rho)
+
+
+@pytest.mark.parametrize("ends", [True, False])
+def test_tangential_flux_follows_the_momenta(lib, ends):
     """Momenta of every size down to 1e-300, zeros and neighbours of other sizes
     among them. Units of 2^-55 of the largest one's power of two: the pair of
     products 1; each momentum cut at 2^-58 with weights up to 3/2 of u_L + u_R
@@ -131,6 +160,10 @@ def test_tangential_flux_follows_the_momenta(lib):
         scale = 2.0 ** -rng.choice([0, 1, 7, 20, 33, 60, 200, 900])
         m = [rng.choice([rng.uniform(-0.65, 0.65), rng.uniform(-0.65, 0.65) * 2.0 ** -rng.randint(0, 70), 0.0]) * scale
              for _ in range(4)]
+        if ends:
+            top = max(bits(scale) >> 52, 4) - 2
+            m = [from_parts(rng.choice(ENDS), max(top - rng.choice([0, 0, 1, 5, 31, 60]), 1), rng.random() < 0.5)
+                 for _ in range(4)]
         us, lr = int(rng.uniform(-3.66, 3.66) * 2 ** 59), int(rng.uniform(0.5, 5.64) * 2 ** 59)
         big = max(map(abs, m))
         em = max((bits(abs(x)) >> 52) for x in m)

@@ -14,8 +14,8 @@ import pytest
 
 from oracle import oracle as O
 from paper_2202_11890_gb300 import workloads as W
-from pairs import oracle_threads, pair
-from test_gpu_3d import gpu_rhs3, pair3
+from pairs import oracle_threads, pair, rel_err
+from test_gpu_3d import gpu_rhs3, pair3, rel3
 from test_gpu_parity import gpu_rhs
 
 pytestmark = pytest.mark.gpu
@@ -199,3 +199,34 @@ def test_rhs3_as_accurate_as_double(kind, amp, wall):
         errors[0].append(gpu_rhs3(cfg, q) - true)
         errors[1].append(O.rhs3(P, q) - true)
     compare(*errors)
+
+
+def end_mantissas(shape, rng):
+    """Momenta of one to 2^-12 of 0.3 whose mantissas are at the ends of their
+    words: all ones, 31 or 32 leading ones, one bit at the words' border."""
+    man = np.array([0, 1, 2 ** 52 - 1, 2 ** 52 - 2, 2 ** 52 - 2 ** 21, 2 ** 52 - 2 ** 20, 2 ** 52 - 2 ** 22, 2 ** 31,
+                    2 ** 21 - 1, 2 ** 32 - 1], np.uint64)
+    e = rng.integers(1009, 1022, shape).astype(np.uint64)
+    x = (rng.choice(man, shape) | e << np.uint64(52)).view(np.float64)
+    return np.where(rng.random(shape) < 0.5, -x, x)
+
+
+def test_momenta_with_mantissas_at_the_ends_of_words():
+    """Against the oracle to the parity norm, 1e-12 of the largest |R|."""
+    rng = np.random.default_rng(61)
+    rho, p = W.rest_primitives(GRID)
+    q = W.conserved(rho, 0 * rho, 0 * rho, p)
+    q[1], q[2] = end_mantissas(rho.shape, rng), end_mantissas(rho.shape, rng)
+    q[3] += 0.5 * (q[1] ** 2 + q[2] ** 2) / rho
+    cfg, P, _ = pair(GRID, 2, dt=0.001)
+    err = rel_err(gpu_rhs(cfg, q), O.rhs(P, q))
+    assert np.all(err < 1e-12), err
+    shape = (GRID3.nz, GRID3.ny, GRID3.nx)
+    rho, p = (np.broadcast_to(f[:, None, :], shape) for f in W.rest_primitives(GRID3.column_grid()))
+    q = W.conserved3(rho, 0 * rho, 0 * rho, 0 * rho, p)
+    for c in (1, 2, 3):
+        q[c] = end_mantissas(shape, rng)
+        q[4] += 0.5 * q[c] ** 2 / rho
+    cfg, P, _ = pair3(GRID3, 2, dt=0.001)
+    err = rel3(gpu_rhs3(cfg, q), O.rhs3(P, q))
+    assert np.all(err < 1e-12), err
